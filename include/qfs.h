@@ -138,10 +138,11 @@ const char* qfs_last_error(void);
 int qfs_device_sms(const qfs_ctx* ctx);
 
 /* Context options (none of them is in the paper; defaults in brackets).
- *   QFS_OPT_WAIT_LIMIT [2^25]: polls (each >= 32 ns) a dependency wait of
- *     the dataflow sweep makes before it gives up; the kernel then sets the
- *     run's error word, every CTA stops taking work and returns, and the call
- *     returns QFS_ETIMEOUT.  The context stays usable; the next call clears
+ *   QFS_OPT_WAIT_LIMIT [2^25]: polls a wait of a whole-sweep launch makes (the
+ *     dataflow sweep for a start's previous step, each poll >= 32 ns; the
+ *     cluster sweep for the environments of the other CTAs) before it gives
+ *     up; the kernel then sets the run's error word, its CTAs return, and the
+ *     call returns QFS_ETIMEOUT.  The context stays usable; the next call clears
  *     the error word.  Must be >= 1.
  *   QFS_OPT_WORKSPACE_CAP [0 = none]: largest device workspace, in bytes, a
  *     call may use; a call that needs more returns QFS_ENOMEM before it
@@ -149,8 +150,9 @@ int qfs_device_sms(const qfs_ctx* ctx);
  *     out-of-memory error, Appendix A).
  *   QFS_OPT_FUSED_UPDATE [1]: per-step sweeps run each gate update in the
  *     backward launch (0: a separate update launch).
- *   QFS_OPT_DATAFLOW [1]: a sweep of all starts is one persistent launch
- *     (0: per-step launches).
+ *   QFS_OPT_DATAFLOW [1]: a sweep of all starts is one launch: the cluster
+ *     sweep where a start's state fits on chip, else the dataflow sweep (0:
+ *     per-step launches).
  *   QFS_OPT_TWO_GATE_FORWARD [1]: the dataflow sweep applies consecutive
  *     forward gates on four distinct qubits in one step (0: one per step).
  *   QFS_OPT_FP64_TARGET_PRODUCT [0]: QFS_MIXED runs form U Psi in FP64

@@ -233,7 +233,10 @@ void prof_harvest(qfs_ctx* ctx) {
 // (plateau, validation) is needed: a launch behind a sweep that met the
 // tolerance returns at once (device stop flag), so the run ends at the same
 // sweep as with one launch per round trip.
-constexpr int kSweepBatch = 4;
+constexpr int kSweepBatch = 64;  // sweeps per host round trip, at most (room for their costs): one launch of
+                                 // the cluster sweep with one CTA per start
+constexpr int kClBatch = 16;     // ... of the cluster sweep, a launch each
+constexpr int kDfBatch = 4;      // ... of the dataflow sweep
 
 // Device buffers of one run, carved from the context's workspace.
 struct Run {
@@ -293,6 +296,13 @@ struct Run {
   int df_nsteps = 0;
   long long df_items = 0;
   double df_bytes = 0.0;    // algorithmic bytes of one dataflow sweep (all starts)
+  ClPlan cl;                // cluster sweep (C = 0: the dataflow or per-step sweep)
+  int4* cl_scale = nullptr;      // per slot: the scales of its fixed-point sweeps (FP64)
+  unsigned* cl_acc = nullptr;
+  double* cl_parts = nullptr;
+  bool cl_check = false;         // checks of training states in one launch
+  bool cl_fx = false;            // fixed-point sweeps or checks: the scales are wanted
+  std::vector<char> cl_plain;    // per slot: its sweeps take the plain FP64 form
   const void* df_key[4] = {};  // what the uploaded table was built for
   int df_key_r = -1;
 };
@@ -331,6 +341,11 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
   R.active = (int*)take((size_t)R.S * sizeof(int));
   R.counters = (unsigned*)take((size_t)(R.S + 1) * sizeof(unsigned));
   R.flag = (int*)take(sizeof(int) * 4);
+  if (R.cl_fx) {
+    R.cl_scale = (int4*)take((size_t)R.T * sizeof(int4));
+    R.cl_acc = (unsigned*)take(5 * sizeof(unsigned));  // (the last: the check's finished columns)
+    R.cl_parts = (double*)take((size_t)R.M * sizeof(double));
+  }
   R.err = R.flag ? R.flag + 1 : nullptr;
   R.envs = need_envs ? (double2*)take((size_t)R.S * R.L * 16 * sizeof(double2)) : nullptr;
   R.df_steps = (DfStep*)take((size_t)std::max(R.df_cap, 1) * sizeof(DfStep));
@@ -420,6 +435,10 @@ int ensure_pinned(qfs_ctx* ctx, size_t n) {
 bool df_usable(const qfs_ctx* ctx, const Run& R, Real r) {
   return ctx->dataflow && ctx->coop && (r == R64 || R.M % 2 == 0) && df_blocks_per_sm(r) > 0;
 }
+
+// Whole-sweep launches: the cluster sweep where a start's state fits on chip,
+// else the dataflow sweep.  (A dataflow trace needs the dataflow sweep.)
+bool whole_usable(const qfs_ctx* ctx, const Run& R, Real r) { return R.cl.C > 0 || df_usable(ctx, R, r); }
 
 // The step table of one sweep (the same steps, in the same order, as
 // sweep()), chunked so that each step offers about two items per resident
@@ -593,9 +612,16 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   R.df_cap = 0;
   R.df_max_nchunk = 0;
   R.df_key_r = -1;
+  R.cl = ClPlan{};
+  if (ctx->dataflow && ctx->coop && !ctx->df_trace)
+    R.cl = cl_plan(prec == QFS_MIXED ? R32 : R64, R.n, M, R.L, S_target, beta != 0.0);
+  R.cl_plain.assign(T, 0);
+  // FP64 cluster sweeps, and the FP64 checks of complex64 runs.
+  R.cl_check = prec == QFS_MIXED && ctx->dataflow && cl_check_fits(R.n, R.L);
+  R.cl_fx = R.cl_check || (R.cl.C > 0 && prec == QFS_FP64);
   {
     const Real rs = prec == QFS_MIXED ? R32 : R64;
-    if (df_usable(ctx, R, rs)) {
+    if (R.cl.C == 0 && df_usable(ctx, R, rs)) {
       std::vector<DfStep> steps;
       double b = 0.0;
       df_build(ctx, R, rs, nullptr, nullptr, nullptr, nullptr, nullptr, steps, &b);
@@ -670,10 +696,18 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     launch_set_identity4(R.vprev + go, (long long)R.spt * R.L, st);
   }
+  int4 sc{0, 0, 0, 0};
+  if (R.cl_scale) {
+    ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
+    CK(cudaMemsetAsync(R.cl_acc + 4, 0, sizeof(unsigned), st));
+    launch_cl_scale(R.n, R.M, R.spt * R.L, R.psi64 + so, R.phil64 + so, R.g64 + go, R.cl_acc, R.cl_scale + t, st);
+    CK(cudaMemcpyAsync(&sc, R.cl_scale + t, sizeof(int4), cudaMemcpyDeviceToHost, st));
+  }
   int flag = 0;
   CK(cudaMemcpyAsync(&flag, R.flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   prof_harvest(ctx);
+  R.cl_plain[t] = sc.x != 0;
   if (flag) return fail(QFS_ENONFINITE, "NaN or Inf in the target, samples or initial gates");
   return QFS_OK;
 }
@@ -882,12 +916,94 @@ int df_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, do
   return QFS_OK;
 }
 
+// The row bits of every gate's qubits.
+void cl_positions(const Run& R, ClArgs& a) {
+  for (int k = 0; k < R.L; ++k) {
+    const Geom g = make_geom(R.n, R.M, R.pairs[2 * k], R.pairs[2 * k + 1]);
+    a.pos[k] = (unsigned char)(g.pos_a | g.pos_b << 4);
+  }
+}
+
+// nsweeps sweeps (sweep0, sweep0 + 1, ... of the batch) by the cluster sweep.
+int cl_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, double2* envs, const int* active,
+             cudaStream_t st, int* stop = nullptr, double stop_tol = -1.0, double* cost_rows = nullptr,
+             double resid_skip = 0.0, int sweep0 = 0, int nsweeps = 1) {
+  ClArgs a{};
+  a.n = R.n;
+  a.M = R.M;
+  a.L = R.L;
+  a.S = R.S;
+  a.spt = std::max(R.spt, 1);
+  a.psi = psi;
+  a.phil = phil;
+  a.g64 = R.g64;
+  a.g32 = R.g32;
+  a.blist = R.B;
+  a.blast = R.phi;
+  a.envs = envs;
+  a.active = active;
+  a.costs = R.costs;
+  a.cost_rows = cost_rows;
+  a.beta = R.beta;
+  a.inv_M = 1.0 / R.M;
+  a.resid_skip = r == R32 ? resid_skip : 0.0;
+  a.stop = stop;
+  a.stop_tol = stop_tol;
+  a.sweep0 = sweep0;
+  a.nsweeps = nsweeps;
+  a.err = R.err;
+  a.wait_limit = ctx->df_wait_limit;
+  cl_positions(R, a);
+  // B list written and read back, Psi and U Psi read.
+  const double bytes = (2.0 * R.L + 2.0) * R.S * (double)R.sN * elem_bytes(r) * nsweeps;
+  a.scale = r == R64 ? R.cl_scale : nullptr;
+  // FP64: the slots whose inputs allow it sweep in fixed point, the others in
+  // plain FP64.
+  bool plain = r == R32, fixed = false;
+  if (r == R64)
+    for (char c : R.cl_plain) (c ? plain : fixed) = true;
+  ProfScope ps(ctx, QFS_PROF_DATAFLOW, bytes, st);
+  if (fixed) CK(launch_sweep_cl(r, R.cl, a, true, st));
+  if (plain) CK(launch_sweep_cl(r, R.cl, a, false, st));
+  return QFS_OK;
+}
+
+// One whole-sweep launch without a batch.
+int whole_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, double2* envs, const int* active,
+                double2* vprev, cudaStream_t st, double resid_skip = 0.0) {
+  if (R.cl.C > 0) return cl_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, -1.0, nullptr, resid_skip);
+  return df_sweep(ctx, R, r, psi, phil, envs, active, vprev, st, nullptr, 0.0, nullptr, resid_skip);
+}
+
 // FP64 sample cost of start s's master gates on states psi with
 // phil = U psi: (1/M) ||phil - C psi||^2 (the training states by default).
 int check64(qfs_ctx* ctx, Run& R, int s, double* out, const double2* psi = nullptr,
             const double2* phil = nullptr) {
   cudaStream_t st = ctx->stream;
   const double2* g = R.g64 + (size_t)s * R.L * 16;
+  if (!psi && R.cl_check && !R.cl_plain[s / R.spt]) {
+    const int t = s / R.spt;
+    ClArgs a{};
+    a.n = R.n;
+    a.M = R.M;
+    a.L = R.L;
+    a.psi = R.psi64 + (size_t)t * R.sN;
+    a.phil = R.phil64 + (size_t)t * R.sN;
+    a.g64 = const_cast<double2*>(g);
+    a.costs = R.cost64r;
+    a.inv_M = 1.0 / R.M;
+    a.scale = R.cl_scale + t;
+    cl_positions(R, a);
+    {
+      ProfScope ps(ctx, QFS_PROF_CHECK, 2.0 * R.sN * sizeof(double2));
+      CK(launch_cl_check(a, R.cl_parts, R.cl_acc + 4, st));
+    }
+    CK(cudaMemcpyAsync(ctx->h_pinned, R.cost64r, sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    prof_harvest(ctx);
+    *out = ctx->h_pinned[0];
+    return QFS_OK;
+  }
   if (!psi) psi = R.psi64 + (size_t)(s / R.spt) * R.sN;
   if (!phil) phil = R.phil64 + (size_t)(s / R.spt) * R.sN;
   const void* in = psi;
@@ -1075,11 +1191,12 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
   std::vector<Outcome> cur(T);
   int left = T;
   SweepGraph graph;
-  const bool df = df_usable(ctx, R, rs);
+  const bool df = whole_usable(ctx, R, rs);
   if (!df) TRY(capture_sweep(ctx, R, rs, psi, phil, graph));
   // Without plateau detection or validation the host decides nothing until
   // some start meets the tolerance, so sweeps go out in batches.
   const bool batch = df && p->plateau_window == 0 && !R.validate;
+  const bool cl_many = R.cl.C == 1 && rs == R64 && T == 1;
   int* stop = R.flag + 2;
   // Complex64 sweeps skip the residual pass of starts whose update-time
   // estimate (error ~1e-7) is far above tol; plateau detection needs every
@@ -1092,12 +1209,26 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
       int room = p->max_sweeps;
       for (int t = 0; t < T; ++t)
         if (busy[t]) room = std::min(room, p->max_sweeps - tsweeps[t]);
-      const int B = batch ? std::max(1, std::min(kSweepBatch, room)) : 1;
+      const int B = batch ? std::max(1, std::min(R.cl.C > 0 ? (cl_many ? kSweepBatch : kClBatch) : kDfBatch, room)) : 1;
       if (df && B > 1) {
-        CK(cudaMemsetAsync(stop, 0, sizeof(int), st));
-        for (int b = 0; b < B; ++b)
-          TRY(df_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, stop, ctol,
-                       R.cost_rows + (size_t)b * S, skip));
+        int per = 1;  // sweeps per launch
+        CK(cudaMemsetAsync(stop, R.cl.C > 0 ? 0x7f : 0, sizeof(int), st));
+        if (R.cl.C > 0) {
+          // FP64 and one target: the run ends at the sweep that meets the
+          // tolerance, so one launch takes the batch and a start that meets
+          // it stops there.  Complex64 runs may go on from that sweep (the
+          // FP64 check decides), so every start has to stand at it.
+          // (One CTA per start only: there the stop word can be looked at
+          // between sweeps, so the other starts end with it.)
+          per = cl_many ? B : 1;
+          for (int b = 0; b < B; b += per)
+            TRY(cl_sweep(ctx, R, rs, psi, phil, nullptr, R.active, st, stop, ctol, R.cost_rows + (size_t)b * S, skip, b,
+                         per));
+        } else {
+          for (int b = 0; b < B; ++b)
+            TRY(df_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, stop, ctol,
+                         R.cost_rows + (size_t)b * S, skip));
+        }
         TRY(read_rows(ctx, R.cost_rows, S, B, rows, R.err));
         // The sweep whose cost met the tolerance ends the batch; the
         // launches behind it returned at once.
@@ -1110,11 +1241,11 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
             break;
           }
         }
-        prof_drop_dataflow(ctx, B - nrows);
+        if (per == 1) prof_drop_dataflow(ctx, B - nrows);
         prof_harvest(ctx);
       } else {
         if (df) {
-          TRY(df_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, nullptr, 0.0, nullptr, skip));
+          TRY(whole_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, skip));
         } else {
           CK(cudaGraphLaunch(graph.exec, st));
           for (int i = 0; i < QFS_PROF_KINDS; ++i) ctx->prof.launches[i] += graph.launches[i];
@@ -1798,8 +1929,8 @@ int qfs_sweep_once(qfs_ctx* ctx, const qfs_circuit* circuit, const double* targe
   const Real rs = precision == QFS_MIXED ? R32 : R64;
   const void* psi = rs == R32 ? (const void*)R.psi32 : (const void*)R.psi64;
   const void* phil = rs == R32 ? (const void*)R.phil32 : (const void*)R.phil64;
-  if (df_usable(ctx, R, rs))
-    TRY(df_sweep(ctx, R, rs, psi, phil, R.envs, nullptr, nullptr, st));
+  if (whole_usable(ctx, R, rs))
+    TRY(whole_sweep(ctx, R, rs, psi, phil, R.envs, nullptr, nullptr, st));
   else
     TRY(sweep(ctx, R, rs, Slice{0, S, S, ctx->stream}, R.g64, R.g32, psi, phil, R.B, R.phi, R.partials,
               R.nblk_max, R.costs, R.envs, nullptr, R.stream_b, nullptr, R.counters));

@@ -132,6 +132,53 @@ int df_blocks_per_sm(Real r);
 cudaError_t launch_sweep_df(Real r, const DfArgs& a, int num_sms, cudaStream_t st);
 void df_chunking(DfStep& st, double bytes_per_unit, double target);
 
+// Cluster sweep (sweep_cl.cu): one thread-block cluster per start, its state
+// in shared memory for the whole sweep.
+constexpr int kClMaxGates = 128;
+struct ClArgs {
+  int n, M, L, S, spt;                  // spt: starts per target
+  int C, e_head, e_shift;               // of the plan (set by the launch)
+  const void* psi; const void* phil;    // per target N x M, in the sweep precision
+  double2* g64; float2* g32;            // S x L x 16 (g32: complex64 sweeps)
+  void* blist;                          // (L - 1) x S x N x M, B_0 .. B_{L-2} in the kernel's own order
+  void* blast;                          // S x N x M: B_{L-1} (complex64 sweeps)
+  double2* envs;                        // nullable: S x L x 16
+  const int* active;                    // nullable
+  double* costs;                        // S: each start's last cost
+  double* cost_rows;                    // nullable: nsweeps x S
+  double beta, inv_M;
+  double resid_skip;                    // as DfArgs
+  int* stop;                            // nullable: the lowest sweep (from sweep0 on) after which a start's cost was
+  double stop_tol;                      //   <= stop_tol; a launch that finds one below its sweep0 returns at once
+  int sweep0, nsweeps;                  // sweeps of this launch; several need C = 1 (a start ends with the sweep in
+                                        // which it or, seen in between, another met stop_tol)
+  int* err; long long wait_limit;       // as DfArgs: polls of an exchange before the kernel gives up
+  const int4* scale;                    // FP64: per target {1: the plain FP64 form, exponents of the column norms
+                                        //   of Psi and U Psi, 0} (launch_cl_scale); null: plain
+  unsigned char pos[kClMaxGates];       // per gate: row bits of its qubits, a | b << 4
+};
+struct ClPlan {
+  int C = 0;                            // CTAs per start; 0: the state does not fit
+  int threads = 0;
+  size_t smem = 0;
+  int e_head = 0, e_shift = 0;          // fixed point: bits of headroom in Psi's scale, shift of E before the
+                                        //   CTAs' sums are added
+};
+// The cluster shape for starts of one target (never of several, so that a
+// target's sums do not depend on what sweeps beside it).
+ClPlan cl_plan(Real r, int n, int M, int L, int spt, bool keep64);
+// fx: the fixed-point form of FP64 sweeps.  Each form takes the targets whose
+// scale says so and leaves the others.
+cudaError_t launch_sweep_cl(Real r, const ClPlan& p, const ClArgs& a, bool fx, cudaStream_t st);
+// (1/M) ||U Psi - C Psi||^2 of the gates a.g64 (one start) on a.psi, a.phil
+// (FP64) with a.scale[0], which must not say plain, into a.costs[0].  parts: M
+// doubles of scratch; count: a word that is zero between launches.
+bool cl_check_fits(int n, int L);
+cudaError_t launch_cl_check(const ClArgs& a, double* parts, unsigned* count, cudaStream_t st);
+// acc: 4 words of scratch.
+void launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
+                     int4* out, cudaStream_t st);
+
 // Set `count` 4x4 complex128 matrices to the identity.
 void launch_set_identity4(double2* v, long long count, cudaStream_t st);
 
