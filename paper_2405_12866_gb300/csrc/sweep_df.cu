@@ -21,7 +21,7 @@
 // back through L2 (ld.global.cg), never from a possibly stale L1 line.
 // Every wait is bounded: when one runs out the CTA sets the run's error word
 // and every CTA stops taking items; the host reports QFS_ETIMEOUT.
-#include "polar4.cuh"
+#include "polar_newton.cuh"
 #include "qfs_common.cuh"
 #include "qfs_kernels.h"
 
@@ -76,25 +76,12 @@ __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
 }
 __device__ __forceinline__ int ld_volatile_i32(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
-// Scratch of the CTA-wide gate update (4x4 matrices in the lane layout
-// M[r][c] at 4c + r).
-struct DfUpd {
-  double2 A[16];             // A = E^dagger scaled by a power of two
-  double2 Q[2][16];          // iterate (double buffer)
-  double2 T[16];             // products
-  double2 X[16];             // the correction factor of the polish step
-  float2 V[16];              // right singular vectors (FP32 Jacobi)
-  float sig[16];             // singular value of column (lane >> 2)
-  int ok;
-};
-
 template <typename T>
 struct DfShared {
   typename C2<T>::t gs[16];
   typename C2<T>::t gs2[16];  // the second gate of a two-gate forward step
   double red[kDfMaxWarps][32];
-  double2 polar[32];
-  DfUpd u;
+  NewtonSh nw;
   long long item;
   int flag;
 };
@@ -600,172 +587,33 @@ __device__ void df_backward_gen(const DfStep& st, int s, int c, DfShared<T>& sh,
   }
 }
 
-// C = op(X) Y for 4x4 complex matrices in shared memory (lane layout),
-// op(X) = X^dagger when AH, by all 128 threads of the CTA.  FP64 arithmetic
-// issues at a fixed cost per warp instruction on this GPU whatever the
-// number of active lanes, so the 256 real products are packed two per
-// thread over four warps (one per SM sub-partition): thread t forms the real
-// (t even) or imaginary part of X[r][k] Y[k][c] for entry t/8, k = (t/2)%4,
-// and the k terms are summed by two shuffles.  POST = 1 stores
-// 1.5 I - 0.5 C instead (the Newton-Schulz factor).  The caller
-// synchronises before and after.
-template <bool AH, int POST>
-__device__ __forceinline__ void mm64_cta(const double2* X, const double2* Y, double2* C) {
-  const int t = threadIdx.x;
-  if (t >= 128) return;  // four warps take part
-  const int e = t >> 3, k = (t >> 1) & 3, part = t & 1;
-  const int r = e & 3, c = e >> 2;
-  double2 x = AH ? X[4 * r + k] : X[4 * k + r];
-  if (AH) x.y = -x.y;
-  const double2 y = Y[4 * c + k];
-  double v = part ? fma(x.x, y.y, x.y * y.x) : fma(x.x, y.x, -(x.y * y.y));
-  v += __shfl_xor_sync(FULL, v, 2);
-  v += __shfl_xor_sync(FULL, v, 4);
-  if (k == 0) {
-    if (POST == 1) v = fma(-0.5, v, (part == 0 && r == c) ? 1.5 : 0.0);
-    reinterpret_cast<double*>(C + e)[part] = v;
-  }
-}
-
-// FP32 part of the update on warp 0 (as in warp_polar4_fast): scale A by an
-// exact power of two, one-sided Jacobi on A V0, Q0 = W V^H.  Leaves the
-// scaled A, Q0 (promoted), V and the singular values in u; returns false
-// when A is zero or too ill-conditioned for the fast path.
-__device__ __forceinline__ bool df_polar_begin(double2 a, double2 v0, DfUpd& u) {
-  const int lane = threadIdx.x & 31;
-  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2;
-  const bool isV = lane >= 16;
-  int e = 0;
-  if (!isV) {
-    const int ex = (__double2hiint(a.x) >> 20) & 0x7ff, ey = (__double2hiint(a.y) >> 20) & 0x7ff;
-    e = max(ex, ey);
-  }
-  e = __reduce_max_sync(FULL, e);
-  if (e == 0) return false;
-  const double sc = __hiloint2double((2046 - e) << 20, 0);
-  const double2 as{a.x * sc, a.y * sc};
-  if (!isV) u.A[l16] = as;
-  const float2 a32{(float)as.x, (float)as.y};
-  const float2 v032{(float)v0.x, (float)v0.y};
-  float2 x;
-  {
-    float2 acc{0.f, 0.f};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 ak = shfl_c(a32, 4 * k + row), vk = shfl_c(v032, 16 + 4 * col + k);
-      acc = cfma(ak, vk, acc);
-    }
-    x = isV ? v032 : acc;
-  }
-  x = jacobi32_sweeps(x);
-  float2 w = shfl_c(x, l16);
-  const float2 v = shfl_c(x, 16 + l16);
-  float nrm = w.x * w.x + w.y * w.y;
-  nrm += __shfl_xor_sync(FULL, nrm, 1);
-  nrm += __shfl_xor_sync(FULL, nrm, 2);
-  float smax = nrm, smin = nrm;
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 4));
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 8));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 4));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 8));
-  if (!(smin > 1e-6f * smax)) return false;
-  const float inv = rsqrtf(nrm);
-  const float sig = nrm * inv;
-  w = float2{w.x * inv, w.y * inv};
-  const float2 q32 = mm_bh(w, v, row, col);
-  if (!isV) {
-    u.Q[0][l16] = double2{(double)q32.x, (double)q32.y};
-    u.V[l16] = v;
-    u.sig[l16] = sig;
-  }
-  return true;
-}
-
-// The update of gate k for start s by the whole CTA: the same mathematics as
-// polar_update_warp / update_from_sum (FP32 Jacobi, two FP64 Newton-Schulz
-// steps, POLISH skew-Hermitian corrections), with the FP64 products spread
-// over the four warps.  Warp 0 holds the summed environment value v (lane j
-// = value j of E) and, in lanes 16..31, the Jacobi start v0 (the gate's V
-// from its previous update, or the identity), loaded by the caller before
-// the partial sums so that its latency is off the chain.  All threads call
-// it.
-template <typename T, int POLISH>
-__device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, double v, double2 v0) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2;
-  DfUpd& u = sh.u;
-  double2* vio = ua.vprev ? ua.vprev + s * ua.g_stride : nullptr;
+// The update of gate k for start s by warp 0 (polar_newton.cuh) from the summed
+// environment, whose value j is in lane j: hi + lo (complex64 sweeps) or e.
+template <typename T>
+__device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, float hi, float lo, double e) {
+  constexpr bool F32 = sizeof(T) == 4;
+  const int lane = threadIdx.x & 31, l16 = lane & 15, at = 4 * (l16 & 3) + (l16 >> 2);
   double2* g64 = ua.g64 + s * ua.g_stride;
-  double2 e{0.0, 0.0}, a{0.0, 0.0};
-  if (warp == 0) {
-    e = double2{__shfl_sync(FULL, v, 2 * l16), __shfl_sync(FULL, v, 2 * l16 + 1)};
-    if (ua.env_out && lane < 16) ua.env_out[s * ua.env_stride + l16] = e;
-    double2 m = e;
-    if (ua.beta != 0.0 && lane < 16) {
-      const double2 go = g64[4 * row + col];
-      m = double2{(1.0 - ua.beta) * m.x + ua.beta * go.x, (1.0 - ua.beta) * m.y - ua.beta * go.y};
-    }
-    a = double2{m.x, -m.y};
-    const bool ok = df_polar_begin(a, v0, u);
-    if (lane == 0) u.ok = ok ? 1 : 0;
+  const bool damp = ua.beta != 0.0;
+  auto env = [&]() { return newton_env(F32 ? (double)hi + (double)lo : e); };
+  auto matrix = [&]() { return damp ? newton_damp(env(), ua.beta, g64) : env(); };
+  const float2 a32 = F32 && !damp ? newton_input32(hi) : newton_input64(matrix(), sh.nw);
+  long long q;
+  const double2 p = newton_update<!F32>(a32, sh.nw, newton_pair(), q) ? newton_entry64(q) : newton_fallback(matrix(), sh.nw);
+  if (lane < 16) {
+    g64[at] = p;
+    if (ua.g32) (ua.g32 + s * ua.g_stride)[at] = float2{(float)p.x, (float)p.y};
   }
-  __syncthreads();
-  bool ok = u.ok != 0;
-  int cur = 0;
-  if (ok) {
-#pragma unroll 1
-    for (int it = 0; it < 2; ++it) {
-      mm64_cta<true, 1>(u.Q[cur], u.Q[cur], u.T);  // T = (3I - Q^H Q) / 2
-      __syncthreads();
-      mm64_cta<false, 0>(u.Q[cur], u.T, u.Q[cur ^ 1]);
-      __syncthreads();
-      cur ^= 1;
-    }
-#pragma unroll 1
-    for (int it = 0; it < POLISH; ++it) {
-      mm64_cta<true, 0>(u.Q[cur], u.A, u.T);  // B = Q^H A
-      __syncthreads();
-      if (warp == 0) {
-        const double2 bm = u.T[l16];
-        const double2 bt = u.T[4 * row + col];  // B[col][row]
-        const float2 k32{0.5f * (float)(bm.x - bt.x), 0.5f * (float)(bm.y + bt.y)};
-        const float2 om = skew_correction(k32, u.V[l16], u.sig[l16], row, col);
-        const float big = max_abs16(om);
-        const int good = it > 0 || big < 1e-3f ? 1 : 0;
-        const double2 xc = exp_skew3(om, big, row, col);
-        if (lane < 16) u.X[l16] = xc;
-        if (lane == 0) u.ok = good;
-      }
-      __syncthreads();
-      if (!u.ok) {
-        ok = false;
-        break;
-      }
-      mm64_cta<false, 0>(u.Q[cur], u.X, u.Q[cur ^ 1]);
-      __syncthreads();
-      cur ^= 1;
-    }
+  if (ua.env_out) {
+    const double2 m = env();
+    if (lane < 16) ua.env_out[s * ua.env_stride + l16] = m;
   }
-  if (warp == 0) {
-    double2 p;
-    if (ok) {
-      p = u.Q[cur][l16];
-      if (vio && lane < 16) vio[l16] = double2{(double)u.V[l16].x, (double)u.V[l16].y};
-    } else {
-      // Zero, ill-conditioned or not converging: the FP64 Jacobi (which
-      // also completes rank-deficient cases), from the identity.
-      p = warp_polar4(a, double2{row == col ? 1.0 : 0.0, 0.0}, sh.polar, vio);
-    }
-    if (lane < 16) {
-      g64[4 * row + col] = p;
-      if (ua.g32) (ua.g32 + s * ua.g_stride)[4 * row + col] = float2{(float)p.x, (float)p.y};
-    }
-    if (ua.cost_out) {
-      double t = lane < 16 ? (p.x * e.x - p.y * e.y) : 0.0;
+  if (ua.cost_out) {
+    const double2 m = env();
+    double t = lane < 16 ? (p.x * m.x - p.y * m.y) : 0.0;
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-      if (lane == 0) ua.cost_out[s] = 2.0 - 2.0 * ua.inv_M * t;
-    }
+    for (int o = 16; o >= 1; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+    if (lane == 0) ua.cost_out[s] = 2.0 - 2.0 * ua.inv_M * t;
   }
 }
 
@@ -884,10 +732,10 @@ __global__ void __launch_bounds__(df_threads<T>(), 1) k_sweep_df(DfArgs a) {
             }
           }
         } else {
-          // The Jacobi start of the update, then the chunk partials summed
-          // by all warps (warp w takes chunks w, w + NW, ...; fixed order).
-          double2 v0{(lane & 3) == ((lane & 15) >> 2) ? 1.0 : 0.0, 0.0};
-          if (warp == 0 && lane >= 16 && st.upd.vprev) v0 = (st.upd.vprev + s * st.upd.g_stride)[lane & 15];
+          // The chunk partials summed by all warps (warp w takes chunks w, w
+          // + NW, ...; fixed order), then over the warps: complex64 sums in
+          // FP32 with their rounding kept (TwoSum), 16 FP64 additions being a
+          // chain of 1000 cycles.
           const T* pp = reinterpret_cast<const T*>(a.partials) + (long long)s * a.part_stride * 32;
           T acc[4] = {T(0), T(0), T(0), T(0)};
           int b = warp;
@@ -896,18 +744,29 @@ __global__ void __launch_bounds__(df_threads<T>(), 1) k_sweep_df(DfArgs a) {
             for (int q = 0; q < 4; ++q) acc[q] += __ldcg(pp + (long long)(b + q * NW) * 32 + lane);
           }
           for (; b < st.nchunk; b += NW) acc[0] += __ldcg(pp + (long long)b * 32 + lane);
-          sh.red[warp][lane] = (double)((acc[0] + acc[1]) + (acc[2] + acc[3]));
+          const T mine = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+          if constexpr (sizeof(T) == 4) reinterpret_cast<float*>(sh.red[warp])[lane] = mine;
+          else sh.red[warp][lane] = mine;
           __syncthreads();
           if (tr && threadIdx.x == 0) tr[2] = globaltimer_ns();
-          double v = 0.0;
+          // complex64 sweeps: the polar factor to FP32 accuracy, the accuracy
+          // of their environments; FP64 sweeps: polar to FP64 rounding.
           if (warp == 0) {
+            float hi = 0.f, lo = 0.f;
+            double e = 0.0;
+            if constexpr (sizeof(T) == 4) {
 #pragma unroll
-            for (int w = 0; w < NW; ++w) v += sh.red[w][lane];
+              for (int w = 0; w < NW; ++w) {
+                float t;
+                two_sum(hi, reinterpret_cast<const float*>(sh.red[w])[lane], hi, t);
+                lo += t;
+              }
+            } else {
+#pragma unroll
+              for (int w = 0; w < NW; ++w) e += sh.red[w][lane];
+            }
+            df_update<T>(st.upd, s, sh, hi, lo, e);
           }
-          // complex64 sweeps: the polar factor to FP32 accuracy, the
-          // accuracy of their environments (no skew-Hermitian correction);
-          // FP64 sweeps: polar to FP64 rounding (two corrections).
-          df_update<T, sizeof(T) == 4 ? 0 : 2>(st.upd, s, sh, v, v0);
           if (st.upd.cost_out != nullptr && threadIdx.x == 0) {
             const double cost = st.upd.cost_out[s];
             if (a.cost_row != nullptr) a.cost_row[s] = cost;
