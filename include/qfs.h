@@ -155,8 +155,8 @@ int qfs_device_sms(const qfs_ctx* ctx);
  *     per-step launches).
  *   QFS_OPT_TWO_GATE_FORWARD [1]: the dataflow sweep applies consecutive
  *     forward gates on four distinct qubits in one step (0: one per step).
- *   QFS_OPT_FP64_TARGET_PRODUCT [0]: QFS_MIXED runs form U Psi in FP64
- *     instead of FP32 pair arithmetic.
+ *   QFS_OPT_FP64_TARGET_PRODUCT [0]: QFS_MIXED runs form U Psi by FP64
+ *     arithmetic instead of digits or fixed point.
  *   QFS_OPT_BATCH_LANES_PER_START [0 = tuned]: the batched form runs every
  *     problem class with this many lanes per start (4, 8, 16 or 32) instead
  *     of the autotuner's choice.
@@ -318,10 +318,11 @@ int qfs_gate_update(qfs_ctx* ctx, int32_t count, const double* envs, const doubl
 
 /* Phi_L = U Psi, the A tensor of Section 3 (the product every instantiation
  * starts from), on device buffers: target_dev N x N and samples_dev N x M
- * complex128 row-major, out_dev N x M (N = 2^n).  precision = QFS_FP64:
- * FP64 arithmetic.  QFS_MIXED: FP32 pair arithmetic (each FP64 operand
- * split into two floats, exact products through FMA, error-tracked sums),
- * about 48 significant bits, the product the mixed-precision runs use.
+ * complex128 row-major, out_dev N x M (N = 2^n).  Either precision gives the
+ * same product, to FP64 accuracy: from n = 7 on by exact products of 8-bit
+ * digits on the tensor cores (the FP64 kernel where a row of U is not of norm
+ * 1 to 10%), below in 64-bit fixed point, in workspace of the context (without
+ * room for it: FP64 arithmetic).
  * Synchronous; uses the context's workspace.  QFS_EINVAL for bad sizes. */
 int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* target_dev,
                            const double* samples_dev, int32_t precision, double* out_dev);

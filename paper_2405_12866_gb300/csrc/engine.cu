@@ -261,6 +261,8 @@ struct Run {
   // state of the sweeps
   void* B = nullptr;    // (L-1) x S x N x M in the sweep precision
   void* phi = nullptr;  // S x N x M in the sweep precision
+  void* oz = nullptr;        // scratch of the target product in digits (null: another form)
+  size_t oz_bytes = 0;
   double2* g64 = nullptr;
   float2* g32 = nullptr;
   double2* vprev = nullptr;  // right singular vectors of each gate's last update
@@ -331,6 +333,9 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
     R.phil32 = (float2*)take((size_t)R.T * R.sN * sizeof(float2));
   }
   R.B = take((size_t)std::max(R.L - 1, 1) * R.S * R.sN * es);
+  // Scratch of the target product: the B list, or a buffer of its own.
+  R.oz = R.oz_bytes == 0 ? nullptr
+         : R.oz_bytes <= (size_t)std::max(R.L - 1, 1) * R.S * R.sN * es ? R.B : take(R.oz_bytes);
   R.phi = take((size_t)R.S * R.sN * es);
   R.g64 = (double2*)take((size_t)R.S * R.L * 16 * sizeof(double2));
   R.g32 = R.prec == QFS_MIXED ? (float2*)take((size_t)R.S * R.L * 16 * sizeof(float2)) : nullptr;
@@ -629,8 +634,15 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
       for (const DfStep& st : steps) R.df_max_nchunk = std::max(R.df_max_nchunk, st.nchunk);
     }
   }
+  R.oz_bytes = oz_scratch_bytes((int)R.N, M, ctx->num_sms);
+  // (Without room for the digits' scratch the product takes another form.)
   const size_t bytes = carve(R, nullptr, need_U, need_envs);
-  TRY(ensure_ws(ctx, bytes));
+  int rc = ensure_ws(ctx, bytes);
+  if (rc == QFS_ENOMEM && R.oz_bytes > 0) {
+    R.oz_bytes = 0;
+    rc = ensure_ws(ctx, carve(R, nullptr, need_U, need_envs));
+  }
+  TRY(rc);
   carve(R, ctx->ws, need_U, need_envs);
   const size_t blist = (size_t)std::max(R.L - 1, 1) * S * R.sN * elem_bytes(prec == QFS_MIXED ? R32 : R64);
   R.stream_b = blist > ctx->l2_bytes / 2;
@@ -639,22 +651,20 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   return QFS_OK;
 }
 
-// Phi_L = U Psi (Sec. 3, the A tensor).  QFS_FP64 runs take the FP64
-// product; mixed runs the FP32 pair-arithmetic product (about 48 bits, far
-// below what the FP64 cost check at dist_tol resolves), with the B list,
-// not in use before the first sweep, as its scratch.  Returns the launches.
+// Phi_L = U Psi (Sec. 3, the A tensor), to FP64 accuracy: from 128 rows on by
+// digits on the tensor cores (n = 7, M = 24: 75 us in FP64, 25 us in its four
+// launches; n = 12, M = 32: 4.28 ms and 0.22), below in fixed point.  (Without
+// room for the digits' scratch, or when a mixed run asks for it, the FP64
+// kernel.)  Returns the launches.
 int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out) {
   cudaStream_t st = ctx->stream;
-  const size_t bbytes = (size_t)std::max(R.L - 1, 1) * R.S * R.sN * elem_bytes(R.prec == QFS_MIXED ? R32 : R64);
-  const size_t split_bytes = align_up((size_t)R.sN * sizeof(float4));
-  if (R.prec == QFS_MIXED && !ctx->upsi_fp64 && bbytes >= 2 * split_bytes) {
-    const int splits = upsi_pair_splits((int)R.N, R.M, ctx->num_sms, bbytes - split_bytes);
-    float4* ps = reinterpret_cast<float4*>(R.B);
-    double2* scratch = reinterpret_cast<double2*>(static_cast<char*>(R.B) + split_bytes);
-    launch_gemm_upsi_pair(U, psi, out, (int)R.N, R.M, ps, scratch, splits, ctx->num_sms, st);
-    return splits > 1 ? 3 : 2;
+  const bool plain = R.prec == QFS_MIXED && ctx->upsi_fp64;
+  if (R.oz && !plain) {
+    launch_oz_product(U, psi, out, (int)R.N, R.M, R.oz, R.err, ctx->num_sms, st);
+    return 4;
   }
-  launch_gemm_upsi(U, psi, out, (int)R.N, R.M, st);
+  if (R.n <= 6 && !plain) launch_fx_product(U, psi, out, R.n, R.M, st);
+  else launch_gemm_upsi(U, psi, out, (int)R.N, R.M, st);
   return 1;
 }
 
@@ -1449,8 +1459,12 @@ int instantiate_restarting(qfs_ctx* ctx, const qfs_circuit* c, const double* tar
     if (validate) {
       draw_states(p->training_distribution, sa, 5u, n, M, h.data());
       CK(cudaMemcpyAsync(R.psi_val64, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
+      CK(cudaMemsetAsync(R.err, 0, sizeof(int), st));
       ctx->prof.launches[QFS_PROF_GEMM] += target_product(ctx, R, R.U, R.psi_val64, R.phil_val64);
+      int err = 0;
+      CK(cudaMemcpyAsync(&err, R.err, sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
+      if (err) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", err);
     }
     CK(cudaMemcpyAsync(R.g64, G.data(), G.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     TRY(setup_inputs(ctx, R));
@@ -1986,17 +2000,25 @@ int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* tar
   const double2* P = reinterpret_cast<const double2*>(samples_dev);
   double2* O = reinterpret_cast<double2*>(out_dev);
   cudaStream_t st = ctx->stream;
-  if (precision == QFS_FP64) {
-    ctx->prof.launches[QFS_PROF_GEMM] += 1;
-    launch_gemm_upsi(U, P, O, N, M, st);
-  } else {
-    const size_t split_bytes = align_up((size_t)N * M * sizeof(float4));
-    const int splits = upsi_pair_splits(N, M, ctx->num_sms, (size_t)16 * N * M * sizeof(double2));
-    TRY(ensure_ws(ctx, split_bytes + align_up((size_t)splits * N * M * sizeof(double2))));
-    ctx->prof.launches[QFS_PROF_GEMM] += splits > 1 ? 3 : 2;
-    launch_gemm_upsi_pair(U, P, O, N, M, reinterpret_cast<float4*>(ctx->ws),
-                          reinterpret_cast<double2*>(ctx->ws + split_bytes), splits, ctx->num_sms, st);
+  // (Without room for the digits' scratch: the FP64 kernel.)
+  const size_t oz = oz_scratch_bytes(N, M, ctx->num_sms);
+  if (oz > 0 && ensure_ws(ctx, 256 + oz) == QFS_OK) {
+    int* err = reinterpret_cast<int*>(ctx->ws);
+    CK(cudaMemsetAsync(err, 0, sizeof(int), st));
+    ctx->prof.launches[QFS_PROF_GEMM] += 4;
+    CK(launch_oz_product(U, P, O, N, M, ctx->ws + 256, err, ctx->num_sms, st));
+    TRY(ensure_pinned(ctx, 1));
+    CK(cudaMemcpyAsync(ctx->h_pinned, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    int e;
+    std::memcpy(&e, ctx->h_pinned, sizeof(int));
+    if (e) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", e);
+    return QFS_OK;
   }
+  g_err.clear();
+  ctx->prof.launches[QFS_PROF_GEMM] += 1;
+  if (n <= 6) launch_fx_product(U, P, O, n, M, st);
+  else launch_gemm_upsi(U, P, O, N, M, st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
   return QFS_OK;

@@ -29,6 +29,7 @@
 // cycles on a random matrix from the identity) and FP64 products, took 10,400
 // and 15,400.
 #pragma once
+#include "fixed.cuh"
 #include "polar4.cuh"
 
 #include <limits.h>
@@ -59,41 +60,6 @@ struct NewtonSh {
   double2 polar[32];            // scratch of the FP64 Jacobi
 };
 
-// Fixed point: a number is (hi, lo) with value hi 2^30 + lo, |lo| <= 2^29, in
-// units of 2^-60; a complex one is int4 {re hi, re lo, im hi, im lo}.
-constexpr int kFxBits = 60, kFxLow = 30;
-__device__ __forceinline__ int2 fx_split(long long v) {
-  return int2{(int)((v + (1LL << (kFxLow - 1))) >> kFxLow), ((int)v << (32 - kFxLow)) >> (32 - kFxLow)};
-}
-// round(x 2^(kFxBits - e)) for |x| < 2^(e + 1), without FP64 instructions.
-__device__ __forceinline__ int2 fx_from(double x, int e) {
-  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
-  long long m = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
-  const int sh = ex - 1075 + kFxBits - e;
-  if (sh >= 0) m = m << min(sh, 10);
-  else m = sh < -54 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
-  return fx_split(hi < 0 ? -m : m);
-}
-__device__ __forceinline__ int4 fx_from2(double2 z, int e) {
-  const int2 x = fx_from(z.x, e), y = fx_from(z.y, e);
-  return int4{x.x, x.y, y.x, y.y};
-}
-// acc + a b of 32-bit numbers, in 64 bits.
-__device__ __forceinline__ long long mad64(int a, int b, long long acc) { return (long long)a * b + acc; }
-// A sum of products of fixed-point numbers: high x high, and the cross terms
-// 2^-30 below.  (low x low, 2^-60 below, is left out.)
-struct FxSum {
-  long long h = 0, c = 0, d = 0;
-  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
-    h = mad64(ah, bh, h);
-    c = mad64(ah, bl, c);
-    d = mad64(al, bh, d);
-  }
-  __device__ __forceinline__ long long value() const {
-    return h + ((c + d + (1LL << (kFxLow - 1))) >> kFxLow);
-  }
-};
-
 // Reciprocal and reciprocal square root of the hardware (about 1 ulp).
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
@@ -105,12 +71,6 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// x with its sign flipped if f (an FP64 negation that is not folded into an
-// FMA costs an FP64 instruction; this is integer).
-__device__ __forceinline__ double neg_if(double x, bool f) {
-  return __hiloint2double(__double2hiint(x) ^ (f ? 0x80000000 : 0), __double2loint(x));
-}
-
 // TwoSum (Knuth): hi + lo = a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& hi, float& lo) {
   hi = __fadd_rn(a, b);
@@ -118,23 +78,34 @@ __device__ __forceinline__ void two_sum(float a, float b, float& hi, float& lo) 
   lo = __fadd_rn(__fsub_rn(a, __fsub_rn(hi, t)), __fsub_rn(b, t));
 }
 
-// x times 2^e for a finite x, exactly, underflow to zero (FP64 arithmetic is
-// scarce; this is integer).
-__device__ __forceinline__ double scale_exp(double x, int e) {
-  const int hi = __double2hiint(x);
-  const int f = ((hi >> 20) & 0x7ff);
-  if (f == 0x7ff) return x;  // Inf and NaN stay what they are
-  if (f == 0 || f + e <= 0) return 0.0;
-  return __hiloint2double(hi + (e << 20), __double2loint(x));
+// Shuffles within each 16-lane half of the warp, and 4x4 products there
+// (entry [r][c] at lane 4c + r of the half).
+__device__ __forceinline__ float2 shfl16(float2 v, int src) {
+  return float2{__shfl_sync(FULL, v.x, src, 16), __shfl_sync(FULL, v.y, src, 16)};
+}
+__device__ __forceinline__ float2 mm16(float2 a, float2 b, int row, int col) {
+  float2 acc{0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc = cfma(shfl16(a, 4 * k + row), shfl16(b, 4 * col + k), acc);
+  return acc;
+}
+__device__ __forceinline__ float2 mm16_ah(float2 a, float2 b, int row, int col) {
+  float2 acc{0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float2 ak = shfl16(a, 4 * row + k), bk = shfl16(b, 4 * col + k);
+    acc = cfma(float2{ak.x, -ak.y}, bk, acc);
+  }
+  return acc;
 }
 
-// Step 1, one warp: x holds A (scaled, largest entry in [1/2, 2)) in lanes
-// 0..15 and again in lanes 16..31.  On success x is the FP32 polar factor and
-// the inverses and scalings are in s (KEEP).  Returns the steps (0: A is
-// singular or too ill-conditioned).  (A butterfly sum is bitwise the same in
-// every lane, so every branch here is uniform.)
-template <bool KEEP>
-__device__ __forceinline__ int newton_polar32(float2& x, NewtonSh& s) {
+// Step 1, one warp: each 16-lane half holds a matrix A in x, its own (HALVES)
+// or both the same.  On success x is the FP32 polar factor and (KEEP; one
+// matrix) the inverses and scalings are in s.  Returns the steps, 0 in a half
+// whose A is singular or too ill-conditioned.  (A butterfly sum is bitwise the
+// same in every lane of a half, so every branch is uniform there.)
+template <bool KEEP, bool HALVES>
+__device__ __forceinline__ int newton_polar32(float2& x, NewtonSh* s) {
   const int lane = threadIdx.x & 31;
   const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2;
   const int r0 = row == 0 ? 1 : 0, r1 = row <= 1 ? 2 : 1, r2 = row <= 2 ? 3 : 2;
@@ -145,9 +116,9 @@ __device__ __forceinline__ int newton_polar32(float2& x, NewtonSh& s) {
   // y = X^{-H}: the conjugate of (cofactor / determinant).
   auto inverse = [&](bool norm) {
     // The 3x3 minor without this lane's row and column, along its first row.
-    const float2 a11 = shfl_c(x, c1 + r1), a22 = shfl_c(x, c2 + r2), a12 = shfl_c(x, c2 + r1), a21 = shfl_c(x, c1 + r2);
-    const float2 a10 = shfl_c(x, c0 + r1), a20 = shfl_c(x, c0 + r2);
-    const float2 a00 = shfl_c(x, c0 + r0), a01 = shfl_c(x, c1 + r0), a02 = shfl_c(x, c2 + r0);
+    const float2 a11 = shfl16(x, c1 + r1), a22 = shfl16(x, c2 + r2), a12 = shfl16(x, c2 + r1), a21 = shfl16(x, c1 + r2);
+    const float2 a10 = shfl16(x, c0 + r1), a20 = shfl16(x, c0 + r2);
+    const float2 a00 = shfl16(x, c0 + r0), a01 = shfl16(x, c1 + r0), a02 = shfl16(x, c2 + r0);
     const float2 m0 = cfma(a11, a22, cmul(float2{-a12.x, -a12.y}, a21));
     const float2 m1 = cfma(a12, a20, cmul(float2{-a10.x, -a10.y}, a22));
     const float2 m2 = cfma(a10, a21, cmul(float2{-a11.x, -a11.y}, a20));
@@ -174,14 +145,17 @@ __device__ __forceinline__ int newton_polar32(float2& x, NewtonSh& s) {
     nx += __shfl_xor_sync(FULL, nx, m);
     nc += __shfl_xor_sync(FULL, nc, m);
   }
-  const float inv0 = __shfl_sync(FULL, inv, 0), ny = nc * inv0;
+  const float inv0 = __shfl_sync(FULL, inv, 0, 16), ny = nc * inv0;
   const float cond2 = nx * ny;
   // (NaN included.)  Cofactors carry rounding of 1e-7 |A|^3, the determinant
   // 1e-7 |A|^4: below 2e-6 |A|^4 it is not known, and of a matrix of rank 2
   // both are rounding, whose quotient says nothing about the condition.
   const float n2 = nx * nx;
-  if (!(cond2 < kNewtonMaxCond * kNewtonMaxCond) || !(n2 * n2 * inv0 < 2.5e11f)) return 0;
+  const bool ok = cond2 < kNewtonMaxCond * kNewtonMaxCond && n2 * n2 * inv0 < 2.5e11f;
+  if (!HALVES && !ok) return 0;
   const int range = cond2 <= 4.6f * 4.6f ? 0 : cond2 <= 83.f * 83.f ? 1 : 2;
+  // The other half may need more steps: further ones only converge further.
+  const int last = 2 + (HALVES ? __reduce_max_sync(FULL, ok ? range : 0) : range);
   // z = (ny / nx)^(1/4) brings the singular values around 1.
   const float t = rsqrt_approx(ny * rcp_approx(nx)), z = rsqrt_approx(t);
   float2 h{0.5f * z, 0.5f * t * z};
@@ -189,16 +163,16 @@ __device__ __forceinline__ int newton_polar32(float2& x, NewtonSh& s) {
 #pragma unroll 1
   for (;;) {
     if (KEEP && lane < 16) {
-      s.Y[it][l16] = y;
-      if (lane == 0) s.z[it] = h;
+      s->Y[it][l16] = y;
+      if (lane == 0) s->z[it] = h;
     }
     x = float2{fmaf(h.x, x.x, h.y * y.x), fmaf(h.x, x.y, h.y * y.y)};
-    if (it == 2 + range) break;
+    if (it == last) break;
     h = kNewtonZ[range][it];
     ++it;
     inverse(false);
   }
-  return it + 1;
+  return ok ? it + 1 : 0;
 }
 
 // The Hermitian R = I - Q^H Q as 16 real values, one per lane of a half warp:
@@ -287,6 +261,24 @@ __device__ __forceinline__ void newton_residual_polar(const NewtonSh& s, float2&
   k32 = im ? float2{ko, k} : float2{k, ko};
 }
 
+// Unitary correction of an FP32 matrix x (lanes 0..15, and a copy in lanes
+// 16..31) that is unitary to 1e-4 or better: q as newton_update returns it.
+// x is left unitary to FP32 rounding.
+__device__ __forceinline__ void newton_unitary(float2& x, NewtonSh& s, const NewtonPair& w, long long& q, bool last) {
+  const int lane = threadIdx.x & 31;
+  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2, im = lane >> 4;
+  constexpr float kUnit = (float)(1LL << kFxBits);
+  // The first correction needs R to FP32 digits only.
+  float2 d = mm(x, newton_entry(w, newton_residual32(x, w)), row, col);
+  q = __float2ll_rn((im ? x.y : x.x) * kUnit) + __float2ll_rn((im ? d.y : d.x) * (0.5f * kUnit));
+  x = float2{fmaf(0.5f, d.x, x.x), fmaf(0.5f, d.y, x.y)};
+  reinterpret_cast<int2*>(&s.Q[l16])[im] = fx_split(q);
+  __syncwarp();
+  if (!last) return;
+  d = mm(x, newton_entry(w, newton_residual_fx(s, w)), row, col);
+  q += __float2ll_rn((im ? d.y : d.x) * (0.5f * kUnit));
+}
+
 // Steps 1 and 2 in one warp for the matrix a32 (E^dagger scaled, its largest
 // entry in [1/2, 2); lanes 0..15 hold [r][c] at 4c + r, lanes 16..31 a copy).
 // POLISH: polar to 2^-59 for the fixed-point matrix in s.A; otherwise unitary
@@ -299,25 +291,11 @@ __device__ __forceinline__ bool newton_update(float2 a32, NewtonSh& s, const New
   const int lane = threadIdx.x & 31;
   const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2, im = lane >> 4;
   float2 x = a32;
-  const int its = newton_polar32<POLISH>(x, s);
+  const int its = newton_polar32<POLISH, false>(x, &s);
   if (!its) return false;
   constexpr float kUnit = (float)(1LL << kFxBits);
-  auto store = [&]() {
-    reinterpret_cast<int2*>(&s.Q[l16])[im] = fx_split(q);
-    __syncwarp();
-  };
-  {
-    // The first unitary correction needs R to FP32 digits only.
-    const float2 d = mm(x, newton_entry(w, newton_residual32(x, w)), row, col);
-    q = __float2ll_rn((im ? x.y : x.x) * kUnit) + __float2ll_rn((im ? d.y : d.x) * (0.5f * kUnit));
-    x = float2{fmaf(0.5f, d.x, x.x), fmaf(0.5f, d.y, x.y)};
-    store();
-  }
-  if (!POLISH) {
-    const float2 d = mm(x, newton_entry(w, newton_residual_fx(s, w)), row, col);
-    q += __float2ll_rn((im ? d.y : d.x) * (0.5f * kUnit));
-    return true;
-  }
+  newton_unitary(x, s, w, q, !POLISH);
+  if (!POLISH) return true;
   bool ok = true;
 #pragma unroll 1
   for (int it = 0;; ++it) {
@@ -349,7 +327,8 @@ __device__ __forceinline__ bool newton_update(float2 a32, NewtonSh& s, const New
     q += __float2ll_rn((im ? d.y : d.x) * kUnit);
     if (big < 1e-10f) break;
     x = float2{x.x + d.x, x.y + d.y};
-    store();
+    reinterpret_cast<int2*>(&s.Q[l16])[im] = fx_split(q);
+    __syncwarp();
   }
   return ok;
 }

@@ -1,0 +1,559 @@
+// Phi_L = U Psi (Section 3 of the paper, the A tensor) to FP64 accuracy on the
+// tensor cores: every number is cut into seven signed 8-bit digits, products
+// of digits are exact in f16 x f16 -> FP32, and sums of products are exact as
+// long as they stay below 2^24 (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59, 2012, for matrix products).
+//
+// Why: FP64 arithmetic runs at 1/64 of FP32's rate here.  The FP64 kernel was
+// at 84% of that pipe's peak (4.28 ms at n = 12, M = 32); the same product in
+// digits is 34 f16 products of the same shape, 73 us of tcgen05 at its peak,
+// beside 40 us to read U once.
+//
+// As a real product: U as it lies in memory is N x 2N reals (re, im
+// interleaved), and Psi becomes 2N x 2M with columns (pr, -pi), (pi, pr), so
+// that columns 2j, 2j + 1 of the result are re and im of column j.
+//
+// Digits: x = sum_i a_i 2^(-6 - 8i), a_i in [-128, 127] for i > 0, from
+// round(x 2^54); Psi's columns are first scaled by a power of two to [1/2, 1).
+// D_d = sum over i + j = d of (a_i b_j), d = 0..7, is one TMEM accumulator of
+// NB columns, and since the digits of Psi lie side by side along the columns
+// of one shared-memory operand, a_i times b_j, b_{j+1}, ... is one MMA that
+// adds into D_{i+j}, D_{i+j+1}, ...  The digits of U are formed on the fly by
+// the warps that load it.  D_0..D_3 are emptied into 64-bit integers after
+// every 256 products, before they can reach 2^24; D_4..D_7 weigh 2^-32 of D_0
+// and less, and may round.  What is left out (d > 7) is below 2^-60 of the
+// result's scale.
+//
+// Below 128 rows there is no tile to fill: k_fx_product forms the product in
+// 64-bit fixed point (fixed.cuh), one component per thread (n = 6, M = 16: 50 us
+// as FP64, 6 us so).
+//
+// U's digits have a fixed scale, so its rows have to have a norm near 1, as a
+// unitary's do.  The kernel sums their squares on the way; if any is outside
+// [0.81, 1.21] (or not a number), the FP64 kernel runs behind it.
+#include <cuda_fp16.h>
+
+#include "fixed.cuh"
+#include "qfs_kernels.h"
+
+#include <algorithm>
+
+namespace qfs {
+
+namespace {
+
+constexpr int kDig = 7;          // digits of a number
+constexpr int kOzK = 32;         // reals of one pipeline step
+constexpr int kOzChunk = 8;      // steps between two readings of D_0..D_3
+constexpr int kOzThreads = 288;  // eight warps for digits and sums, one for the MMAs
+constexpr int kOzProd = 256;
+constexpr int kABytes = kDig * 128 * kOzK * 2;
+constexpr long long kOzWait = 1LL << 24;
+
+__host__ __device__ constexpr int oz_bbytes(int nb) { return kDig * nb * kOzK * 2; }
+constexpr int oz_smem(int nb) { return 2 * (kABytes + oz_bbytes(nb)) + 128; }
+
+__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(uint64_t* b, int n) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ bool bar_wait(uint64_t* b, unsigned parity) {
+  for (long long i = 0; i < kOzWait; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(su32(b)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// The digits of two numbers |x| < 2 as seven f16 pairs, most significant first.
+__device__ __forceinline__ void digits2(double x0, double x1, uint32_t (&d)[kDig]) {
+  unsigned long long t[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double x = k ? x1 : x0;
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
+    const int sh = 1021 - ex;  // x = m 2^(ex - 1075): m 2^(ex - 1021) in units of 2^-54
+    const unsigned long long v = sh <= 0 ? m << min(-sh, 3) : sh > 60 ? 0 : (m + (1ULL << (sh - 1))) >> sh;
+    // Plus 128 in every byte: the bytes are the digits plus 128 (the top one,
+    // which may need a ninth bit, is taken from the upper bits).
+    t[k] = (hi < 0 ? 0 - v : v) + 0x0080808080808080ULL;
+  }
+  const uint32_t l0 = (uint32_t)t[0], l1 = (uint32_t)t[1], h0 = (uint32_t)(t[0] >> 32), h1 = (uint32_t)(t[1] >> 32);
+  // f16 0x6400 | b is 1024 + b; minus 1152 leaves the digit.
+  const __half2 off = __half2half2(__ushort_as_half(0x6480));
+  auto put = [&](int i, uint32_t w0, uint32_t w1, int byte) {
+    const uint32_t p = __byte_perm(w0, w1, byte | (byte + 4) << 4) & 0xffffu;  // bytes: b(w0), b(w1)
+    const uint32_t q = __byte_perm(p, 0x64646464u, 0x4140);                    // b0 64 b1 64
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&q), off);
+    d[i] = *reinterpret_cast<const uint32_t*>(&h);
+  };
+  const int top0 = ((int)h0 >> 16) - 128, top1 = ((int)h1 >> 16) - 128;
+  const __half2 th = __halves2half2(__int2half_rn(top0), __int2half_rn(top1));
+  d[0] = *reinterpret_cast<const uint32_t*>(&th);
+  put(1, h0, h1, 1);
+  put(2, h0, h1, 0);
+  put(3, l0, l1, 3);
+  put(4, l0, l1, 2);
+  put(5, l0, l1, 1);
+  put(6, l0, l1, 0);
+}
+
+// K-major operand without swizzle: 8 rows x 16 bytes are contiguous, `lead`
+// bytes lie between neighbours along K, 128 between groups of 8 rows.
+__device__ __forceinline__ uint64_t oz_desc(uint32_t saddr, uint32_t lead) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(lead >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | (uint64_t)1 << 46;
+}
+
+template <int N32>
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&w)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]),
+        "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15]), "=r"(w[16]),
+        "=r"(w[17]), "=r"(w[18]), "=r"(w[19]), "=r"(w[20]), "=r"(w[21]), "=r"(w[22]), "=r"(w[23]), "=r"(w[24]),
+        "=r"(w[25]), "=r"(w[26]), "=r"(w[27]), "=r"(w[28]), "=r"(w[29]), "=r"(w[30]), "=r"(w[31])
+      : "r"(addr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&w)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]),
+        "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
+      : "r"(addr)
+      : "memory");
+}
+// Zeros into 16 columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_zero16(uint32_t addr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(addr),
+      "r"(0)
+      : "memory");
+}
+
+}  // namespace
+
+// Psi's digits in the order of the product kernel's stages: [column block]
+// [step][K group of 8][digit][column][8].  Block j takes column j of Psi
+// (j >= M: zeros that fill up the last column block); expo[j] its scale.
+// Block 0 also zeroes the row norms and the flag.
+__global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi, int N, int M, int NB, __half* dig, int* expo,
+                                                  float* row2, int* flag) {
+  const int j = blockIdx.x, tid = threadIdx.x;
+  if (row2 != nullptr)
+    for (int i = blockIdx.x * blockDim.x + tid; i < N; i += gridDim.x * blockDim.x) row2[i] = 0.f;
+  if (j == 0 && tid == 0) *flag = 0;
+  int top = 0;  // exponent field of the column's largest entry
+  if (j < M)
+    for (int i = tid; i < N; i += 256) {
+      const double2 z = Psi[(long long)i * M + j];
+      top = max(top, max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff));
+    }
+  __shared__ int red[8];
+  top = __reduce_max_sync(FULL, top);
+  if ((tid & 31) == 0) red[tid >> 5] = top;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) top = max(top, red[w]);
+  const int e = top == 0 ? 0 : top - 1022;  // entries times 2^-e are below 1
+  if (tid == 0) {
+    expo[j] = e;
+    if (top >= 2046) atomicOr(flag, 1);  // Inf, NaN or next to them: the FP64 kernel
+  }
+  auto scaled = [&](double x) {
+    const int hi = __double2hiint(x), f = (hi >> 20) & 0x7ff;
+    return f == 0 || f - e <= 0 ? 0.0 : __hiloint2double(hi - (e << 20), __double2loint(x));
+  };
+  const int c0 = 2 * j, cb = c0 / NB, c = c0 % NB, steps = 2 * N / kOzK;
+  for (int g = tid; g < N / 4; g += 256) {  // a group: 4 complex rows, 8 reals
+    double2 z[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      z[r] = j < M ? Psi[(long long)(4 * g + r) * M + j] : double2{0.0, 0.0};
+      z[r] = double2{scaled(z[r].x), scaled(z[r].y)};
+    }
+    uint32_t a[kDig][4], b[kDig][4];  // columns 2j: (pr, -pi), 2j + 1: (pi, pr)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      uint32_t d[kDig];
+      digits2(z[r].x, -z[r].y, d);
+#pragma unroll
+      for (int i = 0; i < kDig; ++i) a[i][r] = d[i];
+      digits2(z[r].y, z[r].x, d);
+#pragma unroll
+      for (int i = 0; i < kDig; ++i) b[i][r] = d[i];
+    }
+    const int step = g / (kOzK / 8), k8 = g % (kOzK / 8);
+    __half* base = dig + ((long long)cb * steps + step) * (oz_bbytes(NB) / 2) + (long long)k8 * kDig * NB * 8;
+#pragma unroll
+    for (int i = 0; i < kDig; ++i) {
+      *reinterpret_cast<uint4*>(base + (i * NB + c) * 8) = make_uint4(a[i][0], a[i][1], a[i][2], a[i][3]);
+      *reinterpret_cast<uint4*>(base + (i * NB + c + 1) * 8) = make_uint4(b[i][0], b[i][1], b[i][2], b[i][3]);
+    }
+  }
+}
+
+// Grid (N / 128 row tiles, K splits, column blocks).  part: [split][column
+// block][row][NB] sums in units of 2^-54 of the scaled columns.
+template <int NB>
+__global__ void __launch_bounds__(kOzThreads, 1)
+    k_oz_product(const double* __restrict__ U, const __half* __restrict__ dig, int N, long long* part, float* row2, int* err) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  constexpr int kB = oz_bbytes(NB), kStage = kABytes + kB, HC = NB / 2;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + 2 * kStage);
+  uint64_t *empty = full + 2, *accfull = full + 4, *accfree = full + 5;
+  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 6);
+  volatile int* gave_up = reinterpret_cast<volatile int*>(slot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int steps = 2 * N / kOzK;
+  const int k0 = (int)((long long)blockIdx.y * steps / gridDim.y), k1 = (int)((long long)(blockIdx.y + 1) * steps / gridDim.y);
+  const int nk = k1 - k0, nchunk = (nk + kOzChunk - 1) / kOzChunk;
+  const int row0 = blockIdx.x * 128;
+
+  if (tid == 0) {
+    bar_init(&full[0], kOzProd + 1);
+    bar_init(&full[1], kOzProd + 1);
+    bar_init(&empty[0], 1);
+    bar_init(&empty[1], 1);
+    bar_init(accfull, 1);
+    bar_init(accfree, kOzProd);
+    *gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(slot)), "r"(8 * NB)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *slot;
+
+  if (warp == 8) {
+    // ------------------------------------------------------------- the MMAs
+    if (lane == 0) {
+      constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(128 >> 4) << 24);
+      bool ok = true;
+      for (int i = 0; i < nk && ok; ++i) {
+        const int s = i & 1;
+        if (i % kOzChunk == 0) ok = bar_wait(accfree, (unsigned)(i / kOzChunk) & 1u);
+        ok = ok && bar_wait(&full[s], (unsigned)(i >> 1) & 1u) && !*gave_up;
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = su32(sm + s * kStage), b0 = a0 + kABytes;
+        // a_i times digits j .. j + w - 1 of Psi into D_{i+j} ...: at most four
+        // digits (256 columns) at a time, D_0..D_3 apart from D_4..D_7.
+        auto mma = [&](int kk, int i_, int j, int w) {
+          const uint64_t ad = oz_desc(a0 + (uint32_t)(i_ * 128 * kOzK * 2 + kk * 2 * 128 * 16), 128 * 16);
+          const uint64_t bd = oz_desc(b0 + (uint32_t)(kk * 2 * kDig * NB * 16 + j * NB * 16), kDig * NB * 16);
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)((i_ + j) * NB)),
+              "l"(ad), "l"(bd), "r"(idesc | (uint32_t)(w * NB >> 3) << 17), "r"(1)
+              : "memory");
+        };
+#pragma unroll
+        for (int kk = 0; kk < kOzK / 16; ++kk) {
+#pragma unroll
+          for (int d = 0; d < kDig; ++d) {
+            if (d < 4) mma(kk, d, 0, 4 - d);
+            const int j = d < 4 ? 4 - d : 0, last = d == 0 ? 6 : 7 - d;  // i + j from 4 (or i) to 7 (j <= 6)
+            mma(kk, d, j, last - j + 1);
+          }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&empty[s]))
+                     : "memory");
+        if ((i + 1) % kOzChunk == 0 || i + 1 == nk)
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(accfull))
+                       : "memory");
+      }
+      if (!ok) *gave_up = 1;
+    }
+    __syncwarp();
+  } else {
+    // ---------------------------------------------- digits of U, sums of D
+    // Lane: row lane & 7 of a group of eight, K group lane >> 3 of four, so
+    // that eight lanes store 128 contiguous bytes; two rows per thread.
+    const int r = warp * 8 + (lane & 7), k8 = lane >> 3;
+    const double* u0 = U + (long long)(row0 + r) * 2 * N + k8 * 8;
+    const double* u1 = u0 + 64LL * 2 * N;
+    double2 x[2][4];
+    float n0 = 0.f, n1 = 0.f;
+    auto load = [&](int k) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        x[0][q] = __ldg(reinterpret_cast<const double2*>(u0 + (long long)k * kOzK) + q);
+        x[1][q] = __ldg(reinterpret_cast<const double2*>(u1 + (long long)k * kOzK) + q);
+      }
+    };
+    const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * HC);
+    long long hi[HC];
+#pragma unroll
+    for (int c = 0; c < HC; ++c) hi[c] = 0;
+    auto zero = [&](int from, int to) {
+      for (int d = from; d < to; ++d)
+#pragma unroll
+        for (int c = 0; c < HC; c += 16) tmem_zero16(lanes + (uint32_t)(d * NB + c));
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    };
+    auto read = [&](int d, uint32_t (&w)[32]) {
+      if constexpr (HC == 32) tmem_ld32<HC>(lanes + (uint32_t)(d * NB), w);
+      else tmem_ld16(lanes + (uint32_t)(d * NB), w);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    };
+    auto gather = [&](int chunk) {  // D_0..D_3 into hi
+      if (!bar_wait(accfull, (unsigned)chunk & 1u)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int d = 0; d < 4; ++d) {
+        uint32_t w[32];
+        read(d, w);
+#pragma unroll
+        for (int c = 0; c < HC; ++c) hi[c] += (long long)__float2int_rn(__uint_as_float(w[c])) << (8 * (3 - d));
+      }
+      return true;
+    };
+    bool ok = true;
+    int issued = 0;
+    zero(0, 8);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    bar_arrive(accfree);
+    if (nk > 0) load(k0);
+    for (int i = 0; i < nk; ++i) {
+      const int s = i & 1;
+      ok = bar_wait(&empty[s], ((unsigned)(i >> 1) & 1u) ^ 1u) && !*gave_up;
+      if (!ok) break;
+      unsigned char* st = sm + s * kStage;
+      if (tid == 0) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[s])), "r"(kB) : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(st + kABytes)),
+            "l"(dig + ((long long)blockIdx.z * steps + k0 + i) * (kB / 2)), "r"(kB), "r"(su32(&full[s]))
+            : "memory");
+        ++issued;
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t d[4][kDig];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          digits2(x[h][q].x, x[h][q].y, d[q]);
+          const float fx = (float)x[h][q].x, fy = (float)x[h][q].y;
+          (h ? n1 : n0) = fmaf(fx, fx, fmaf(fy, fy, h ? n1 : n0));
+        }
+#pragma unroll
+        for (int p = 0; p < kDig; ++p)
+          *reinterpret_cast<uint4*>(st + p * 128 * kOzK * 2 + k8 * 128 * 16 + (r + 64 * h) * 16) =
+              make_uint4(d[0][p], d[1][p], d[2][p], d[3][p]);
+      }
+      if (i + 1 < nk) load(k0 + i + 1);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bar_arrive(&full[s]);
+      // The previous chunk's sums, with this step's operands already staged.
+      if (i > 0 && i % kOzChunk == 0) {
+        ok = gather(i / kOzChunk - 1);
+        if (!ok) break;
+        zero(0, 4);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        bar_arrive(accfree);
+      }
+    }
+    if (ok && nk > 0) ok = gather(nchunk - 1);
+    if (!ok) {
+      *gave_up = 1;
+      if (tid == 0)  // the copies in flight land first (bounded)
+        for (int i = max(0, issued - 2); i < issued; ++i) bar_wait(&full[i & 1], (unsigned)(i >> 1) & 1u);
+    } else {
+      long long* out = part + (((long long)blockIdx.y * gridDim.z + blockIdx.z) * N + row0 + (warp & 3) * 32 + lane) * NB +
+                       (warp >> 2) * HC;
+      long long low[HC];
+#pragma unroll
+      for (int c = 0; c < HC; ++c) low[c] = 0;
+      if (nk > 0) {
+#pragma unroll
+        for (int d = 4; d < 8; ++d) {
+          uint32_t w[32];
+          read(d, w);
+#pragma unroll
+          for (int c = 0; c < HC; ++c) low[c] += (long long)__float2int_rn(__uint_as_float(w[c])) << (8 * (7 - d));
+        }
+      }
+      // hi in 2^-36, low in 2^-68; together in 2^-54.
+#pragma unroll
+      for (int c = 0; c < HC; c += 2)
+        *reinterpret_cast<longlong2*>(out + c) =
+            longlong2{(hi[c] << 18) + ((low[c] + (1 << 13)) >> 14), (hi[c + 1] << 18) + ((low[c + 1] + (1 << 13)) >> 14)};
+      if (blockIdx.z == 0) {
+        n0 += __shfl_xor_sync(FULL, n0, 8);
+        n1 += __shfl_xor_sync(FULL, n1, 8);
+        n0 += __shfl_xor_sync(FULL, n0, 16);
+        n1 += __shfl_xor_sync(FULL, n1, 16);
+        if (lane < 8) {
+          atomicAdd(row2 + row0 + r, n0);
+          atomicAdd(row2 + row0 + r + 64, n1);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (tid == 0 && *gave_up) atomicOr(err, 1);
+  if (warp == 8) {
+    if (lane == 0 && *gave_up) {
+      // MMAs already issued finish (bounded) before their accumulator goes.
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&empty[0]))
+                   : "memory");
+      for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(8 * NB) : "memory");
+  }
+}
+
+// The splits' sums (exact), to FP64; *flag |= 1 when a row of U was not of norm 1.
+__global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__ part, const int* __restrict__ expo,
+                                                    const float* __restrict__ row2, int N, int M, int NB, int splits, int cblocks,
+                                                    double2* out, int* flag) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)N * M) return;
+  const int row = (int)(i / M), j = (int)(i - (long long)row * M);
+  const int cb = 2 * j / NB, c = 2 * j % NB;
+  long long re = 0, im = 0;
+  for (int s = 0; s < splits; ++s) {
+    const longlong2 v =
+        __ldcs(reinterpret_cast<const longlong2*>(part + (((long long)s * cblocks + cb) * N + row) * NB + c));
+    re += v.x;
+    im += v.y;
+  }
+  const int e = expo[j];
+  out[i] = double2{ldexp((double)re, e - 54), ldexp((double)im, e - 54)};
+  if (j == 0) {
+    const float n2 = row2[row];
+    if (!(n2 > 0.81f && n2 < 1.21f)) atomicOr(flag, 1);
+  }
+}
+
+// out = U Psi for N <= 64 rows: grid (N / 8 row tiles (at least 1), column tiles
+// of 32).  Scales from the largest entries of the block's rows of U and columns
+// of Psi, with room for 2 N terms: the high sums stay below 2^62, each cross sum
+// below 2^62 and both together below 2^63.  Entries next to FP64's largest
+// exponent, Inf and NaN take FP64 arithmetic.
+constexpr int kFxRows = 8, kFxCols = 32;
+__global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ U, const double2* __restrict__ Psi,
+                                                    double2* __restrict__ out, int n, int M) {
+  __shared__ int4 su[kFxRows * 64], sp[64 * kFxCols];
+  __shared__ int red[2][8];
+  const int N = 1 << n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = blockIdx.x * kFxRows, rows = min(kFxRows, N - r0), c0 = blockIdx.y * kFxCols, cols = min(kFxCols, M - c0);
+  int tu = 0, tp = 0;
+  auto top = [](int t, double2 z) {
+    return max(t, max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff));
+  };
+  for (int i = tid; i < rows * N; i += 256) tu = top(tu, U[(long long)r0 * N + i]);
+  for (int i = tid; i < N * cols; i += 256) tp = top(tp, Psi[(long long)(i / cols) * M + c0 + i % cols]);
+  tu = __reduce_max_sync(FULL, tu);
+  tp = __reduce_max_sync(FULL, tp);
+  if (lane == 0) {
+    red[0][warp] = tu;
+    red[1][warp] = tp;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    tu = max(tu, red[0][w]);
+    tp = max(tp, red[1][w]);
+  }
+  const bool plain = tu >= 2040 || tp >= 2040;
+  const int eu = tu - 1022 + n - 1, ep = tp - 1022 + max(n - 2, 1);
+  if (!plain) {
+    for (int i = tid; i < rows * N; i += 256) su[i] = fx_from2(U[(long long)r0 * N + i], eu);
+    for (int i = tid; i < N * cols; i += 256) sp[i] = fx_from2(Psi[(long long)(i / cols) * M + c0 + i % cols], ep);
+  }
+  __syncthreads();
+  for (int c = tid; c < 2 * rows * cols; c += 256) {
+    const int im = c & 1, i = (c >> 1) / cols, j = (c >> 1) % cols;
+    double v = 0.0;
+    if (plain) {
+      for (int k = 0; k < N; ++k) {
+        const double2 x = U[(long long)(r0 + i) * N + k], y = Psi[(long long)k * M + c0 + j];
+        v = im ? fma(x.x, y.y, fma(x.y, y.x, v)) : fma(x.x, y.x, fma(-x.y, y.y, v));
+      }
+    } else {
+      FxSum t;
+      for (int k = 0; k < N; ++k) {
+        const int4 x = su[i * N + k], y = sp[k * cols + j];
+        t.add(x.x, x.y, im ? y.z : y.x, im ? y.w : y.y);
+        t.add(im ? x.z : -x.z, im ? x.w : -x.w, im ? y.x : y.z, im ? y.y : y.w);
+      }
+      v = scale_exp((double)t.value(), eu + ep - kFxBits);
+    }
+    reinterpret_cast<double*>(out + (long long)(r0 + i) * M + c0 + j)[im] = v;
+  }
+}
+
+namespace {
+
+struct OzShape {
+  int nb, cblocks, splits;
+  size_t dig, part, row2, expo, total;
+};
+OzShape oz_shape(int N, int M, int num_sms) {
+  OzShape s;
+  s.nb = 2 * M <= 32 ? 32 : 64;
+  s.cblocks = (2 * M + s.nb - 1) / s.nb;
+  const int steps = 2 * N / kOzK;
+  s.splits = std::max(1, std::min(steps / 2, num_sms / (N / 128 * s.cblocks)));
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  s.dig = up((size_t)s.cblocks * steps * oz_bbytes(s.nb));
+  s.part = up((size_t)s.splits * s.cblocks * N * s.nb * sizeof(long long));
+  s.row2 = up((size_t)N * sizeof(float));
+  s.expo = up((size_t)s.cblocks * s.nb / 2 * sizeof(int) + 2 * sizeof(int));
+  s.total = s.dig + s.part + s.row2 + s.expo;
+  return s;
+}
+
+}  // namespace
+
+size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 128 ? 0 : oz_shape(N, M, num_sms).total; }
+
+cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
+                              int num_sms, cudaStream_t st) {
+  const OzShape s = oz_shape(N, M, num_sms);
+  char* p = static_cast<char*>(scratch);
+  __half* dig = reinterpret_cast<__half*>(p);
+  long long* part = reinterpret_cast<long long*>(p + s.dig);
+  float* row2 = reinterpret_cast<float*>(p + s.dig + s.part);
+  int* flag = reinterpret_cast<int*>(p + s.dig + s.part + s.row2);
+  int* expo = flag + 2;
+  cudaError_t e = cudaFuncSetAttribute(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem(s.nb));
+  if (e != cudaSuccess) return e;
+  k_oz_prep<<<s.cblocks * s.nb / 2, 256, 0, st>>>(Psi, N, M, s.nb, dig, expo, row2, flag);
+  const dim3 grid(N / 128, s.splits, s.cblocks);
+  if (s.nb == 64) k_oz_product<64><<<grid, kOzThreads, oz_smem(64), st>>>((const double*)U, dig, N, part, row2, err);
+  else k_oz_product<32><<<grid, kOzThreads, oz_smem(32), st>>>((const double*)U, dig, N, part, row2, err);
+  k_oz_finish<<<(unsigned)(((long long)N * M + 255) / 256), 256, 0, st>>>(part, expo, row2, N, M, s.nb, s.splits, s.cblocks,
+                                                                        out, flag);
+  launch_gemm_upsi(U, Psi, out, N, M, st, flag);
+  return cudaGetLastError();
+}
+
+void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st) {
+  k_fx_product<<<dim3(std::max(1, (1 << n) / kFxRows), (M + kFxCols - 1) / kFxCols), 256, 0, st>>>(U, Psi, out, n, M);
+}
+
+}  // namespace qfs

@@ -46,8 +46,8 @@ namespace qfs {
 namespace {
 
 constexpr int kClMaxC = 16;
-constexpr int kMaxSmem = 200 * 1024;
-constexpr int kClRing = 4;  // rounds of B in flight per thread (complex64)
+constexpr int kMaxSmem = 211 * 1024;  // (beside 15 KB of static shared memory)
+constexpr int kClRing = 3;  // rounds of B in flight per thread (complex64)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -94,16 +94,6 @@ __device__ __forceinline__ void cp_wait() {
 }
 __device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
-// Where entry e = (column << n) | row of a slice sits: bits 4 and 5 are folded
-// into the bank bits, so that the units of a gate on any two neighbouring row
-// bits (whose lanes skip those bits) spread over the banks.  Linear over XOR,
-// and a permutation of every 16 entries: below 16 rows a slice need not be a
-// multiple of that, so there nothing is folded (fold = 0).
-__device__ __forceinline__ uint32_t swz(uint32_t e, uint32_t fold) {
-  return e ^ (((e >> 4) & fold) * 5u) ^ (((e >> 5) & fold) * 10u);
-}
-__device__ __forceinline__ uint32_t swz_fold(int n) { return n >= 4 ? 1u : 0u; }
-
 struct ClShared {
   unsigned long long exch[2][kClMaxC][32];  // environment sums of the cluster's CTAs, two exchanges deep
   unsigned long long red[16][32];           // per-warp sums
@@ -111,11 +101,6 @@ struct ClShared {
   NewtonSh nw;
   long long out[32];  // the new gate for the warp that writes it out: components of newton_update, or FP64
   int flag, out_fx;
-};
-
-// The row bits of a gate's two qubits.
-struct ClGeo {
-  int pa, pb, lo, hi;
 };
 
 // Sum of the CTAs' values: each CTA's warp 0 brings one 8-byte value per lane;
@@ -241,51 +226,7 @@ __device__ __forceinline__ bool cl_sum_double(ClShared& sh, uint32_t C, uint32_t
   return true;
 }
 
-__device__ __forceinline__ ClGeo cl_geo(const ClArgs& a, int k) {
-  const int p = a.pos[k], pa = p & 15, pb = p >> 4;
-  return ClGeo{pa, pb, min(pa, pb), max(pa, pb)};
-}
-
-// Fixed point: out = G in (adj: G^dagger in) on a slice of `units` units, one
-// component of one output row per lane.  out = sum p v.x + q v.y in three
-// integer FMAs per product.  In place when out = in.
-template <int NT>
-__device__ __forceinline__ void fx_apply(const int4* in, int4* out, const int4* gate, const ClGeo& g, bool adj, int units, int n) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rbits = n - 2;
-  const uint32_t fold = swz_fold(n);
-  const int x = (lane >> 1) & 3, im = lane & 1;
-  int2 p[4], q[4];
-  uint32_t xo[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int4 w = gate[adj ? 4 * j + x : 4 * x + j];
-    const int sy = adj ? -1 : 1;  // conj(G) for the adjoint
-    const int2 re{w.x, w.y}, iy{sy * w.z, sy * w.w};
-    p[j] = im ? iy : re;
-    q[j] = im ? re : int2{-iy.x, -iy.y};
-    xo[j] = swz(((uint32_t)(j >> 1) << g.pa) | ((uint32_t)(j & 1) << g.pb), fold);
-  }
-  const uint32_t mine = xo[x];
-  for (int u0 = warp * 4; u0 < units; u0 += NT / 8) {
-    const int u = u0 + (lane >> 3);
-    const uint32_t b = swz(((uint32_t)(u >> rbits) << n) |
-                           insert_two_zero_bits((uint32_t)u & ((1u << rbits) - 1u), g.lo, g.hi), fold);
-    FxSum t;
-    if (u < units) {
-      int4 v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = in[b ^ xo[j]];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        t.add(p[j].x, p[j].y, v[j].x, v[j].y);
-        t.add(q[j].x, q[j].y, v[j].z, v[j].w);
-      }
-    }
-    const int2 r = fx_split(t.value());
-    __syncwarp();  // (in place: the eight lanes of a unit have read it)
-    if (u < units) reinterpret_cast<int2*>(out + (b ^ mine))[im] = r;
-  }
-}
+__device__ __forceinline__ PairBits cl_geo(const ClArgs& a, int k) { return pair_bits(a.pos[k] & 15, a.pos[k] >> 4); }
 
 }  // namespace
 
@@ -396,7 +337,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
   // FP64: out = G in, one component of one output row per lane; ADJ: G^dagger.
   auto apply64 = [&](int k, const T2* in, T2* out, bool adj) {
     if constexpr (!F32) {
-      const ClGeo g = cl_geo(a, k);
+      const PairBits g = cl_geo(a, k);
       const int x = (lane >> 1) & 3, im = lane & 1;
       double p[4], q[4];  // out = sum p v.x + q v.y
 #pragma unroll
@@ -460,7 +401,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
     __syncthreads();
     if constexpr (F32) {
       for (int k = 0; k < L; ++k) {
-        const ClGeo g = cl_geo(a, k);
+        const PairBits g = cl_geo(a, k);
         uint32_t xo[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) xo[j] = swz(((uint32_t)(j >> 1) << g.pa) | ((uint32_t)(j & 1) << g.pb), fold);
@@ -510,7 +451,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
     // --------------------------------------------------------------- backward
     double cost = 0.0;
     for (int k = L - 1; k >= 0; --k) {
-      const ClGeo g = cl_geo(a, k);
+      const PairBits g = cl_geo(a, k);
       uint32_t xo[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) xo[j] = swz(((uint32_t)(j >> 1) << g.pa) | ((uint32_t)(j & 1) << g.pb), fold);
@@ -725,7 +666,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
       // The residual cost (1/M) sum |g_1^dagger Phi_1 - Psi|^2, unless the
       // update's estimate is so far above the tolerance that it decides nothing.
       if (!(a.resid_skip > 0.0 && cost > a.resid_skip)) {
-        const ClGeo g = cl_geo(a, 0);
+        const PairBits g = cl_geo(a, 0);
         T2 gd[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -824,7 +765,7 @@ int cl_resident(Real r, int nt, bool fx, int C, size_t smem) {
   static std::map<std::tuple<int, int, int, int, size_t>, int> known;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  const auto key = std::make_tuple(dev, (int)r * 2 + (int)fx, nt, C, (smem + 4095) / 4096);
+  const auto key = std::make_tuple(dev, (int)r * 2 + (int)fx, nt, C, smem);
   {
     std::lock_guard<std::mutex> lock(mu);
     const auto it = known.find(key);
@@ -835,7 +776,7 @@ int cl_resident(Real r, int nt, bool fx, int C, size_t smem) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(64 * C));
   cfg.blockDim = dim3((unsigned)nt);
-  cfg.dynamicSmemBytes = (smem + 4095) / 4096 * 4096;
+  cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)C;
@@ -883,10 +824,10 @@ __global__ void __launch_bounds__(NT) k_cl_check(ClArgs a, double* parts, unsign
     __syncthreads();
   }
   double t = 0.0;
-  auto full = [](int hi, int lo) { return ((long long)hi << kFxLow) + lo; };
   for (int i = tid; i < N; i += NT) {
     const int4 x = X[swz((uint32_t)i, fold)], y = fx_from2(__ldg(phil + (long long)i * M + j), e);
-    const double dx = (double)(full(y.x, y.y) - full(x.x, x.y)), dy = (double)(full(y.z, y.w) - full(x.z, x.w));
+    const double dx = (double)(fx_value(y.x, y.y) - fx_value(x.x, x.y)),
+                 dy = (double)(fx_value(y.z, y.w) - fx_value(x.z, x.w));
     t = fma(dx, dx, fma(dy, dy, t));
   }
 #pragma unroll
