@@ -2131,13 +2131,40 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
   const int stream_b = (size_t)std::max(R.L - 1, 1) * S * state > tmp.l2_bytes / 2;
 
   cudaStream_t st = tmp.stream;
-  // The fused update's counters must start at zero; a call that stopped
-  // part-way could have left them otherwise.
-  CK(cudaMemsetAsync(R.counters, 0, (size_t)S * sizeof(unsigned), st));
   if (gates_out_dev != gates_in_dev)
     CK(cudaMemcpyAsync(gates_out_dev, gates_in_dev, (size_t)S * R.L * 16 * sizeof(double2),
                        cudaMemcpyDeviceToDevice, st));
-  launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st);
+  // Phi_L = U Psi: digits where their scratch still fits behind the sweep's.
+  const size_t oz = oz_scratch_bytes((int)R.N, M, sms);
+  if (R.n <= 6) {
+    launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st);
+  } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
+    int* err = reinterpret_cast<int*>(take(sizeof(int)));
+    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), err, sms, st));
+  } else {
+    launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st);
+  }
+  // The cluster sweep where it takes the problem (n = 6, 10 gates, M = 16, 8
+  // starts: 305 us as 40 launches, 90 us as 5).  Nothing comes back to the host
+  // in between, so both forms are queued and the one the inputs are not for
+  // returns at once.
+  R.cl = cl_plan(R64, R.n, M, R.L, S, beta != 0.0);
+  if (R.cl.C > 0) {
+    char* aux = reinterpret_cast<char*>(R.partials);  // (not used by this sweep; at least 256 bytes)
+    R.cl_acc = reinterpret_cast<unsigned*>(aux);
+    R.cl_scale = reinterpret_cast<int4*>(aux + 64);
+    R.err = reinterpret_cast<int*>(aux + 128);
+    R.costs = costs_out_dev ? costs_out_dev : reinterpret_cast<double*>(R.phi);
+    R.spt = S;
+    R.cl_plain = {0, 1};
+    launch_cl_scale(R.n, M, S * R.L, R.psi64, R.phil64, R.g64, R.cl_acc, R.cl_scale, st);
+    TRY(cl_sweep(&tmp, R, R64, R.psi64, R.phil64, reinterpret_cast<double2*>(envs_out_dev), nullptr, st));
+    CK(cudaGetLastError());
+    return QFS_OK;
+  }
+  // The fused update's counters must start at zero; a call that stopped
+  // part-way could have left them otherwise.
+  CK(cudaMemsetAsync(R.counters, 0, (size_t)S * sizeof(unsigned), st));
   TRY(sweep(&tmp, R, R64, Slice{0, S, S, st}, R.g64, nullptr, R.psi64, R.phil64, R.B, R.phi, R.partials,
             R.nblk_max, costs_out_dev, reinterpret_cast<double2*>(envs_out_dev), nullptr, stream_b,
             nullptr, R.counters));
