@@ -4,15 +4,14 @@
 // Work is handed out in units: a unit is one problem and 32/G of its starts,
 // run by one warp with G lanes per start (G = 32: a warp per start; G = 16,
 // 8 or 4: two, four or eight starts share a warp).  Each start keeps its
-// running state B and Phi (N x M complex, N <= 32, M <= 16), its gates and
-// the right singular vectors of their last updates in its own slice of
-// shared memory and sweeps as in Section 3 of the paper; the list of
+// running state B and Phi (N x M complex, N <= 32, M <= 16) and its gates in
+// its own slice of shared memory and sweeps as in Section 3 of the paper; the list of
 // intermediate states is replaced by walking B back with the old gate
 // (B_{k-1} = g_k^dagger B_k), so nothing leaves the SM between sweeps.  The
 // starts' state arithmetic (gate applications, environment sums) runs side
 // by side in their lane groups; each group reduces its environment over its
 // own lanes, and the warp then updates the unit's gates one after another
-// (Eq. 2: the FP32 Jacobi polar factor, FP64 Jacobi for ill-conditioned
+// (Eq. 2: the FP32 Newton polar factor, FP64 Jacobi for ill-conditioned
 // environments).  Units come from an atomic work
 // queue ordered largest problem first; the schedule G (and the warps per
 // block) of each class of problems (n, L, M) is chosen by the host's
@@ -23,7 +22,7 @@
 // multistarts would return.  A finishing kernel then makes the selected
 // gates unitary in FP64, checks the cost in FP64 and, if needed, refines
 // with FP64 sweeps.
-#include "polar4.cuh"
+#include "polar_newton.cuh"
 #include "qfs_common.cuh"
 #include "qfs_kernels.h"
 
@@ -33,60 +32,27 @@ namespace qfs {
 
 namespace {
 
-// Polar factor in FP32 (batched complex64 sweeps) of A (lanes 0..15, A[r][c]
-// at 4c + r): one-sided Jacobi on X = A V0, V0 the right singular vectors of
-// the gate's previous update (16 complex at v_io, V[r][c] at 4c + r), whose
-// columns are already nearly orthogonal once the sweeps settle, so few
-// rotation sweeps are needed.  The new V, made unitary to FP32 rounding by
-// one Newton-Schulz step (so that no drift accumulates over sweeps), is
-// written back to v_io.  Returns false when sigma_min < 1e-3 sigma_max (the
-// caller then takes the FP64 Jacobi, which also completes rank-deficient
-// cases).
-__device__ __forceinline__ bool warp_polar4_f32_warm(float2 a, float2* v_io, float2* q_out) {
-  const int lane = threadIdx.x & 31;
-  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2;
-  const bool isV = lane >= 16;
-  const float2 v0 = v_io[l16];  // every lane: V0[row][col]
-  float2 x;
-  {
-    float2 acc{0.f, 0.f};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 ak = shfl_c(a, 4 * k + row), vk = shfl_c(v0, 4 * col + k);
-      acc = cfma(ak, vk, acc);
-    }
-    x = isV ? v0 : acc;
-  }
-  bool rotated = false;
-  x = jacobi32_sweeps(x, &rotated);
-  float2 w = shfl_c(x, l16);
-  float2 v = shfl_c(x, 16 + l16);
-  float nrm = w.x * w.x + w.y * w.y;
-  nrm += __shfl_xor_sync(FULL, nrm, 1);
-  nrm += __shfl_xor_sync(FULL, nrm, 2);
-  float smax = nrm, smin = nrm;
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 4));
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 8));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 4));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 8));
-  if (!(smin > 1e-6f * smax)) return false;
-  const float inv = rsqrtf(nrm);
-  w = float2{w.x * inv, w.y * inv};
-  // Q = W V^H, unitary to the Jacobi tolerance (~1e-6), with no
-  // Newton-Schulz step: the batched sweeps see that deviation only
-  // quadratically in their residual cost, each update starts afresh, and the
-  // finishing kernel makes the answer unitary in FP64.  V carries over
-  // between sweeps, so it is renormalised.
-  *q_out = mm_bh(w, v, row, col);
-  if (rotated) {  // an unrotated V is the stored one: nothing to renormalise
-    const float2 gv = mm_ah(v, v, row, col);
-    const float2 tv{(row == col ? 1.5f : 0.f) - 0.5f * gv.x, -0.5f * gv.y};
-    v = mm(v, tv, row, col);
-    __syncwarp();
-    if (lane < 16) v_io[l16] = v;
-  }
-  __syncwarp();
-  return true;
+// Polar factor in FP32 (batched complex64 sweeps): each 16-lane half of the
+// warp holds a matrix A (entry [r][c] at lane 4c + r), its own (HALVES) or
+// both the same.  The scaled Newton iteration of polar_newton.cuh and one
+// Newton-Schulz step, which leaves the factor unitary to FP32 rounding (the
+// finishing kernel makes the answer unitary in FP64).  False in a half whose
+// matrix is singular or too ill-conditioned (the caller then takes the FP64
+// Jacobi, which also completes rank-deficient cases).
+//
+// Against the one-sided Jacobi with the gate's previous singular vectors as
+// start that it replaces, an update needs no state between sweeps and a fixed
+// 3 to 5 steps of 380 cycles where a Jacobi sweep took 750 and three to five
+// of them were needed in the first sweeps of a run.
+template <bool HALVES>
+__device__ __forceinline__ bool batch_polar32(float2 a, float2* q_out) {
+  const int l16 = threadIdx.x & 15, row = l16 & 3, col = l16 >> 2;
+  const int its = newton_polar32<false, HALVES>(a, nullptr);
+  if (!HALVES && !its) return false;
+  const float2 g = mm16_ah(a, a, row, col);
+  const float2 t{(row == col ? 1.5f : 0.f) - 0.5f * g.x, -0.5f * g.y};
+  *q_out = mm16(a, t, row, col);
+  return its != 0;
 }
 
 template <typename T> struct BT;
@@ -184,212 +150,56 @@ __device__ void group_env_acc(const T2* Bs, const T2* Ph, int n, int M, int qa, 
   }
 }
 
-// New gate from E (E[c][r] in lane 4c + r): the polar factor of E^dagger.
-template <typename T2>
-__device__ void warp_update(T2 e, T2* g, double2* sm, float2* v);
-
-// v: the gate's right singular vectors from its previous update (the Jacobi
-// start; identity at the first sweep), updated in place.
-template <>
-__device__ void warp_update<float2>(float2 e, float2* g, double2* sm, float2* v) {
+// New gate from E (E[c][r] in lane 4c + r of both halves): the polar factor
+// of E^dagger.
+__device__ void warp_update(float2 e, float2* g, double2* sm) {
   const int lane = threadIdx.x & 31;
   const int l16 = lane & 15, r = l16 & 3, c = l16 >> 2;
   const float2 a32{e.x, -e.y};  // A[r][c] = conj(E[c][r])
   float2 q;
-  if (!warp_polar4_f32_warm(a32, v, &q)) {
+  if (!batch_polar32<false>(a32, &q)) {
     const double2 p =
         warp_polar4(double2{(double)e.x, -(double)e.y}, double2{r == c ? 1.0 : 0.0, 0.0}, sm, nullptr);
     q = float2{(float)p.x, (float)p.y};
-    if (lane < 16) v[l16] = float2{r == c ? 1.f : 0.f, 0.f};  // restart from the identity
   }
   if (lane < 16) g[4 * r + c] = q;
   __syncwarp();
 }
-
-template <>
-__device__ void warp_update<double2>(double2 e, double2* g, double2* sm, float2* v) {
-  (void)v;
+__device__ void warp_update64(double2 e, double2* g, double2* sm) {
   double2 p;
   polar_update_warp<2>(e, nullptr, 0.0, sm, g, nullptr, &p, nullptr);
   __syncwarp();
-}
-
-// ---------------------------------------------------------------------------
-// Two updates side by side, one per 16-lane half of the warp (the schedule
-// with 16 lanes per start).  Each lane of a half holds one entry of X = A V
-// and the same entry of V (M[row][col] at lane 4 col + row of the half), so
-// a Jacobi round needs no exchange between an X lane and a V lane; every
-// shuffle stays inside its half (width 16).
-
-__device__ __forceinline__ float2 shfl16(float2 v, int src) {
-  return float2{__shfl_sync(FULL, v.x, src, 16), __shfl_sync(FULL, v.y, src, 16)};
-}
-__device__ __forceinline__ float2 mm16(float2 a, float2 b, int row, int col) {
-  float2 acc{0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) acc = cfma(shfl16(a, 4 * k + row), shfl16(b, 4 * col + k), acc);
-  return acc;
-}
-__device__ __forceinline__ float2 mm16_ah(float2 a, float2 b, int row, int col) {
-  float2 acc{0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float2 ak = shfl16(a, 4 * row + k), bk = shfl16(b, 4 * col + k);
-    acc = cfma(float2{ak.x, -ak.y}, bk, acc);
-  }
-  return acc;
-}
-__device__ __forceinline__ float2 mm16_bh(float2 a, float2 b, int row, int col) {
-  float2 acc{0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float2 ak = shfl16(a, 4 * k + row), bk = shfl16(b, 4 * k + col);
-    acc = cfma(ak, float2{bk.x, -bk.y}, acc);
-  }
-  return acc;
-}
-// Whether every column pair of this half's X has |gamma|^2 <= kJac32Tol
-// alpha beta (the Gram-matrix test of jacobi32_converged), as a
-// warp-uniform two-bit mask (bit h: half h).
-__device__ __forceinline__ unsigned half_converged(float2 x, int row, int col) {
-  const float2 g = mm16_ah(x, x, row, col);
-  const float dr = __shfl_sync(FULL, g.x, 5 * row, 16), dc = __shfl_sync(FULL, g.x, 5 * col, 16);
-  const bool ok = row == col || (g.x * g.x + g.y * g.y) <= kJac32Tol * dr * dc;
-  const unsigned b = __ballot_sync(FULL, ok);
-  return ((b & 0xffffu) == 0xffffu ? 1u : 0u) | ((b >> 16) == 0xffffu ? 2u : 0u);
-}
-
-// The polar factor of A (A[row][col] at lane 4 col + row of each half), the
-// Jacobi started from V0 = v_io (that half's gate's right singular vectors
-// from its previous update) and the new V written back, as
-// warp_polar4_f32_warm does for one matrix.  Returns, warp-uniformly, a
-// two-bit mask of the halves whose fast path succeeded; a half that failed
-// (zero or too ill-conditioned) has not written v_io and its *q_out is
-// undefined.  `act` (per half): whether this half's result is wanted.
-__device__ unsigned halfwarp_polar4_f32_warm(float2 a, float2* v_io, bool act, float2* q_out) {
-  const int lane = threadIdx.x & 31;
-  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2, h = lane >> 4;
-  const float2 v0 = act ? v_io[l16] : float2{row == col ? 1.f : 0.f, 0.f};
-  if (!act) a = float2{row == col ? 1.f : 0.f, 0.f};
-  float2 x = mm16(a, v0, row, col);
-  float2 v = v0;
-  unsigned done = half_converged(x, row, col);
-  bool rotated = false;
-  for (int sweep = 0; sweep < 12 && done != 3u; ++sweep) {
-    const bool mine_done = (done >> h) & 1u;
-    bool any = false;
-#pragma unroll
-    for (int m = 1; m <= 3; ++m) {
-      const float2 y = shfl16(x, l16 ^ (4 * m)), yv = shfl16(v, l16 ^ (4 * m));
-      const bool isP = col < (col ^ m);
-      float nown = x.x * x.x + x.y * x.y;
-      float npar = y.x * y.x + y.y * y.y;
-      float2 g = isP ? float2{x.x * y.x + x.y * y.y, x.x * y.y - x.y * y.x}
-                     : float2{y.x * x.x + y.y * x.y, y.x * x.y - y.y * x.x};
-#pragma unroll
-      for (int o = 1; o <= 2; o <<= 1) {
-        nown += __shfl_xor_sync(FULL, nown, o);
-        npar += __shfl_xor_sync(FULL, npar, o);
-        g.x += __shfl_xor_sync(FULL, g.x, o);
-        g.y += __shfl_xor_sync(FULL, g.y, o);
-      }
-      const float alpha = isP ? nown : npar, beta = isP ? npar : nown;
-      const float ag2 = g.x * g.x + g.y * g.y;
-      float cs = 1.f, sn = 0.f, px = 1.f, py = 0.f;
-      if (!mine_done && ag2 > kJac32Tol * alpha * beta && ag2 > 1e-36f) {
-        const float rg = rsqrtf(ag2);
-        const float zeta = 0.5f * (beta - alpha) * rg;
-        const float q = fmaf(zeta, zeta, 1.f);
-        const float t = fabsf(zeta) > 1e18f ? __fdividef(0.5f, zeta)
-                                             : copysignf(__fdividef(1.f, fabsf(zeta) + q * rsqrtf(q)), zeta);
-        cs = rsqrtf(fmaf(t, t, 1.f));
-        sn = t * cs;
-        px = g.x * rg;
-        py = -g.y * rg;
-        any = true;
-      }
-      if (isP) {
-        const float tx = px * y.x - py * y.y, ty = px * y.y + py * y.x;
-        const float ux = px * yv.x - py * yv.y, uy = px * yv.y + py * yv.x;
-        x = float2{cs * x.x - sn * tx, cs * x.y - sn * ty};
-        v = float2{cs * v.x - sn * ux, cs * v.y - sn * uy};
-      } else {
-        const float tx = px * x.x - py * x.y, ty = px * x.y + py * x.x;
-        const float ux = px * v.x - py * v.y, uy = px * v.y + py * v.x;
-        x = float2{sn * y.x + cs * tx, sn * y.y + cs * ty};
-        v = float2{sn * yv.x + cs * ux, sn * yv.y + cs * uy};
-      }
-    }
-    // A half with no rotation in a whole sweep is done; else the Gram test.
-    const unsigned b = __ballot_sync(FULL, any);
-    rotated |= ((b >> (16 * h)) & 0xffffu) != 0u;
-    const unsigned none = ((b & 0xffffu) == 0u ? 1u : 0u) | ((b >> 16) == 0u ? 2u : 0u);
-    done |= none;
-    if (done != 3u) done |= half_converged(x, row, col);
-  }
-  float nrm = x.x * x.x + x.y * x.y;
-  nrm += __shfl_xor_sync(FULL, nrm, 1);
-  nrm += __shfl_xor_sync(FULL, nrm, 2);
-  float smax = nrm, smin = nrm;
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 4));
-  smax = fmaxf(smax, __shfl_xor_sync(FULL, smax, 8));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 4));
-  smin = fminf(smin, __shfl_xor_sync(FULL, smin, 8));
-  const bool good = smin > 1e-6f * smax;
-  const unsigned gb = __ballot_sync(FULL, good);
-  const unsigned okmask = ((gb & 0xffffu) == 0xffffu ? 1u : 0u) | ((gb >> 16) == 0xffffu ? 2u : 0u);
-  const float inv = rsqrtf(good ? nrm : 1.f);
-  const float2 w{x.x * inv, x.y * inv};
-  // Q = W V^H, unitary to the Jacobi tolerance (~1e-6): the batched sweeps'
-  // residual cost sees that deviation only quadratically, every update
-  // starts afresh from its environment, and the finishing kernel makes the
-  // answer unitary in FP64 before the FP64 cost check.
-  *q_out = mm16_bh(w, v, row, col);
-  // Renormalise a rotated V (one Newton-Schulz step) so no drift
-  // accumulates over sweeps; an unrotated V is the stored one.
-  if (__any_sync(FULL, rotated)) {
-    const float2 gv = mm16_ah(v, v, row, col);
-    const float2 tv{(row == col ? 1.5f : 0.f) - 0.5f * gv.x, -0.5f * gv.y};
-    v = mm16(v, tv, row, col);
-    __syncwarp();
-    if (act && ((okmask >> h) & 1u) && rotated) v_io[l16] = v;
-  }
-  __syncwarp();
-  return okmask;
 }
 
 // The unit's two gate updates at once (16 lanes per start): half h updates
 // the gate of start h from its environment e (E[c][r] at lane 4c + r of the
 // half).  A half whose fast path fails takes the FP64 Jacobi (warp-wide, one
 // half after the other), as warp_update does.
-__device__ void halfwarp_update(float2 e, float2* g, double2* sm, float2* v, bool act) {
+__device__ void halfwarp_update(float2 e, float2* g, double2* sm, bool act) {
   const int lane = threadIdx.x & 31;
   const int l16 = lane & 15, r = l16 & 3, c = l16 >> 2, h = lane >> 4;
-  const float2 a32{e.x, -e.y};  // A[r][c] = conj(E[c][r])
+  // A[r][c] = conj(E[c][r]); an idle half carries the identity along.
+  const float2 a32 = act ? float2{e.x, -e.y} : float2{r == c ? 1.f : 0.f, 0.f};
   float2 q;
-  const unsigned act_mask = __ballot_sync(FULL, act);
-  const unsigned acts = ((act_mask & 0xffffu) ? 1u : 0u) | ((act_mask >> 16) ? 2u : 0u);
-  const unsigned ok = halfwarp_polar4_f32_warm(a32, v, act, &q);
+  const bool fine = batch_polar32<true>(a32, &q);
+  const unsigned bad = __ballot_sync(FULL, !fine);
   for (int hh = 0; hh < 2; ++hh) {
-    if (!((acts >> hh) & 1u) || ((ok >> hh) & 1u)) continue;
+    if (!((bad >> (16 * hh)) & 1u)) continue;
     // The FP64 Jacobi of half hh's matrix on the whole warp: A in lanes 0..15.
     const float2 ah{__shfl_sync(FULL, a32.x, 16 * hh + l16), __shfl_sync(FULL, a32.y, 16 * hh + l16)};
     const double2 p = warp_polar4(double2{(double)ah.x, (double)ah.y}, double2{r == c ? 1.0 : 0.0, 0.0}, sm, nullptr);
     const float2 pf{(float)p.x, (float)p.y};
     const float2 pq{__shfl_sync(FULL, pf.x, l16), __shfl_sync(FULL, pf.y, l16)};
-    if (h == hh) {
-      q = pq;
-      v[l16] = float2{r == c ? 1.f : 0.f, 0.f};  // restart from the identity
-    }
+    if (h == hh) q = pq;
   }
   if (act) g[4 * r + c] = q;
   __syncwarp();
 }
 
 // Per-start smem slice (complex64): B (E_max), Phi (E_max), gates (16 L_max),
-// right singular vectors (16 L_max), environment (16).
+// environment (16).
 __host__ __device__ __forceinline__ int batch_slice_f2(int max_elems, int max_L) {
-  return 2 * max_elems + 32 * max_L + 16;
+  return 2 * max_elems + 16 * max_L + 16;
 }
 
 // One sweep (Section 3) of every active start of a unit: forward to B_{L-1}
@@ -410,8 +220,7 @@ __device__ float group_sweep(float2* slice, int slice_f2, int E_max, int L_max, 
   float2* Bs = slice + gi * slice_f2;
   float2* Ph = Bs + E_max;
   float2* Gt = Ph + E_max;
-  float2* V = Gt + 16 * L_max;
-  float* Env = reinterpret_cast<float*>(V + 16 * L_max);
+  float* Env = reinterpret_cast<float*>(Gt + 16 * L_max);
   const int E = M << n;
   if (act) {
     for (int i = gl; i < E; i += G) {
@@ -434,7 +243,7 @@ __device__ float group_sweep(float2* slice, int slice_f2, int E_max, int L_max, 
       const float v = warp_reduce_scatter32<float>(acc, lane);
       const int l16 = lane & 15;
       const float2 e{__shfl_sync(FULL, v, 2 * l16), __shfl_sync(FULL, v, 2 * l16 + 1)};
-      if (act) warp_update<float2>(e, Gt + 16 * (k - 1), sm, V + 16 * (k - 1));
+      if (act) warp_update(e, Gt + 16 * (k - 1), sm);
     } else if constexpr (G == 16) {
       // After the reduce-scatter lane gl holds two of its start's 32
       // environment floats; gather E[c][r] to lane 4c + r of each half
@@ -444,7 +253,7 @@ __device__ float group_sweep(float2* slice, int slice_f2, int E_max, int L_max, 
       Env[base + 1] = acc[1];
       __syncwarp();
       const float2 e{Env[2 * gl], Env[2 * gl + 1]};
-      halfwarp_update(e, Gt + 16 * (k - 1), sm, V + 16 * (k - 1), act);
+      halfwarp_update(e, Gt + 16 * (k - 1), sm, act);
     } else {
       const int base = group_reduce_scatter<G, float>(acc, gl);
 #pragma unroll
@@ -456,9 +265,9 @@ __device__ float group_sweep(float2* slice, int slice_f2, int E_max, int L_max, 
       for (int j = 0; j < NG; ++j) {
         if (!((act_mask >> j) & 1u)) continue;
         float2* sj = slice + j * slice_f2;
-        const float* envj = reinterpret_cast<const float*>(sj + 2 * E_max + 32 * L_max);
+        const float* envj = reinterpret_cast<const float*>(sj + 2 * E_max + 16 * L_max);
         const float2 e{envj[2 * l16], envj[2 * l16 + 1]};
-        warp_update<float2>(e, sj + 2 * E_max + 16 * (k - 1), sm, sj + 2 * E_max + 16 * L_max + 16 * (k - 1));
+        warp_update(e, sj + 2 * E_max + 16 * (k - 1), sm);
       }
     }
     __syncwarp();
@@ -508,7 +317,7 @@ __device__ void warp_sweep64(double2* Bs, double2* Ph, double2* G, const double2
     const double v = warp_reduce_scatter32<double>(acc, lane);
     const int l16 = lane & 15;
     const double2 e{__shfl_sync(FULL, v, 2 * l16), __shfl_sync(FULL, v, 2 * l16 + 1)};
-    warp_update<double2>(e, G + 16 * (k - 1), sm, nullptr);
+    warp_update64(e, G + 16 * (k - 1), sm);
     if (k > 1) {
       group_apply<32, double2>(Bs, G + 16 * (k - 2), n, M, pairs[2 * (k - 2)], pairs[2 * (k - 2) + 1], true, lane);
       group_apply<32, double2>(Ph, G + 16 * (k - 1), n, M, qa, qb, true, lane);
@@ -519,29 +328,82 @@ __device__ void warp_sweep64(double2* Bs, double2* Ph, double2* G, const double2
 
 }  // namespace
 
-// Per-problem set-up: Phi_L = U Psi in FP64 and complex64 copies of Psi and
-// Phi_L.  One block per problem.
-__global__ void k_batch_prep(BatchArgs a) {
+namespace {
+// Largest exponent field of `count` complex numbers, by a whole block.
+__device__ int block_exponent(const double2* z, int count, int* red) {
+  int top = 0;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) {
+    const double2 v = z[i];
+    top = max(top, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+  }
+  top = __reduce_max_sync(FULL, top);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) top = max(top, red[w]);
+  return top;
+}
+}  // namespace
+
+// Per-problem set-up: Phi_L = U Psi to FP64 accuracy and complex64 copies of
+// Psi and Phi_L.  One block per problem, one component of the product per
+// thread at a time, in fixed point: with a scale from the largest entry and
+// room for the 2 N terms (at most 5 + 4 bits) an entry has 55 bits below the
+// largest, as FP64 gives the entries of a unitary on up to six qubits.  (1024
+// problems of 3 to 5 qubits: 110 us in FP64, whose pipe it filled by a third.)
+// Entries out of the scale's range (Inf, NaN) take the FP64 form.
+__global__ void __launch_bounds__(128) k_batch_prep(BatchArgs a) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ int red[4];
   const int p = blockIdx.x;
   if (p >= a.P) return;
   const BatchProblem pr = a.probs[p];
   const int N = 1 << pr.n, M = pr.M;
   const double2* U = a.targets + pr.target_off;
   const double2* psi = a.psi64 + pr.state_off;
+  double2* phil64 = a.phil64 + pr.state_off;
+  float2* phil32 = a.phil32 + pr.state_off;
+  if (threadIdx.x == 0) a.s_star[p] = INT_MAX;
   for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
-    const int i = e / M, j = e - i * M;
-    double2 acc{0.0, 0.0};
-    for (int k = 0; k < N; ++k) {
-      const double2 u = U[(size_t)i * N + k], s = psi[(size_t)k * M + j];
-      acc.x = fma(u.x, s.x, fma(-u.y, s.y, acc.x));
-      acc.y = fma(u.x, s.y, fma(u.y, s.x, acc.y));
-    }
-    a.phil64[pr.state_off + e] = acc;
-    a.phil32[pr.state_off + e] = float2{(float)acc.x, (float)acc.y};
     const double2 s = psi[e];
     a.psi32[pr.state_off + e] = float2{(float)s.x, (float)s.y};
   }
-  if (threadIdx.x == 0) a.s_star[p] = INT_MAX;
+  const int tu = block_exponent(U, N * N, red), tp = block_exponent(psi, N * M, red);
+  if (tu >= 2040 || tp >= 2040) {
+    for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
+      const int i = e / M, j = e - i * M;
+      double2 acc{0.0, 0.0};
+      for (int k = 0; k < N; ++k) {
+        const double2 u = U[(size_t)i * N + k], s = psi[(size_t)k * M + j];
+        acc.x = fma(u.x, s.x, fma(-u.y, s.y, acc.x));
+        acc.y = fma(u.x, s.y, fma(u.y, s.x, acc.y));
+      }
+      phil64[e] = acc;
+      phil32[e] = float2{(float)acc.x, (float)acc.y};
+    }
+    return;
+  }
+  // Room for 2 N terms: the high sums stay below 2^62, each cross sum below
+  // 2^62 and both together below 2^63.
+  const int eu = tu - 1022 + pr.n - 1, ep = tp - 1022 + max(pr.n - 2, 1);
+  int4* su = reinterpret_cast<int4*>(dsm);
+  int4* sp = su + N * N;
+  for (int e = threadIdx.x; e < N * N; e += blockDim.x) su[e] = fx_from2(U[e], eu);
+  for (int e = threadIdx.x; e < N * M; e += blockDim.x) sp[e] = fx_from2(psi[e], ep);
+  __syncthreads();
+  for (int c = threadIdx.x; c < 2 * N * M; c += blockDim.x) {
+    const int e = c >> 1, im = c & 1, i = e / M, j = e - i * M;
+    const int4 *u = su + i * N, *s = sp + j;
+    FxSum t;
+    for (int k = 0; k < N; ++k) {
+      const int4 x = u[k], y = s[k * M];
+      t.add(x.x, x.y, im ? y.z : y.x, im ? y.w : y.y);
+      t.add(im ? x.z : -x.z, im ? x.w : -x.w, im ? y.x : y.z, im ? y.y : y.w);
+    }
+    const double v = scale_exp((double)t.value(), eu + ep - kFxBits);
+    reinterpret_cast<double*>(phil64 + e)[im] = v;
+    reinterpret_cast<float*>(phil32 + e)[im] = (float)v;
+  }
 }
 
 // One unit (a problem and up to 32/G of its starts) swept by the warp to
@@ -562,14 +424,11 @@ __device__ __forceinline__ void batch_run_unit(const BatchArgs& a, const BatchUn
   bool act = gi < u.ns;
   float2* mine = region + gi * sf;
   float2* Gt = mine + 2 * E;
-  float2* V = Gt + 16 * L;
   const size_t goff = pr.gate_off + (size_t)s * L * 16;
   if (act) {
     for (int i = gl; i < 16 * L; i += G) {
       const double2 g = a.init_gates[goff + i];
       Gt[i] = float2{(float)g.x, (float)g.y};
-      const int e = i & 15;
-      V[i] = float2{(e & 3) == (e >> 2) ? 1.f : 0.f, 0.f};
     }
   }
   __syncwarp();
@@ -647,58 +506,74 @@ __global__ void k_batch_sweep(BatchArgs a, const BatchUnit* units, int nunits, i
   }
 }
 
-// One warp per problem: pick the start, make its gates unitary in FP64, FP64
-// cost check, FP64 refinement sweeps while the cost is above tol.
-__global__ void k_batch_finalize(BatchArgs a) {
+// One block per problem: pick the start, make its gates unitary, check the
+// cost, FP64 refinement sweeps while the cost is above tol.
+//
+// Gates are made unitary by one warp each and the cost's circuit is applied in
+// fixed point (fixed.cuh), each to FP64 accuracy: bound by integer issue.  As
+// one warp of FP64 instructions a problem took 30 to 80 us (1024 problems of 3
+// to 5 qubits: 172 us).
+__global__ void __launch_bounds__(128) k_batch_finalize(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  __shared__ double2 sm_polar[32];
+  __shared__ NewtonSh nw[4];
+  __shared__ double red[4];
+  __shared__ int redi[4];
   const int p = blockIdx.x;
   if (p >= a.P) return;
-  const int lane = threadIdx.x & 31;
-  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int l16 = lane & 15, row = l16 & 3, col = l16 >> 2, im = lane >> 4;
   const BatchProblem pr = a.probs[p];
-  const int E = pr.M << pr.n;
-  double2* Bs = reinterpret_cast<double2*>(dsm);
+  const int E = pr.M << pr.n, n = pr.n, M = pr.M;
+  double2* Bs = reinterpret_cast<double2*>(dsm);  // (refinement sweeps)
   double2* Ph = Bs + a.max_elems;
   double2* G = Ph + a.max_elems;
+  int4* X = reinterpret_cast<int4*>(G + 16 * a.max_L);
+  int4* GX = X + a.max_elems;
   // Selection: among starts converged at the earliest converged sweep, the
   // lowest cost (lowest index on ties); if none converged, the lowest cost.
-  int best = 0;
   const int sst = a.s_star[p];
+  int best = 0;
   double bc = 1e300;
-  for (int s = 0; s < a.S; ++s) {
+  for (int s = lane; s < a.S; s += 32) {
     const size_t ri = (size_t)p * a.S + s;
-    const bool eligible = sst == INT_MAX || a.conv_sweep[ri] == sst;
     const double c = a.final_cost[ri];
-    if (eligible && c < bc) {
+    if ((sst == INT_MAX || a.conv_sweep[ri] == sst) && c < bc) {
       bc = c;
       best = s;
     }
   }
-  int sweeps = sst == INT_MAX ? a.sweeps_run[(size_t)p * a.S + best] : sst;
-  const size_t goff = pr.gate_off + (size_t)best * pr.L * 16;
-  // FP64 copy of the gates, made unitary by two Newton-Schulz steps.
-  for (int k = 0; k < pr.L; ++k) {
-    const float2 g32 = a.gates32[goff + 16 * k + (4 * row + col)];  // lane 4col+row holds g[row][col]
-    double2 q{(double)g32.x, (double)g32.y};
-    for (int it = 0; it < 2; ++it) {
-      const double2 gq = mm64_ah(q, q, row, col, lane < 16);
-      const double2 t{(row == col ? 1.5 : 0.0) - 0.5 * gq.x, -0.5 * gq.y};
-      q = mm64(q, t, row, col, lane < 16);
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    const double oc = __shfl_xor_sync(FULL, bc, m);
+    const int ob = __shfl_xor_sync(FULL, best, m);
+    if (oc < bc || (oc == bc && ob < best)) {
+      bc = oc;
+      best = ob;
     }
-    if (lane < 16) G[16 * k + 4 * row + col] = q;
   }
-  __syncwarp();
+  const int sweeps = sst == INT_MAX ? a.sweeps_run[(size_t)p * a.S + best] : sst;
+  const size_t goff = pr.gate_off + (size_t)best * pr.L * 16;
+  const NewtonPair pair = newton_pair();
+  for (int k = warp; k < pr.L; k += 4) {
+    float2 x = a.gates32[goff + 16 * k + (4 * row + col)];  // lane 4col+row holds g[row][col]
+    long long q;
+    newton_unitary(x, nw[warp], pair, q, true);
+    reinterpret_cast<int2*>(GX + 16 * k + 4 * row + col)[im] = fx_split(q);
+    reinterpret_cast<double*>(G + 16 * k + 4 * row + col)[im] = scale_exp((double)q, -kFxBits);
+    __syncwarp();
+  }
   const int* pairs = a.pairs + pr.pair_off;
   const double2* psi = a.psi64 + pr.state_off;
   const double2* phil = a.phil64 + pr.state_off;
-  // FP64 cost: (1/M) || Phi_L - C Psi ||^2.
-  auto cost64 = [&]() {
+  // FP64 cost: (1/M) || Phi_L - C Psi ||^2.  One scale for both sides, with
+  // room for an entry to grow to its column's norm (3 bits).
+  const int top = max(block_exponent(psi, E, redi), block_exponent(phil, E, redi));
+  double c;
+  auto cost64 = [&]() {  // (warp 0, in FP64: refined gates, and numbers out of the scale's range)
     for (int i = lane; i < E; i += 32) Bs[i] = psi[i];
     __syncwarp();
     for (int k = 1; k <= pr.L; ++k) {
-      group_apply<32, double2>(Bs, G + 16 * (k - 1), pr.n, pr.M, pairs[2 * (k - 1)], pairs[2 * (k - 1) + 1], false,
-                               lane);
+      group_apply<32, double2>(Bs, G + 16 * (k - 1), n, M, pairs[2 * (k - 1)], pairs[2 * (k - 1) + 1], false, lane);
       __syncwarp();
     }
     double acc = 0.0;
@@ -708,17 +583,52 @@ __global__ void k_batch_finalize(BatchArgs a) {
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-    return acc / pr.M;
+    return acc / M;
   };
-  double c = cost64();
-  int refine = 0;
-  while (c > a.tol && refine < a.refine_max && (sst != INT_MAX || a.refine_unconverged)) {
-    warp_sweep64(Bs, Ph, G, psi, phil, pairs, pr.n, pr.M, pr.L, sm_polar);
-    ++refine;
-    c = cost64();
+  if (top < 2040) {
+    const int e = top - 1022 + 3;
+    const uint32_t fold = swz_fold(n);
+    for (int i = tid; i < E; i += 128) {
+      const int r = i / M, j = i - r * M;
+      X[swz(((uint32_t)j << n) | (uint32_t)r, fold)] = fx_from2(psi[i], e);
+    }
+    __syncthreads();
+    for (int k = 0; k < pr.L; ++k) {
+      fx_apply<128>(X, X, GX + 16 * k, pair_bits(n - 1 - pairs[2 * k], n - 1 - pairs[2 * k + 1]), false, E >> 2, n);
+      __syncthreads();
+    }
+    double acc = 0.0;
+    for (int i = tid; i < E; i += 128) {
+      const int r = i / M, j = i - r * M;
+      const int4 x = X[swz(((uint32_t)j << n) | (uint32_t)r, fold)], y = fx_from2(phil[i], e);
+      const double dx = (double)(fx_value(y.x, y.y) - fx_value(x.x, x.y)), dy = (double)(fx_value(y.z, y.w) - fx_value(x.z, x.w));
+      acc = fma(dx, dx, fma(dy, dy, acc));
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if (lane == 0) red[warp] = acc;
+    __syncthreads();
+    c = ldexp((red[0] + red[1]) + (red[2] + red[3]), 2 * (e - kFxBits)) / M;
+  } else {
+    __syncthreads();
+    if (warp == 0) {
+      c = cost64();
+      if (lane == 0) red[0] = c;
+    }
+    __syncthreads();
+    c = red[0];
   }
-  for (int i = lane; i < 16 * pr.L; i += 32) a.gates_out[pr.gate_out_off + i] = G[i];
-  if (lane == 0) {
+  int refine = 0;
+  if (warp == 0) {
+    while (c > a.tol && refine < a.refine_max && (sst != INT_MAX || a.refine_unconverged)) {
+      warp_sweep64(Bs, Ph, G, psi, phil, pairs, n, M, pr.L, nw[0].polar);
+      ++refine;
+      c = cost64();
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < 16 * pr.L; i += 128) a.gates_out[pr.gate_out_off + i] = G[i];
+  if (tid == 0) {
     a.res_cost[p] = c;
     a.res_sweeps[p] = sweeps;
     a.res_best[p] = best;
@@ -727,7 +637,9 @@ __global__ void k_batch_finalize(BatchArgs a) {
 }
 
 void launch_batch_prep(const BatchArgs& a, cudaStream_t st) {
-  k_batch_prep<<<a.P, 128, 0, st>>>(a);
+  const size_t smem = (size_t)a.max_prep * sizeof(int4);
+  cudaFuncSetAttribute(k_batch_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_batch_prep<<<a.P, 128, smem, st>>>(a);
 }
 
 int batch_region_f2(int G, int max_elems, int max_L) { return (32 / G) * batch_slice_f2(max_elems, max_L); }
@@ -771,9 +683,9 @@ void launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int n
 }
 
 void launch_batch_finalize(const BatchArgs& a, cudaStream_t st) {
-  const size_t smem = (size_t)(2 * a.max_elems + 16 * a.max_L) * sizeof(double2);
+  const size_t smem = (size_t)(3 * a.max_elems + 32 * a.max_L) * sizeof(double2);
   cudaFuncSetAttribute(k_batch_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_batch_finalize<<<a.P, 32, smem, st>>>(a);
+  k_batch_finalize<<<a.P, 128, smem, st>>>(a);
 }
 
 }  // namespace qfs

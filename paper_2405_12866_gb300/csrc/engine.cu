@@ -2401,7 +2401,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
                 p->training_distribution);
   std::vector<BatchProblem> probs(P);
   long long pair_off = 0, state_off = 0, target_off = 0, gate_off = 0, gout_off = 0;
-  int max_elems = 0, max_L = 0;
+  int max_elems = 0, max_L = 0, max_prep = 0;
   for (int i = 0; i < P; ++i) {
     const int n = ns[i], L = Ls[i];
     if (n < 2 || n > 6) return fail(QFS_EUNSUPPORTED, "problem %d: n = %d (batched form: 2..6)", i, n);
@@ -2419,6 +2419,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
     gout_off += (long long)L * 16;
     max_elems = std::max(max_elems, N * M);
     max_L = std::max(max_L, L);
+    max_prep = std::max(max_prep, N * N + N * M);
   }
   TRY(ctx_check(ctx));
   TRY(set_device(ctx));
@@ -2485,6 +2486,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
   a.min_sweeps = p->min_sweeps;
   a.max_elems = max_elems;
   a.max_L = max_L;
+  a.max_prep = max_prep;
   a.gates_out = reinterpret_cast<double2*>(w + o_gout);
   a.res_cost = reinterpret_cast<double*>(w + o_rc);
   a.res_sweeps = reinterpret_cast<int*>(w + o_rs);

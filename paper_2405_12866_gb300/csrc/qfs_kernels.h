@@ -280,6 +280,7 @@ struct BatchArgs {
   double diff_tol_r;      //   improvement > diff_tol_r (App. A), once min_sweeps have run
   int min_sweeps;
   int max_elems, max_L;   // largest N*M and L in the batch (shared-memory slices)
+  int max_prep;           // largest N*N + N*M (the set-up's shared memory)
   double2* gates_out;     // selected gates, FP64 (L x 16 per problem)
   double* res_cost;
   int* res_sweeps;
