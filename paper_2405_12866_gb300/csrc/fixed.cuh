@@ -35,7 +35,7 @@ __device__ __forceinline__ int2 fx_from(double x, int e) {
   const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
   long long m = ((long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
   const int sh = ex - 1075 + kFxBits - e;
-  if (sh >= 0) m = m << min(sh, 10);
+  if (sh >= 0) m = ex == 0 ? 0 : m << min(sh, 10);
   else m = sh < -54 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
   return fx_split(hi < 0 ? -m : m);
 }
@@ -43,6 +43,10 @@ __device__ __forceinline__ int4 fx_from2(double2 z, int e) {
   const int2 x = fx_from(z.x, e), y = fx_from(z.y, e);
   return int4{x.x, x.y, y.x, y.y};
 }
+// Whether exponent field t of a matrix' largest entry (0: all zeros) is too far
+// out for products scaled back by scale_exp (which knows neither overflow nor
+// denormals); so are Inf and NaN.
+__device__ __forceinline__ bool fx_out_of_range(int t) { return t != 0 && (t < 500 || t > 1500); }
 // acc + a b of 32-bit numbers, in 64 bits.
 __device__ __forceinline__ long long mad64(int a, int b, long long acc) { return (long long)a * b + acc; }
 // A sum of products of fixed-point numbers: high x high, and the cross terms

@@ -670,7 +670,8 @@ void launch_cast_c128_to_c64(const double2* in, float2* out, long long count, cu
   k_cast<<<(int)blocks, 256, 0, st>>>(in, out, count);
 }
 
-__global__ void k_nonfinite(const double* x, long long count, int* flag) {
+__global__ void k_nonfinite(const double* x, long long count, int* flag, const int* only_if) {
+  if (only_if != nullptr && *only_if == 0) return;
   int bad = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
        i += (long long)gridDim.x * blockDim.x) {
@@ -680,11 +681,11 @@ __global__ void k_nonfinite(const double* x, long long count, int* flag) {
   if (__any_sync(FULL, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
 }
 
-void launch_nonfinite_check(const double* x, long long count, int* flag, cudaStream_t st) {
+void launch_nonfinite_check(const double* x, long long count, int* flag, cudaStream_t st, const int* only_if) {
   if (count <= 0) return;
   long long blocks = (count + 255) / 256;
   if (blocks > 2048) blocks = 2048;
-  k_nonfinite<<<(int)blocks, 256, 0, st>>>(x, count, flag);
+  k_nonfinite<<<(int)blocks, 256, 0, st>>>(x, count, flag, only_if);
 }
 
 }  // namespace qfs

@@ -74,18 +74,25 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, unsigned parity) {
 }
 
 // The digits of two numbers |x| < 2 as seven f16 pairs, most significant first.
+// The kernel's producers are bound by these instructions, so: two 32-bit
+// funnel shifts instead of a 64-bit shift by a variable, no conversions.
 __device__ __forceinline__ void digits2(double x0, double x1, uint32_t (&d)[kDig]) {
   unsigned long long t[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const double x = k ? x1 : x0;
-    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
-    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
-    const int sh = 1021 - ex;  // x = m 2^(ex - 1075): m 2^(ex - 1021) in units of 2^-54
-    const unsigned long long v = sh <= 0 ? m << min(-sh, 3) : sh > 60 ? 0 : (m + (1ULL << (sh - 1))) >> sh;
+    const int h = __double2hiint(x);
+    const uint32_t l = (uint32_t)__double2loint(x), mh = ((uint32_t)h & 0xfffffu) | 0x100000u;
+    // |x| 2^55 = (m << 3) >> (1023 - exponent field) for the 53-bit mantissa m.
+    const uint32_t m1 = mh << 3 | l >> 29, m0 = l << 3;
+    const int sh = min(max(1023 - ((h >> 20) & 0x7ff), 0), 63);
+    const bool far = sh >= 32;
+    const uint32_t a1 = far ? 0u : m1, a0 = far ? m1 : m0;
+    const unsigned long long y = (unsigned long long)(a1 >> (sh & 31)) << 32 | __funnelshift_r(a0, a1, sh);
+    const unsigned long long v = (y + 1) >> 1;  // rounded to 2^-54
     // Plus 128 in every byte: the bytes are the digits plus 128 (the top one,
     // which may need a ninth bit, is taken from the upper bits).
-    t[k] = (hi < 0 ? 0 - v : v) + 0x0080808080808080ULL;
+    t[k] = (h < 0 ? 0 - v : v) + 0x0080808080808080ULL;
   }
   const uint32_t l0 = (uint32_t)t[0], l1 = (uint32_t)t[1], h0 = (uint32_t)(t[0] >> 32), h1 = (uint32_t)(t[1] >> 32);
   // f16 0x6400 | b is 1024 + b; minus 1152 leaves the digit.
@@ -105,6 +112,14 @@ __device__ __forceinline__ void digits2(double x0, double x1, uint32_t (&d)[kDig
   put(4, l0, l1, 2);
   put(5, l0, l1, 1);
   put(6, l0, l1, 0);
+}
+
+// x rounded toward zero to FP32 (zero below 2^-126), from its bits: an FP64
+// conversion occupies the FP64 pipe.
+__device__ __forceinline__ float trunc32(double x) {
+  const int h = __double2hiint(x), f = ((h >> 20) & 0x7ff) - 896;
+  const uint32_t m = ((uint32_t)h & 0xfffffu) << 3 | (uint32_t)__double2loint(x) >> 29;
+  return __uint_as_float(f <= 0 ? 0u : (uint32_t)min(f, 255) << 23 | m);  // (Inf or NaN stays one; the sign is not wanted)
 }
 
 // K-major operand without swizzle: 8 rows x 16 bytes are contiguous, `lead`
@@ -148,14 +163,15 @@ __device__ __forceinline__ void tmem_zero16(uint32_t addr) {
 
 // Psi's digits in the order of the product kernel's stages: [column block]
 // [step][K group of 8][digit][column][8].  Block j takes column j of Psi
-// (j >= M: zeros that fill up the last column block); expo[j] its scale.
-// Block 0 also zeroes the row norms and the flag.
+// (j >= M: zeros that fill up the last column block) and a chunk of the rows
+// (blockIdx.y; all of them look over the whole column for its scale expo[j]).
+// Block (0, 0) also zeroes the flag.
 __global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi, int N, int M, int NB, __half* dig, int* expo,
                                                   float* row2, int* flag) {
   const int j = blockIdx.x, tid = threadIdx.x;
-  if (row2 != nullptr)
-    for (int i = blockIdx.x * blockDim.x + tid; i < N; i += gridDim.x * blockDim.x) row2[i] = 0.f;
-  if (j == 0 && tid == 0) *flag = 0;
+  for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + tid; i < N; i += gridDim.x * gridDim.y * blockDim.x)
+    row2[i] = 0.f;
+  if (j == 0 && blockIdx.y == 0 && tid == 0) *flag = 0;
   int top = 0;  // exponent field of the column's largest entry
   if (j < M)
     for (int i = tid; i < N; i += 256) {
@@ -168,16 +184,15 @@ __global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi
   __syncthreads();
   for (int w = 0; w < 8; ++w) top = max(top, red[w]);
   const int e = top == 0 ? 0 : top - 1022;  // entries times 2^-e are below 1
-  if (tid == 0) {
-    expo[j] = e;
-    if (top >= 2046) atomicOr(flag, 1);  // Inf, NaN or next to them: the FP64 kernel
-  }
+  // (Far out, Inf or NaN: 2^20 stands for it, and the FP64 kernel runs.)
+  if (tid == 0 && blockIdx.y == 0) expo[j] = top != 0 && (top < 100 || top > 1900) ? 1 << 20 : e;
   auto scaled = [&](double x) {
     const int hi = __double2hiint(x), f = (hi >> 20) & 0x7ff;
     return f == 0 || f - e <= 0 ? 0.0 : __hiloint2double(hi - (e << 20), __double2loint(x));
   };
   const int c0 = 2 * j, cb = c0 / NB, c = c0 % NB, steps = 2 * N / kOzK;
-  for (int g = tid; g < N / 4; g += 256) {  // a group: 4 complex rows, 8 reals
+  const int g0 = (int)((long long)blockIdx.y * (N / 4) / gridDim.y), g1 = (int)((long long)(blockIdx.y + 1) * (N / 4) / gridDim.y);
+  for (int g = g0 + tid; g < g1; g += 256) {  // a group: 4 complex rows, 8 reals
     double2 z[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -292,12 +307,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const double* u1 = u0 + 64LL * 2 * N;
     double2 x[2][4];
     float n0 = 0.f, n1 = 0.f;
-    auto load = [&](int k) {
+    auto load = [&](int h, int k) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        x[0][q] = __ldg(reinterpret_cast<const double2*>(u0 + (long long)k * kOzK) + q);
-        x[1][q] = __ldg(reinterpret_cast<const double2*>(u1 + (long long)k * kOzK) + q);
-      }
+      for (int q = 0; q < 4; ++q) x[h][q] = __ldg(reinterpret_cast<const double2*>((h ? u1 : u0) + (long long)k * kOzK) + q);
     };
     const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * HC);
     long long hi[HC];
@@ -331,7 +343,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     zero(0, 8);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     bar_arrive(accfree);
-    if (nk > 0) load(k0);
+    if (nk > 0) {
+      load(0, k0);
+      load(1, k0);
+    }
     for (int i = 0; i < nk; ++i) {
       const int s = i & 1;
       ok = bar_wait(&empty[s], ((unsigned)(i >> 1) & 1u) ^ 1u) && !*gave_up;
@@ -351,15 +366,16 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           digits2(x[h][q].x, x[h][q].y, d[q]);
-          const float fx = (float)x[h][q].x, fy = (float)x[h][q].y;
+          const float fx = trunc32(x[h][q].x), fy = trunc32(x[h][q].y);
           (h ? n1 : n0) = fmaf(fx, fx, fmaf(fy, fy, h ? n1 : n0));
         }
 #pragma unroll
         for (int p = 0; p < kDig; ++p)
           *reinterpret_cast<uint4*>(st + p * 128 * kOzK * 2 + k8 * 128 * 16 + (r + 64 * h) * 16) =
               make_uint4(d[0][p], d[1][p], d[2][p], d[3][p]);
+        // This row's next numbers, at once: 32 KB a CTA stay in flight.
+        if (i + 1 < nk) load(h, k0 + i + 1);
       }
-      if (i + 1 < nk) load(k0 + i + 1);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       bar_arrive(&full[s]);
       // The previous chunk's sums, with this step's operands already staged.
@@ -440,18 +456,19 @@ __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__
     im += v.y;
   }
   const int e = expo[j];
-  out[i] = double2{ldexp((double)re, e - 54), ldexp((double)im, e - 54)};
+  out[i] = double2{scale_exp((double)re, e - 54), scale_exp((double)im, e - 54)};
   if (j == 0) {
     const float n2 = row2[row];
     if (!(n2 > 0.81f && n2 < 1.21f)) atomicOr(flag, 1);
   }
+  if (e == 1 << 20 && row == 0) atomicOr(flag, 1);
 }
 
 // out = U Psi for N <= 64 rows: grid (N / 8 row tiles (at least 1), column tiles
 // of 32).  Scales from the largest entries of the block's rows of U and columns
 // of Psi, with room for 2 N terms: the high sums stay below 2^62, each cross sum
-// below 2^62 and both together below 2^63.  Entries next to FP64's largest
-// exponent, Inf and NaN take FP64 arithmetic.
+// below 2^62 and both together below 2^63.  Entries far from 1, Inf and NaN take
+// FP64 arithmetic.
 constexpr int kFxRows = 8, kFxCols = 32;
 __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ U, const double2* __restrict__ Psi,
                                                     double2* __restrict__ out, int n, int M) {
@@ -477,7 +494,7 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
     tu = max(tu, red[0][w]);
     tp = max(tp, red[1][w]);
   }
-  const bool plain = tu >= 2040 || tp >= 2040;
+  const bool plain = fx_out_of_range(tu) || fx_out_of_range(tp);
   const int eu = tu - 1022 + n - 1, ep = tp - 1022 + max(n - 2, 1);
   if (!plain) {
     for (int i = tid; i < rows * N; i += 256) su[i] = fx_from2(U[(long long)r0 * N + i], eu);
@@ -530,6 +547,11 @@ OzShape oz_shape(int N, int M, int num_sms) {
 
 size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 128 ? 0 : oz_shape(N, M, num_sms).total; }
 
+const int* oz_flag(const void* scratch, int N, int M, int num_sms) {
+  const OzShape s = oz_shape(N, M, num_sms);
+  return reinterpret_cast<const int*>(static_cast<const char*>(scratch) + s.dig + s.part + s.row2);
+}
+
 cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
                               int num_sms, cudaStream_t st) {
   const OzShape s = oz_shape(N, M, num_sms);
@@ -542,7 +564,7 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
   cudaError_t e = cudaFuncSetAttribute(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem(s.nb));
   if (e != cudaSuccess) return e;
-  k_oz_prep<<<s.cblocks * s.nb / 2, 256, 0, st>>>(Psi, N, M, s.nb, dig, expo, row2, flag);
+  k_oz_prep<<<dim3(s.cblocks * s.nb / 2, std::max(1, std::min(16, N / 512))), 256, 0, st>>>(Psi, N, M, s.nb, dig, expo, row2, flag);
   const dim3 grid(N / 128, s.splits, s.cblocks);
   if (s.nb == 64) k_oz_product<64><<<grid, kOzThreads, oz_smem(64), st>>>((const double*)U, dig, N, part, row2, err);
   else k_oz_product<32><<<grid, kOzThreads, oz_smem(32), st>>>((const double*)U, dig, N, part, row2, err);

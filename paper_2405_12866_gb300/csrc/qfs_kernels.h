@@ -231,6 +231,9 @@ void launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N,
 // The same product, for N >= 128, from 8-bit digits on the tensor cores
 // (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1.
 // err: device word, bit 0 set when a bounded wait ran out.
+// The word in its scratch that is not zero, once it has run, when the FP64 kernel
+// ran too: for one, whenever U or Psi holds Inf or NaN.
+const int* oz_flag(const void* scratch, int N, int M, int num_sms);
 // The same for n <= 6 in 64-bit fixed point.
 void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st);
 size_t oz_scratch_bytes(int N, int M, int num_sms);
@@ -239,8 +242,9 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
 
 void launch_cast_c128_to_c64(const double2* in, float2* out, long long count, cudaStream_t st);
 
-// flag[0] |= 1 when any of the `count` doubles is NaN or infinite.
-void launch_nonfinite_check(const double* x, long long count, int* flag, cudaStream_t st);
+// flag[0] |= 1 when any of the `count` doubles is NaN or infinite.  only_if
+// (nullable, device): nothing is read when it holds zero.
+void launch_nonfinite_check(const double* x, long long count, int* flag, cudaStream_t st, const int* only_if = nullptr);
 
 // ---------------------------------------------------------------- batches
 

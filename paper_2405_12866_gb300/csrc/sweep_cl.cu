@@ -870,7 +870,7 @@ __global__ void k_cl_scale(int N, int M, int gates, const double2* psi, const do
       a = fmaf(ux, ux, fmaf(uy, uy, a));
       b = fmaf(vx, vx, fmaf(vy, vy, b));
     }
-    __shared__ float s[2][8];
+    __shared__ float s[2][32];
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) {
       a += __shfl_xor_sync(FULL, a, m);
@@ -933,7 +933,8 @@ __global__ void k_cl_scale(int N, int M, int gates, const double2* psi, const do
 void launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
                      int4* out, cudaStream_t st) {
   cudaMemsetAsync(acc, 0, 4 * sizeof(unsigned), st);
-  k_cl_scale<<<M + (gates + 255) / 256, 256, 0, st>>>(1 << n, M, gates, psi, phil, g, acc, out);
+  const int nt = n >= 11 ? 1024 : 256;
+  k_cl_scale<<<M + (gates + nt - 1) / nt, nt, 0, st>>>(1 << n, M, gates, psi, phil, g, acc, out);
 }
 
 ClPlan cl_plan(Real r, int n, int M, int L, int spt, bool keep64) {

@@ -70,11 +70,14 @@ def test_product_of_structured_targets(ctx, n, what):
 
 
 @pytest.mark.parametrize("n", [5, 8])
-@pytest.mark.parametrize("what", ["target_times_2", "target_times_1e-9", "one_row_times_3", "columns_of_all_sizes"])
+@pytest.mark.parametrize("what", ["target_times_2", "target_times_1e-9", "one_row_times_3", "columns_of_all_sizes", "no_states",
+                                  "tiny_states", "huge_states"])
 def test_product_of_inputs_without_unit_norms(ctx, n, what):
     U, Psi = _brick(n), w.sample_states(6, n, 8).copy()
     if what == "columns_of_all_sizes" and n >= 7:
         Psi *= np.array([1, 1e-200, 0, 1e100, 1e-3, 7, 1e8, 1])[None, :]
+    elif what.endswith("_states"):
+        Psi *= {"no": 0.0, "tiny": 1e-290, "huge": 1e290}[what.split("_")[0]]
     elif what == "one_row_times_3":
         U[3] *= 3
     elif what != "columns_of_all_sizes":
