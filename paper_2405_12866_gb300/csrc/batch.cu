@@ -27,6 +27,9 @@
 #include "qfs_kernels.h"
 
 #include <climits>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 namespace qfs {
 
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(128) k_batch_prep(BatchArgs a) {
     a.psi32[pr.state_off + e] = float2{(float)s.x, (float)s.y};
   }
   const int tu = block_exponent(U, N * N, red), tp = block_exponent(psi, N * M, red);
-  if (tu >= 2040 || tp >= 2040) {
+  if (fx_out_of_range(tu) || fx_out_of_range(tp)) {
     for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
       const int i = e / M, j = e - i * M;
       double2 acc{0.0, 0.0};
@@ -585,7 +588,7 @@ __global__ void __launch_bounds__(128) k_batch_finalize(BatchArgs a) {
     for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
     return acc / M;
   };
-  if (top < 2040) {
+  if (!fx_out_of_range(top)) {
     const int e = top - 1022 + 3;
     const uint32_t fold = swz_fold(n);
     for (int i = tid; i < E; i += 128) {
@@ -661,19 +664,38 @@ int blocks_per_sm_g(int warps, size_t smem) {
 }
 }  // namespace
 
+// (Asked about 180 times a call of a thousand problems in 21 classes; the driver's
+// two calls behind an answer took 190 us of the call together, so answers are
+// kept, by device and launch shape.)
 int batch_sweep_blocks_per_sm(int G, int warps, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, size_t>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const auto key = std::make_tuple(dev, G, warps, smem);
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  int b = 0;
   switch (G) {
-    case 4: return blocks_per_sm_g<4>(warps, smem);
-    case 8: return blocks_per_sm_g<8>(warps, smem);
-    case 16: return blocks_per_sm_g<16>(warps, smem);
-    case 32: return blocks_per_sm_g<32>(warps, smem);
-    default: return 0;
+    case 4: b = blocks_per_sm_g<4>(warps, smem); break;
+    case 8: b = blocks_per_sm_g<8>(warps, smem); break;
+    case 16: b = blocks_per_sm_g<16>(warps, smem); break;
+    case 32: b = blocks_per_sm_g<32>(warps, smem); break;
+    default: break;
   }
+  if (known.size() >= 4096) known.clear();
+  known[key] = b;
+  return b;
 }
 
 void launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
                         int warps, int region_f2, cudaStream_t st) {
   const size_t smem = (size_t)warps * region_f2 * sizeof(float2);
+  const void* kernels[4] = {(const void*)k_batch_sweep<4>, (const void*)k_batch_sweep<8>, (const void*)k_batch_sweep<16>,
+                            (const void*)k_batch_sweep<32>};
+  cudaFuncSetAttribute(kernels[G == 4 ? 0 : G == 8 ? 1 : G == 16 ? 2 : 3], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)smem);
   switch (G) {
     case 4: k_batch_sweep<4><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
     case 8: k_batch_sweep<8><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
