@@ -81,6 +81,21 @@ class Result(C.Structure):
                 ("best_start", C.c_int32), ("fp64_sweeps", C.c_int32), ("training_states", C.c_int32)]
 
 
+# The same records as a numpy array (columns out of thousands of them in one go:
+# reading a ctypes structure field by field costs a microsecond a problem).
+_RESULT = np.dtype([("cost", "f8"), ("sweeps", "i4"), ("converged", "i4"), ("best_start", "i4"),
+                    ("fp64_sweeps", "i4"), ("training_states", "i4")], align=True)
+
+
+def _result_dicts(res) -> list:
+    """One dict per record of a Result array."""
+    r = np.frombuffer(res, dtype=_RESULT, count=len(res))
+    return [{"cost": c, "sweeps": s, "converged": v, "best_start": b, "fp64_sweeps": f, "training_states": t}
+            for c, s, v, b, f, t in zip(r["cost"].tolist(), r["sweeps"].tolist(), (r["converged"] != 0).tolist(),
+                                        r["best_start"].tolist(), r["fp64_sweeps"].tolist(),
+                                        r["training_states"].tolist())]
+
+
 _lib = None
 _P = C.c_void_p
 _D = C.POINTER(C.c_double)
@@ -411,9 +426,7 @@ class Context:
                                            targets.ctypes.data, sm.ctypes.data if sm is not None else None,
                                            ig.ctypes.data if ig is not None else None, C.byref(params),
                                            out.ctypes.data, res))
-        info = [dict(cost=r.cost, sweeps=r.sweeps, converged=bool(r.converged), best_start=r.best_start,
-                     fp64_sweeps=r.fp64_sweeps, training_states=r.training_states) for r in res]
-        return out, info
+        return out, _result_dicts(res)
 
     def batch_schedules(self):
         """The batched form's tuned shapes: (list of dicts per class, list of
@@ -479,9 +492,7 @@ class Context:
         _check(lib().qfs_instantiate_batch(self._h, P, ns.ctypes.data, Ls.ctypes.data, pr.ctypes.data,
                                            t.ctypes.data, None, ig.ctypes.data if ig is not None else None,
                                            C.byref(params), out.ctypes.data, res))
-        r = np.frombuffer(res, dtype=np.dtype([("cost", "f8"), ("sweeps", "i4"), ("converged", "i4"),
-                                                ("best_start", "i4"), ("fp64_sweeps", "i4"),
-                                                ("training_states", "i4")], align=True), count=P)
+        r = np.frombuffer(res, dtype=_RESULT, count=P)
         return out, r["cost"].copy(), r["sweeps"].copy(), r["converged"].astype(bool), r["best_start"].copy()
 
     def instantiate_batch_dev(self, ns, Ls, pairs, targets, samples, init_gates, params: Params, out):
@@ -496,8 +507,10 @@ class Context:
         _check(lib().qfs_instantiate_batch_dev(self._h, P, ns.ctypes.data, Ls.ctypes.data, pairs.ctypes.data,
                                                targets.data_ptr(), samples.data_ptr(), init_gates.data_ptr(),
                                                C.byref(params), out.data_ptr(), res))
-        return [dict(cost=r.cost, sweeps=r.sweeps, converged=bool(r.converged), best_start=r.best_start,
-                     fp64_sweeps=r.fp64_sweeps) for r in res]
+        info = _result_dicts(res)
+        for r in info:
+            del r["training_states"]  # (the host entry's record has it)
+        return info
 
     def gemm_bf16(self, A, B, bias=None, gelu=False, want_f32=True, want_bf16=False, M_valid=0):
         """C = A B^T (+ bias, GELU) for bf16 CUDA tensors A (M x K), B (N x K)."""
@@ -649,9 +662,7 @@ class WarmStart:
         st = (C.c_int64 * 4)()
         _check(lib().qfs_ws_instantiate(self._h, P, t.ctypes.data, fg.ctypes.data if fg is not None else None,
                                         C.byref(params), first_sweeps, out.ctypes.data, res, st))
-        r = np.frombuffer(res, dtype=np.dtype([("cost", "f8"), ("sweeps", "i4"), ("converged", "i4"),
-                                                ("best_start", "i4"), ("fp64_sweeps", "i4"),
-                                                ("training_states", "i4")], align=True), count=P).copy()
+        r = np.frombuffer(res, dtype=_RESULT, count=P).copy()
         return out, r, dict(first_converged=int(st[0]), first_start_sweeps=int(st[1]),
                             fallback_start_sweeps=int(st[2]), fallback_targets=int(st[3]))
 
