@@ -295,6 +295,7 @@ struct Run {
   double* df_resid = nullptr;
   int df_cap = 0;           // steps the table holds
   int df_max_nchunk = 0;    // largest chunks per start of any step
+  int df_part_len = 32;     // partial sums of a chunk
   int df_nsteps = 0;
   long long df_items = 0;
   double df_bytes = 0.0;    // algorithmic bytes of one dataflow sweep (all starts)
@@ -356,7 +357,8 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
   R.df_steps = (DfStep*)take((size_t)std::max(R.df_cap, 1) * sizeof(DfStep));
   R.df_ctrl_cap = 1 + ((size_t)R.df_cap + 1) * R.S;
   R.df_ctrl = (unsigned*)take(sizeof(unsigned) * 2 * R.df_ctrl_cap);  // two slots: this sweep's, the next's
-  R.df_partials = (double*)take(sizeof(double) * 32 * (size_t)R.S * std::max(R.df_max_nchunk, 1));
+  R.df_partials = (double*)take(std::max(sizeof(double) * 32, sizeof(float) * R.df_part_len) * (size_t)R.S *
+                                std::max(R.df_max_nchunk, 1));
   // The residual pass keeps its double partials apart: in complex64 the
   // environment partials are floats, and one start's residual slots would
   // overlap another start's environment slots while that start still sweeps.
@@ -476,77 +478,10 @@ void df_build(const qfs_ctx* ctx, const Run& R, Real r, const void* psi, const v
     df_chunking(st, bytes_per_unit, target);
     *bytes += bytes_per_unit * st.units * S;
   };
-  // Forward: gates k and k+1 on four distinct qubits go in one step (B_k is
-  // then written but not read back), others one at a time.
-  for (int k = 1; k <= L - 1;) {
-    DfStep st{};
-    st.in = k == 1 ? psi : B_ptr(k - 1);
-    st.in_stride = k == 1 ? 0 : sN;
-    st.in_gstride = k == 1 ? sN : 0;
-    st.out = B_ptr(k);
-    st.gate = gate_ptr(k - 1);
-    st.gate_stride = gstride;
-    const int a1 = R.pairs[2 * (k - 1)], b1 = R.pairs[2 * (k - 1) + 1];
-    bool two = ctx->df_fwd2 && k + 1 <= L - 1;
-    if (two) {
-      const int a2 = R.pairs[2 * k], b2 = R.pairs[2 * k + 1];
-      two = a2 != a1 && a2 != b1 && b2 != a1 && b2 != b1;
-      if (two) st.bg = make_bwd_geom(n, M, a1, b1, a2, b2);
-    }
-    if (two) {
-      st.kind = DF_FWD2;
-      st.out2 = B_ptr(k + 1);
-      st.gate2 = gate_ptr(k);
-      st.units = (1 << (n - 4)) * (M / vec);
-      chunk_it(st, 16.0 * vec * es * 3.0);
-      k += 2;
-    } else {
-      st.kind = DF_FWD;
-      st.fg = make_geom(n, M, a1, b1);
-      st.units = (1 << (n - 2)) * (M / vec);
-      chunk_it(st, 4.0 * vec * es * 2.0);
-      k += 1;
-    }
-    steps.push_back(st);
-  }
-  for (int k = L; k >= 1; --k) {
-    DfStep st{};
-    const int qa = R.pairs[2 * (k - 1)], qb = R.pairs[2 * (k - 1) + 1];
-    int ua = qa, ub = qb;
-    st.in = k == 1 ? psi : B_ptr(k - 1);
-    st.in_stride = k == 1 ? 0 : sN;
-    st.in_gstride = k == 1 ? sN : 0;
-    if (k == L) {
-      st.phi_in = phil;
-      st.phi_in_stride = 0;
-      st.phi_in_gstride = sN;
-      st.phi_out = nullptr;
-      st.gate = nullptr;
-    } else {
-      st.phi_in = k == L - 1 ? phil : R.phi;
-      st.phi_in_stride = k == L - 1 ? 0 : sN;
-      st.phi_in_gstride = k == L - 1 ? sN : 0;
-      st.phi_out = R.phi;
-      st.gate = gate_ptr(k);
-      ua = R.pairs[2 * k];
-      ub = R.pairs[2 * k + 1];
-    }
-    st.gate_stride = gstride;
-    st.bg = make_bwd_geom(n, M, ua, ub, qa, qb);
-    const int U = st.bg.U, ea = st.bg.ea, eb = st.bg.eb;
-    int v = vec;
-    if (U == 4) st.kind = DF_BWD4;
-    else if (U == 2) st.kind = ea == 1 ? DF_BWD2_10 : DF_BWD2_01;
-    else {
-      v = 1;
-      st.kind = ea == 2 ? DF_BWD3_20 : eb == 2 ? DF_BWD3_02 : ea == 1 ? DF_BWD3_10 : DF_BWD3_01;
-    }
-    st.units = (1 << (n - U)) * (M / v);
-    // Phi_k is stored by every backward step but the first (k = L).
-    chunk_it(st, (double)(1 << U) * v * es * (k < L ? 3.0 : 2.0));
-    UpdateArgs& u = st.upd;
+  auto update_args = [&](int k, int nblk) {
+    UpdateArgs u{};
     u.partials = R.df_partials;
-    u.nblk = st.nchunk;  // (the dataflow kernel sums the chunk slots itself)
+    u.nblk = nblk;  // (the dataflow kernel sums the chunk slots itself)
     u.partials_f32 = r == R32;
     u.g64 = R.g64 ? R.g64 + (size_t)(k - 1) * 16 : nullptr;
     u.g_stride = gstride;
@@ -561,19 +496,161 @@ void df_build(const qfs_ctx* ctx, const Run& R, Real r, const void* psi, const v
     u.S = S;
     u.active = active;
     u.vprev = vprev ? vprev + (size_t)(k - 1) * 16 : nullptr;
+    return u;
+  };
+  auto distinct = [&](int k) {  // gates k and k + 1 on four distinct qubits
+    const int a1 = R.pairs[2 * (k - 1)], b1 = R.pairs[2 * (k - 1) + 1], a2 = R.pairs[2 * k], b2 = R.pairs[2 * k + 1];
+    return a2 != a1 && a2 != b1 && b2 != a1 && b2 != b1;
+  };
+  // Groups of gates, in circuit order: {k} or {k, k + 1} on four distinct
+  // qubits.  complex64 sweeps take both gates of a group in one backward step;
+  // FP64 sweeps do not (the doubled arithmetic of that step would cost more
+  // than the pass over memory it saves).  Paired from the end, so that a gate
+  // left over is gate 1, whose step the residual continues.
+  const bool pairs = r == R32 && ctx->df_fwd2;
+  std::vector<std::pair<int, int>> groups;  // first gate, gates
+  if (pairs) {
+    for (int k = L; k >= 1;) {
+      const int len = k >= 2 && distinct(k - 1) ? 2 : 1;
+      groups.insert(groups.begin(), {k - len + 1, len});
+      k -= len;
+    }
+  } else {
+    for (int k = 1; k <= L - 1;) {
+      const int len = ctx->df_fwd2 && k + 1 <= L - 1 && distinct(k) ? 2 : 1;
+      groups.push_back({k, len});
+      k += len;
+    }
+    groups.push_back({L, 1});
+  }
+  // Forward: all groups but the last, a step each.
+  for (size_t gi = 0; gi + 1 < groups.size(); ++gi) {
+    const auto [k, len] = groups[gi];
+    DfStep st{};
+    st.in = k == 1 ? psi : B_ptr(k - 1);
+    st.in_stride = k == 1 ? 0 : sN;
+    st.in_gstride = k == 1 ? sN : 0;
+    st.gate = gate_ptr(k - 1);
+    st.gate_stride = gstride;
+    const int a1 = R.pairs[2 * (k - 1)], b1 = R.pairs[2 * (k - 1) + 1];
+    if (len == 2) {
+      st.kind = DF_FWD2;
+      st.bg = make_bwd_geom(n, M, a1, b1, R.pairs[2 * k], R.pairs[2 * k + 1]);
+      st.out = pairs ? nullptr : B_ptr(k);  // (a pair's environments need B_{k-1} only)
+      st.out2 = B_ptr(k + 1);
+      st.gate2 = gate_ptr(k);
+      st.units = (1 << (n - 4)) * (M / vec);
+      chunk_it(st, 16.0 * vec * es * (pairs ? 2.0 : 3.0));
+    } else {
+      st.kind = DF_FWD;
+      st.out = B_ptr(k);
+      st.fg = make_geom(n, M, a1, b1);
+      st.units = (1 << (n - 2)) * (M / vec);
+      chunk_it(st, 4.0 * vec * es * 2.0);
+    }
     steps.push_back(st);
+  }
+  // Backward.  Phi starts as U Psi, shared by a target's starts, and is the
+  // start's own from the first step that stores it on.
+  bool own = false;
+  int pending = 0;  // gate whose adjoint Phi still lacks
+  auto phi_from = [&](DfStep& st) {
+    st.phi_in = own ? R.phi : phil;
+    st.phi_in_stride = own ? sN : 0;
+    st.phi_in_gstride = own ? 0 : sN;
+  };
+  auto carry = [&](int k, int len, int resid) {  // Phi past gates k .. k + len - 1
+    DfStep st{};
+    st.in = own ? R.phi : phil;
+    st.in_stride = own ? sN : 0;
+    st.in_gstride = own ? 0 : sN;
+    st.adj = 1;
+    st.resid = resid;
+    st.gate_stride = gstride;
+    if (len == 2) {
+      st.kind = DF_FWD2;
+      st.bg = make_bwd_geom(n, M, R.pairs[2 * k], R.pairs[2 * k + 1], R.pairs[2 * (k - 1)], R.pairs[2 * (k - 1) + 1]);
+      st.gate = gate_ptr(k);
+      st.gate2 = gate_ptr(k - 1);
+      st.out2 = R.phi;
+      st.units = (1 << (n - 4)) * (M / vec);
+      chunk_it(st, 16.0 * vec * es * 2.0);
+    } else {
+      st.kind = DF_FWD;
+      st.fg = make_geom(n, M, R.pairs[2 * (k - 1)], R.pairs[2 * (k - 1) + 1]);
+      st.gate = gate_ptr(k - 1);
+      st.out = R.phi;
+      st.units = (1 << (n - 2)) * (M / vec);
+      chunk_it(st, 4.0 * vec * es * 2.0);
+    }
+    steps.push_back(st);
+    own = true;
+  };
+  std::vector<std::pair<int, int>> back;  // backward groups, in the order they run
+  for (int k = L; k >= 1;) {
+    const int len = pairs && k >= 2 && distinct(k - 1) ? 2 : 1;
+    back.push_back({k - len + 1, len});
+    k -= len;
+  }
+  for (const auto& [k0, len] : back) {
+    DfStep st{};
+    const int qa = R.pairs[2 * (k0 - 1)], qb = R.pairs[2 * (k0 - 1) + 1];
+    st.gate_stride = gstride;
+    if (len == 2) {
+      if (pending) carry(pending, 1, 0);
+      pending = 0;
+      st.kind = DF_ENV16;
+      st.in = k0 == 1 ? psi : B_ptr(k0 - 1);
+      st.in_stride = k0 == 1 ? 0 : sN;
+      st.in_gstride = k0 == 1 ? sN : 0;
+      phi_from(st);
+      st.bg = make_bwd_geom(n, M, R.pairs[2 * k0], R.pairs[2 * k0 + 1], qa, qb);
+      st.units = (1 << (n - 4)) * (M / vec);
+      chunk_it(st, 16.0 * vec * es * 2.0);
+      st.upd = update_args(k0 + 1, st.nchunk);
+      st.upd2 = update_args(k0, st.nchunk);
+      steps.push_back(st);
+      carry(k0, 2, k0 == 1 ? 1 : 0);
+      continue;
+    }
+    int ua = qa, ub = qb;
+    st.in = k0 == 1 ? psi : B_ptr(k0 - 1);
+    st.in_stride = k0 == 1 ? 0 : sN;
+    st.in_gstride = k0 == 1 ? sN : 0;
+    phi_from(st);
+    if (pending) {
+      st.phi_out = R.phi;
+      st.gate = gate_ptr(pending - 1);
+      ua = R.pairs[2 * (pending - 1)];
+      ub = R.pairs[2 * (pending - 1) + 1];
+      own = true;
+    }
+    st.bg = make_bwd_geom(n, M, ua, ub, qa, qb);
+    const int U = st.bg.U, ea = st.bg.ea, eb = st.bg.eb;
+    int v = vec;
+    if (U == 4) st.kind = DF_BWD4;
+    else if (U == 2) st.kind = ea == 1 ? DF_BWD2_10 : DF_BWD2_01;
+    else {
+      v = 1;
+      st.kind = ea == 2 ? DF_BWD3_20 : eb == 2 ? DF_BWD3_02 : ea == 1 ? DF_BWD3_10 : DF_BWD3_01;
+    }
+    st.units = (1 << (n - U)) * (M / v);
+    // Phi is stored by a step that carries a gate into it.
+    chunk_it(st, (double)(1 << U) * v * es * (pending ? 3.0 : 2.0));
+    st.upd = update_args(k0, st.nchunk);
+    steps.push_back(st);
+    pending = k0;
   }
   if (r == R32) {
     DfStep st{};
     st.kind = DF_RESID;
+    st.resid = 1;
     st.in = psi;
     st.in_stride = 0;
     st.in_gstride = sN;
-    st.phi_in = L == 1 ? phil : R.phi;
-    st.phi_in_stride = L == 1 ? 0 : sN;
-    st.phi_in_gstride = L == 1 ? sN : 0;
+    phi_from(st);
     st.phi_out = nullptr;
-    st.gate = gate_ptr(0);
+    st.gate = pending ? gate_ptr(0) : nullptr;
     st.gate_stride = gstride;
     st.bg = make_bwd_geom(n, M, R.pairs[0], R.pairs[1], R.pairs[0], R.pairs[1]);
     st.units = (1 << (n - 2)) * (M / vec);
@@ -616,6 +693,7 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   }
   R.df_cap = 0;
   R.df_max_nchunk = 0;
+  R.df_part_len = 32;
   R.df_key_r = -1;
   R.cl = ClPlan{};
   if (ctx->dataflow && ctx->coop && !ctx->df_trace)
@@ -631,7 +709,10 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
       double b = 0.0;
       df_build(ctx, R, rs, nullptr, nullptr, nullptr, nullptr, nullptr, steps, &b);
       R.df_cap = (int)steps.size();
-      for (const DfStep& st : steps) R.df_max_nchunk = std::max(R.df_max_nchunk, st.nchunk);
+      for (const DfStep& st : steps) {
+        R.df_max_nchunk = std::max(R.df_max_nchunk, st.nchunk);
+        if (st.kind == DF_ENV16) R.df_part_len = 512;
+      }
     }
   }
   R.oz_bytes = oz_scratch_bytes((int)R.N, M, ctx->num_sms);
@@ -905,6 +986,7 @@ int df_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, do
   a.err = R.err;
   a.wait_limit = ctx->df_wait_limit;
   a.partials = R.df_partials;
+  a.part_len = R.df_part_len;
   a.resid_partials = R.df_resid;
   a.part_stride = R.df_max_nchunk;
   a.resid_cost = R.costs;

@@ -85,6 +85,7 @@ enum DfKind {
   DF_BWD3_01 = 7,
   DF_RESID = 8,    // residual cost (1/M) sum |g_1^dagger Phi_1 - Psi|^2
   DF_FWD2 = 9,     // B_k = g_k B_{k-1} and B_{k+1} = g_{k+1} B_k, gates on four distinct qubits
+  DF_ENV16 = 10,   // environments and updates of gates k and k - 1 on four distinct qubits (complex64)
 };
 struct DfStep {
   int kind;
@@ -103,6 +104,9 @@ struct DfStep {
   Geom fg;
   BwdGeom bg;
   UpdateArgs upd;                       // backward steps: the update of gate k
+  UpdateArgs upd2;                      // DF_ENV16: of gate k - 1
+  int adj;                              // DF_FWD, DF_FWD2: apply the adjoint gates
+  int resid;                            // the step serves the residual (skipped with it)
 };
 struct DfArgs {
   const DfStep* steps; int nsteps; int S;
@@ -113,7 +117,8 @@ struct DfArgs {
   unsigned* done;                       // S: steps finished per start
   int* err;                             // bit 0: a bounded wait ran out
   long long wait_limit;                 // polls of a dependency wait before it gives up
-  void* partials;                       // S x part_stride x 32 environment partials (float or double)
+  void* partials;                       // S x part_stride x part_len environment partials (float or double)
+  int part_len;                         // 32, or 512 with DF_ENV16 steps
   double* resid_partials;               // S x part_stride x 32, residual step only
   int part_stride;                      // slots per start: the most chunks of any step
   double* resid_cost; double inv_M;     // residual step output

@@ -113,13 +113,17 @@ __device__ __forceinline__ const T2* df_phi_in(const DfStep& st, int s) {
   return reinterpret_cast<const T2*>(st.phi_in) + s * st.phi_in_stride + (long long)(s / st.spt) * st.phi_in_gstride;
 }
 
+// Entry i of a gate of start s, or of its adjoint.
+template <typename T2>
+__device__ __forceinline__ T2 gate_entry(const DfStep& st, const void* gate, int s, int i) {
+  const T2 g = __ldcg(reinterpret_cast<const T2*>(gate) + s * st.gate_stride + (st.adj ? 4 * (i & 3) + (i >> 2) : i));
+  return T2{g.x, st.adj ? -g.y : g.y};
+}
 // Gate of this start (16 complex) into shared memory.
 template <typename T>
 __device__ __forceinline__ void load_gate(const DfStep& st, int s, DfShared<T>& sh) {
   using T2 = typename C2<T>::t;
-  if (threadIdx.x < 16)
-    sh.gs[threadIdx.x] = st.gate ? __ldcg(reinterpret_cast<const T2*>(st.gate) + s * st.gate_stride + threadIdx.x)
-                                 : T2{};
+  if (threadIdx.x < 16) sh.gs[threadIdx.x] = st.gate ? gate_entry<T2>(st, st.gate, s, threadIdx.x) : T2{};
   __syncthreads();
 }
 
@@ -211,10 +215,13 @@ __host__ __device__ constexpr int df_stage_bytes() {
 
 // Two forward steps in one pass over 16-row units (gates k and k+1 on four
 // distinct qubits; geometry bg with gate k's pair on local bits 3, 2 and
-// gate k+1's on local bits 1, 0): B_k = g_k B_{k-1} and B_{k+1} = g_{k+1}
-// B_k, both stored, B_k never read back.  Four lanes share a unit: lane
+// gate k+1's on local bits 1, 0): B_k = g_k B_{k-1}, stored where something
+// reads it, and B_{k+1} = g_{k+1} B_k.  The same step with the adjoints of two
+// updated gates carries Phi past both, in place.  Four lanes share a unit: lane
 // quarter qx holds the four rows of one value of gate k+1's bits and applies
-// g_k to them; g_{k+1} then mixes the four quarters through shuffles.  Rows
+// g_k to them; after a transpose over the four lanes it applies g_{k+1}.  (Sixteen
+// shuffles a round; fetching every row where it is used took 64, and 16 warps
+// of those were the step's bound: 11.9 us an item of 420 KB.)  Rows
 // are staged by cp.async into the thread's own slots (kDfFwd2Stages - 1
 // rounds in flight).
 constexpr int kDfFwd2Stages = 4;
@@ -227,18 +234,12 @@ __device__ void df_forward2(const DfStep& st, int s, int c, DfShared<T>& sh, uin
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int qx = lane >> 3, v = lane & 7;
-  if (threadIdx.x < 16)
-    sh.gs[threadIdx.x] = __ldcg(reinterpret_cast<const T2*>(st.gate) + s * st.gate_stride + threadIdx.x);
-  else if (threadIdx.x < 32)
-    sh.gs2[threadIdx.x - 16] =
-        __ldcg(reinterpret_cast<const T2*>(st.gate2) + s * st.gate_stride + (threadIdx.x - 16));
+  if (threadIdx.x < 16) sh.gs[threadIdx.x] = gate_entry<T2>(st, st.gate, s, threadIdx.x);
+  else if (threadIdx.x < 32) sh.gs2[threadIdx.x - 16] = gate_entry<T2>(st, st.gate2, s, threadIdx.x - 16);
   __syncthreads();
   T2 g1[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) g1[i] = sh.gs[i];
-  T2 g2[4];  // row qx of g_{k+1}
-#pragma unroll
-  for (int m = 0; m < 4; ++m) g2[m] = sh.gs2[4 * qx + m];
   const T2* X = df_in<T2>(st, s);
   T2* Y1 = reinterpret_cast<T2*>(st.out) + s * st.bg.sN;
   T2* Y2 = reinterpret_cast<T2*>(st.out2) + s * st.bg.sN;
@@ -300,29 +301,39 @@ __device__ void df_forward2(const DfStep& st, int s, int c, DfShared<T>& sh, uin
         for (int xp = 1; xp < 4; ++xp) acc = cfma(g1[4 * x + xp], b[xp][q], acc);
         y[x][q] = acc;
       }
-    if (valid) {
+    if (valid && st.out != nullptr) {
 #pragma unroll
       for (int x = 0; x < 4; ++x) stg<T, VEC>(Y1 + o + joff[x], y[x]);
     }
-    // z = g_{k+1} y over the quarters, summed in the order of the one-gate
-    // forward step (quarter 0 first); quarter xp sits xor 8 (qx ^ xp) away.
+    // The quarters' rows change places (4 x 4 transpose of 16-byte entries over
+    // the unit's four lanes, two exchanges): lane qx then holds row qx of gate
+    // k's index for all four of gate k+1's.
+    auto swap = [&](T2 (&p)[VEC], T2 (&q)[VEC], bool upper, int m) {
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
+      for (int e = 0; e < VEC; ++e) {
+        const T2 send = upper ? p[e] : q[e];
+        const T2 got{__shfl_xor_sync(FULL, send.x, m), __shfl_xor_sync(FULL, send.y, m)};
+        if (upper) p[e] = got;
+        else q[e] = got;
+      }
+    };
+    swap(y[0], y[1], qx & 1, 8);
+    swap(y[2], y[3], qx & 1, 8);
+    swap(y[0], y[2], qx >> 1, 16);
+    swap(y[1], y[3], qx >> 1, 16);
+    // z = g_{k+1} y, summed in the order of the one-gate forward step.
+    const uint32_t oz = o - xoff + ((qx >> 1) ? d3 : 0u) + ((qx & 1) ? d2 : 0u);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
       T2 z[VEC];
 #pragma unroll
       for (int q = 0; q < VEC; ++q) {
-        T2 w[4];
+        T2 acc = cmul(sh.gs2[4 * r], y[0][q]);
 #pragma unroll
-        for (int xp = 0; xp < 4; ++xp) {
-          w[xp].x = __shfl_xor_sync(FULL, y[x][q].x, 8 * (qx ^ xp));
-          w[xp].y = __shfl_xor_sync(FULL, y[x][q].y, 8 * (qx ^ xp));
-        }
-        T2 acc = cmul(g2[0], w[0]);
-#pragma unroll
-        for (int xp = 1; xp < 4; ++xp) acc = cfma(g2[xp], w[xp], acc);
+        for (int xp = 1; xp < 4; ++xp) acc = cfma(sh.gs2[4 * r + xp], y[xp][q], acc);
         z[q] = acc;
       }
-      if (valid) stg<T, VEC>(Y2 + o + joff[x], z);
+      if (valid) stg<T, VEC>(Y2 + oz + ((r >> 1) ? d1 : 0u) + ((r & 1) ? d0 : 0u), z);
     }
   }
   cp_async_wait<0>();
@@ -587,10 +598,127 @@ __device__ void df_backward_gen(const DfStep& st, int s, int c, DfShared<T>& sh,
   }
 }
 
+// Environments of two gates on four distinct qubits in one pass (complex64):
+// F[x][y] = sum B[x] conj(Phi[y]) over the 16 x 16 row pairs of a unit, B the
+// state before both gates, Phi carried past everything behind them.  Both 4x4
+// environments, the second one with the first gate already updated, are sums
+// over F with the other gate (df_update_pair), so B and Phi are read once for
+// two gates where a step per gate reads B, reads Phi and writes Phi twice:
+// 6 N M s bytes a pair of gates with its forward step and Phi's, against 9.  At
+// n = 12, M = 32, 32 starts: 484 -> 461 us a sweep (with the transposed forward
+// step); what is left is issue-bound, 9.8 us an item of 512 units at 256 FMAs a
+// thread and round, not bound by the bytes.
+//
+// The price is arithmetic, 16 complex FMAs per entry instead of 8, so F is
+// formed as a small matrix product: a tile of 16 rows x 64 columns' pairs of B
+// and Phi in shared memory (cp.async, kEnvStages deep, rows padded by 32 bytes
+// so that the four rows of an access lie in different banks), 16 threads per
+// 16 x 16 block with 4 x 4 entries each: 128 FMAs per eight 16-byte reads.
+constexpr int kEnvStages = 4, kEnvCols = 64, kEnvRow = kEnvCols * 16 + 32, kEnvStage = 32 * kEnvRow;
+static_assert(kEnvStages * kEnvStage <= df_stage_bytes<float>(), "environment stages fit the stage buffer");
+static_assert(16 * 512 * 4 + 2 * 512 * 4 <= df_stage_bytes<float>(), "and its sums");
+
+__device__ __forceinline__ void cp_async16_zero(void* smem, const void* gmem, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+
+__device__ void df_env16(const DfStep& st, int s, int c, float* part, unsigned char* stage) {
+  constexpr int NT = df_threads<float>();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float2* B = df_in<float2>(st, s);
+  const float2* P = df_phi_in<float2>(st, s);
+  const uint32_t M = (uint32_t)st.bg.M;
+  const int MV = st.bg.M / 2;
+  const int u0 = c * st.chunk, u1 = min(u0 + st.chunk, st.units);
+  const int rounds = (u1 - u0 + kEnvCols - 1) / kEnvCols;
+  // Copies: this thread's column pair and four rows, two of B and two of Phi.
+  const int col = tid & (kEnvCols - 1), rg = tid >> 6;
+  auto row_off = [&](int t) {
+    return ((((uint32_t)t & 1u) << st.bg.pos[0]) | (((uint32_t)t >> 1 & 1u) << st.bg.pos[1]) |
+            (((uint32_t)t >> 2 & 1u) << st.bg.pos[2]) | (((uint32_t)t >> 3 & 1u) << st.bg.pos[3])) * M;
+  };
+  const uint32_t ra = row_off(rg), rb = row_off(rg + 8);
+  auto issue = [&](int rd) {
+    if (rd < rounds) {
+      const int u = u0 + rd * kEnvCols + col;
+      const bool valid = u < u1;
+      const int r = (valid ? u : u0) / MV, jv = (valid ? u : u0) - r * MV;
+      uint32_t base = (uint32_t)r;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int p = st.bg.ins[i];
+        base = ((base >> p) << (p + 1)) | (base & ((1u << p) - 1u));
+      }
+      const uint32_t o = base * M + (uint32_t)jv * 2;
+      unsigned char* d = stage + (rd % kEnvStages) * kEnvStage + col * 16;
+      cp_async16_zero(d + rg * kEnvRow, B + o + ra, valid);
+      cp_async16_zero(d + (rg + 8) * kEnvRow, B + o + rb, valid);
+      cp_async16_zero(d + (rg + 16) * kEnvRow, P + o + ra, valid);
+      cp_async16_zero(d + (rg + 24) * kEnvRow, P + o + rb, valid);
+    }
+    cp_async_commit();
+  };
+  // Sums: entries F[4 r + i][4 q + j].
+  const int i = tid & 3, j = (tid >> 2) & 3, g = tid >> 4;
+  float acc[4][4][2];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[r][q][0] = acc[r][q][1] = 0.f;
+  __syncthreads();  // (the stages may still be read as another step's)
+#pragma unroll
+  for (int rd = 0; rd < kEnvStages - 1; ++rd) issue(rd);
+  for (int rd = 0; rd < rounds; ++rd) {
+    cp_async_wait<kEnvStages - 2>();
+    __syncthreads();  // round rd is there for everybody, round rd - 1 is read
+    issue(rd + kEnvStages - 1);
+    const unsigned char* d = stage + (rd % kEnvStages) * kEnvStage;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned char* e = d + (h * 32 + g) * 16;
+      float4 b[4], p[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) b[r] = *reinterpret_cast<const float4*>(e + (4 * r + i) * kEnvRow);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) p[q] = *reinterpret_cast<const float4*>(e + (16 + 4 * q + j) * kEnvRow);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          cfma_conj(acc[r][q][0], acc[r][q][1], float2{b[r].x, b[r].y}, float2{p[q].x, p[q].y});
+          cfma_conj(acc[r][q][0], acc[r][q][1], float2{b[r].z, b[r].w}, float2{p[q].z, p[q].w});
+        }
+    }
+  }
+  cp_async_wait<0>();
+  // The warp's two groups, then the warps (TwoSum, fixed order).
+  float* buf = reinterpret_cast<float*>(stage);
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float re = acc[r][q][0] + __shfl_xor_sync(FULL, acc[r][q][0], 16);
+      const float im = acc[r][q][1] + __shfl_xor_sync(FULL, acc[r][q][1], 16);
+      if (lane < 16) *reinterpret_cast<float2*>(buf + warp * 512 + 2 * ((4 * r + i) * 16 + 4 * q + j)) = float2{re, im};
+    }
+  __syncthreads();
+  float hi = 0.f, lo = 0.f;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    float t;
+    two_sum(hi, buf[w * 512 + tid], hi, t);
+    lo += t;
+  }
+  __stcg(part + tid, hi + lo);
+}
+
 // The update of gate k for start s by warp 0 (polar_newton.cuh) from the summed
 // environment, whose value j is in lane j: hi + lo (complex64 sweeps) or e.
 template <typename T>
-__device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, float hi, float lo, double e) {
+__device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, float hi, float lo, double e, float2* keep = nullptr) {
   constexpr bool F32 = sizeof(T) == 4;
   const int lane = threadIdx.x & 31, l16 = lane & 15, at = 4 * (l16 & 3) + (l16 >> 2);
   double2* g64 = ua.g64 + s * ua.g_stride;
@@ -602,7 +730,9 @@ __device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, float hi
   const double2 p = newton_update<!F32>(a32, sh.nw, newton_pair(), q) ? newton_entry64(q) : newton_fallback(matrix(), sh.nw);
   if (lane < 16) {
     g64[at] = p;
-    if (ua.g32) (ua.g32 + s * ua.g_stride)[at] = float2{(float)p.x, (float)p.y};
+    const float2 pf{(float)p.x, (float)p.y};
+    if (ua.g32) (ua.g32 + s * ua.g_stride)[at] = pf;
+    if (keep) keep[at] = pf;
   }
   if (ua.env_out) {
     const double2 m = env();
@@ -617,14 +747,53 @@ __device__ void df_update(const UpdateArgs& ua, int s, DfShared<T>& sh, float hi
   }
 }
 
+// The two updates behind df_env16, by warp 0: F (hi + lo, 16 x 16 complex) in
+// shared memory, gate k on the upper index pair of x = 4 xa + xb, gate k - 1 on
+// the lower.  E_k[xa][ya] = sum g_{k-1}[z][xb] F[xa xb][ya z] with the old gate
+// k - 1 (it makes B_{k-1} of B_{k-2}), E_{k-1}[xb][yb] = sum g_k[ya][z]
+// F[z xb][ya yb] with the new gate k (its adjoint makes Phi_{k-1} of Phi_k).
+__device__ void df_update_pair(const UpdateArgs& up, const UpdateArgs& lower, int s, DfShared<float>& sh, const float2* fh,
+                               const float2* fl) {
+  const int lane = threadIdx.x & 31, x = lane >> 3, y = (lane >> 1) & 3, im = lane & 1;
+  if (lane < 16) sh.gs[lane] = __ldcg(lower.g32 + s * lower.g_stride + lane);
+  __syncwarp();
+  auto term = [&](float2 g, float2 f, float& acc) {  // component im of g f
+    acc = fmaf(g.x, im ? f.y : f.x, acc);
+    acc = fmaf(im ? g.y : -g.y, im ? f.x : f.y, acc);
+  };
+  float a = 0.f, b = 0.f, l = 0.f, hi, lo;
+#pragma unroll
+  for (int z = 0; z < 4; ++z)
+#pragma unroll
+    for (int xb = 0; xb < 4; ++xb) {
+      const int at = (4 * x + xb) * 16 + 4 * y + z;
+      term(sh.gs[4 * z + xb], fh[at], (xb & 1) ? b : a);
+      term(sh.gs[4 * z + xb], fl[at], l);
+    }
+  two_sum(a, b, hi, lo);
+  df_update<float>(up, s, sh, hi, lo + l, 0.0, sh.gs2);
+  __syncwarp();
+  a = b = l = 0.f;
+#pragma unroll
+  for (int z = 0; z < 4; ++z)
+#pragma unroll
+    for (int ya = 0; ya < 4; ++ya) {
+      const int at = (4 * z + x) * 16 + 4 * ya + y;
+      term(sh.gs2[4 * ya + z], fh[at], (ya & 1) ? b : a);
+      term(sh.gs2[4 * ya + z], fl[at], l);
+    }
+  two_sum(a, b, hi, lo);
+  df_update<float>(lower, s, sh, hi, lo + l, 0.0);
+}
+
 // Partial-sum slots: start s owns slots s * stride .. s * stride + stride - 1
 // (stride = the most chunks of any step), so starts that are at different
 // steps, with different chunk counts, never share a slot.
 template <typename T>
 __device__ void df_process(const DfStep& st, int s, int c, DfShared<T>& sh, void* partials, double* resid,
-                           int stride, uint4* stage) {
+                           int stride, int len, uint4* stage) {
   constexpr int V2 = sizeof(T) == 4 ? 2 : 1;  // samples per thread for 4- and 16-row units
-  T* part = reinterpret_cast<T*>(partials) + ((long long)s * stride + c) * 32;
+  T* part = reinterpret_cast<T*>(partials) + ((long long)s * stride + c) * len;
   double* part64 = resid + ((long long)s * stride + c) * 32;
   switch (st.kind) {
     case DF_FWD: df_forward<T, V2>(st, s, c, sh); break;
@@ -637,6 +806,9 @@ __device__ void df_process(const DfStep& st, int s, int c, DfShared<T>& sh, void
     case DF_BWD3_10: df_backward_gen<T, 1, 0, 3, 1, 0>(st, s, c, sh, part); break;
     case DF_BWD3_01: df_backward_gen<T, 1, 0, 3, 0, 1>(st, s, c, sh, part); break;
     case DF_RESID: df_backward_gen<T, V2, 1, 2, 1, 0>(st, s, c, sh, part64); break;
+    case DF_ENV16:
+      if constexpr (sizeof(T) == 4) df_env16(st, s, c, part, reinterpret_cast<unsigned char*>(stage));
+      break;
     default: break;
   }
 }
@@ -700,10 +872,10 @@ __global__ void __launch_bounds__(df_threads<T>(), 1) k_sweep_df(DfArgs a) {
     // update is far above the tolerance is skipped: it could not decide
     // anything (the estimate, accurate to ~1e-7 absolute, stands).
     const bool act = (a.active == nullptr || a.active[s] != 0) &&
-                     !(st.kind == DF_RESID && a.resid_skip > 0.0 && __ldcg(a.resid_cost + s) > a.resid_skip);
+                     !(st.resid && a.resid_skip > 0.0 && __ldcg(a.resid_cost + s) > a.resid_skip);
     if (a.trace && threadIdx.x == 0 && c == 0) a.trace[((long long)i * a.S + s) * 4] = globaltimer_ns();
     if (itr && threadIdx.x == 0) itr[1] = globaltimer_ns();
-    if (act) df_process<T>(st, s, c, sh, a.partials, a.resid_partials, a.part_stride, df_stage);
+    if (act) df_process<T>(st, s, c, sh, a.partials, a.resid_partials, a.part_stride, a.part_len, df_stage);
     // Publish this chunk; the last chunk of (step, start) finishes the step.
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -731,19 +903,46 @@ __global__ void __launch_bounds__(df_threads<T>(), 1) k_sweep_df(DfArgs a) {
               if (a.stop != nullptr && t * a.inv_M <= a.stop_tol) atomicExch(a.stop, 1);
             }
           }
+        } else if (sizeof(T) == 4 && st.kind == DF_ENV16) {
+          if constexpr (sizeof(T) == 4) {
+            // One of the 512 values of F per thread, over the chunks.
+            float* fh = reinterpret_cast<float*>(df_stage);
+            float* fl = fh + 512;
+            const float* pp = reinterpret_cast<const float*>(a.partials) + (long long)s * a.part_stride * a.part_len + threadIdx.x;
+            float hi = 0.f, lo = 0.f;
+            for (int b0 = 0; b0 < st.nchunk; b0 += 8) {  // (eight loads in flight)
+              float v[8];
+#pragma unroll
+              for (int b = 0; b < 8; ++b) v[b] = b0 + b < st.nchunk ? __ldcg(pp + (long long)(b0 + b) * a.part_len) : 0.f;
+#pragma unroll
+              for (int b = 0; b < 8; ++b) {
+                float t;
+                two_sum(hi, v[b], hi, t);
+                lo += t;
+              }
+            }
+            fh[threadIdx.x] = hi;
+            fl[threadIdx.x] = lo;
+            __syncthreads();
+            if (tr && threadIdx.x == 0) tr[2] = globaltimer_ns();
+            if (warp == 0)
+              df_update_pair(st.upd, st.upd2, s, sh, reinterpret_cast<const float2*>(fh), reinterpret_cast<const float2*>(fl));
+            if (st.upd2.cost_out != nullptr && threadIdx.x == 0 && a.cost_row != nullptr)
+              a.cost_row[s] = st.upd2.cost_out[s];
+          }
         } else {
           // The chunk partials summed by all warps (warp w takes chunks w, w
           // + NW, ...; fixed order), then over the warps: complex64 sums in
           // FP32 with their rounding kept (TwoSum), 16 FP64 additions being a
           // chain of 1000 cycles.
-          const T* pp = reinterpret_cast<const T*>(a.partials) + (long long)s * a.part_stride * 32;
+          const T* pp = reinterpret_cast<const T*>(a.partials) + (long long)s * a.part_stride * a.part_len;
           T acc[4] = {T(0), T(0), T(0), T(0)};
           int b = warp;
           for (; b + 3 * NW < st.nchunk; b += 4 * NW) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += __ldcg(pp + (long long)(b + q * NW) * 32 + lane);
+            for (int q = 0; q < 4; ++q) acc[q] += __ldcg(pp + (long long)(b + q * NW) * a.part_len + lane);
           }
-          for (; b < st.nchunk; b += NW) acc[0] += __ldcg(pp + (long long)b * 32 + lane);
+          for (; b < st.nchunk; b += NW) acc[0] += __ldcg(pp + (long long)b * a.part_len + lane);
           const T mine = (acc[0] + acc[1]) + (acc[2] + acc[3]);
           if constexpr (sizeof(T) == 4) reinterpret_cast<float*>(sh.red[warp])[lane] = mine;
           else sh.red[warp][lane] = mine;
