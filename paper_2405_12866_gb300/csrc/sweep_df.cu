@@ -605,7 +605,7 @@ __device__ void df_backward_gen(const DfStep& st, int s, int c, DfShared<T>& sh,
 // over F with the other gate (df_update_pair), so B and Phi are read once for
 // two gates where a step per gate reads B, reads Phi and writes Phi twice:
 // 6 N M s bytes a pair of gates with its forward step and Phi's, against 9.  At
-// n = 12, M = 32, 32 starts: 484 -> 461 us a sweep (with the transposed forward
+// n = 12, M = 32, 32 starts: 491 -> 477 us a sweep (461 with the transposed forward
 // step); what is left is issue-bound, 9.8 us an item of 512 units at 256 FMAs a
 // thread and round, not bound by the bytes.
 //
