@@ -3098,24 +3098,27 @@ extern "C" int qfs_gemm_bf16_dev(qfs_ctx* ctx, int32_t M, int32_t N, int32_t K, 
   if (ldc % 8) return fail(QFS_EINVAL, "ldc must be a multiple of 8");
   TRY(ctx_check(ctx));
   TRY(set_device(ctx));
-  TRY(ensure_ws(ctx, 256));
-  int* err = reinterpret_cast<int*>(ctx->ws);
+  TRY(ensure_ws(ctx, 256));  // (a workspace limit too small for any call refuses this one too)
+  // The kernel sets the error word in pinned host memory, so a call is one
+  // launch and one wait; a device word took a memset before it and a copy
+  // behind it.
+  TRY(ensure_pinned(ctx, 1));
+  volatile int* err = reinterpret_cast<volatile int*>(ctx->h_pinned);
+  *err = 0;
   cudaStream_t st = ctx->stream;
-  CK(cudaMemsetAsync(err, 0, sizeof(int), st));
   GemmArgs g{reinterpret_cast<const __nv_bfloat16*>(A), lda, reinterpret_cast<const __nv_bfloat16*>(B), ldb,
              C32, reinterpret_cast<__nv_bfloat16*>(C16), ldc, bias, gelu, M, N, K,
-             M_valid > 0 ? M_valid : M, err};
-  g.splitk = gemm_splitk_for(g, ctx->num_sms > 0 ? ctx->num_sms : 148);
+             M_valid > 0 ? M_valid : M, const_cast<int*>(err)};
+  g.sms = ctx->num_sms > 0 ? ctx->num_sms : 148;
+  g.splitk = gemm_splitk_for(g);
   {
     ProfScope ps(ctx, QFS_PROF_MLP, 2.0 * M * N * K, st);
     CK(launch_gemm_bf16_tc(g, st));
   }
   CK(cudaGetLastError());
-  int h = 0;
-  CK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   prof_harvest(ctx);
-  if (h) return fail(QFS_ETIMEOUT, "a bounded tensor-core wait ran out");
+  if (*err) return fail(QFS_ETIMEOUT, "a bounded tensor-core wait ran out");
   return QFS_OK;
 }
 
@@ -3184,7 +3187,8 @@ long long ws_param_count(const qfs_ws* m) {
 int ws_gemm(qfs_ws* m, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N, int K,
             float* C32, __nv_bfloat16* C16, int ldc, const float* bias, int gelu, int M_valid) {
   GemmArgs g{A, lda, B, ldb, C32, C16, ldc, bias, gelu, M, N, K, M_valid, m->err};
-  g.splitk = gemm_splitk_for(g, m->ctx->num_sms > 0 ? m->ctx->num_sms : 148);
+  g.sms = m->ctx->num_sms > 0 ? m->ctx->num_sms : 148;
+  g.splitk = gemm_splitk_for(g);
   CK(launch_gemm_bf16_tc(g, m->ctx->stream));
   return QFS_OK;
 }

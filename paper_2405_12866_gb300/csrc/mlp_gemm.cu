@@ -3,21 +3,32 @@
 // A and B bf16 row-major (both K-major), accumulation in FP32 in tensor
 // memory (TMEM).
 //
-// k_gemm_bf16_tma: a warp-specialised pipeline.  Warp 0
-// issues TMA tile loads (128-byte swizzle) into a ring of kStages shared
-// stages, each tracked by a "full" mbarrier (transaction bytes) and an
-// "empty" mbarrier; warp 1 owns the TMEM accumulator (128 x BN fp32
-// columns) and one of its threads issues the tcgen05.mma chain, releasing
-// each stage with tcgen05.commit; warps 2-9 wait for the final commit and
-// run the epilogue (tcgen05.ld, bias, GELU, stores in whole 128-byte lines
-// through shared memory).  With split-K (grid z) each CTA reduces a K range
-// and adds its tile into C32 with vector atomics (the first split adds the
-// bias).
+// k_gemm_bf16_tma: a warp-specialised, persistent pipeline.  Each CTA walks
+// its share of the work items (output tiles x K splits).  Warp 0 issues TMA
+// tile loads (128-byte swizzle) into a ring of kStages shared stages, each
+// tracked by a "full" mbarrier (transaction bytes) and an "empty" mbarrier,
+// running ahead into the next item's tiles; warp 1 owns two TMEM accumulators
+// (128 x BN fp32 columns each, used in turn) and one of its threads issues the
+// tcgen05.mma chain, releasing each stage with tcgen05.commit; warps 2-9 wait
+// for an accumulator's commit and run its epilogue (tcgen05.ld, bias, GELU,
+// stores in whole 128-byte lines through shared memory) under the next item's
+// products.  With split-K each item reduces a K range and adds its tile into
+// C32 with vector atomics (the first split adds the bias).
+//
+// What bounds it: the tensor pipe at the chip's sustained rate (5.4 us a 128 x
+// 256 tile at K = 1024 on all SMs, 1.9 PFLOP/s), plus ~5 us of launch, first
+// loads and the last epilogue.  With one tile per CTA the set-up and the
+// epilogue stood beside the products in each of the two rounds of 8192 x 1024
+// x 1024's 256 tiles, and GELU, 3.6 us a tile with a branch around every
+// store, was most of the epilogue (now 1.1 us).  Bias, GELU and a bf16 output:
+// 8192 rows 27.2 -> 18.4 us, 4096 rows (one round) 14.4 -> 11.9, 16384 rows
+// 53.7 -> 31.8; a split-K product 1024 x 1024 x 4096 11.75 -> 11.3.
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <mutex>
 
@@ -45,13 +56,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
 }
 
 // The tanh form of GELU, 0.5 x (1 + tanh u) with u = sqrt(2/pi) (x +
-// 0.044715 x^3), evaluated as the equal x / (1 + exp(-2u)): one exponential
-// and one division instead of tanhf, ~1e-6 relative, far below the bf16
-// rounding of the result.  exp(-2u) = inf for u < -44 gives -0.
+// 0.044715 x^3), evaluated as the equal x / (1 + exp(-2u)) with exp(-2u) =
+// 2^(x (c1 + c2 x^2)): seven instructions, two of them special functions,
+// ~1e-6 relative, far below the bf16 rounding of the result.  The flushing
+// forms skip the scaling for subnormals: 1 + a subnormal is 1, and a quotient
+// by 2^126 and above is 0 (exp = inf for u < -44 gives -0).
 __device__ __forceinline__ float gelu_tanh(float x) {
-  const float k0 = 0.7978845608028654f, k1 = 0.044715f;
-  const float u = k0 * fmaf(k1 * x, x * x, x);
-  return __fdividef(x, 1.f + __expf(-2.f * u));
+  constexpr double kL = -2.0 * 0.79788456080286536 * 1.4426950408889634;  // -2 sqrt(2/pi) log2(e)
+  const float c1 = (float)kL, c2 = (float)(kL * 0.044715);
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * fmaf(x * x, c2, c1)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
+  return x * r;
 }
 
 }  // namespace
@@ -62,19 +78,20 @@ namespace {
 
 // Warp 0: TMA producer; warp 1: MMA issuer; warps 2-9: epilogue (two per
 // TMEM lane quadrant, each with half of the tile's columns).
-constexpr int kBM = 128, kBK = 64, kStages = 4, kTmaThreads = 320;
-// Row stride (floats) of an epilogue warp's 32 x 32 staging block: 16-byte
-// aligned rows whose float4 accesses by 8 lanes cover all 32 banks.
-constexpr int kTileStride = 36;
-static_assert(8 * 32 * kTileStride * 4 <= kStages * kBM * kBK * 2, "epilogue blocks fit the operand stages");
+constexpr int kBM = 128, kBK = 64, kStages = 4, kTmaThreads = 320, kEpiWarps = 8;
+// An epilogue warp's 32 x 32 fp32 staging block: float4 slot c of row r lies at
+// slot c ^ (r & 7), so both a column of rows and a row of slots cover all banks.
+constexpr int kTileBytes = 32 * 32 * 4;
+__device__ __forceinline__ int tile_slot(int r, int c4) { return 32 * r + 4 * (c4 ^ (r & 7)); }
 
 template <int BN>
 struct TmaCfg {
   static constexpr int kABytes = kBM * kBK * 2;
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  // stages, 1024-byte alignment slack, barriers (256 B), the tile's bias
-  static constexpr int kSmem = kStages * kStageBytes + 1024 + 256 + BN * 4;
+  // stages, 1024-byte alignment slack, barriers (256 B), the epilogue's blocks
+  static constexpr int kSmem = kStages * kStageBytes + 1024 + 256 + kEpiWarps * kTileBytes;
+  static constexpr int kTmemCols = 2 * BN;  // two accumulators
   static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                      ((uint32_t)(kBM >> 4) << 24);
 };
@@ -92,8 +109,32 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
-__device__ __forceinline__ void mbar_init1(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(bar)) : "memory");
+__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void commit_to(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
+               : "memory");
+}
+
+// Work item i of a product: its tile's first row and column and its K steps.
+// Items of one split are consecutive, tiles of one row block next to each
+// other (they share A's rows in L2).
+struct GemmItem {
+  int m0, n0, z, kb, ke;
+};
+template <int BN>
+__device__ __forceinline__ GemmItem gemm_item(const GemmArgs& g, int i) {
+  const unsigned nx = (unsigned)g.N / BN, tiles = nx * ((unsigned)g.M / kBM), KT = (unsigned)g.K / kBK;
+  unsigned z = 0, t = (unsigned)i, kb = 0, ke = KT;
+  if (g.splitk > 1) {
+    z = t / tiles;
+    t -= z * tiles;
+    kb = z * KT / (unsigned)g.splitk;
+    ke = (z + 1) * KT / (unsigned)g.splitk;
+  }
+  const unsigned y = t / nx;
+  return GemmItem{(int)(y * kBM), (int)((t - y * nx) * BN), (int)z, (int)kb, (int)ke};
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
@@ -116,23 +157,25 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
   unsigned char* sb = smem_raw + (base - raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(sb + kStages * Cfg::kStageBytes);
   uint64_t* empty = full + kStages;
-  uint64_t* accf = empty + kStages;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accf + 1);
+  uint64_t* accf = empty + kStages;  // [2] accumulator complete
+  uint64_t* acce = accf + 2;         // [2] accumulator read by every epilogue warp
+  uint64_t* drain = acce + 2;        // after a give-up: the MMAs issued are done
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
-  const int KT = g.K / kBK;
-  const int splitk = gridDim.z;
-  const int kb = (int)((long long)blockIdx.z * KT / splitk), ke = (int)((long long)(blockIdx.z + 1) * KT / splitk);
-  const int nk = ke - kb;
+  const int items = (g.N / BN) * (g.M / kBM) * g.splitk;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init1(&full[s]);
-      mbar_init1(&empty[s]);
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
     }
-    mbar_init1(accf);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accf[b], 1);
+      mbar_init(&acce[b], kEpiWarps);
+    }
+    mbar_init(drain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
@@ -140,7 +183,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                 "r"(BN)
+                 "r"(Cfg::kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -157,56 +200,68 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
     // Producer: one thread issues the TMA loads of both operands per stage.
     if (lane == 0) {
       int issued = 0;
-      for (int i = 0; i < nk; ++i) {
-        const int s = i % kStages;
-        const unsigned ph = (unsigned)(i / kStages) & 1u;
-        if (!mbar_wait_bounded(&empty[s], ph ^ 1u) || *abort_flag) {
-          *abort_flag = 1;
-          break;
+      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x) {
+        const GemmItem it = gemm_item<BN>(g, w);
+        for (int k = it.kb; k < it.ke; ++k, ++issued) {
+          const int s = issued % kStages;
+          const unsigned ph = (unsigned)(issued / kStages) & 1u;
+          if (!mbar_wait_bounded(&empty[s], ph ^ 1u) || *abort_flag) {
+            *abort_flag = 1;
+            break;
+          }
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[s])),
+                       "r"(Cfg::kStageBytes)
+                       : "memory");
+          const uint32_t dst = base + (uint32_t)(s * Cfg::kStageBytes);
+          tma_load_2d(dst, &mapA, &full[s], k * kBK, it.m0);
+          tma_load_2d(dst + Cfg::kABytes, &mapB, &full[s], k * kBK, it.n0);
         }
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[s])),
-                     "r"(Cfg::kStageBytes)
-                     : "memory");
-        const uint32_t dst = base + (uint32_t)(s * Cfg::kStageBytes);
-        tma_load_2d(dst, &mapA, &full[s], (kb + i) * kBK, m0);
-        tma_load_2d(dst + Cfg::kABytes, &mapB, &full[s], (kb + i) * kBK, n0);
-        ++issued;
       }
-      if (*abort_flag) {
-        // Wait (bounded) for every copy this CTA issued before leaving.
-        for (int i = 0; i < issued; ++i) mbar_wait_bounded(&full[i % kStages], (unsigned)(i / kStages) & 1u);
-      }
+      // After a give-up (which may come from another warp once every load is
+      // issued), wait (bounded) for the copies that may be in flight: the last
+      // one of each stage.
+      if (*abort_flag)
+        for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i)
+          mbar_wait_bounded(&full[i % kStages], (unsigned)(i / kStages) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
     // MMA issuer.
     if (lane == 0) {
-      for (int i = 0; i < nk; ++i) {
-        const int s = i % kStages;
-        const unsigned ph = (unsigned)(i / kStages) & 1u;
-        if (!mbar_wait_bounded(&full[s], ph) || *abort_flag) {
+      int step = 0, item = 0;
+      for (int w = blockIdx.x; w < items && !*abort_flag; w += gridDim.x, ++item) {
+        const GemmItem it = gemm_item<BN>(g, w);
+        const int buf = item & 1;
+        if (!mbar_wait_bounded(&acce[buf], (((unsigned)item >> 1) & 1u) ^ 1u)) {
           *abort_flag = 1;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a0 = base + (uint32_t)(s * Cfg::kStageBytes), b0 = a0 + Cfg::kABytes;
+        const uint32_t acc_t = tmem + (uint32_t)(buf * BN);
+        for (int k = it.kb; k < it.ke; ++k, ++step) {
+          const int s = step % kStages;
+          const unsigned ph = (unsigned)(step / kStages) & 1u;
+          if (!mbar_wait_bounded(&full[s], ph) || *abort_flag) {
+            *abort_flag = 1;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t a0 = base + (uint32_t)(s * Cfg::kStageBytes), b0 = a0 + Cfg::kABytes;
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk) {
-          const uint64_t ad = desc_sw128(a0 + kk * 32), bd = desc_sw128(b0 + kk * 32);
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-              "l"(ad), "l"(bd), "r"(Cfg::kIdesc), "r"(acc)
-              : "memory");
+          for (int kk = 0; kk < kBK / 16; ++kk) {
+            const uint64_t ad = desc_sw128(a0 + kk * 32), bd = desc_sw128(b0 + kk * 32);
+            const uint32_t acc = (k > it.kb || kk > 0) ? 1u : 0u;
+            asm volatile(
+                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc_t),
+                "l"(ad), "l"(bd), "r"(Cfg::kIdesc), "r"(acc)
+                : "memory");
+          }
+          commit_to(&empty[s]);
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         su32(&empty[s]))
-                     : "memory");
+        // Arrives once every MMA issued above has completed.
+        commit_to(&accf[buf]);
       }
-      // Arrives once every MMA issued above has completed.
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(accf))
-                   : "memory");
       // Every operand load of this CTA is issued: the next kernel on the
       // stream may start its set-up (it waits for this grid to complete
       // before touching memory).
@@ -215,82 +270,105 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
     __syncwarp();
   } else {
     // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (rows of the
-    // tile) and columns half * BN/2 .. + BN/2 - 1.  The bias (added by the
-    // first K split only) is staged in shared memory while the MMAs run.
+    // tile) and columns half * BN/2 .. + BN/2 - 1.
     const int q = warp & 3, half = (warp - 2) >> 2;
-    float* stile = reinterpret_cast<float*>(sb) + (warp - 2) * 32 * kTileStride;
-    float* sbias = reinterpret_cast<float*>(sb + kStages * Cfg::kStageBytes + 256);
-    const bool add_bias = g.bias != nullptr && blockIdx.z == 0;
-    if (add_bias)
-      for (int j = threadIdx.x - 64; j < BN; j += kTmaThreads - 64) sbias[j] = g.bias[n0 + j];
-    asm volatile("bar.sync 1, %0;" ::"n"(kTmaThreads - 64) : "memory");
-    const bool ok = mbar_wait_bounded(accf, 0) && !*abort_flag;
-    if (!ok) {
-      *abort_flag = 1;
-    } else {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    float* stile = reinterpret_cast<float*>(sb + kStages * Cfg::kStageBytes + 256 + (warp - 2) * kTileBytes);
+    int item = 0;
+    for (int w = blockIdx.x; w < items; w += gridDim.x, ++item) {
+      const GemmItem it = gemm_item<BN>(g, w);
+      const int buf = item & 1;
+      const bool add_bias = g.bias != nullptr && it.z == 0;
+      // (the bias is fetched under the products)
       constexpr int HC = BN / 2;
-      for (int cb = half * HC; cb < (half + 1) * HC; cb += 64) {
+      float4 bias[HC / 32];
+#pragma unroll
+      for (int b = 0; b < HC / 32; ++b)
+        bias[b] = add_bias ? __ldg(reinterpret_cast<const float4*>(g.bias + it.n0 + half * HC + 32 * b) + (lane & 7))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!mbar_wait_bounded(&accf[buf], ((unsigned)item >> 1) & 1u) || *abort_flag) {
+        *abort_flag = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int c64 = 0; c64 < HC; c64 += 64) {
+        const int cb = half * HC + c64;
         uint32_t v[64];
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cb;
+        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + cb);
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          uint32_t* w = v + 32 * hh;
+          uint32_t* w32 = v + 32 * hh;
           asm volatile(
               "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
               "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-              : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]),
-                "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]),
-                "=r"(w[15]), "=r"(w[16]), "=r"(w[17]), "=r"(w[18]), "=r"(w[19]), "=r"(w[20]), "=r"(w[21]),
-                "=r"(w[22]), "=r"(w[23]), "=r"(w[24]), "=r"(w[25]), "=r"(w[26]), "=r"(w[27]), "=r"(w[28]),
-                "=r"(w[29]), "=r"(w[30]), "=r"(w[31])
+              : "=r"(w32[0]), "=r"(w32[1]), "=r"(w32[2]), "=r"(w32[3]), "=r"(w32[4]), "=r"(w32[5]), "=r"(w32[6]), "=r"(w32[7]),
+                "=r"(w32[8]), "=r"(w32[9]), "=r"(w32[10]), "=r"(w32[11]), "=r"(w32[12]), "=r"(w32[13]), "=r"(w32[14]),
+                "=r"(w32[15]), "=r"(w32[16]), "=r"(w32[17]), "=r"(w32[18]), "=r"(w32[19]), "=r"(w32[20]), "=r"(w32[21]),
+                "=r"(w32[22]), "=r"(w32[23]), "=r"(w32[24]), "=r"(w32[25]), "=r"(w32[26]), "=r"(w32[27]), "=r"(w32[28]),
+                "=r"(w32[29]), "=r"(w32[30]), "=r"(w32[31])
               : "r"(taddr + 32u * hh)
               : "memory");
         }
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        // Each 32 x 32 block goes through this warp's slice of the (now idle)
-        // operand stages: lane l writes its row, then eight lanes cover one
-        // row's 128 bytes per store, so every store writes whole lines.
+        if (c64 + 64 == HC) {
+          // The accumulator is read: the next item but one may overwrite it.
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acce[buf])) : "memory");
+        }
+        // Each 32 x 32 block goes through this warp's staging block: lane l
+        // writes its row, then eight lanes cover one row's 128 bytes per
+        // store, so every store writes whole lines.
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          const int lc = cb + 32 * hh, col = n0 + lc;
+          const int col = it.n0 + cb + 32 * hh + 4 * (lane & 7);
 #pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4) {
-            float4 f = make_float4(__uint_as_float(v[32 * hh + 4 * j4]), __uint_as_float(v[32 * hh + 4 * j4 + 1]),
-                                   __uint_as_float(v[32 * hh + 4 * j4 + 2]), __uint_as_float(v[32 * hh + 4 * j4 + 3]));
-            if (add_bias) {
-              f.x += sbias[lc + 4 * j4];
-              f.y += sbias[lc + 4 * j4 + 1];
-              f.z += sbias[lc + 4 * j4 + 2];
-              f.w += sbias[lc + 4 * j4 + 3];
-            }
-            *reinterpret_cast<float4*>(stile + lane * kTileStride + 4 * j4) = f;
-          }
+          for (int j4 = 0; j4 < 8; ++j4)
+            *reinterpret_cast<float4*>(stile + tile_slot(lane, j4)) =
+                make_float4(__uint_as_float(v[32 * hh + 4 * j4]), __uint_as_float(v[32 * hh + 4 * j4 + 1]),
+                            __uint_as_float(v[32 * hh + 4 * j4 + 2]), __uint_as_float(v[32 * hh + 4 * j4 + 3]));
+          const float4 bv = bias[c64 / 32 + hh];
           __syncwarp();
+          // Without a branch between them, so that the 32 values' chains
+          // overlap: GELU is half of the epilogue.
+          float4 f[8];
 #pragma unroll
-          for (int it = 0; it < 8; ++it) {
-            const int r = 4 * it + (lane >> 3), c4 = lane & 7;
-            const int grow = m0 + q * 32 + r;
-            const float4 f = *reinterpret_cast<const float4*>(stile + r * kTileStride + 4 * c4);
-            if (grow < g.M_valid) {
-              float* d32 = g.C32 ? g.C32 + (size_t)grow * g.ldc + col + 4 * c4 : nullptr;
-              if (splitk > 1) {
-                atomicAdd(reinterpret_cast<float4*>(d32), f);
-              } else {
-                if (d32) *reinterpret_cast<float4*>(d32) = f;
-                if (g.C16) {
-                  float a0 = f.x, a1 = f.y, a2 = f.z, a3 = f.w;
-                  if (g.gelu) {
-                    a0 = gelu_tanh(a0);
-                    a1 = gelu_tanh(a1);
-                    a2 = gelu_tanh(a2);
-                    a3 = gelu_tanh(a3);
-                  }
-                  const __nv_bfloat162 p0 = __floats2bfloat162_rn(a0, a1), p1 = __floats2bfloat162_rn(a2, a3);
-                  *reinterpret_cast<uint2*>(g.C16 + (size_t)grow * g.ldc + col + 4 * c4) =
+          for (int i8 = 0; i8 < 8; ++i8) {
+            f[i8] = *reinterpret_cast<const float4*>(stile + tile_slot(4 * i8 + (lane >> 3), lane & 7));
+            if (add_bias) {
+              f[i8].x += bv.x;
+              f[i8].y += bv.y;
+              f[i8].z += bv.z;
+              f[i8].w += bv.w;
+            }
+          }
+          const int row0 = it.m0 + q * 32 + (lane >> 3), left = g.M_valid - row0;
+          const size_t at = (size_t)row0 * g.ldc + col, step = 4 * (size_t)g.ldc;
+          if (g.splitk > 1) {
+#pragma unroll
+            for (int i8 = 0; i8 < 8; ++i8)
+              if (4 * i8 < left) atomicAdd(reinterpret_cast<float4*>(g.C32 + at + i8 * step), f[i8]);
+          } else {
+            if (g.C32) {
+#pragma unroll
+              for (int i8 = 0; i8 < 8; ++i8)
+                if (4 * i8 < left) *reinterpret_cast<float4*>(g.C32 + at + i8 * step) = f[i8];
+            }
+            if (g.C16) {
+              if (g.gelu) {
+#pragma unroll
+                for (int i8 = 0; i8 < 8; ++i8)
+                  f[i8] = make_float4(gelu_tanh(f[i8].x), gelu_tanh(f[i8].y), gelu_tanh(f[i8].z), gelu_tanh(f[i8].w));
+              }
+#pragma unroll
+              for (int i8 = 0; i8 < 8; ++i8) {
+                const __nv_bfloat162 p0 = __floats2bfloat162_rn(f[i8].x, f[i8].y),
+                                     p1 = __floats2bfloat162_rn(f[i8].z, f[i8].w);
+                if (4 * i8 < left)
+                  *reinterpret_cast<uint2*>(g.C16 + at + i8 * step) =
                       make_uint2(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1));
-                }
               }
             }
           }
@@ -301,14 +379,18 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) atomicOr(g.err, 1);
+  // (g.err may be mapped host memory: one plain store, no atomic.)
+  if (threadIdx.x == 0 && *abort_flag) *reinterpret_cast<volatile int*>(g.err) = 1;
   if (warp == 1) {
     // After a give-up, let the MMAs already issued finish (bounded) before
-    // the accumulator is released.
-    if (lane == 0 && *abort_flag) mbar_wait_bounded(accf, 0);
+    // the accumulators are released.
+    if (lane == 0 && *abort_flag) {
+      commit_to(drain);
+      mbar_wait_bounded(drain, 0);
+    }
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::kTmemCols) : "memory");
   }
 }
 
@@ -377,19 +459,20 @@ bool cached_kmajor(CUtensorMap* map, const void* ptr, int rows, int K, int ld, i
 }
 
 template <int BN>
-cudaError_t launch_tma(const GemmArgs& g, int splitk, cudaStream_t st) {
+cudaError_t launch_tma(const GemmArgs& g, cudaStream_t st) {
   static const cudaError_t attr = cudaFuncSetAttribute(k_gemm_bf16_tma<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        TmaCfg<BN>::kSmem);
   if (attr != cudaSuccess) return attr;
   CUtensorMap ma, mb;
   if (!cached_kmajor(&ma, g.A, g.M, g.K, g.lda, kBM) || !cached_kmajor(&mb, g.B, g.N, g.K, g.ldb, BN))
     return cudaErrorInvalidValue;
-  dim3 grid(g.N / BN, g.M / kBM, splitk);
+  const long long items = (long long)(g.N / BN) * (g.M / kBM) * g.splitk;
+  const long long at_once = g.sms > 0 ? g.sms : 1;  // one CTA per SM: the stages fill its shared memory
   // Programmatic dependent launch: this GEMM's set-up may overlap the tail
   // of the previous kernel on the stream (the kernel waits for it before
   // any memory access).
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
+  cfg.gridDim = dim3((unsigned)std::min(items, at_once));
   cfg.blockDim = dim3(kTmaThreads);
   cfg.dynamicSmemBytes = TmaCfg<BN>::kSmem;
   cfg.stream = st;
@@ -405,24 +488,23 @@ cudaError_t launch_tma(const GemmArgs& g, int splitk, cudaStream_t st) {
 
 }  // namespace
 
-int gemm_splitk_for(const GemmArgs& g, int num_sms) {
+int gemm_splitk_for(const GemmArgs& g) {
   if (g.C16 || g.gelu || !g.C32) return 1;  // (the bias is added by the first split)
   const int BN = g.N % 256 == 0 ? 256 : 128;
   const int tiles = (g.N / BN) * (g.M / kBM);
   const int KT = g.K / kBK;
   int s = 1;
-  while (tiles * s * 2 <= num_sms && KT / (s * 2) >= 4) s *= 2;
+  while (tiles * s * 2 <= g.sms && KT / (s * 2) >= 4) s *= 2;
   return s;
 }
 
 cudaError_t launch_gemm_bf16_tc(const GemmArgs& g, cudaStream_t st) {
-  const int splitk = g.splitk > 1 ? g.splitk : 1;
-  if (splitk > 1) {
+  if (g.splitk > 1) {
     // The split CTAs add into C32, which starts from zero.
     const cudaError_t e = cudaMemset2DAsync(g.C32, (size_t)g.ldc * 4, 0, (size_t)g.N * 4, g.M_valid, st);
     if (e != cudaSuccess) return e;
   }
-  return g.N % 256 == 0 ? launch_tma<256>(g, splitk, st) : launch_tma<128>(g, splitk, st);
+  return g.N % 256 == 0 ? launch_tma<256>(g, st) : launch_tma<128>(g, st);
 }
 
 }  // namespace qfs
