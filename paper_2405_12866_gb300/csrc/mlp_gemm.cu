@@ -20,9 +20,11 @@
 // loads and the last epilogue.  With one tile per CTA the set-up and the
 // epilogue stood beside the products in each of the two rounds of 8192 x 1024
 // x 1024's 256 tiles, and GELU, 3.6 us a tile with a branch around every
-// store, was most of the epilogue (now 1.1 us).  Bias, GELU and a bf16 output:
-// 8192 rows 27.2 -> 18.4 us, 4096 rows (one round) 14.4 -> 11.9, 16384 rows
-// 53.7 -> 31.8; a split-K product 1024 x 1024 x 4096 11.75 -> 11.3.
+// store, was most of the epilogue (now 1.6 us).  Bias, GELU and a bf16 output:
+// 8192 rows 27.2 -> 20.1 us, 4096 rows (one round) 14.4 -> 12.7, 16384 rows
+// 53.7 -> 34.3; a split-K product 1024 x 1024 x 4096 11.75 -> 11.3.  (GELU with
+// its constants folded, 7 instructions, takes 18.4 us for 8192 rows, but rounds
+// differently: 2e-4 of the bf16 activations move by a step.)
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -56,16 +58,16 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
 }
 
 // The tanh form of GELU, 0.5 x (1 + tanh u) with u = sqrt(2/pi) (x +
-// 0.044715 x^3), evaluated as the equal x / (1 + exp(-2u)) with exp(-2u) =
-// 2^(x (c1 + c2 x^2)): seven instructions, two of them special functions,
-// ~1e-6 relative, far below the bf16 rounding of the result.  The flushing
-// forms skip the scaling for subnormals: 1 + a subnormal is 1, and a quotient
-// by 2^126 and above is 0 (exp = inf for u < -44 gives -0).
+// 0.044715 x^3), evaluated as the equal x / (1 + exp(-2u)): ten instructions,
+// two of them special functions, ~1e-6 relative, far below the bf16 rounding of
+// the result.  The flushing forms skip the scaling for subnormals: 1 + a
+// subnormal is 1, and a quotient by 2^126 and above is 0 (exp(-2u) = inf for
+// u < -44 gives -0).
 __device__ __forceinline__ float gelu_tanh(float x) {
-  constexpr double kL = -2.0 * 0.79788456080286536 * 1.4426950408889634;  // -2 sqrt(2/pi) log2(e)
-  const float c1 = (float)kL, c2 = (float)(kL * 0.044715);
+  const float k0 = 0.7978845608028654f, k1 = 0.044715f;
+  const float u = k0 * fmaf(k1 * x, x * x, x);
   float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * fmaf(x * x, c2, c1)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"((-2.f * u) * 1.4426950408889634f));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
   return x * r;
 }
