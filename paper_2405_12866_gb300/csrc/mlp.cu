@@ -25,27 +25,100 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 }
 }  // namespace
 
+// A double as the unevaluated sum of two floats, hi its truncation to 24 bits,
+// by integer operations and one integer conversion: FP64 conversions run at
+// 1/64 of FP32's rate.  ok is cleared where the split or a product of two such
+// pairs could leave FP32's normal range (0 itself is fine).
+__device__ __forceinline__ float2 split_f32(double x, bool& ok) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const unsigned up = (unsigned)(u >> 32), ex = (up >> 20) & 0x7FFu;
+  if ((u << 1) == 0) return float2{__uint_as_float(up & 0x80000000u), 0.f};
+  ok &= ex - (1023u - 40u) <= 60u;  // 2^-40 <= |x| < 2^21
+  const unsigned sign = up & 0x80000000u, e32 = ex - 896u;
+  const float hi = __uint_as_float(sign | (e32 << 23) | ((unsigned)(u >> 29) & 0x7FFFFFu));
+  // The low 29 bits, in units of 2^-52 of x's binade.
+  const float lo = __fmul_rn((float)((unsigned)u & 0x1FFFFFFFu), __uint_as_float(sign | ((e32 - 52u) << 23)));
+  return float2{hi, lo};
+}
+
+// a b as p + e, e exact to 2^-24 of itself (2^-47 of the product).
+__device__ __forceinline__ float2 mul_pair(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  return float2{p, __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.x, -p)))};
+}
+// The float next to s - t.
+__device__ __forceinline__ float sub_pair(float2 s, float2 t) {
+  const float d = __fsub_rn(s.x, t.x), v = __fsub_rn(d, s.x);
+  const float err = __fsub_rn(__fsub_rn(s.x, __fsub_rn(d, v)), __fadd_rn(t.x, v));
+  return __fadd_rn(d, __fadd_rn(err, __fsub_rn(s.y, t.y)));
+}
+
 // Features of target t: the 16 x 8 complex matrix U_t Phi_fix as 256 reals
 // (row-major, re/im interleaved), bf16, row t of X (ld = 256).  Rows
-// count..rows-1 are zero.
-__global__ void k_ws_features(const double2* __restrict__ U, const double2* __restrict__ phif, int count,
-                              int rows, __nv_bfloat16* __restrict__ X) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;  // one complex output
-  if (e >= (long long)rows * 128) return;
-  const int t = (int)(e / 128), k = (int)(e % 128), i = k / 8, j = k % 8;
-  float re = 0.f, im = 0.f;
-  if (t < count) {
-    const double2* u = U + (size_t)t * 256 + i * 16;
-    for (int q = 0; q < 16; ++q) {
-      const double2 a = u[q], b = phif[q * 8 + j];
-      re += (float)(a.x * b.x - a.y * b.y);
-      im += (float)(a.x * b.y + a.y * b.x);
-    }
+// count..rows-1 are zero.  Every product of two complex entries is rounded to
+// FP32 and the 16 of an output are added in FP32.
+//
+// The products in FP64 were bound by that pipe (95 us for 4096 targets; the
+// targets are 17 MB, 2.5 us of memory time), so they are formed from pairs of
+// floats, which gives the same rounded float but for one in ~2^23.  A block
+// walks over targets: its 128 threads, one per output, keep their column of
+// Phi_fix in registers and share the split target.  A target with an entry
+// outside the pairs' range takes the FP64 products.  Now 21 us.
+constexpr int kFeatStride = 17;  // float4s a row: four rows' reads lie in different banks
+__global__ void __launch_bounds__(128) k_ws_features(const double2* __restrict__ U, const double2* __restrict__ phif,
+                                                     int count, int rows, __nv_bfloat16* __restrict__ X) {
+  __shared__ float4 su[16 * kFeatStride];
+  const int k = threadIdx.x, i = k / 8, j = k % 8;
+  float2 bx[16], by[16];
+  bool phi_ok = true;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const double2 b = phif[q * 8 + j];
+    bx[q] = split_f32(b.x, phi_ok);
+    by[q] = split_f32(b.y, phi_ok);
   }
-  // Scaled by sqrt(16) = 4 so that the features have unit variance per
-  // complex entry (the columns of U Phi_fix are unit vectors of length 16).
-  X[(size_t)t * 256 + 2 * k] = __float2bfloat16(4.f * re);
-  X[(size_t)t * 256 + 2 * k + 1] = __float2bfloat16(4.f * im);
+  double2 next[2];
+  auto fetch = [&](int t) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) next[h] = t < count ? __ldg(U + (size_t)t * 256 + k + 128 * h) : double2{0.0, 0.0};
+  };
+  fetch(blockIdx.x);
+  for (int t = blockIdx.x; t < rows; t += gridDim.x) {
+    float re = 0.f, im = 0.f;
+    if (t < count) {
+      bool ok = phi_ok;
+      float4 mine[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 ax = split_f32(next[h].x, ok), ay = split_f32(next[h].y, ok);
+        mine[h] = make_float4(ax.x, ax.y, ay.x, ay.y);
+      }
+      __syncthreads();  // the last target's entries are read
+#pragma unroll
+      for (int h = 0; h < 2; ++h) su[((k + 128 * h) / 16) * kFeatStride + (k & 15)] = mine[h];
+      const bool pairs = __syncthreads_and(ok);
+      fetch(t + gridDim.x);  // (under this target's products)
+      if (pairs) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          const float4 a = su[i * kFeatStride + q];
+          const float2 ax{a.x, a.y}, ay{a.z, a.w}, nby{-by[q].x, -by[q].y};
+          re = __fadd_rn(re, sub_pair(mul_pair(ax, bx[q]), mul_pair(ay, by[q])));
+          im = __fadd_rn(im, sub_pair(mul_pair(ay, bx[q]), mul_pair(ax, nby)));
+        }
+      } else {
+        const double2* u = U + (size_t)t * 256 + i * 16;
+        for (int q = 0; q < 16; ++q) {
+          const double2 a = u[q], b = phif[q * 8 + j];
+          re += (float)(a.x * b.x - a.y * b.y);
+          im += (float)(a.x * b.y + a.y * b.x);
+        }
+      }
+    }
+    // Scaled by sqrt(16) = 4 so that the features have unit variance per
+    // complex entry (the columns of U Phi_fix are unit vectors of length 16).
+    *reinterpret_cast<__nv_bfloat162*>(X + (size_t)t * 256 + 2 * k) = __floats2bfloat162_rn(4.f * re, 4.f * im);
+  }
 }
 
 // dst[c][r] = src[r][c] (bf16), 32 x 32 tiles; R, C multiples of 32.
@@ -242,8 +315,8 @@ static int blocks_for(long long n, int threads = 256, int cap = 4096) {
 
 void launch_ws_features(const double2* U, const double2* phif, int count, int rows, __nv_bfloat16* X,
                         cudaStream_t st) {
-  const long long n = (long long)rows * 128;
-  k_ws_features<<<(int)((n + 255) / 256), 256, 0, st>>>(U, phif, count, rows, X);
+  // (two blocks an SM by their registers; each splits Phi_fix once)
+  k_ws_features<<<std::min(rows, 304), 128, 0, st>>>(U, phif, count, rows, X);
 }
 void launch_ws_gates_adjoint(const float* Y, int ldy, int count, double2* E, cudaStream_t st) {
   const long long n = (long long)count * 96;
