@@ -3157,7 +3157,8 @@ struct qfs_ws {
   __nv_bfloat16* X16 = nullptr;  // B_cap x 256
   __nv_bfloat16* H16[kLayers];   // B_cap x dout
   float* Z32[kLayers];           // B_cap x dout
-  float *dA32, *dB32;            // B_cap x 1024 scratch (fp32 gradients)
+  float* dH32;                   // B_cap x 1024: a layer's input gradient
+  double* lab64 = nullptr;       // B_cap x 192: the labels as given
   __nv_bfloat16 *dA16, *dB16, *T1, *T2;  // bf16 gradient and transposes (1024 x B_cap)
   float* Tlab = nullptr;         // B_cap x 192 labels
   double* loss_part = nullptr;   // 1024
@@ -3207,47 +3208,37 @@ void ws_forward(qfs_ws* m, int B) {
   }
 }
 
-// Loss and gradients for B rows (B_valid real) with labels in m->Tlab.  The
-// mean loss goes to *loss (host, synchronising) and/or is added to
-// *loss_acc_dev (device, asynchronous).
-int ws_backward(qfs_ws* m, int B, int B_valid, double* loss, double* loss_acc_dev = nullptr) {
+// Loss and gradients for B rows (B_valid real) with labels in m->Tlab; the
+// loss's partial sums go to m->loss_part (their number to *parts) and, scaled,
+// are added to *loss_acc_dev (device).  layer_done (nullable): event l is
+// recorded once layer l's gradients are complete.
+int ws_backward(qfs_ws* m, int B, int B_valid, int* parts, double* loss_acc_dev, cudaEvent_t* layer_done) {
   cudaStream_t st = m->ctx->stream;
   const int L = qfs_ws::kLayers;
-  const int nparts = launch_ws_loss_grad(m->Z32[L - 1], m->dout[L - 1], m->Tlab, m->n_out, B, B_valid, m->dA32,
-                                         m->dA16, m->loss_part, st);
-  float* g32 = m->dA32;
   __nv_bfloat16* g16 = m->dA16;
+  const int nparts = launch_ws_loss_grad(m->Z32[L - 1], m->dout[L - 1], m->Tlab, m->n_out, B, B_valid, g16, m->T1,
+                                         m->gb[L - 1], m->loss_part, st);
+  if (parts) *parts = nparts;
   for (int l = L - 1; l >= 0; --l) {
     const int N = m->dout[l], K = m->din[l];
-    launch_colsum(g32, B, N, m->gb[l], st);
-    launch_transpose_bf16(g16, B, N, m->T1, st);  // N x B
     const __nv_bfloat16* hin = l == 0 ? m->X16 : m->H16[l - 1];
     launch_transpose_bf16(hin, B, K, m->T2, st);  // K x B
-    float* o32 = g32 == m->dA32 ? m->dB32 : m->dA32;
     __nv_bfloat16* o16 = g16 == m->dA16 ? m->dB16 : m->dA16;
     {
       // The layer's weight gradient and (below the first layer) dH = g W
       // (B x K), back to back under one pair of events.
       ProfScope ps(m->ctx, QFS_PROF_MLP, (l > 0 ? 4.0 : 2.0) * N * K * B, nullptr, l > 0 ? 2 : 1);
       TRY(ws_gemm(m, m->T1, B, m->T2, B, N, K, B, m->gW[l], nullptr, K, nullptr, 0, N));
-      if (l > 0) TRY(ws_gemm(m, g16, N, m->WT16[l], N, B, K, N, o32, nullptr, K, nullptr, 0, B));
+      if (l > 0) TRY(ws_gemm(m, g16, N, m->WT16[l], N, B, K, N, m->dH32, nullptr, K, nullptr, 0, B));
     }
+    if (layer_done) CK(cudaEventRecord(layer_done[l], st));
     if (l > 0) {
-      // dZ = dH * gelu'(Z_{l-1}).
-      launch_gelu_back(o32, m->Z32[l - 1], (long long)B * K, K, B_valid, o32, o16, st);
-      g32 = o32;
+      // g of the layer below, its transpose and its bias gradient.
+      launch_gelu_back(m->dH32, m->Z32[l - 1], B, K, B_valid, o16, m->T1, m->gb[l - 1], st);
       g16 = o16;
     }
   }
   if (loss_acc_dev) launch_loss_accumulate(m->loss_part, nparts, 1.0 / ((double)B_valid * m->n_out), loss_acc_dev, st);
-  if (loss) {
-    std::vector<double> parts(nparts);
-    CK(cudaMemcpyAsync(parts.data(), m->loss_part, sizeof(double) * nparts, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    double s = 0.0;
-    for (double x : parts) s += x;
-    *loss = s / ((double)B_valid * m->n_out);
-  }
   return QFS_OK;
 }
 
@@ -3304,7 +3295,7 @@ extern "C" int qfs_ws_create(qfs_ctx* ctx, uint64_t seed, int32_t batch_cap, qfs
     oH[l] = take((size_t)batch_cap * m->dout[l] * 2); oZ[l] = take((size_t)batch_cap * m->dout[l] * 4);
   }
   const size_t ophif = take(sizeof(double2) * 128), oX = take((size_t)batch_cap * 256 * 2),
-               odA32 = take((size_t)batch_cap * 1024 * 4), odB32 = take((size_t)batch_cap * 1024 * 4),
+               odH32 = take((size_t)batch_cap * 1024 * 4), olab = take((size_t)batch_cap * 192 * 8),
                odA16 = take((size_t)batch_cap * 1024 * 2), odB16 = take((size_t)batch_cap * 1024 * 2),
                oT1 = take((size_t)batch_cap * 1024 * 2), oT2 = take((size_t)batch_cap * 1024 * 2),
                oT = take((size_t)batch_cap * 192 * 4), olp = take(1040 * sizeof(double)),
@@ -3326,7 +3317,7 @@ extern "C" int qfs_ws_create(qfs_ctx* ctx, uint64_t seed, int32_t batch_cap, qfs
   }
   m->phif = (double2*)(b + ophif);
   m->X16 = (__nv_bfloat16*)(b + oX);
-  m->dA32 = (float*)(b + odA32); m->dB32 = (float*)(b + odB32);
+  m->dH32 = (float*)(b + odH32); m->lab64 = (double*)(b + olab);
   m->dA16 = (__nv_bfloat16*)(b + odA16); m->dB16 = (__nv_bfloat16*)(b + odB16);
   m->T1 = (__nv_bfloat16*)(b + oT1); m->T2 = (__nv_bfloat16*)(b + oT2);
   m->Tlab = (float*)(b + oT); m->loss_part = (double*)(b + olp);
@@ -3405,22 +3396,50 @@ extern "C" int qfs_ws_loss_grad(qfs_ws* m, int32_t count, const double* targets,
   TRY(set_device(m->ctx));
   cudaStream_t st = m->ctx->stream;
   const int B = (count + 127) / 128 * 128;
-  TRY(ws_load_features(m, targets, count, B));
-  std::vector<float> t((size_t)count * 192);
-  for (size_t i = 0; i < t.size(); ++i) t[i] = (float)labels[i];
-  CK(cudaMemcpyAsync(m->Tlab, t.data(), t.size() * 4, cudaMemcpyHostToDevice, st));
-  ws_forward(m, B);
-  TRY(ws_backward(m, B, count, loss));
-  if (grads_out) {
-    long long off = 0;
-    for (int l = 0; l < qfs_ws::kLayers; ++l) {
-      const size_t nw = (size_t)m->dout[l] * m->din[l], nb = m->dout[l];
-      CK(cudaMemcpyAsync(grads_out + off, m->gW[l], nw * 4, cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(grads_out + off + nw, m->gb[l], nb * 4, cudaMemcpyDeviceToHost, st));
-      off += nw + nb;
+  // The labels are copied (and rounded to FP32 on the device) on a second
+  // stream under the forward pass, which does not read them, and each layer's
+  // gradients leave on it under the backward pass of the layers below.
+  constexpr int L = qfs_ws::kLayers;
+  qfs_ctx* ctx = m->ctx;
+  TRY(ensure_group_streams(ctx, L));
+  cudaStream_t cs = ctx->gstream[0];
+  std::vector<double> parts(1024);
+  auto run = [&]() -> int {
+    CK(cudaEventRecord(ctx->fork_event, st));
+    TRY(ws_load_features(m, targets, count, B));
+    ws_forward(m, B);
+    CK(cudaStreamWaitEvent(cs, ctx->fork_event, 0));
+    CK(cudaMemcpyAsync(m->lab64, labels, sizeof(double) * 192 * (size_t)count, cudaMemcpyHostToDevice, cs));
+    launch_cast_f64_f32(m->lab64, m->Tlab, 192LL * count, cs);
+    CK(cudaEventRecord(ctx->gevent[0], cs));
+    CK(cudaStreamWaitEvent(st, ctx->gevent[0], 0));
+    int nparts = 0;
+    TRY(ws_backward(m, B, count, &nparts, nullptr, ctx->gevent));
+    if (grads_out) {
+      float* out = grads_out + ws_param_count(m);
+      for (int l = L - 1; l >= 0; --l) {
+        const size_t nw = (size_t)m->dout[l] * m->din[l], nb = m->dout[l];
+        out -= nw + nb;
+        CK(cudaStreamWaitEvent(cs, ctx->gevent[l], 0));
+        CK(cudaMemcpyAsync(out, m->gW[l], nw * 4, cudaMemcpyDeviceToHost, cs));
+        CK(cudaMemcpyAsync(out + nw, m->gb[l], nb * 4, cudaMemcpyDeviceToHost, cs));
+      }
     }
-  }
-  CK(cudaStreamSynchronize(st));
+    if (loss) {
+      CK(cudaMemcpyAsync(parts.data(), m->loss_part, sizeof(double) * nparts, cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      double s = 0.0;
+      for (int i = 0; i < nparts; ++i) s += parts[i];
+      *loss = s / ((double)count * m->n_out);
+    }
+    return QFS_OK;
+  };
+  const int rc = run();
+  // (The caller's buffers are in use until both streams are done.)
+  const cudaError_t e1 = cudaStreamSynchronize(cs), e2 = cudaStreamSynchronize(st);
+  if (rc != QFS_OK) return rc;
+  CK(e1);
+  CK(e2);
   return check_err_word(m);
 }
 
@@ -3454,17 +3473,16 @@ extern "C" int qfs_ws_train(qfs_ws* m, int32_t count, const double* targets, con
   }
   int rc = QFS_OK;
   {
-    std::vector<float> lb((size_t)m->B_cap * 192);
     for (int s0 = 0; s0 < count && rc == QFS_OK; s0 += m->B_cap) {
       const int bv = std::min(m->B_cap, count - s0);
       if (cudaMemcpyAsync(m->tgt, targets + (size_t)s0 * 512, sizeof(double2) * 256 * (size_t)bv,
                           cudaMemcpyHostToDevice, st) != cudaSuccess)
         rc = fail(QFS_ECUDA, "copy of targets failed");
       launch_ws_features(m->tgt, m->phif, bv, bv, Xall + (size_t)s0 * 256, st);
-      for (size_t i = 0; i < (size_t)bv * 192; ++i) lb[i] = (float)labels[(size_t)s0 * 192 + i];
-      if (cudaMemcpyAsync(Tall + (size_t)s0 * 192, lb.data(), sizeof(float) * 192 * (size_t)bv,
+      if (cudaMemcpyAsync(m->lab64, labels + (size_t)s0 * 192, sizeof(double) * 192 * (size_t)bv,
                           cudaMemcpyHostToDevice, st) != cudaSuccess)
         rc = fail(QFS_ECUDA, "copy of labels failed");
+      launch_cast_f64_f32(m->lab64, Tall + (size_t)s0 * 192, 192LL * bv, st);
       cudaStreamSynchronize(st);
     }
   }
@@ -3514,7 +3532,7 @@ extern "C" int qfs_ws_train(qfs_ws* m, int32_t count, const double* targets, con
     cudaStream_t s = m->ctx->stream;
     launch_ws_gather(Xall, Tall, didx, bv, B, m->X16, m->Tlab, s, jstep, batch);
     ws_forward(m, B);
-    TRY(ws_backward(m, B, bv, nullptr, ep_acc));
+    TRY(ws_backward(m, B, bv, nullptr, ep_acc, nullptr));
     for (int k = 0; k < qfs_ws::kLayers; ++k) {
       launch_adam(m->W[k], m->mW[k], m->vW[k], m->gW[k], (long long)m->dout[k] * m->din[k], 0.f, b1, b2, eps, 1.f,
                   1.f, m->W16[k], s, sched, gstep);

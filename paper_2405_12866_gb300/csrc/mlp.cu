@@ -158,73 +158,151 @@ __global__ void k_cast_f32_bf16(const float* __restrict__ a, __nv_bfloat16* __re
     b[i] = __float2bfloat16(a[i]);
 }
 
-// Output gradient of the mean squared error over the first n_out columns of
-// the first B_valid rows: dY = 2 (Y - T) / (B_valid n_out) (fp32 and bf16),
-// zero elsewhere; loss partial sums per block into loss_part[blockIdx.x].
-__global__ void k_ws_loss_grad(const float* __restrict__ Y, int ldy, const float* __restrict__ T, int n_out,
-                               int rows, int B_valid, float* __restrict__ dY32, __nv_bfloat16* __restrict__ dY16,
-                               double* __restrict__ loss_part) {
-  __shared__ double red[256];
-  double acc = 0.0;
-  const double scale = 2.0 / ((double)B_valid * n_out);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * ldy; e += gridDim.x * blockDim.x) {
-    const int r = e / ldy, c = e - r * ldy;
-    float g = 0.f;
-    if (r < B_valid && c < n_out) {
-      const double d = (double)Y[e] - (double)T[(size_t)r * n_out + c];
-      acc += d * d;
-      g = (float)(scale * d);
-    }
-    dY32[e] = g;
-    dY16[e] = __float2bfloat16(g);
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) loss_part[blockIdx.x] = red[0];
+__global__ void k_cast_f64_f32(const double* __restrict__ a, float* __restrict__ b, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    b[i] = (float)a[i];
 }
 
-// dZ = dH * gelu'(Z) (fp32 and bf16), rows >= B_valid zeroed.
-// Four elements per thread (n and ld multiples of 4); row-major, so the
-// first B_valid rows are exactly the elements below B_valid * ld.  dZ32 may
-// be dH (in place: each thread reads its four elements before writing them).
-__global__ void k_gelu_back(const float* dH, const float* __restrict__ Z, long long n, int ld, int B_valid,
-                            float* dZ32, __nv_bfloat16* __restrict__ dZ16) {
-  const long long nvalid = (long long)B_valid * ld;
-  for (long long i = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < n;
-       i += 4LL * gridDim.x * blockDim.x) {
-    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i < nvalid) {
-      const float4 h = *reinterpret_cast<const float4*>(dH + i), z = *reinterpret_cast<const float4*>(Z + i);
-      g = make_float4(h.x * gelu_grad_f(z.x), h.y * gelu_grad_f(z.y), h.z * gelu_grad_f(z.z), h.w * gelu_grad_f(z.w));
-    }
-    *reinterpret_cast<float4*>(dZ32 + i) = g;
-    const __nv_bfloat162 a = __floats2bfloat162_rn(g.x, g.y), b = __floats2bfloat162_rn(g.z, g.w);
-    *reinterpret_cast<uint2*>(dZ16 + i) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-  }
+// A 64 x 64 tile of a layer's output gradient G (256 threads; thread (tx, ty)
+// holds columns 4 tx .. + 3 of rows ty, ty + 16, ...): what the two products of
+// the layer's backward pass and its bias gradient need of it, while it is in
+// registers.  bf16 rows to G16 (rows x cols), the transposed tile to GT16 (cols
+// x rows) through shared memory, the column sums to db (zero before) by one
+// atomic per column and tile.
+//
+// As four kernels (gradient in FP32 and bf16, column sums, transpose, each
+// reading what the last one wrote) a hidden layer of 4096 x 1024 took 19.0 us
+// and the output layer 35; memory traffic 84 MB, here 50 (L2 holds most of
+// it).  Now 8.2 and 17 us, each with its column sums' memset (1.7 us).
+struct GradTile {
+  __nv_bfloat162 t[64][33];  // row stride 33 words: 2-way conflicts at most in the transposed reads
+  float sum[16][64];
+};
+__device__ __forceinline__ void grad_tile_row(GradTile& s, int r, int tx, float4 g, float4& acc,
+                                              __nv_bfloat16* __restrict__ row16) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(g.x, g.y), b = __floats2bfloat162_rn(g.z, g.w);
+  *reinterpret_cast<uint2*>(row16 + 4 * tx) =
+      make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  s.t[r][2 * tx] = a;
+  s.t[r][2 * tx + 1] = b;
+  acc.x += g.x;
+  acc.y += g.y;
+  acc.z += g.z;
+  acc.w += g.w;
 }
-
-// db[c] += sum over rows of G[r][c]: block (32 columns x 8 row lanes) over a
-// slice of the rows, reduced in shared memory, one atomic per column and
-// block (db is zeroed by the launcher).
-__global__ void k_colsum(const float* __restrict__ G, int rows, int cols, float* __restrict__ db) {
-  __shared__ float red[8][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  float s = 0.f;
-  if (c < cols)
-    for (int r = blockIdx.y * 8 + threadIdx.y; r < rows; r += 8 * gridDim.y) s += G[(size_t)r * cols + c];
-  red[threadIdx.y][threadIdx.x] = s;
+__device__ __forceinline__ void grad_tile_end(GradTile& s, int tid, float4 acc, int r0, int c0, int rows,
+                                              __nv_bfloat16* __restrict__ GT16, float* __restrict__ db) {
+  *reinterpret_cast<float4*>(&s.sum[tid >> 4][4 * (tid & 15)]) = acc;
   __syncthreads();
-  if (threadIdx.y == 0 && c < cols) {
+  if (tid < 64) {
     float t = 0.f;
 #pragma unroll
-    for (int y = 0; y < 8; ++y) t += red[y][threadIdx.x];
-    atomicAdd(db + c, t);
+    for (int y = 0; y < 16; ++y) t += s.sum[y][tid];
+    atomicAdd(db + c0 + tid, t);
   }
+  const __nv_bfloat16* tile = reinterpret_cast<const __nv_bfloat16*>(s.t);
+  const int lane = tid & 31;
+#pragma unroll
+  for (int c = tid >> 5; c < 64; c += 8) {
+    __nv_bfloat162 v;
+    v.x = tile[(2 * lane) * 66 + c];
+    v.y = tile[(2 * lane + 1) * 66 + c];
+    *reinterpret_cast<__nv_bfloat162*>(GT16 + (size_t)(c0 + c) * rows + r0 + 2 * lane) = v;
+  }
+}
+
+// Output gradient of the mean squared error over the first n_out columns of
+// the first B_valid rows: G = 2 (Y - T) / (B_valid n_out), zero elsewhere;
+// loss partial sums per block into loss_part[block] (at most 1024).  Block
+// column x walks the row tiles y, y + gridDim.y, ...
+//
+// Y - T, its square and its scaled value are pairs of floats (exact, 2^-45 and
+// the same rounded float as from FP64 but for one in ~2^20): FP64 conversions
+// and products for every entry were 24 us of that pipe.  Differences outside
+// the pairs' range take FP64.
+__global__ void __launch_bounds__(256)
+    k_ws_loss_grad(const float* __restrict__ Y, int ldy, const float* __restrict__ T, int n_out, int rows, int B_valid,
+                   double scale, __nv_bfloat16* __restrict__ G16, __nv_bfloat16* __restrict__ GT16, float* __restrict__ db,
+                   double* __restrict__ loss_part) {
+  __shared__ GradTile s;
+  __shared__ double red[8];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, c0 = blockIdx.x * 64;
+  const float sh = (float)scale, sl = (float)(scale - (double)sh);
+  double acc = 0.0;
+  for (int r0 = 64 * blockIdx.y; r0 < rows; r0 += 64 * gridDim.y) {
+    float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
+    float q_hi = 0.f, q_lo = 0.f;
+    const int c = c0 + 4 * tx;
+    float4 ly[4], lt[4];
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const int r = r0 + ty + 16 * y;
+      const bool in = r < B_valid && c < n_out;
+      ly[y] = in ? *reinterpret_cast<const float4*>(Y + (size_t)r * ldy + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      lt[y] = in ? *reinterpret_cast<const float4*>(T + (size_t)r * n_out + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const int r = r0 + ty + 16 * y;
+      float g[4];  // (0 where the loads gave 0)
+      {
+        const float4 v = ly[y], w = lt[y];
+        const float vy[4] = {v.x, v.y, v.z, v.w}, vt[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // d + de = Y - T exactly.
+          const float d = __fsub_rn(vy[e], vt[e]), b = __fsub_rn(d, vy[e]);
+          const float de = __fsub_rn(__fsub_rn(vy[e], __fsub_rn(d, b)), __fadd_rn(vt[e], b));
+          const float m = fabsf(d);
+          if (d == 0.f || (m >= 1e-18f && m <= 1e18f)) {
+            const float p = __fmul_rn(d, sh);
+            g[e] = __fadd_rn(p, __fmaf_rn(de, sh, __fmaf_rn(d, sl, __fmaf_rn(d, sh, -p))));
+            const float q = __fmul_rn(d, d), qe = __fmaf_rn(2.f * d, de, __fmaf_rn(d, d, -q));
+            const float t = __fadd_rn(q_hi, q), tb = __fsub_rn(t, q_hi);
+            q_lo = __fadd_rn(q_lo, __fadd_rn(__fadd_rn(__fsub_rn(q_hi, __fsub_rn(t, tb)), __fsub_rn(q, tb)), qe));
+            q_hi = t;
+          } else {
+            const double dd = (double)vy[e] - (double)vt[e];
+            acc += dd * dd;
+            g[e] = (float)(scale * dd);
+          }
+        }
+      }
+      grad_tile_row(s, ty + 16 * y, tx, make_float4(g[0], g[1], g[2], g[3]), col, G16 + (size_t)r * ldy + c0);
+    }
+    acc += (double)q_hi + (double)q_lo;
+    grad_tile_end(s, tid, col, r0, c0, rows, GT16, db);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) acc += __shfl_xor_sync(~0u, acc, m);
+  if ((tid & 31) == 0) red[tid >> 5] = acc;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < 8; ++w) acc += red[w];
+    loss_part[blockIdx.y * gridDim.x + blockIdx.x] = acc;
+  }
+}
+
+// G = dH * gelu'(Z) of a hidden layer, rows >= B_valid zero.
+__global__ void __launch_bounds__(256)
+    k_gelu_back(const float* __restrict__ dH, const float* __restrict__ Z, int rows, int cols, int B_valid,
+                __nv_bfloat16* __restrict__ G16, __nv_bfloat16* __restrict__ GT16, float* __restrict__ db) {
+  __shared__ GradTile s;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+  float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    const int r = r0 + ty + 16 * y;
+    const size_t at = (size_t)r * cols + c0 + 4 * tx;
+    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < B_valid) {
+      const float4 h = *reinterpret_cast<const float4*>(dH + at), z = *reinterpret_cast<const float4*>(Z + at);
+      g = make_float4(h.x * gelu_grad_f(z.x), h.y * gelu_grad_f(z.y), h.z * gelu_grad_f(z.z), h.w * gelu_grad_f(z.w));
+    }
+    grad_tile_row(s, ty + 16 * y, tx, g, col, G16 + (size_t)r * cols + c0);
+  }
+  grad_tile_end(s, tid, col, r0, c0, rows, GT16, db);
 }
 
 // acc += (sum of parts[0..n)) * scale (one block).
@@ -337,20 +415,21 @@ void launch_transpose_bf16(const __nv_bfloat16* src, int R, int C, __nv_bfloat16
 void launch_cast_f32_bf16(const float* a, __nv_bfloat16* b, long long n, cudaStream_t st) {
   k_cast_f32_bf16<<<blocks_for(n), 256, 0, st>>>(a, b, n);
 }
-int launch_ws_loss_grad(const float* Y, int ldy, const float* T, int n_out, int rows, int B_valid, float* dY32,
-                        __nv_bfloat16* dY16, double* loss_part, cudaStream_t st) {
-  const int blocks = blocks_for((long long)rows * ldy, 256, 1024);
-  k_ws_loss_grad<<<blocks, 256, 0, st>>>(Y, ldy, T, n_out, rows, B_valid, dY32, dY16, loss_part);
-  return blocks;
+void launch_cast_f64_f32(const double* a, float* b, long long n, cudaStream_t st) {
+  k_cast_f64_f32<<<blocks_for(n), 256, 0, st>>>(a, b, n);
 }
-void launch_gelu_back(const float* dH, const float* Z, long long n, int ld, int B_valid, float* dZ32,
-                      __nv_bfloat16* dZ16, cudaStream_t st) {
-  k_gelu_back<<<blocks_for(n / 4), 256, 0, st>>>(dH, Z, n, ld, B_valid, dZ32, dZ16);
+int launch_ws_loss_grad(const float* Y, int ldy, const float* T, int n_out, int rows, int B_valid, __nv_bfloat16* G16,
+                        __nv_bfloat16* GT16, float* db, double* loss_part, cudaStream_t st) {
+  const dim3 grid(ldy / 64, std::min(rows / 64, 1024 / (ldy / 64)));
+  cudaMemsetAsync(db, 0, sizeof(float) * (size_t)ldy, st);
+  k_ws_loss_grad<<<grid, 256, 0, st>>>(Y, ldy, T, n_out, rows, B_valid, 2.0 / ((double)B_valid * n_out), G16, GT16, db,
+                                       loss_part);
+  return (int)(grid.x * grid.y);
 }
-void launch_colsum(const float* G, int rows, int cols, float* db, cudaStream_t st) {
+void launch_gelu_back(const float* dH, const float* Z, int rows, int cols, int B_valid, __nv_bfloat16* G16,
+                      __nv_bfloat16* GT16, float* db, cudaStream_t st) {
   cudaMemsetAsync(db, 0, sizeof(float) * (size_t)cols, st);
-  const int ychunks = std::max(1, std::min(64, rows / 64));
-  k_colsum<<<dim3((cols + 31) / 32, ychunks), dim3(32, 8), 0, st>>>(G, rows, cols, db);
+  k_gelu_back<<<dim3(cols / 64, rows / 64), 256, 0, st>>>(dH, Z, rows, cols, B_valid, G16, GT16, db);
 }
 void launch_loss_accumulate(const double* parts, int n, double scale, double* acc, cudaStream_t st) {
   k_loss_accumulate<<<1, 256, 0, st>>>(parts, n, scale, acc);

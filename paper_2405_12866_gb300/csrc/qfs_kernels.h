@@ -361,12 +361,15 @@ void launch_ws_gather(const __nv_bfloat16* Xall, const float* Tall, const int* i
 // *jstep += 1 and *gstep += 1 on the device (the end of a training step).
 void launch_ws_step_advance(int* jstep, int* gstep, cudaStream_t st);
 void launch_cast_f32_bf16(const float* a, __nv_bfloat16* b, long long n, cudaStream_t st);
-// Returns the number of loss partial sums written.
-int launch_ws_loss_grad(const float* Y, int ldy, const float* T, int n_out, int rows, int B_valid, float* dY32,
-                        __nv_bfloat16* dY16, double* loss_part, cudaStream_t st);
-void launch_gelu_back(const float* dH, const float* Z, long long n, int ld, int B_valid, float* dZ32,
-                      __nv_bfloat16* dZ16, cudaStream_t st);
-void launch_colsum(const float* G, int rows, int cols, float* db, cudaStream_t st);
+void launch_cast_f64_f32(const double* a, float* b, long long n, cudaStream_t st);
+// A layer's output gradient, rows x cols (multiples of 64): bf16, bf16
+// transposed, and its column sums in db.  Of the loss (ldy columns, the first
+// n_out a multiple of 4; returns the number of loss partial sums written):
+int launch_ws_loss_grad(const float* Y, int ldy, const float* T, int n_out, int rows, int B_valid, __nv_bfloat16* G16,
+                        __nv_bfloat16* GT16, float* db, double* loss_part, cudaStream_t st);
+// ... and of a hidden layer from the gradient of its activations.
+void launch_gelu_back(const float* dH, const float* Z, int rows, int cols, int B_valid, __nv_bfloat16* G16,
+                      __nv_bfloat16* GT16, float* db, cudaStream_t st);
 // sched (nullable, device): lr, bc1, bc2 of step *sched_step (3 floats per
 // step), in place of the lr, bc1, bc2 arguments.
 void launch_adam(float* w, float* m, float* v, const float* g, long long n, float lr, float b1, float b2, float eps,
