@@ -93,3 +93,22 @@ def test_product_passes_nan_and_inf_on(ctx, n):
     got = _product(ctx, U, Psi, 0)
     assert np.isnan(got[3]).all() and not np.isfinite(got[4]).any()
     assert np.isfinite(np.delete(got, [3, 4], axis=0)).all()
+
+
+@pytest.mark.parametrize("n, M", [(2, 3), (3, 8), (5, 31), (6, 64)])
+def test_small_product_column_by_column_and_row_by_row(ctx, n, M):
+    """Up to 6 qubits: rows of U and columns of Psi of very different sizes in
+    one block, each to FP64 accuracy of its own.  The exact product comes from
+    integers: entries are multiples of 2^-20, scaled by powers of two.  A result
+    rounds by 2^-53 twice at most, its inputs by 2^-56 of the row's and the
+    column's largest entry times the sum of the others (2 2^n terms)."""
+    N = 1 << n
+    rng = np.random.default_rng(9)
+    u, p = (rng.integers(-(1 << 20), 1 << 20, s).astype(np.int64) for s in ((2, N, N), (2, N, M)))
+    ru, cp = rng.integers(-300, 300, (N, 1)), rng.integers(-200, 200, (1, M))
+    U, Psi = np.ldexp(u * 2.0**-20, ru), np.ldexp(p * 2.0**-20, cp)
+    want = np.ldexp((u[0] @ p[0] - u[1] @ p[1]) * 2.0**-40, ru + cp), np.ldexp((u[0] @ p[1] + u[1] @ p[0]) * 2.0**-40, ru + cp)
+    got = _product(ctx, U[0] + 1j * U[1], Psi[0] + 1j * Psi[1], 0)
+    size = np.abs(U).max(axis=(0, 2))[:, None] * np.abs(Psi).max(axis=(0, 1))[None, :]
+    for g, e in zip((got.real, got.imag), want):
+        assert np.all(np.abs(g - e) <= 2.0**-52 * np.abs(e) + 2 * N * 2.0**-55 * size)
