@@ -308,6 +308,7 @@ struct Run {
   std::vector<char> cl_plain;    // per slot: its sweeps take the plain FP64 form
   const void* df_key[4] = {};  // what the uploaded table was built for
   int df_key_r = -1;
+  bool lean = false;           // the workspace has room for the smallest buffers only
 };
 
 size_t elem_bytes(Real r) { return r == R32 ? sizeof(float2) : sizeof(double2); }
@@ -343,7 +344,7 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
   R.vprev = (double2*)take((size_t)R.S * R.L * 16 * sizeof(double2));
   R.partials = (double*)take((size_t)R.S * R.nblk_max * 32 * sizeof(double));
   R.costs = (double*)take((size_t)R.S * sizeof(double));
-  R.cost_rows = (double*)take((size_t)kSweepBatch * R.S * sizeof(double));
+  R.cost_rows = (double*)take((size_t)(R.lean ? kDfBatch : kSweepBatch) * R.S * sizeof(double));
   R.active = (int*)take((size_t)R.S * sizeof(int));
   R.counters = (unsigned*)take((size_t)(R.S + 1) * sizeof(unsigned));
   R.flag = (int*)take(sizeof(int) * 4);
@@ -357,8 +358,10 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
   R.df_steps = (DfStep*)take((size_t)std::max(R.df_cap, 1) * sizeof(DfStep));
   R.df_ctrl_cap = 1 + ((size_t)R.df_cap + 1) * R.S;
   R.df_ctrl = (unsigned*)take(sizeof(unsigned) * 2 * R.df_ctrl_cap);  // two slots: this sweep's, the next's
-  R.df_partials = (double*)take(std::max(sizeof(double) * 32, sizeof(float) * R.df_part_len) * (size_t)R.S *
-                                std::max(R.df_max_nchunk, 1));
+  // (lean: where the per-step launches keep theirs; a run takes one form or the other)
+  const size_t parts = std::max(sizeof(double) * 32, sizeof(float) * R.df_part_len) * (size_t)R.S *
+                       std::max(R.df_max_nchunk, 1);
+  R.df_partials = R.lean && parts <= sizeof(double) * 32 * (size_t)R.S * R.nblk_max ? R.partials : (double*)take(parts);
   // The residual pass keeps its double partials apart: in complex64 the
   // environment partials are floats, and one start's residual slots would
   // overlap another start's environment slots while that start still sweeps.
@@ -507,7 +510,7 @@ void df_build(const qfs_ctx* ctx, const Run& R, Real r, const void* psi, const v
   // FP64 sweeps do not (the doubled arithmetic of that step would cost more
   // than the pass over memory it saves).  Paired from the end, so that a gate
   // left over is gate 1, whose step the residual continues.
-  const bool pairs = r == R32 && ctx->df_fwd2;
+  const bool pairs = r == R32 && ctx->df_fwd2 && !R.lean;
   std::vector<std::pair<int, int>> groups;  // first gate, gates
   if (pairs) {
     for (int k = L; k >= 1;) {
@@ -691,19 +694,22 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
     R.nblk_max = std::max(R.nblk_max, make_bwd_shape(R.n, M, shape_starts(S), rs, ctx->num_sms, U).nblk);
     R.nblk64_max = std::max(R.nblk64_max, make_bwd_shape(R.n, M, 1, R64, ctx->num_sms, U).nblk);
   }
-  R.df_cap = 0;
-  R.df_max_nchunk = 0;
-  R.df_part_len = 32;
-  R.df_key_r = -1;
-  R.cl = ClPlan{};
-  if (ctx->dataflow && ctx->coop && !ctx->df_trace)
-    R.cl = cl_plan(prec == QFS_MIXED ? R32 : R64, R.n, M, R.L, S_target, beta != 0.0);
-  R.cl_plain.assign(T, 0);
-  // FP64 cluster sweeps, and the FP64 checks of complex64 runs.
-  R.cl_check = prec == QFS_MIXED && ctx->dataflow && cl_check_fits(R.n, R.L);
-  R.cl_fx = R.cl_check || (R.cl.C > 0 && prec == QFS_FP64);
-  {
-    const Real rs = prec == QFS_MIXED ? R32 : R64;
+  const Real rs = prec == QFS_MIXED ? R32 : R64;
+  // What the sweep and the product keep in the workspace.  lean: no cluster
+  // sweep, no digits and one gate per backward step, whose buffers are the
+  // smallest, for a run that a memory limit leaves no more room for.
+  auto plan = [&](bool lean) -> size_t {
+    R.lean = lean;
+    R.df_cap = 0;
+    R.df_max_nchunk = 0;
+    R.df_part_len = 32;
+    R.df_key_r = -1;
+    R.cl = ClPlan{};
+    if (!lean && ctx->dataflow && ctx->coop && !ctx->df_trace)
+      R.cl = cl_plan(rs, R.n, M, R.L, S_target, beta != 0.0);
+    // FP64 cluster sweeps, and the FP64 checks of complex64 runs.
+    R.cl_check = !lean && prec == QFS_MIXED && ctx->dataflow && cl_check_fits(R.n, R.L);
+    R.cl_fx = R.cl_check || (R.cl.C > 0 && prec == QFS_FP64);
     if (R.cl.C == 0 && df_usable(ctx, R, rs)) {
       std::vector<DfStep> steps;
       double b = 0.0;
@@ -714,15 +720,16 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
         if (st.kind == DF_ENV16) R.df_part_len = 512;
       }
     }
-  }
-  R.oz_bytes = oz_scratch_bytes((int)R.N, M, ctx->num_sms);
-  // (Without room for the digits' scratch the product takes another form.)
-  const size_t bytes = carve(R, nullptr, need_U, need_envs);
-  int rc = ensure_ws(ctx, bytes);
+    R.oz_bytes = lean ? 0 : oz_scratch_bytes((int)R.N, M, ctx->num_sms);
+    return carve(R, nullptr, need_U, need_envs);
+  };
+  R.cl_plain.assign(T, 0);
+  int rc = ensure_ws(ctx, plan(false));
   if (rc == QFS_ENOMEM && R.oz_bytes > 0) {
-    R.oz_bytes = 0;
+    R.oz_bytes = 0;  // (the product first: the sweep runs many times)
     rc = ensure_ws(ctx, carve(R, nullptr, need_U, need_envs));
   }
+  if (rc == QFS_ENOMEM) rc = ensure_ws(ctx, plan(true));
   TRY(rc);
   carve(R, ctx->ws, need_U, need_envs);
   const size_t blist = (size_t)std::max(R.L - 1, 1) * S * R.sN * elem_bytes(prec == QFS_MIXED ? R32 : R64);
