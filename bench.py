@@ -140,8 +140,8 @@ def bf16_peak(sustained=True):
 
 
 KERNEL_SOURCES = {
-    "k_sweep_df": ("sweep_df.cu", "polar4.cuh", "qfs_common.cuh", "qfs_kernels.h"),
-    "k_batch_sweep": ("batch.cu", "polar4.cuh", "qfs_common.cuh", "qfs_kernels.h"),
+    "k_sweep_df": ("sweep_df.cu", "polar_newton.cuh", "fixed.cuh", "polar4.cuh", "qfs_common.cuh", "qfs_kernels.h"),
+    "k_batch_sweep": ("batch.cu", "polar_newton.cuh", "fixed.cuh", "polar4.cuh", "qfs_common.cuh", "qfs_kernels.h"),
     "k_backward_q4": ("kernels_sweep.cu", "polar4.cuh", "qfs_common.cuh", "qfs_kernels.h"),
 }
 
