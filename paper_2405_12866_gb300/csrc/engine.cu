@@ -739,11 +739,11 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   return QFS_OK;
 }
 
-// Phi_L = U Psi (Sec. 3, the A tensor), to FP64 accuracy: from 128 rows on by
-// digits on the tensor cores (n = 7, M = 24: 75 us in FP64, 25 us in its four
-// launches; n = 12, M = 32: 4.28 ms and 0.22), below in fixed point.  (Without
-// room for the digits' scratch, or when a mixed run asks for it, the FP64
-// kernel.)  Returns the launches.
+// Phi_L = U Psi (Sec. 3, the A tensor), to FP64 accuracy: from 512 rows on by
+// digits on the tensor cores (a call at n = 9, M = 24: 302 us in FP64, 57 so; n =
+// 12, M = 32: 4.28 ms and 0.19), below in fixed point (n = 8, M = 24: 163 us in
+// FP64, 53 by digits, 40 so).  (Without room for the digits' scratch, or when a
+// mixed run asks for it, the FP64 kernel.)  Returns the launches.
 int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out) {
   cudaStream_t st = ctx->stream;
   const bool plain = R.prec == QFS_MIXED && ctx->upsi_fp64;
@@ -751,7 +751,7 @@ int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, d
     launch_oz_product(U, psi, out, (int)R.N, R.M, R.oz, R.err, ctx->num_sms, st);
     return 4;
   }
-  if (R.n <= 6 && !plain) launch_fx_product(U, psi, out, R.n, R.M, st);
+  if (R.n <= kFxProductQubits && !plain) launch_fx_product(U, psi, out, R.n, R.M, st);
   else launch_gemm_upsi(U, psi, out, (int)R.N, R.M, st);
   return 1;
 }
@@ -2094,22 +2094,21 @@ int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* tar
   cudaStream_t st = ctx->stream;
   // (Without room for the digits' scratch: the FP64 kernel.)
   const size_t oz = oz_scratch_bytes(N, M, ctx->num_sms);
-  if (oz > 0 && ensure_ws(ctx, 256 + oz) == QFS_OK) {
-    int* err = reinterpret_cast<int*>(ctx->ws);
-    CK(cudaMemsetAsync(err, 0, sizeof(int), st));
-    ctx->prof.launches[QFS_PROF_GEMM] += 4;
-    CK(launch_oz_product(U, P, O, N, M, ctx->ws + 256, err, ctx->num_sms, st));
+  if (oz > 0 && ensure_ws(ctx, oz) == QFS_OK) {
+    // (The kernel sets the error word in pinned host memory: no memset before it
+    // and no copy behind it.)
     TRY(ensure_pinned(ctx, 1));
-    CK(cudaMemcpyAsync(ctx->h_pinned, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    volatile int* err = reinterpret_cast<volatile int*>(ctx->h_pinned);
+    *err = 0;
+    ctx->prof.launches[QFS_PROF_GEMM] += 4;
+    CK(launch_oz_product(U, P, O, N, M, ctx->ws, const_cast<int*>(err), ctx->num_sms, st));
     CK(cudaStreamSynchronize(st));
-    int e;
-    std::memcpy(&e, ctx->h_pinned, sizeof(int));
-    if (e) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", e);
+    if (*err) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", *err);
     return QFS_OK;
   }
   g_err.clear();
   ctx->prof.launches[QFS_PROF_GEMM] += 1;
-  if (n <= 6) launch_fx_product(U, P, O, n, M, st);
+  if (n <= kFxProductQubits) launch_fx_product(U, P, O, n, M, st);
   else launch_gemm_upsi(U, P, O, N, M, st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
@@ -2228,7 +2227,7 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
                        cudaMemcpyDeviceToDevice, st));
   // Phi_L = U Psi: digits where their scratch still fits behind the sweep's.
   const size_t oz = oz_scratch_bytes((int)R.N, M, sms);
-  if (R.n <= 6) {
+  if (R.n <= kFxProductQubits) {
     launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st);
   } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
     int* err = reinterpret_cast<int*>(take(sizeof(int)));

@@ -24,9 +24,9 @@
 // and less, and may round.  What is left out (d > 7) is below 2^-60 of the
 // result's scale.
 //
-// Below 128 rows there is no tile to fill: k_fx_product forms the product in
-// 64-bit fixed point (fixed.cuh), one component per thread (n = 6, M = 16: 50 us
-// as FP64, 6 us so).
+// Up to 256 rows there are at most two tiles to fill: k_fx_product forms the
+// product in 64-bit fixed point (fixed.cuh), a component by one or two threads (n
+// = 6, M = 16: 50 us as FP64, 6 us so).
 //
 // U's digits have a fixed scale, so its rows have to have a norm near 1, as a
 // unitary's do.  The kernel sums their squares on the way; if any is outside
@@ -464,8 +464,7 @@ __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__
   if (e == 1 << 20 && row == 0) atomicOr(flag, 1);
 }
 
-// out = U Psi for N <= 64 rows: grid (N / 8 row tiles (at least 1), column tiles
-// of 32).  A scale for every row of U and every column of Psi, from its largest
+// out = U Psi for N <= 256 rows: grid (N / 8 row tiles (at least 1), column tiles).  A scale for every row of U and every column of Psi, from its largest
 // entry, with room for 2 N terms: the high sums stay below 2^62, each cross sum
 // below 2^62 and both together below 2^63.  Where a row's or a column's entries
 // are far from 1, Inf or NaN, its results take FP64 arithmetic.
@@ -475,10 +474,16 @@ __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__
 // cross sums below 2^-60 count here, because the room for 2 N terms puts the
 // result's scale up to 2^9 above the result (without them 1.3e-15 of the norm at
 // n = 6, FP64 arithmetic 3.8e-16; with them 2.2e-16, in the same time).
-constexpr int kFxRows = 8, kFxCols = 32;
+//
+// At n = 7 and 8 too, in tiles of 8 columns with KS = 2 threads to a component
+// (which take every second term each): one launch takes less than the four of the
+// digits (a call with M = 24: n = 7 61 -> 33 us, n = 8 53 -> 40, n = 9 by digits 54).
+constexpr int kFxRows = 8;
+template <int kFxCols, int KS>
 __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ U, const double2* __restrict__ Psi,
                                                     double2* __restrict__ out, int n, int M) {
-  __shared__ int4 su[kFxRows * 64], sp[64 * kFxCols];
+  extern __shared__ int4 su[];  // kFxRows x N, then N x kFxCols
+  int4* sp = su + (kFxRows << n);
   __shared__ int tu[kFxRows], tp[kFxCols];  // largest exponent fields
   const int N = 1 << n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = blockIdx.x * kFxRows, rows = min(kFxRows, N - r0), c0 = blockIdx.y * kFxCols, cols = min(kFxCols, M - c0);
@@ -498,8 +503,23 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
   for (int i = tid; i < rows * N; i += 256) su[i] = fx_from2(U[(long long)r0 * N + i], eu(i >> n));
   for (int i = tid; i < N * cols; i += 256) sp[i] = fx_from2(Psi[(long long)(i / cols) * M + c0 + i % cols], ep(i % cols));
   __syncthreads();
-  for (int c = tid; c < 2 * rows * cols; c += 256) {
-    const int im = c & 1, i = (c >> 1) / cols, j = (c >> 1) % cols;
+  for (int e = tid; e < 2 * KS * rows * cols; e += 256) {  // (KS = 2: a multiple of 32, so warps are whole)
+    const int c = e / KS, part = e % KS, im = c & 1, i = (c >> 1) / cols, j = (c >> 1) % cols;
+    FxSum t;
+    long long low = 0;  // low x low, in units of 2^-112
+    for (int k = part; k < N; k += KS) {
+      const int4 x = su[i * N + k], y = sp[k * cols + j];
+      const int b1 = im ? y.w : y.y, a2 = im ? x.w : -x.w, b2 = im ? y.y : y.w;
+      t.add(x.x, x.y, im ? y.z : y.x, b1);
+      t.add(im ? x.z : -x.z, a2, im ? y.x : y.z, b2);
+      low += (mad64(x.y, b1, 0) >> 8) + (mad64(a2, b2, 0) >> 8);
+    }
+    long long cross = t.c + t.d + (low >> 22);
+    if constexpr (KS == 2) {
+      t.h += __shfl_xor_sync(FULL, t.h, 1);
+      cross += __shfl_xor_sync(FULL, cross, 1);
+      if (part) continue;
+    }
     double v = 0.0;
     if (fx_out_of_range(tu[i]) || fx_out_of_range(tp[j])) {
       for (int k = 0; k < N; ++k) {
@@ -507,16 +527,7 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
         v = im ? fma(x.x, y.y, fma(x.y, y.x, v)) : fma(x.x, y.x, fma(-x.y, y.y, v));
       }
     } else {
-      FxSum t;
-      long long low = 0;  // low x low, in units of 2^-112
-      for (int k = 0; k < N; ++k) {
-        const int4 x = su[i * N + k], y = sp[k * cols + j];
-        const int b1 = im ? y.w : y.y, a2 = im ? x.w : -x.w, b2 = im ? y.y : y.w;
-        t.add(x.x, x.y, im ? y.z : y.x, b1);
-        t.add(im ? x.z : -x.z, a2, im ? y.x : y.z, b2);
-        low += (mad64(x.y, b1, 0) >> 8) + (mad64(a2, b2, 0) >> 8);
-      }
-      v = scale_exp(fma((double)(t.c + t.d + (low >> 22)), 1.0 / (1LL << kFxLow), (double)t.h), eu(i) + ep(j) - kFxBits);
+      v = scale_exp(fma((double)cross, 1.0 / (1LL << kFxLow), (double)t.h), eu(i) + ep(j) - kFxBits);
     }
     reinterpret_cast<double*>(out + (long long)(r0 + i) * M + c0 + j)[im] = v;
   }
@@ -545,7 +556,7 @@ OzShape oz_shape(int N, int M, int num_sms) {
 
 }  // namespace
 
-size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 128 ? 0 : oz_shape(N, M, num_sms).total; }
+size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 512 ? 0 : oz_shape(N, M, num_sms).total; }
 
 const int* oz_flag(const void* scratch, int N, int M, int num_sms) {
   const OzShape s = oz_shape(N, M, num_sms);
@@ -575,7 +586,16 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
 }
 
 void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st) {
-  k_fx_product<<<dim3(std::max(1, (1 << n) / kFxRows), (M + kFxCols - 1) / kFxCols), 256, 0, st>>>(U, Psi, out, n, M);
+  const unsigned tiles = (unsigned)std::max(1, (1 << n) / kFxRows);
+  const int cols = n <= 6 ? 32 : 8;
+  const size_t smem = sizeof(int4) * (size_t)(kFxRows + cols) << n;  // (n = 8: 64 KB)
+  const dim3 grid(tiles, (M + cols - 1) / cols);
+  if (n <= 6) {
+    k_fx_product<32, 1><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
+  } else {
+    cudaFuncSetAttribute(k_fx_product<8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_fx_product<8, 2><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
+  }
 }
 
 }  // namespace qfs

@@ -233,13 +233,14 @@ void launch_gate_update_batch(int count, const double2* envs, const double2* g_o
 // only_if (nullable, device): the kernel does nothing when it holds zero.
 void launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
                       cudaStream_t st, const int* only_if = nullptr);
-// The same product, for N >= 128, from 8-bit digits on the tensor cores
+// The same product, for N >= 512, from 8-bit digits on the tensor cores
 // (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1.
 // err: device word, bit 0 set when a bounded wait ran out.
 // The word in its scratch that is not zero, once it has run, when the FP64 kernel
 // ran too: for one, whenever U or Psi holds Inf or NaN.
 const int* oz_flag(const void* scratch, int N, int M, int num_sms);
-// The same for n <= 6 in 64-bit fixed point.
+// The same for n <= 8 in 64-bit fixed point.
+constexpr int kFxProductQubits = 8;
 void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st);
 size_t oz_scratch_bytes(int N, int M, int num_sms);
 cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,

@@ -1,5 +1,5 @@
-"""U Psi from 8-bit digits on the tensor cores (n >= 7) and in fixed point (n
-<= 6) against complex128 numpy, at the sizes where a tile, a column block or a
+"""U Psi from 8-bit digits on the tensor cores (n >= 9) and in fixed point (n
+<= 8) against complex128 numpy, at the sizes where a tile, a column block or a
 split ends, on targets whose digits are all alike or mostly zero, and on inputs
 outside the digits' scale (the FP64 kernel behind them).
 
@@ -95,9 +95,9 @@ def test_product_passes_nan_and_inf_on(ctx, n):
     assert np.isfinite(np.delete(got, [3, 4], axis=0)).all()
 
 
-@pytest.mark.parametrize("n, M", [(2, 3), (3, 8), (5, 31), (6, 64)])
+@pytest.mark.parametrize("n, M", [(2, 3), (3, 8), (5, 31), (6, 64), (7, 9), (7, 128), (8, 1), (8, 50)])
 def test_small_product_column_by_column_and_row_by_row(ctx, n, M):
-    """Up to 6 qubits: rows of U and columns of Psi of very different sizes in
+    """Up to 8 qubits: rows of U and columns of Psi of very different sizes in
     one block, each to FP64 accuracy of its own.  The exact product comes from
     integers: entries are multiples of 2^-20, scaled by powers of two.  A result
     rounds by 2^-53 twice at most, its inputs by 2^-56 of the row's and the
@@ -112,3 +112,23 @@ def test_small_product_column_by_column_and_row_by_row(ctx, n, M):
     size = np.abs(U).max(axis=(0, 2))[:, None] * np.abs(Psi).max(axis=(0, 1))[None, :]
     for g, e in zip((got.real, got.imag), want):
         assert np.all(np.abs(g - e) <= 2.0**-52 * np.abs(e) + 2 * N * 2.0**-55 * size)
+
+
+@pytest.mark.parametrize("what", ["identity", "minus_identity", "hadamard", "hadamard_of_hadamard", "permutation", "basis_states"])
+def test_digits_of_structured_targets(ctx, what):
+    test_product_of_structured_targets(ctx, 9, what)
+
+
+@pytest.mark.parametrize("what", ["target_times_2", "target_times_1e-9", "one_row_times_3", "columns_of_all_sizes", "no_states",
+                                  "tiny_states", "huge_states"])
+def test_digits_of_inputs_without_unit_norms(ctx, what):
+    test_product_of_inputs_without_unit_norms(ctx, 9, what)
+
+
+@pytest.mark.parametrize("M", [1, 16, 17, 32, 33])
+def test_digits_match_numpy(ctx, M):
+    test_product_matches_numpy(ctx, 9, M, 0)
+
+
+def test_digits_pass_nan_and_inf_on(ctx):
+    test_product_passes_nan_and_inf_on(ctx, 9)
