@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(128) k_batch_finalize(BatchArgs a) {
 
 void launch_batch_prep(const BatchArgs& a, cudaStream_t st) {
   const size_t smem = (size_t)a.max_prep * sizeof(int4);
-  cudaFuncSetAttribute(k_batch_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_batch_prep, kBatchPrepSmem);
   k_batch_prep<<<a.P, 128, smem, st>>>(a);
 }
 
@@ -654,7 +654,7 @@ size_t batch_sweep_smem(int G, int warps, int max_elems, int max_L) {
 namespace {
 template <int G>
 int blocks_per_sm_g(int warps, size_t smem) {
-  cudaFuncSetAttribute(k_batch_sweep<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_batch_sweep<G>, kBatchSweepSmem);
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_sweep<G>, 32 * warps, smem) != cudaSuccess) {
     cudaGetLastError();
@@ -692,21 +692,14 @@ int batch_sweep_blocks_per_sm(int G, int warps, size_t smem) {
 void launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
                         int warps, int region_f2, cudaStream_t st) {
   const size_t smem = (size_t)warps * region_f2 * sizeof(float2);
-  const void* kernels[4] = {(const void*)k_batch_sweep<4>, (const void*)k_batch_sweep<8>, (const void*)k_batch_sweep<16>,
-                            (const void*)k_batch_sweep<32>};
-  cudaFuncSetAttribute(kernels[G == 4 ? 0 : G == 8 ? 1 : G == 16 ? 2 : 3], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
-  switch (G) {
-    case 4: k_batch_sweep<4><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
-    case 8: k_batch_sweep<8><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
-    case 16: k_batch_sweep<16><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
-    default: k_batch_sweep<32><<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2); break;
-  }
+  const auto kernel = G == 4 ? k_batch_sweep<4> : G == 8 ? k_batch_sweep<8> : G == 16 ? k_batch_sweep<16> : k_batch_sweep<32>;
+  allow_smem(kernel, kBatchSweepSmem);
+  kernel<<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2);
 }
 
 void launch_batch_finalize(const BatchArgs& a, cudaStream_t st) {
   const size_t smem = (size_t)(3 * a.max_elems + 32 * a.max_L) * sizeof(double2);
-  cudaFuncSetAttribute(k_batch_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_batch_finalize, kBatchFinalizeSmem);
   k_batch_finalize<<<a.P, 128, smem, st>>>(a);
 }
 

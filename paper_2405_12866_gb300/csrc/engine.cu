@@ -2299,7 +2299,7 @@ int batch_warps_region(int G, int region_f2) {
   int best = 0, best_res = 0;
   for (int w : {4, 2, 8}) {
     const size_t smem = (size_t)w * region_f2 * sizeof(float2);
-    if (smem > 200 * 1024) continue;
+    if (smem > kBatchSweepSmem) continue;
     const int res = w * batch_sweep_blocks_per_sm(G, w, smem);
     if (res > best_res) {
       best_res = res;
@@ -2495,11 +2495,11 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
   int max_elems = 0, max_L = 0, max_prep = 0;
   for (int i = 0; i < P; ++i) {
     const int n = ns[i], L = Ls[i];
-    if (n < 2 || n > 6) return fail(QFS_EUNSUPPORTED, "problem %d: n = %d (batched form: 2..6)", i, n);
-    if (L < 1 || L > 32) return fail(QFS_EUNSUPPORTED, "problem %d: L = %d (batched form: 1..32)", i, L);
+    if (n < 2 || n > kBatchMaxQubits) return fail(QFS_EUNSUPPORTED, "problem %d: n = %d (batched form: 2..6)", i, n);
+    if (L < 1 || L > kBatchMaxGates) return fail(QFS_EUNSUPPORTED, "problem %d: L = %d (batched form: 1..32)", i, L);
     const int N = 1 << n;
     int M = p->M > 0 ? std::min(p->M, N) : N / 2;
-    if (M * N > 1024) return fail(QFS_EUNSUPPORTED, "problem %d: N*M = %d > 1024", i, M * N);
+    if (M * N > kBatchMaxElems) return fail(QFS_EUNSUPPORTED, "problem %d: N*M = %d > 1024", i, M * N);
     qfs_circuit c{n, L, pairs + pair_off};
     TRY(check_circuit(&c));
     probs[i] = BatchProblem{n, L, M, (int)pair_off, state_off, target_off, gate_off, gout_off};
@@ -2639,7 +2639,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
       c.warps = 0;
       for (int wv : {4, 2, 8}) {
         const size_t smem = batch_sweep_smem(c.G, wv, c.M << c.n, c.L);
-        if (smem <= 200 * 1024 && batch_sweep_blocks_per_sm(c.G, wv, smem) >= 1) {
+        if (smem <= kBatchSweepSmem && batch_sweep_blocks_per_sm(c.G, wv, smem) >= 1) {
           c.warps = wv;
           break;
         }

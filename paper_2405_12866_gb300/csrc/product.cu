@@ -593,7 +593,7 @@ void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n
   if (n <= 6) {
     k_fx_product<32, 1><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
   } else {
-    cudaFuncSetAttribute(k_fx_product<8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_fx_product<8, 2>, sizeof(int4) * (size_t)(kFxRows + 8) << kFxProductQubits);
     k_fx_product<8, 2><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
   }
 }

@@ -13,6 +13,16 @@ namespace qfs {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// Lets launches of a kernel take up to `bytes` of dynamic shared memory.  The
+// limit belongs to the function on its device, not to the calling thread, so
+// every caller passes the same: the most any launch of that kernel takes.  (A
+// limit of this launch's size could be lowered by another host thread between
+// here and the launch, which then fails.)
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 template <typename T> struct C2;
 template <> struct C2<float>  { using t = float2;  };
 template <> struct C2<double> { using t = double2; };

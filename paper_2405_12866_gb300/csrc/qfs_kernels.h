@@ -255,6 +255,11 @@ void launch_nonfinite_check(const double* x, long long count, int* flag, cudaStr
 // ---------------------------------------------------------------- batches
 
 constexpr int kBatchMaxWarps = 8;
+// What the batched form takes, and the shared memory its kernels may need then.
+constexpr int kBatchMaxQubits = 6, kBatchMaxGates = 32, kBatchMaxElems = 1024;  // (N M)
+constexpr size_t kBatchPrepSmem = ((size_t)(1 << 2 * kBatchMaxQubits) + kBatchMaxElems) * 16;
+constexpr size_t kBatchFinalizeSmem = (size_t)(3 * kBatchMaxElems + 32 * kBatchMaxGates) * 16;
+constexpr size_t kBatchSweepSmem = 200 * 1024;  // a block's, at most: launch shapes above it are not considered
 
 // One instantiation problem of a batch; offsets are in complex elements
 // (pairs: in ints) into the packed arrays of BatchArgs.
