@@ -639,10 +639,9 @@ __global__ void __launch_bounds__(128) k_batch_finalize(BatchArgs a) {
   }
 }
 
-void launch_batch_prep(const BatchArgs& a, cudaStream_t st) {
-  const size_t smem = (size_t)a.max_prep * sizeof(int4);
-  allow_smem(k_batch_prep, kBatchPrepSmem);
-  k_batch_prep<<<a.P, 128, smem, st>>>(a);
+cudaError_t launch_batch_prep(const BatchArgs& a, cudaStream_t st) {
+  const cudaError_t e = allow_smem(k_batch_prep, kBatchPrepSmem);
+  return e != cudaSuccess ? e : launch_kernel(k_batch_prep, a.P, 128, (size_t)a.max_prep * sizeof(int4), st, a);
 }
 
 int batch_region_f2(int G, int max_elems, int max_L) { return (32 / G) * batch_slice_f2(max_elems, max_L); }
@@ -689,18 +688,18 @@ int batch_sweep_blocks_per_sm(int G, int warps, size_t smem) {
   return b;
 }
 
-void launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
-                        int warps, int region_f2, cudaStream_t st) {
+cudaError_t launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
+                               int warps, int region_f2, cudaStream_t st) {
   const size_t smem = (size_t)warps * region_f2 * sizeof(float2);
   const auto kernel = G == 4 ? k_batch_sweep<4> : G == 8 ? k_batch_sweep<8> : G == 16 ? k_batch_sweep<16> : k_batch_sweep<32>;
-  allow_smem(kernel, kBatchSweepSmem);
-  kernel<<<blocks, 32 * warps, smem, st>>>(a, units, nunits, queue, region_f2);
+  const cudaError_t e = allow_smem(kernel, kBatchSweepSmem);
+  return e != cudaSuccess ? e : launch_kernel(kernel, blocks, 32 * warps, smem, st, a, units, nunits, queue, region_f2);
 }
 
-void launch_batch_finalize(const BatchArgs& a, cudaStream_t st) {
+cudaError_t launch_batch_finalize(const BatchArgs& a, cudaStream_t st) {
   const size_t smem = (size_t)(3 * a.max_elems + 32 * a.max_L) * sizeof(double2);
-  allow_smem(k_batch_finalize, kBatchFinalizeSmem);
-  k_batch_finalize<<<a.P, 128, smem, st>>>(a);
+  const cudaError_t e = allow_smem(k_batch_finalize, kBatchFinalizeSmem);
+  return e != cudaSuccess ? e : launch_kernel(k_batch_finalize, a.P, 128, smem, st, a);
 }
 
 }  // namespace qfs

@@ -743,17 +743,19 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
 // digits on the tensor cores (a call at n = 9, M = 24: 302 us in FP64, 57 so; n =
 // 12, M = 32: 4.28 ms and 0.19), below in fixed point (n = 8, M = 24: 163 us in
 // FP64, 53 by digits, 40 so).  (Without room for the digits' scratch, or when a
-// mixed run asks for it, the FP64 kernel.)  Returns the launches.
-int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out) {
+// mixed run asks for it, the FP64 kernel.)  Adds its launches to *launches.
+int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out, long long* launches) {
   cudaStream_t st = ctx->stream;
   const bool plain = R.prec == QFS_MIXED && ctx->upsi_fp64;
   if (R.oz && !plain) {
-    launch_oz_product(U, psi, out, (int)R.N, R.M, R.oz, R.err, ctx->num_sms, st);
-    return 4;
+    CK(launch_oz_product(U, psi, out, (int)R.N, R.M, R.oz, R.err, ctx->num_sms, st));
+    *launches += 4;
+    return QFS_OK;
   }
-  if (R.n <= kFxProductQubits && !plain) launch_fx_product(U, psi, out, R.n, R.M, st);
-  else launch_gemm_upsi(U, psi, out, (int)R.N, R.M, st);
-  return 1;
+  if (R.n <= kFxProductQubits && !plain) CK(launch_fx_product(U, psi, out, R.n, R.M, st));
+  else CK(launch_gemm_upsi(U, psi, out, (int)R.N, R.M, st));
+  *launches += 1;
+  return QFS_OK;
 }
 
 // Phi_L = U Psi, complex64 copies for the mixed sweeps, gate copies.
@@ -775,7 +777,8 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
   }
   {
     ProfScope ps(ctx, QFS_PROF_GEMM, 8.0 * R.N * R.N * R.M);  // flops, not bytes
-    ctx->prof.launches[QFS_PROF_GEMM] += target_product(ctx, R, R.Uslot[t], R.psi64 + so, R.phil64 + so) - 1;
+    --ctx->prof.launches[QFS_PROF_GEMM];  // (the scope counts one, the product all of its own)
+    TRY(target_product(ctx, R, R.Uslot[t], R.psi64 + so, R.phil64 + so, &ctx->prof.launches[QFS_PROF_GEMM]));
   }
   {
     // The product in digits has read all of U: only where it met something out
@@ -801,7 +804,7 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
   if (R.cl_scale) {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     CK(cudaMemsetAsync(R.cl_acc + 4, 0, sizeof(unsigned), st));
-    launch_cl_scale(R.n, R.M, R.spt * R.L, R.psi64 + so, R.phil64 + so, R.g64 + go, R.cl_acc, R.cl_scale + t, st);
+    CK(launch_cl_scale(R.n, R.M, R.spt * R.L, R.psi64 + so, R.phil64 + so, R.g64 + go, R.cl_acc, R.cl_scale + t, st));
     CK(cudaMemcpyAsync(&sc, R.cl_scale + t, sizeof(int4), cudaMemcpyDeviceToHost, st));
   }
   int flag = 0;
@@ -1552,7 +1555,7 @@ int instantiate_restarting(qfs_ctx* ctx, const qfs_circuit* c, const double* tar
       draw_states(p->training_distribution, sa, 5u, n, M, h.data());
       CK(cudaMemcpyAsync(R.psi_val64, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
       CK(cudaMemsetAsync(R.err, 0, sizeof(int), st));
-      ctx->prof.launches[QFS_PROF_GEMM] += target_product(ctx, R, R.U, R.psi_val64, R.phil_val64);
+      TRY(target_product(ctx, R, R.U, R.psi_val64, R.phil_val64, &ctx->prof.launches[QFS_PROF_GEMM]));
       int err = 0;
       CK(cudaMemcpyAsync(&err, R.err, sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
@@ -2108,8 +2111,8 @@ int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* tar
   }
   g_err.clear();
   ctx->prof.launches[QFS_PROF_GEMM] += 1;
-  if (n <= kFxProductQubits) launch_fx_product(U, P, O, n, M, st);
-  else launch_gemm_upsi(U, P, O, N, M, st);
+  if (n <= kFxProductQubits) CK(launch_fx_product(U, P, O, n, M, st));
+  else CK(launch_gemm_upsi(U, P, O, N, M, st));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
   return QFS_OK;
@@ -2228,12 +2231,12 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
   // Phi_L = U Psi: digits where their scratch still fits behind the sweep's.
   const size_t oz = oz_scratch_bytes((int)R.N, M, sms);
   if (R.n <= kFxProductQubits) {
-    launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st);
+    CK(launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st));
   } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
     int* err = reinterpret_cast<int*>(take(sizeof(int)));
     CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), err, sms, st));
   } else {
-    launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st);
+    CK(launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st));
   }
   // The cluster sweep where it takes the problem (n = 6, 10 gates, M = 16, 8
   // starts: 305 us as 40 launches, 90 us as 5).  Nothing comes back to the host
@@ -2248,7 +2251,7 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
     R.costs = costs_out_dev ? costs_out_dev : reinterpret_cast<double*>(R.phi);
     R.spt = S;
     R.cl_plain = {0, 1};
-    launch_cl_scale(R.n, M, S * R.L, R.psi64, R.phil64, R.g64, R.cl_acc, R.cl_scale, st);
+    CK(launch_cl_scale(R.n, M, S * R.L, R.psi64, R.phil64, R.g64, R.cl_acc, R.cl_scale, st));
     TRY(cl_sweep(&tmp, R, R64, R.psi64, R.phil64, reinterpret_cast<double2*>(envs_out_dev), nullptr, st));
     CK(cudaGetLastError());
     return QFS_OK;
@@ -2414,8 +2417,8 @@ int autotune_batch(qfs_ctx* ctx, BatchArgs a, const std::vector<BatchProblem>& p
       for (int rep = 0; rep < 3; ++rep) {  // the first run warms up
         CK(cudaMemsetAsync(queue_dev, 0, sizeof(int), st));
         CK(cudaEventRecord(e0, st));
-        launch_batch_sweep(G, t, units_dev, (int)u.size(), queue_dev, blocks, w, batch_region_f2(G, c.M << c.n, c.L),
-                           st);
+        CK(launch_batch_sweep(G, t, units_dev, (int)u.size(), queue_dev, blocks, w, batch_region_f2(G, c.M << c.n, c.L),
+                              st));
         CK(cudaEventRecord(e1, st));
         CK(cudaEventSynchronize(e1));
         CK(cudaGetLastError());
@@ -2653,7 +2656,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
       for (auto& kv : ctx->batch_tuned) f |= kv.first == batch_class_key(c.n, c.L, c.M, S, true);
       untuned |= !f;
     }
-    if (untuned) launch_batch_prep(a, st);
+    if (untuned) CK(launch_batch_prep(a, st));
     TRY(autotune_batch(ctx, a, probs, classes, units_dev, a.queue, max_units));
   }
   // Builds (or finds in the cache) and launches the graph of one plan: the
@@ -2736,7 +2739,7 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
       cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(int) * 64, cs);
       {
         ProfScope ps(ctx, QFS_PROF_OTHER, 0.0, cs);
-        launch_batch_prep(a, cs);
+        if (e == cudaSuccess) e = launch_batch_prep(a, cs);
       }
       if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_event, cs);
       for (size_t li = 0; li < launches.size() && e == cudaSuccess; ++li) {
@@ -2752,16 +2755,16 @@ int batch_common(qfs_ctx* ctx, int32_t P, const int32_t* ns, const int32_t* Ls, 
           ProfScope ps(ctx, QFS_PROF_BATCH, 0.0, ls);
           BatchArgs al = a;
           al.unit_trace = trace ? trace + 4 * (size_t)L.unit0 : nullptr;
-          launch_batch_sweep(L.G, al, units_dev + L.unit0, L.nunits, a.queue + li, blocks, L.warps, L.region, ls);
+          e = launch_batch_sweep(L.G, al, units_dev + L.unit0, L.nunits, a.queue + li, blocks, L.warps, L.region, ls);
         }
-        if (li > 0) {
+        if (li > 0 && e == cudaSuccess) {
           e = cudaEventRecord(ctx->gevent[gs], ls);
           if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ctx->gevent[gs], 0);
         }
       }
       if (!in.sweep_once) {
         ProfScope ps(ctx, QFS_PROF_CHECK, 0.0, cs);
-        launch_batch_finalize(a, cs);
+        if (e == cudaSuccess) e = launch_batch_finalize(a, cs);
       }
       ctx->prof.capturing = false;
       cudaGraph_t graph = nullptr;

@@ -649,10 +649,10 @@ __global__ void k_gemm_upsi(const double2* __restrict__ U, const double2* __rest
   }
 }
 
-void launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
-                      cudaStream_t st, const int* only_if) {
+cudaError_t launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
+                             cudaStream_t st, const int* only_if) {
   dim3 grid((N + 15) / 16, (M + 31) / 32);
-  k_gemm_upsi<<<grid, dim3(32, 8), 0, st>>>(U, Psi, out, N, M, only_if);
+  return launch_kernel(k_gemm_upsi, grid, dim3(32, 8), 0, st, U, Psi, out, N, M, only_if);
 }
 
 __global__ void k_cast(const double2* in, float2* out, long long count) {

@@ -575,27 +575,24 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
   cudaError_t e = cudaFuncSetAttribute(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem(s.nb));
   if (e != cudaSuccess) return e;
-  k_oz_prep<<<dim3(s.cblocks * s.nb / 2, std::max(1, std::min(16, N / 512))), 256, 0, st>>>(Psi, N, M, s.nb, dig, expo, row2, flag);
-  const dim3 grid(N / 128, s.splits, s.cblocks);
-  if (s.nb == 64) k_oz_product<64><<<grid, kOzThreads, oz_smem(64), st>>>((const double*)U, dig, N, part, row2, err);
-  else k_oz_product<32><<<grid, kOzThreads, oz_smem(32), st>>>((const double*)U, dig, N, part, row2, err);
-  k_oz_finish<<<(unsigned)(((long long)N * M + 255) / 256), 256, 0, st>>>(part, expo, row2, N, M, s.nb, s.splits, s.cblocks,
-                                                                        out, flag);
-  launch_gemm_upsi(U, Psi, out, N, M, st, flag);
-  return cudaGetLastError();
+  e = launch_kernel(k_oz_prep, dim3(s.cblocks * s.nb / 2, std::max(1, std::min(16, N / 512))), 256, 0, st, Psi, N, M, s.nb, dig,
+                    expo, row2, flag);
+  if (e != cudaSuccess) return e;
+  e = launch_kernel(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>, dim3(N / 128, s.splits, s.cblocks), kOzThreads,
+                    oz_smem(s.nb), st, (const double*)U, dig, N, part, row2, err);
+  if (e != cudaSuccess) return e;
+  e = launch_kernel(k_oz_finish, (unsigned)(((long long)N * M + 255) / 256), 256, 0, st, part, expo, row2, N, M, s.nb, s.splits,
+                    s.cblocks, out, flag);
+  return e != cudaSuccess ? e : launch_gemm_upsi(U, Psi, out, N, M, st, flag);
 }
 
-void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st) {
-  const unsigned tiles = (unsigned)std::max(1, (1 << n) / kFxRows);
+cudaError_t launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st) {
   const int cols = n <= 6 ? 32 : 8;
   const size_t smem = sizeof(int4) * (size_t)(kFxRows + cols) << n;  // (n = 8: 64 KB)
-  const dim3 grid(tiles, (M + cols - 1) / cols);
-  if (n <= 6) {
-    k_fx_product<32, 1><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
-  } else {
-    allow_smem(k_fx_product<8, 2>, sizeof(int4) * (size_t)(kFxRows + 8) << kFxProductQubits);
-    k_fx_product<8, 2><<<grid, 256, smem, st>>>(U, Psi, out, n, M);
-  }
+  const dim3 grid((unsigned)std::max(1, (1 << n) / kFxRows), (M + cols - 1) / cols);
+  if (n <= 6) return launch_kernel(k_fx_product<32, 1>, grid, 256, smem, st, U, Psi, out, n, M);
+  const cudaError_t e = allow_smem(k_fx_product<8, 2>, sizeof(int4) * (size_t)(kFxRows + 8) << kFxProductQubits);
+  return e != cudaSuccess ? e : launch_kernel(k_fx_product<8, 2>, grid, 256, smem, st, U, Psi, out, n, M);
 }
 
 }  // namespace qfs

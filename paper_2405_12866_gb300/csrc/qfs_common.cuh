@@ -23,6 +23,18 @@ inline cudaError_t allow_smem(K* kernel, size_t bytes) {
   return cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// A launch that returns its own error.  (<<<>>> leaves it in the thread's last
+// error, among whatever other code left there.)
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <typename T> struct C2;
 template <> struct C2<float>  { using t = float2;  };
 template <> struct C2<double> { using t = double2; };

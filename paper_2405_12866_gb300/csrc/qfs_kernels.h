@@ -181,8 +181,8 @@ cudaError_t launch_sweep_cl(Real r, const ClPlan& p, const ClArgs& a, bool fx, c
 bool cl_check_fits(int n, int L);
 cudaError_t launch_cl_check(const ClArgs& a, double* parts, unsigned* count, cudaStream_t st);
 // acc: 4 words of scratch.
-void launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
-                     int4* out, cudaStream_t st);
+cudaError_t launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
+                            int4* out, cudaStream_t st);
 
 // Set `count` 4x4 complex128 matrices to the identity.
 void launch_set_identity4(double2* v, long long count, cudaStream_t st);
@@ -231,8 +231,8 @@ void launch_gate_update_batch(int count, const double2* envs, const double2* g_o
 
 // out (N x M, complex128) = U (N x N) * Psi (N x M), all row-major.
 // only_if (nullable, device): the kernel does nothing when it holds zero.
-void launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
-                      cudaStream_t st, const int* only_if = nullptr);
+cudaError_t launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
+                             cudaStream_t st, const int* only_if = nullptr);
 // The same product, for N >= 512, from 8-bit digits on the tensor cores
 // (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1.
 // err: device word, bit 0 set when a bounded wait ran out.
@@ -241,7 +241,7 @@ void launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N,
 const int* oz_flag(const void* scratch, int N, int M, int num_sms);
 // The same for n <= 8 in 64-bit fixed point.
 constexpr int kFxProductQubits = 8;
-void launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st);
+cudaError_t launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st);
 size_t oz_scratch_bytes(int N, int M, int num_sms);
 cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
                               int num_sms, cudaStream_t st);
@@ -315,7 +315,7 @@ struct BatchUnit {
   int p, s0, ns;
 };
 
-void launch_batch_prep(const BatchArgs& a, cudaStream_t st);
+cudaError_t launch_batch_prep(const BatchArgs& a, cudaStream_t st);
 // A warp's shared memory (float2) with G lanes per start, for problems of
 // at most max_elems = N * M amplitudes and max_L gates.
 int batch_region_f2(int G, int max_elems, int max_L);
@@ -326,9 +326,9 @@ size_t batch_sweep_smem(int G, int warps, int max_elems, int max_L);
 int batch_sweep_blocks_per_sm(int G, int warps, size_t smem);
 // The persistent sweep over `units` (queue: a zeroed counter), G in
 // {4, 8, 16, 32}; region_f2: each warp's shared memory in float2.
-void launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
-                        int warps, int region_f2, cudaStream_t st);
-void launch_batch_finalize(const BatchArgs& a, cudaStream_t st);
+cudaError_t launch_batch_sweep(int G, const BatchArgs& a, const BatchUnit* units, int nunits, int* queue, int blocks,
+                               int warps, int region_f2, cudaStream_t st);
+cudaError_t launch_batch_finalize(const BatchArgs& a, cudaStream_t st);
 
 // ---------------------------------------------------------- learned part
 

@@ -930,11 +930,12 @@ __global__ void k_cl_scale(int N, int M, int gates, const double2* psi, const do
   }
 }
 
-void launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
-                     int4* out, cudaStream_t st) {
-  cudaMemsetAsync(acc, 0, 4 * sizeof(unsigned), st);
+cudaError_t launch_cl_scale(int n, int M, int gates, const double2* psi, const double2* phil, const double2* g, unsigned* acc,
+                            int4* out, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
   const int nt = n >= 11 ? 1024 : 256;
-  k_cl_scale<<<M + (gates + nt - 1) / nt, nt, 0, st>>>(1 << n, M, gates, psi, phil, g, acc, out);
+  return launch_kernel(k_cl_scale, M + (gates + nt - 1) / nt, nt, 0, st, 1 << n, M, gates, psi, phil, g, acc, out);
 }
 
 ClPlan cl_plan(Real r, int n, int M, int L, int spt, bool keep64) {
@@ -1010,8 +1011,7 @@ cudaError_t launch_cl_check(const ClArgs& a, double* parts, unsigned* count, cud
   const auto kernel = wide ? k_cl_check<512> : k_cl_check<128>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
-  kernel<<<a.M, wide ? 512 : 128, smem, st>>>(a, parts, count);
-  return cudaGetLastError();
+  return launch_kernel(kernel, a.M, wide ? 512 : 128, smem, st, a, parts, count);
 }
 
 }  // namespace qfs
