@@ -731,6 +731,7 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   }
   if (rc == QFS_ENOMEM) rc = ensure_ws(ctx, plan(true));
   TRY(rc);
+  g_err.clear();  // (a refused plan's message, where a smaller one fits)
   carve(R, ctx->ws, need_U, need_envs);
   const size_t blist = (size_t)std::max(R.L - 1, 1) * S * R.sN * elem_bytes(prec == QFS_MIXED ? R32 : R64);
   R.stream_b = blist > ctx->l2_bytes / 2;
