@@ -63,6 +63,33 @@ struct FxSum {
   }
 };
 
+// The entries of a matrix product of 2^n terms, one component per thread, with a
+// scale for every row of the left matrix and every column of the right one, from
+// their largest exponent fields t, and room for 2 2^n terms: the high sums stay
+// below 2^62, each cross sum below 2^62 and both together below 2^63.  That room
+// puts the result's scale up to 2^9 above the result, so the low x low products
+// and the bits of the cross sums below 2^-60 count here.
+__device__ __forceinline__ int fx_top(double2 z) {
+  return max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff);
+}
+__device__ __forceinline__ int fx_row_exp(int t, int n) { return t - 1022 + n - 1; }
+__device__ __forceinline__ int fx_col_exp(int t, int n) { return t - 1022 + max(n - 2, 1); }
+struct FxDot {
+  FxSum t;
+  long long low = 0;  // low x low, in units of 2^-112
+  // Component im of x y.
+  __device__ __forceinline__ void add(int4 x, int4 y, int im) {
+    const int b1 = im ? y.w : y.y, a2 = im ? x.w : -x.w, b2 = im ? y.y : y.w;
+    t.add(x.x, x.y, im ? y.z : y.x, b1);
+    t.add(im ? x.z : -x.z, a2, im ? y.x : y.z, b2);
+    low += (mad64(x.y, b1, 0) >> 8) + (mad64(a2, b2, 0) >> 8);
+  }
+  __device__ __forceinline__ long long cross() const { return t.c + t.d + (low >> 22); }
+};
+__device__ __forceinline__ double fx_dot_value(long long high, long long cross, int e) {
+  return scale_exp(fma((double)cross, 1.0 / (1LL << kFxLow), (double)high), e - kFxBits);
+}
+
 // Where entry e = (column << n) | row of a slice sits: bits 4 and 5 are folded
 // into the bank bits, so that the units of a gate on any two neighbouring row
 // bits (whose lanes skip those bits) spread over the banks.  Linear over XOR,

@@ -464,16 +464,12 @@ __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__
   if (e == 1 << 20 && row == 0) atomicOr(flag, 1);
 }
 
-// out = U Psi for N <= 256 rows: grid (N / 8 row tiles (at least 1), column tiles).  A scale for every row of U and every column of Psi, from its largest
-// entry, with room for 2 N terms: the high sums stay below 2^62, each cross sum
-// below 2^62 and both together below 2^63.  Where a row's or a column's entries
-// are far from 1, Inf or NaN, its results take FP64 arithmetic.
+// out = U Psi for N <= 256 rows (fixed.cuh: FxDot): grid (N / 8 row tiles (at least 1), column tiles).  Where a row's
+// or a column's entries are far from 1, Inf or NaN, its results take FP64 arithmetic.
 //
 // A warp reads a row of U, so its exponent is one reduction; columns, read along
-// rows of Psi, meet in shared memory.  Low x low products and the bits of the
-// cross sums below 2^-60 count here, because the room for 2 N terms puts the
-// result's scale up to 2^9 above the result (without them 1.3e-15 of the norm at
-// n = 6, FP64 arithmetic 3.8e-16; with them 2.2e-16, in the same time).
+// rows of Psi, meet in shared memory.  (Without the low x low products 1.3e-15 of
+// the norm at n = 6, FP64 arithmetic 3.8e-16; with them 2.2e-16, in the same time.)
 //
 // At n = 7 and 8 too, in tiles of 8 columns with KS = 2 threads to a component
 // (which take every second term each): one launch takes less than the four of the
@@ -487,36 +483,28 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
   __shared__ int tu[kFxRows], tp[kFxCols];  // largest exponent fields
   const int N = 1 << n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = blockIdx.x * kFxRows, rows = min(kFxRows, N - r0), c0 = blockIdx.y * kFxCols, cols = min(kFxCols, M - c0);
-  auto top = [](double2 z) { return max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff); };
   if (tid < kFxCols) tp[tid] = 0;
   if (warp < rows) {
     int t = 0;
-    for (int k = lane; k < N; k += 32) t = max(t, top(U[(long long)(r0 + warp) * N + k]));
+    for (int k = lane; k < N; k += 32) t = max(t, fx_top(U[(long long)(r0 + warp) * N + k]));
     t = __reduce_max_sync(FULL, t);
     if (lane == 0) tu[warp] = t;
   }
   __syncthreads();
-  for (int i = tid; i < N * cols; i += 256) atomicMax(&tp[i % cols], top(Psi[(long long)(i / cols) * M + c0 + i % cols]));
+  for (int i = tid; i < N * cols; i += 256) atomicMax(&tp[i % cols], fx_top(Psi[(long long)(i / cols) * M + c0 + i % cols]));
   __syncthreads();
-  auto eu = [&](int i) { return tu[i] - 1022 + n - 1; };
-  auto ep = [&](int j) { return tp[j] - 1022 + max(n - 2, 1); };
+  auto eu = [&](int i) { return fx_row_exp(tu[i], n); };
+  auto ep = [&](int j) { return fx_col_exp(tp[j], n); };
   for (int i = tid; i < rows * N; i += 256) su[i] = fx_from2(U[(long long)r0 * N + i], eu(i >> n));
   for (int i = tid; i < N * cols; i += 256) sp[i] = fx_from2(Psi[(long long)(i / cols) * M + c0 + i % cols], ep(i % cols));
   __syncthreads();
   for (int e = tid; e < 2 * KS * rows * cols; e += 256) {  // (KS = 2: a multiple of 32, so warps are whole)
     const int c = e / KS, part = e % KS, im = c & 1, i = (c >> 1) / cols, j = (c >> 1) % cols;
-    FxSum t;
-    long long low = 0;  // low x low, in units of 2^-112
-    for (int k = part; k < N; k += KS) {
-      const int4 x = su[i * N + k], y = sp[k * cols + j];
-      const int b1 = im ? y.w : y.y, a2 = im ? x.w : -x.w, b2 = im ? y.y : y.w;
-      t.add(x.x, x.y, im ? y.z : y.x, b1);
-      t.add(im ? x.z : -x.z, a2, im ? y.x : y.z, b2);
-      low += (mad64(x.y, b1, 0) >> 8) + (mad64(a2, b2, 0) >> 8);
-    }
-    long long cross = t.c + t.d + (low >> 22);
+    FxDot t;
+    for (int k = part; k < N; k += KS) t.add(su[i * N + k], sp[k * cols + j], im);
+    long long high = t.t.h, cross = t.cross();
     if constexpr (KS == 2) {
-      t.h += __shfl_xor_sync(FULL, t.h, 1);
+      high += __shfl_xor_sync(FULL, high, 1);
       cross += __shfl_xor_sync(FULL, cross, 1);
       if (part) continue;
     }
@@ -527,7 +515,7 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
         v = im ? fma(x.x, y.y, fma(x.y, y.x, v)) : fma(x.x, y.x, fma(-x.y, y.y, v));
       }
     } else {
-      v = scale_exp(fma((double)cross, 1.0 / (1LL << kFxLow), (double)t.h), eu(i) + ep(j) - kFxBits);
+      v = fx_dot_value(high, cross, eu(i) + ep(j));
     }
     reinterpret_cast<double*>(out + (long long)(r0 + i) * M + c0 + j)[im] = v;
   }
