@@ -19,10 +19,13 @@
 // NB columns, and since the digits of Psi lie side by side along the columns
 // of one shared-memory operand, a_i times b_j, b_{j+1}, ... is one MMA that
 // adds into D_{i+j}, D_{i+j+1}, ...  The digits of U are formed on the fly by
-// the warps that load it.  D_0..D_3 are emptied into 64-bit integers after
-// every 256 products, before they can reach 2^24; D_4..D_7 weigh 2^-32 of D_0
-// and less, and may round.  What is left out (d > 7) is below 2^-60 of the
-// result's scale.
+// the warps that load it.  D_0..D_4 are emptied into 64-bit integers before they
+// can pass 2^24, D_4 after every 256 products, and D_5 with it (81920 a product at
+// most, so its last additions may round to 2^-52 where every digit is extreme);
+// D_6, 2^-48 of D_0, after every 4096.  D_7 may round, and what is left out (d > 7)
+// is below 2^-60 of the result's scale.  (With D_4 and D_5 read only at the end the
+// sums of constant rows and columns were off by up to 1e-11 from n = 13 on, in one
+// split of 8192 products and more.)
 //
 // Up to 256 rows there are at most two tiles to fill: k_fx_product forms the
 // product in 64-bit fixed point (fixed.cuh), a component by one or two threads (n
@@ -44,7 +47,8 @@ namespace {
 
 constexpr int kDig = 7;          // digits of a number
 constexpr int kOzK = 32;         // reals of one pipeline step
-constexpr int kOzChunk = 8;      // steps between two readings of D_0..D_3
+constexpr int kOzChunk = 8;      // steps between two readings of D_3..D_5 (D_0..D_2: fewer)
+constexpr int kOzLow = 16;       // chunks between two readings of D_6
 constexpr int kOzThreads = 288;  // eight warps for digits and sums, one for the MMAs
 constexpr int kOzProd = 256;
 constexpr int kABytes = kDig * 128 * kOzK * 2;
@@ -128,20 +132,7 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t saddr, uint32_t lead) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(lead >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | (uint64_t)1 << 46;
 }
 
-template <int N32>
-__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&w)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]),
-        "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15]), "=r"(w[16]),
-        "=r"(w[17]), "=r"(w[18]), "=r"(w[19]), "=r"(w[20]), "=r"(w[21]), "=r"(w[22]), "=r"(w[23]), "=r"(w[24]),
-        "=r"(w[25]), "=r"(w[26]), "=r"(w[27]), "=r"(w[28]), "=r"(w[29]), "=r"(w[30]), "=r"(w[31])
-      : "r"(addr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&w)[32]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&w)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
       "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -149,6 +140,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&w)[32]) {
         "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
       : "r"(addr)
       : "memory");
+}
+// Loads done; the registers stand here so that nothing reads them before.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&w)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7]),
+                 "+r"(w[8]), "+r"(w[9]), "+r"(w[10]), "+r"(w[11]), "+r"(w[12]), "+r"(w[13]), "+r"(w[14]), "+r"(w[15])
+               :
+               : "memory");
 }
 // Zeros into 16 columns of this warp's 32 lanes.
 __device__ __forceinline__ void tmem_zero16(uint32_t addr) {
@@ -315,32 +314,50 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     long long hi[HC];
 #pragma unroll
     for (int c = 0; c < HC; ++c) hi[c] = 0;
-    auto zero = [&](int from, int to) {
-      for (int d = from; d < to; ++d)
-#pragma unroll
-        for (int c = 0; c < HC; c += 16) tmem_zero16(lanes + (uint32_t)(d * NB + c));
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    };
-    auto read = [&](int d, uint32_t (&w)[32]) {
-      if constexpr (HC == 32) tmem_ld32<HC>(lanes + (uint32_t)(d * NB), w);
-      else tmem_ld16(lanes + (uint32_t)(d * NB), w);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    };
-    auto gather = [&](int chunk) {  // D_0..D_3 into hi
+    // D_0..D_5 into hi, 16 columns at a time: while one part is added the next is
+    // on its way and the last one is zeroed.  Before a sum can pass 2^24: a product
+    // adds at most 2^12 to D_0, 2^14 to D_1 (both read after every fourth chunk),
+    // 2^15 to D_2 (every second), 49152 to D_3 and 2^16 to D_4 (every one).
+    constexpr int P = HC / 16;
+    auto at = [&](int q) { return lanes + (uint32_t)(q / P * NB + q % P * 16); };
+    auto gather = [&](int chunk, bool clear) {  // clear: another chunk follows
       if (!bar_wait(accfull, (unsigned)chunk & 1u)) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // (P = 1 takes parts of two sums together: it starts at an even one.)
+      const int d0 = !clear || chunk % 4 == 3 ? 0 : P == 1 || chunk % 2 == 1 ? 2 : 3;
+      uint32_t wa[16], wb[16];
+      tmem_ld16(at(d0 * P), wa);
+      auto pair = [&](int q, int weight_a, int weight_b, bool top) {  // parts q and q + 1
+        auto add = [&](const uint32_t (&w)[16], int c0, int weight) {
 #pragma unroll
-      for (int d = 0; d < 4; ++d) {
-        uint32_t w[32];
-        read(d, w);
+          for (int c = 0; c < 16; ++c) {
+            const int v = __float2int_rn(__uint_as_float(w[c]));
+            if (top) hi[c0 + c] += (long long)(v * weight) << 32;
+            else hi[c0 + c] = mad64(v, weight, hi[c0 + c]);
+          }
+        };
+        tmem_wait_ld(wa);
+        tmem_ld16(at(q + 1), wb);
+        if (clear) tmem_zero16(at(q));
+        add(wa, 0, weight_a);
+        tmem_wait_ld(wb);
+        if (q + 2 < 6 * P) tmem_ld16(at(q + 2), wa);
+        if (clear) tmem_zero16(at(q + 1));
+        add(wb, P == 2 ? 16 : 0, weight_b);
+      };
+      // (|D_0| <= 2^22 and |D_1| <= 2^24 weigh 2^40 and 2^32.)
+      if (d0 == 0) {
 #pragma unroll
-        for (int c = 0; c < HC; ++c) hi[c] += (long long)__float2int_rn(__uint_as_float(w[c])) << (8 * (3 - d));
+        for (int q = 0; q < 2 * P; q += 2) pair(q, 1 << (8 - 8 * (q / P)), 1 << (8 - 8 * ((q + 1) / P)), true);
       }
+#pragma unroll 1
+      for (int q = max(d0, 2) * P; q < 6 * P; q += 2) pair(q, 1 << (40 - 8 * (q / P)), 1 << (40 - 8 * ((q + 1) / P)), false);
       return true;
     };
     bool ok = true;
     int issued = 0;
-    zero(0, 8);
+    for (int q = 0; q < 8 * P; ++q) tmem_zero16(at(q));
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     bar_arrive(accfree);
     if (nk > 0) {
@@ -380,14 +397,25 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       bar_arrive(&full[s]);
       // The previous chunk's sums, with this step's operands already staged.
       if (i > 0 && i % kOzChunk == 0) {
-        ok = gather(i / kOzChunk - 1);
+        ok = gather(i / kOzChunk - 1, true);
         if (!ok) break;
-        zero(0, 4);
+        if (i % (kOzChunk * kOzLow) == 0) {
+#pragma unroll
+          for (int h = 0; h < P; ++h) {
+            uint32_t w[16];
+            tmem_ld16(at(6 * P + h), w);
+            tmem_wait_ld(w);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) hi[16 * h + c] += (__float2int_rn(__uint_as_float(w[c])) + 128) >> 8;
+            tmem_zero16(at(6 * P + h));
+          }
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         bar_arrive(accfree);
       }
     }
-    if (ok && nk > 0) ok = gather(nchunk - 1);
+    if (ok && nk > 0) ok = gather(nchunk - 1, false);
     if (!ok) {
       *gave_up = 1;
       if (tid == 0)  // the copies in flight land first (bounded)
@@ -395,23 +423,25 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     } else {
       long long* out = part + (((long long)blockIdx.y * gridDim.z + blockIdx.z) * N + row0 + (warp & 3) * 32 + lane) * NB +
                        (warp >> 2) * HC;
-      long long low[HC];
+      // hi in 2^-52, D_6 in 2^-60, D_7 in 2^-68; together in 2^-54.
 #pragma unroll
-      for (int c = 0; c < HC; ++c) low[c] = 0;
-      if (nk > 0) {
+      for (int h = 0; h < P; ++h) {
+        uint32_t w6[16], w7[16];
 #pragma unroll
-        for (int d = 4; d < 8; ++d) {
-          uint32_t w[32];
-          read(d, w);
-#pragma unroll
-          for (int c = 0; c < HC; ++c) low[c] += (long long)__float2int_rn(__uint_as_float(w[c])) << (8 * (7 - d));
+        for (int c = 0; c < 16; ++c) w6[c] = w7[c] = 0u;
+        if (nk > 0) {
+          tmem_ld16(at(6 * P + h), w6);
+          tmem_ld16(at(7 * P + h), w7);
+          tmem_wait_ld(w6);
+          tmem_wait_ld(w7);
         }
-      }
-      // hi in 2^-36, low in 2^-68; together in 2^-54.
+        auto sum = [&](int c) {
+          const long long low = ((long long)__float2int_rn(__uint_as_float(w6[c])) << 8) + __float2int_rn(__uint_as_float(w7[c]));
+          return (hi[16 * h + c] << 2) + ((low + (1 << 13)) >> 14);
+        };
 #pragma unroll
-      for (int c = 0; c < HC; c += 2)
-        *reinterpret_cast<longlong2*>(out + c) =
-            longlong2{(hi[c] << 18) + ((low[c] + (1 << 13)) >> 14), (hi[c + 1] << 18) + ((low[c + 1] + (1 << 13)) >> 14)};
+        for (int c = 0; c < 16; c += 2) *reinterpret_cast<longlong2*>(out + 16 * h + c) = longlong2{sum(c), sum(c + 1)};
+      }
       if (blockIdx.z == 0) {
         n0 += __shfl_xor_sync(FULL, n0, 8);
         n1 += __shfl_xor_sync(FULL, n1, 8);

@@ -1,0 +1,77 @@
+"""U Psi from 8-bit digits (n >= 9) against exact integers, at the sizes where a
+CTA runs through many chunks, a part of a chunk or a second column block, for
+targets and states whose digits are all alike, so that the digits' sums grow as
+fast as they can.
+
+Entries are integers: of U times 2^-(22 + n/2) (rows of norm 1 to a few percent),
+of Psi below 2^23 times 2^-23, so every digit is exact and no product of digits
+is left out.  What rounds is the result (2^-53 of it) and its unit (2^-54 of the
+column's scale, a split at a time; at most 32 splits).  Where all digits are
+alike, sums of digits may pass 2^24 between two readings: 2^-52 at three of 256
+products (d = 5) and 2^-48 per 4096 (d = 6).  Entries constant over a row and a
+column have 53 bits: then the inputs round too, by 2^-55 of 1 a product each."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2405_12866_gb300 import build, qfs
+    build.build()
+    with qfs.Context(0) as c:
+        yield c
+
+
+SIZES = [(9, 5), (10, 16), (11, 1), (11, 17), (11, 65), (12, 32), (12, 33), (12, 300), (13, 20), (13, 64)]
+
+
+@pytest.mark.parametrize("n,M", SIZES)
+@pytest.mark.parametrize("alike", [False, True])
+def test_digits_against_exact_integers(ctx, n, M, alike):
+    import torch
+    N = 1 << n
+    gen = torch.Generator(device="cuda").manual_seed(100 * n + M)
+
+    def ints(lo, hi, shape):
+        return torch.randint(lo, hi, shape, generator=gen, device="cuda", dtype=torch.int64)
+
+    one = int((0.5 if n % 2 else np.sqrt(0.5)) * (1 << 22))
+    if alike:  # one value and sign for a row and for a column, but for the low bits
+        u = torch.stack([one - ints(0, 1 << 16, (N, 1)) + ints(0, 1 << 10, (N, N)) for _ in range(2)])
+        p = torch.stack([ints(1 << 22, (1 << 23) - 1024, (1, M)) + ints(0, 1 << 10, (N, M)) for _ in range(2)])
+    else:
+        a = int(one * np.sqrt(3.0))
+        u, p = ints(-a, a + 1, (2, N, N)), ints(-(1 << 23) + 1, 1 << 23, (2, N, M))
+    U = torch.complex(*(torch.ldexp(x.double(), torch.tensor(-(22 + n // 2), device="cuda")) for x in u))
+    Psi = torch.complex(*(torch.ldexp(x.double(), torch.tensor(-23, device="cuda")) for x in p))
+    got = ctx.target_product(n, U, Psi, 0).cpu().numpy()
+    rows = np.unique(np.concatenate([[0, 1, 127, 128, N - 128, N - 1], np.random.default_rng(n).integers(0, N, 18)]))
+    u, p = u[:, torch.from_numpy(rows).cuda()].cpu().numpy(), p.cpu().numpy()
+    unit = 2.0 ** -(45 + n // 2)
+    want = (u[0] @ p[0] - u[1] @ p[1]).astype(np.longdouble) * unit, (u[0] @ p[1] + u[1] @ p[0]).astype(np.longdouble) * unit
+    slack = 2 * N * (3 / 256 * 2.0**-52 + 2.0**-48 / 4096) if alike else 0.0
+    for g, e in zip((got[rows].real, got[rows].imag), want):
+        assert np.all(np.abs(g - e) <= 2.0**-53 * np.abs(e) + 32 * 2.0**-55 + slack)
+
+
+@pytest.mark.parametrize("n,M", SIZES)
+def test_digits_of_constant_rows_and_columns(ctx, n, M):
+    import torch
+    N = 1 << n
+    rng = np.random.default_rng(100 * n + M)
+    c = (rng.uniform(0.93, 1.07, N) * np.exp(2j * np.pi * rng.uniform(size=N))) / np.sqrt(N)
+    d = rng.uniform(0.5, 0.999, M) + 1j * rng.uniform(-0.999, 0.999, M)
+    U = torch.from_numpy(c).cuda()[:, None].expand(N, N).contiguous()
+    Psi = torch.from_numpy(d).cuda()[None, :].expand(N, M).contiguous()
+    got = ctx.target_product(n, U, Psi, 1).cpu().numpy()
+    cr, ci, dr, di = (x.astype(np.longdouble) for x in (c.real, c.imag, d.real, d.imag))
+    want = N * (np.outer(cr, dr) - np.outer(ci, di)), N * (np.outer(cr, di) + np.outer(ci, dr))
+    # (U's and Psi's entries are below 1; a quarter more for what is above.)
+    tol = 2 * N * 2.0**-55 * (1.25 + np.abs(c).max())
+    for g, e in zip((got.real, got.imag), want):
+        assert np.all(np.abs(g - e) <= 2.0**-53 * np.abs(e) + tol)
