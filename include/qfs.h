@@ -491,12 +491,21 @@ int qfs_ws_instantiate(qfs_ws* ws, int32_t P, const double* targets, const doubl
  * cudaGetSymbolAddress (with that device current) and caches it for the
  * rest of the process, which assumes the device's primary context lives as
  * long (after a cudaDeviceReset the cached address is stale); make that
- * first call before any stream capture. */
+ * first call before any stream capture.
+ *
+ * The call does not wait for its kernels, so it cannot return QFS_ETIMEOUT:
+ * where a bounded device wait runs out (QFS_OPT_WAIT_LIMIT's default), the
+ * start concerned gets NaN for its cost, its gates and its environments. */
 #define QFS_NOALLOC_SCRATCH_BYTES (16u << 20)
 int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circuit, const double* target_dev,
                            const double* samples_dev, int32_t M, int32_t S, double beta,
                            const double* gates_in_dev, double* gates_out_dev,
                            double* costs_out_dev, double* envs_out_dev);
+/* The same with the polls of a wait (as QFS_OPT_WAIT_LIMIT, >= 1) given. */
+int qfs_sweep_once_noalloc_limit(void* cuda_stream, const qfs_circuit* circuit, const double* target_dev,
+                                 const double* samples_dev, int32_t M, int32_t S, double beta,
+                                 const double* gates_in_dev, double* gates_out_dev,
+                                 double* costs_out_dev, double* envs_out_dev, int64_t wait_limit);
 
 #ifdef __cplusplus
 }

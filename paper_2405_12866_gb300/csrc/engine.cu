@@ -87,6 +87,8 @@ struct Prof {
 
 constexpr int kMaxGroups = 8;
 
+constexpr long long kWaitLimit = 1LL << 25;
+
 struct qfs_ctx {
   Prof prof;
   // Streams for groups of starts swept concurrently, forked from and joined
@@ -109,7 +111,7 @@ struct qfs_ctx {
   double df_item_bytes = 1024.0 * 1024.0;  // largest streaming bytes of one dataflow work item (QFS_DF_ITEM_KB)
   double df_items_per_cta = 1.5;           // work items per CTA and backward step (QFS_DF_ITEMS_PER_CTA)
   double df_items_per_cta_fwd = 1.0;       // ... and forward step (QFS_DF_ITEMS_PER_CTA_FWD)
-  long long df_wait_limit = 1LL << 25;     // polls before a dataflow dependency wait gives up (QFS_OPT_WAIT_LIMIT)
+  long long df_wait_limit = kWaitLimit;    // polls before a wait of a whole-sweep launch gives up (QFS_OPT_WAIT_LIMIT)
   // Batched form: the tuned launch shape per problem class (n, L, M) and the
   // captured graphs of recent batch shapes (replayed when a call repeats one).
   std::vector<std::pair<long long, std::pair<int, int>>> batch_tuned;  // class key -> (G, warps)
@@ -2165,7 +2167,17 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
                                       int32_t M, int32_t S, double beta, const double* gates_in_dev,
                                       double* gates_out_dev, double* costs_out_dev,
                                       double* envs_out_dev) {
+  return qfs_sweep_once_noalloc_limit(cuda_stream, circuit, target_dev, samples_dev, M, S, beta, gates_in_dev,
+                                      gates_out_dev, costs_out_dev, envs_out_dev, kWaitLimit);
+}
+
+extern "C" int qfs_sweep_once_noalloc_limit(void* cuda_stream, const qfs_circuit* circuit,
+                                            const double* target_dev, const double* samples_dev,
+                                            int32_t M, int32_t S, double beta, const double* gates_in_dev,
+                                            double* gates_out_dev, double* costs_out_dev,
+                                            double* envs_out_dev, int64_t wait_limit) {
   g_err.clear();
+  if (wait_limit < 1) return fail(QFS_EINVAL, "wait_limit = %lld < 1", (long long)wait_limit);
   TRY(check_circuit(circuit));
   TRY(check_run_params(circuit->n, M, S, 1, QFS_FP64, beta, 0.0));
   if (!target_dev || !samples_dev || !gates_in_dev || !gates_out_dev)
@@ -2182,6 +2194,7 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
   tmp.stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   tmp.num_sms = sms;
   tmp.l2_bytes = (size_t)l2;
+  tmp.df_wait_limit = wait_limit;
 
   Run R;
   R.n = circuit->n;
@@ -2234,8 +2247,7 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
   if (R.n <= kFxProductQubits) {
     CK(launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st));
   } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
-    int* err = reinterpret_cast<int*>(take(sizeof(int)));
-    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), err, sms, st));
+    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), nullptr, sms, st));
   } else {
     CK(launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st));
   }
@@ -2248,7 +2260,7 @@ extern "C" int qfs_sweep_once_noalloc(void* cuda_stream, const qfs_circuit* circ
     char* aux = reinterpret_cast<char*>(R.partials);  // (not used by this sweep; at least 256 bytes)
     R.cl_acc = reinterpret_cast<unsigned*>(aux);
     R.cl_scale = reinterpret_cast<int4*>(aux + 64);
-    R.err = reinterpret_cast<int*>(aux + 128);
+    R.err = nullptr;  // (the kernel says NaN where a wait ran out)
     R.costs = costs_out_dev ? costs_out_dev : reinterpret_cast<double*>(R.phi);
     R.spt = S;
     R.cl_plain = {0, 1};

@@ -33,7 +33,8 @@
 //
 // U's digits have a fixed scale, so its rows have to have a norm near 1, as a
 // unitary's do.  The kernel sums their squares on the way; if any is outside
-// [0.81, 1.21] (or not a number), the FP64 kernel runs behind it.
+// [0.81, 1.21] (or not a number), the FP64 kernel runs behind it; so it does where
+// a bounded wait ran out.
 #include <cuda_fp16.h>
 
 #include "fixed.cuh"
@@ -223,7 +224,8 @@ __global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi
 // block][row][NB] sums in units of 2^-54 of the scaled columns.
 template <int NB>
 __global__ void __launch_bounds__(kOzThreads, 1)
-    k_oz_product(const double* __restrict__ U, const __half* __restrict__ dig, int N, long long* part, float* row2, int* err) {
+    k_oz_product(const double* __restrict__ U, const __half* __restrict__ dig, int N, long long* part, float* row2, int* flag,
+                 int* err) {
   extern __shared__ __align__(128) unsigned char sm[];
   constexpr int kB = oz_bbytes(NB), kStage = kABytes + kB, HC = NB / 2;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + 2 * kStage);
@@ -456,7 +458,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (tid == 0 && *gave_up) atomicOr(err, 1);
+  if (tid == 0 && *gave_up) {
+    atomicOr(flag, 1);  // (the FP64 kernel forms the product)
+    if (err != nullptr) atomicOr(err, 1);
+  }
   if (warp == 8) {
     if (lane == 0 && *gave_up) {
       // MMAs already issued finish (bounded) before their accumulator goes.
@@ -597,7 +602,7 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
                     expo, row2, flag);
   if (e != cudaSuccess) return e;
   e = launch_kernel(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>, dim3(N / 128, s.splits, s.cblocks), kOzThreads,
-                    oz_smem(s.nb), st, (const double*)U, dig, N, part, row2, err);
+                    oz_smem(s.nb), st, (const double*)U, dig, N, part, row2, flag, err);
   if (e != cudaSuccess) return e;
   e = launch_kernel(k_oz_finish, (unsigned)(((long long)N * M + 255) / 256), 256, 0, st, part, expo, row2, N, M, s.nb, s.splits,
                     s.cblocks, out, flag);

@@ -157,7 +157,7 @@ struct ClArgs {
   double stop_tol;                      //   <= stop_tol; a launch that finds one below its sweep0 returns at once
   int sweep0, nsweeps;                  // sweeps of this launch; several need C = 1 (a start ends with the sweep in
                                         // which it or, seen in between, another met stop_tol)
-  int* err; long long wait_limit;       // as DfArgs: polls of an exchange before the kernel gives up
+  int* err; long long wait_limit;       // as DfArgs: polls of an exchange before the kernel gives up; err may be null
   const int4* scale;                    // FP64: per target {1: the plain FP64 form, exponents of the column norms
                                         //   of Psi and U Psi, 0} (launch_cl_scale); null: plain
   unsigned char pos[kClMaxGates];       // per gate: row bits of its qubits, a | b << 4
@@ -234,8 +234,8 @@ void launch_gate_update_batch(int count, const double2* envs, const double2* g_o
 cudaError_t launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
                              cudaStream_t st, const int* only_if = nullptr);
 // The same product, for N >= 512, from 8-bit digits on the tensor cores
-// (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1.
-// err: device word, bit 0 set when a bounded wait ran out.
+// (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1 or a
+// bounded wait ran out.  err: device word, bit 0 set when one did (may be null).
 // The word in its scratch that is not zero, once it has run, when the FP64 kernel
 // ran too: for one, whenever U or Psi holds Inf or NaN.
 const int* oz_flag(const void* scratch, int N, int M, int num_sms);

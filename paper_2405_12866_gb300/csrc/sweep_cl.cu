@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
     if (cost <= a.stop_tol && a.nsweeps > 1) break;  // (this start has met the tolerance: it sweeps no further)
     __syncthreads();
   }
-  if (!alive && tid == 0) atomicOr(a.err, 1);
+  if (!alive && tid == 0 && a.err != nullptr) atomicOr(a.err, 1);
   // No CTA leaves while copies of its own are in flight or a peer may still
   // store to its shared memory.  A CTA that saw every exchange complete has
   // received all there is; one that gave up waits (bounded) for what its peers
@@ -735,6 +735,14 @@ __global__ void __launch_bounds__(NT, 1) k_sweep_cl(ClArgs a) {
     cluster_arrive();
     cluster_wait();
     if (!alive) {
+      // What this start has is not a sweep's: NaN, for a caller that has no error
+      // word.  (Behind the barrier: the CTAs have written what they write.)
+      const double nan = __longlong_as_double(-1LL);
+      for (int i = tid; i < L * 16; i += NT) {
+        g64[i] = double2{nan, nan};
+        if (a.envs != nullptr) a.envs[(long long)s * L * 16 + i] = double2{nan, nan};
+      }
+      if (tid == 0) a.costs[s] = nan;
       for (int i = 0; i < 256; ++i) __nanosleep(1000);
     }
   }

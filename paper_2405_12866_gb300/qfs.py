@@ -44,7 +44,7 @@ EXPORTS = [
     "qfs_generate_inputs", "qfs_generate_states", "qfs_instantiate", "qfs_instantiate_many",
     "qfs_instantiate_many_dev", "qfs_instantiate_ex", "qfs_instantiate_dev",
     "qfs_sweep_once", "qfs_gate_update", "qfs_profile_enable", "qfs_profile_reset",
-    "qfs_profile_read", "qfs_sweep_once_noalloc", "qfs_instantiate_batch",
+    "qfs_profile_read", "qfs_sweep_once_noalloc", "qfs_sweep_once_noalloc_limit", "qfs_instantiate_batch",
     "qfs_instantiate_batch_dev", "qfs_gemm_bf16_dev", "qfs_ws_create", "qfs_ws_destroy", "qfs_ws_params",
     "qfs_ws_loss_grad", "qfs_ws_train", "qfs_ws_predict",
     "qfs_dataflow_trace_enable", "qfs_dataflow_trace_read", "qfs_target_product_dev",
@@ -151,6 +151,7 @@ def lib():
     L.qfs_batch_trace_read.argtypes = [_P, _P, C.c_int64, C.POINTER(C.c_int64)]
     L.qfs_sweep_once_noalloc.argtypes = [_P, C.POINTER(Circuit), _P, _P, C.c_int32, C.c_int32,
                                          C.c_double, _P, _P, _P, _P]
+    L.qfs_sweep_once_noalloc_limit.argtypes = L.qfs_sweep_once_noalloc.argtypes + [C.c_int64]
     L.qfs_profile_enable.argtypes = [_P, C.c_int]
     L.qfs_set_option.argtypes = [_P, C.c_int32, C.c_int64]
     L.qfs_batch_schedules.argtypes = [_P, C.c_int32, _P, C.POINTER(C.c_int32), _P, _P, C.POINTER(C.c_int32),
