@@ -46,11 +46,25 @@ __device__ __forceinline__ float2 mul_pair(float2 a, float2 b) {
   const float p = __fmul_rn(a.x, b.x);
   return float2{p, __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.x, -p)))};
 }
+// d + e rounded to a float; sure is cleared where a number within 2^-43 size of
+// d + e rounds to another one.  The pairs are good to that at worst and FP64
+// arithmetic to 2^-52, so where sure stands both round to the same float.
+__device__ __forceinline__ float round_pair(float d, float e, float size, bool& sure) {
+  constexpr float kSlack = 1.f / (1LL << 43);
+  const float r = __fadd_rn(d, __fmaf_rn(size, kSlack, e));
+  sure &= r == __fadd_rn(d, __fmaf_rn(size, -kSlack, e));
+  return r;
+}
 // The float next to s - t.
-__device__ __forceinline__ float sub_pair(float2 s, float2 t) {
+__device__ __forceinline__ float sub_pair(float2 s, float2 t, bool& sure) {
   const float d = __fsub_rn(s.x, t.x), v = __fsub_rn(d, s.x);
   const float err = __fsub_rn(__fsub_rn(s.x, __fsub_rn(d, v)), __fadd_rn(t.x, v));
-  return __fadd_rn(d, __fadd_rn(err, __fsub_rn(s.y, t.y)));
+  return round_pair(d, __fadd_rn(err, __fsub_rn(s.y, t.y)), __fadd_rn(fabsf(s.x), fabsf(t.x)), sure);
+}
+// A float of normal size (or 0) as a double, by integer operations.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x);
+  return x == 0.f ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
 }
 
 // Features of target t: the 16 x 8 complex matrix U_t Phi_fix as 256 reals
@@ -60,10 +74,11 @@ __device__ __forceinline__ float sub_pair(float2 s, float2 t) {
 //
 // The products in FP64 were bound by that pipe (95 us for 4096 targets; the
 // targets are 17 MB, 2.5 us of memory time), so they are formed from pairs of
-// floats, which gives the same rounded float but for one in ~2^23.  A block
-// walks over targets: its 128 threads, one per output, keep their column of
-// Phi_fix in registers and share the split target.  A target with an entry
-// outside the pairs' range takes the FP64 products.  Now 21 us.
+// floats, which give the same rounded float except next to the middle between
+// two: an output with such a product (one in ~2000) takes FP64 products, and so does
+// a target with an entry outside the pairs' range.  A block walks over targets: its
+// 128 threads, one per output, keep their column of Phi_fix in registers and share
+// the split target.  24 us (without the check 22).
 constexpr int kFeatStride = 17;  // float4s a row: four rows' reads lie in different banks
 __global__ void __launch_bounds__(128) k_ws_features(const double2* __restrict__ U, const double2* __restrict__ phif,
                                                      int count, int rows, __nv_bfloat16* __restrict__ X) {
@@ -99,12 +114,30 @@ __global__ void __launch_bounds__(128) k_ws_features(const double2* __restrict__
       const bool pairs = __syncthreads_and(ok);
       fetch(t + gridDim.x);  // (under this target's products)
       if (pairs) {
+        bool sure = true;
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
           const float4 a = su[i * kFeatStride + q];
           const float2 ax{a.x, a.y}, ay{a.z, a.w}, nby{-by[q].x, -by[q].y};
-          re = __fadd_rn(re, sub_pair(mul_pair(ax, bx[q]), mul_pair(ay, by[q])));
-          im = __fadd_rn(im, sub_pair(mul_pair(ay, bx[q]), mul_pair(ax, nby)));
+          re = __fadd_rn(re, sub_pair(mul_pair(ax, bx[q]), mul_pair(ay, by[q]), sure));
+          im = __fadd_rn(im, sub_pair(mul_pair(ay, bx[q]), mul_pair(ax, nby), sure));
+        }
+        // Outputs (about one in 2000) with an unsure product, a warp at a time: a
+        // lane forms one component of one product in FP64.
+        for (unsigned todo = __ballot_sync(FULL, !sure); todo; todo &= todo - 1) {
+          const int lane = k & 31, src = __ffs(todo) - 1, o = (k & ~31) | src, q = lane >> 1;
+          const double2 x = U[(size_t)t * 256 + o / 8 * 16 + q], y = phif[q * 8 + o % 8];
+          const float v = (float)(lane & 1 ? x.x * y.y + x.y * y.x : x.x * y.x - x.y * y.y);
+          float sx = 0.f, sy = 0.f;
+#pragma unroll
+          for (int p = 0; p < 16; ++p) {
+            sx = __fadd_rn(sx, __shfl_sync(FULL, v, 2 * p));
+            sy = __fadd_rn(sy, __shfl_sync(FULL, v, 2 * p + 1));
+          }
+          if (lane == src) {
+            re = sx;
+            im = sy;
+          }
         }
       } else {
         const double2* u = U + (size_t)t * 256 + i * 16;
@@ -216,10 +249,12 @@ __device__ __forceinline__ void grad_tile_end(GradTile& s, int tid, float4 acc, 
 // loss partial sums per block into loss_part[block] (at most 1024).  Block
 // column x walks the row tiles y, y + gridDim.y, ...
 //
-// Y - T, its square and its scaled value are pairs of floats (exact, 2^-45 and
-// the same rounded float as from FP64 but for one in ~2^20): FP64 conversions
-// and products for every entry were 24 us of that pipe.  Differences outside
-// the pairs' range take FP64.
+// Y - T is a pair of floats (exactly) and so is its scaled value, which gives the
+// same rounded float as FP64 except next to the middle between two, and there it
+// takes FP64; the sum of squares is FP64's, of differences widened by integer
+// operations.  (Squares as pairs, 16 to a sum: 1.6e-15 of the loss away from the
+// exact one; so 2e-16.)  FP64 conversions and products for everything were 24 us of
+// that pipe.  Differences outside the pairs' range take FP64.
 __global__ void __launch_bounds__(256)
     k_ws_loss_grad(const float* __restrict__ Y, int ldy, const float* __restrict__ T, int n_out, int rows, int B_valid,
                    double scale, __nv_bfloat16* __restrict__ G16, __nv_bfloat16* __restrict__ GT16, float* __restrict__ db,
@@ -228,10 +263,9 @@ __global__ void __launch_bounds__(256)
   __shared__ double red[8];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, c0 = blockIdx.x * 64;
   const float sh = (float)scale, sl = (float)(scale - (double)sh);
-  double acc = 0.0;
+  double acc[2] = {0.0, 0.0};
   for (int r0 = 64 * blockIdx.y; r0 < rows; r0 += 64 * gridDim.y) {
     float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
-    float q_hi = 0.f, q_lo = 0.f;
     const int c = c0 + 4 * tx;
     float4 ly[4], lt[4];
 #pragma unroll
@@ -244,43 +278,47 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
       const int r = r0 + ty + 16 * y;
+      const float4 v = ly[y], w = lt[y];
+      const float vy[4] = {v.x, v.y, v.z, v.w}, vt[4] = {w.x, w.y, w.z, w.w};
       float g[4];  // (0 where the loads gave 0)
-      {
-        const float4 v = ly[y], w = lt[y];
-        const float vy[4] = {v.x, v.y, v.z, v.w}, vt[4] = {w.x, w.y, w.z, w.w};
+      double dd[4];
+      bool sure = true;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        // d + de = Y - T exactly.
+        const float d = __fsub_rn(vy[e], vt[e]), b = __fsub_rn(d, vy[e]);
+        const float de = __fsub_rn(__fsub_rn(vy[e], __fsub_rn(d, b)), __fadd_rn(vt[e], b));
+        const float m = fabsf(d), p = __fmul_rn(d, sh);
+        sure &= d == 0.f || (m >= 1e-18f && m <= 1e18f);
+        g[e] = round_pair(p, __fmaf_rn(de, sh, __fmaf_rn(d, sl, __fmaf_rn(d, sh, -p))), fabsf(p), sure);
+        dd[e] = widen(d) + widen(de);
+      }
+      if (!sure) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          // d + de = Y - T exactly.
-          const float d = __fsub_rn(vy[e], vt[e]), b = __fsub_rn(d, vy[e]);
-          const float de = __fsub_rn(__fsub_rn(vy[e], __fsub_rn(d, b)), __fadd_rn(vt[e], b));
-          const float m = fabsf(d);
-          if (d == 0.f || (m >= 1e-18f && m <= 1e18f)) {
-            const float p = __fmul_rn(d, sh);
-            g[e] = __fadd_rn(p, __fmaf_rn(de, sh, __fmaf_rn(d, sl, __fmaf_rn(d, sh, -p))));
-            const float q = __fmul_rn(d, d), qe = __fmaf_rn(2.f * d, de, __fmaf_rn(d, d, -q));
-            const float t = __fadd_rn(q_hi, q), tb = __fsub_rn(t, q_hi);
-            q_lo = __fadd_rn(q_lo, __fadd_rn(__fadd_rn(__fsub_rn(q_hi, __fsub_rn(t, tb)), __fsub_rn(q, tb)), qe));
-            q_hi = t;
-          } else {
-            const double dd = (double)vy[e] - (double)vt[e];
-            acc += dd * dd;
-            g[e] = (float)(scale * dd);
-          }
+          dd[e] = (double)vy[e] - (double)vt[e];
+          g[e] = (float)(scale * dd[e]);
         }
+      }
+      if (c < n_out) {  // (n_out is a multiple of 64: whole blocks)
+        acc[0] = fma(dd[0], dd[0], acc[0]);
+        acc[1] = fma(dd[1], dd[1], acc[1]);
+        acc[0] = fma(dd[2], dd[2], acc[0]);
+        acc[1] = fma(dd[3], dd[3], acc[1]);
       }
       grad_tile_row(s, ty + 16 * y, tx, make_float4(g[0], g[1], g[2], g[3]), col, G16 + (size_t)r * ldy + c0);
     }
-    acc += (double)q_hi + (double)q_lo;
     grad_tile_end(s, tid, col, r0, c0, rows, GT16, db);
     __syncthreads();
   }
+  double sum = acc[0] + acc[1];
 #pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) acc += __shfl_xor_sync(~0u, acc, m);
-  if ((tid & 31) == 0) red[tid >> 5] = acc;
+  for (int m = 16; m >= 1; m >>= 1) sum += __shfl_xor_sync(~0u, sum, m);
+  if ((tid & 31) == 0) red[tid >> 5] = sum;
   __syncthreads();
   if (tid == 0) {
-    for (int w = 1; w < 8; ++w) acc += red[w];
-    loss_part[blockIdx.y * gridDim.x + blockIdx.x] = acc;
+    for (int w = 1; w < 8; ++w) sum += red[w];
+    loss_part[blockIdx.y * gridDim.x + blockIdx.x] = sum;
   }
 }
 
