@@ -320,9 +320,10 @@ int qfs_gate_update(qfs_ctx* ctx, int32_t count, const double* envs, const doubl
  * starts from), on device buffers: target_dev N x N and samples_dev N x M
  * complex128 row-major, out_dev N x M (N = 2^n).  Either precision gives the
  * same product, to FP64 accuracy: from n = 9 on by exact products of 8-bit
- * digits on the tensor cores (the FP64 kernel where a row of U is not of norm
- * 1 to 10%), below in 64-bit fixed point, in workspace of the context (without
- * room for it: FP64 arithmetic).
+ * digits on the tensor cores (in a second pass where a row of U is not of norm
+ * 1 to 10%), below in 64-bit fixed point, in workspace of the context (at most
+ * 256 MB, but for one block of 32 columns at least; without room for it: FP64
+ * arithmetic).
  * Synchronous; uses the context's workspace.  QFS_EINVAL for bad sizes. */
 int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* target_dev,
                            const double* samples_dev, int32_t precision, double* out_dev);

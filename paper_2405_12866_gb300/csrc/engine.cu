@@ -274,6 +274,7 @@ struct Run {
   int* active = nullptr;
   int* flag = nullptr;
   unsigned* counters = nullptr;  // S + 1 "last block done" counters (fused update)
+  int* rows = nullptr;           // device word: rows of U out of the digits' scale
   int* err = nullptr;            // device error word: bit 0 = a bounded device wait ran out
   double2* envs = nullptr;
   // FP64 single-start buffers (mixed precision: cost check and refinement)
@@ -355,7 +356,9 @@ size_t carve(Run& R, char* base, bool need_U, bool need_envs) {
     R.cl_acc = (unsigned*)take(5 * sizeof(unsigned));  // (the last: the check's finished columns)
     R.cl_parts = (double*)take((size_t)R.M * sizeof(double));
   }
-  R.err = R.flag ? R.flag + 1 : nullptr;
+  // Words: NaN or Inf in an input, rows out of the product's scale, the error word, the stop word.
+  R.rows = R.flag ? R.flag + 1 : nullptr;
+  R.err = R.flag ? R.flag + 2 : nullptr;
   R.envs = need_envs ? (double2*)take((size_t)R.S * R.L * 16 * sizeof(double2)) : nullptr;
   R.df_steps = (DfStep*)take((size_t)std::max(R.df_cap, 1) * sizeof(DfStep));
   R.df_ctrl_cap = 1 + ((size_t)R.df_cap + 1) * R.S;
@@ -747,12 +750,17 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
 // 12, M = 32: 4.28 ms and 0.19), below in fixed point (n = 8, M = 24: 163 us in
 // FP64, 53 by digits, 40 so).  (Without room for the digits' scratch, or when a
 // mixed run asks for it, the FP64 kernel.)  Adds its launches to *launches.
-int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out, long long* launches) {
+// Digits: where R.rows says afterwards that rows are out of scale, the caller runs
+// it again, scaled.
+int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, double2* out, long long* launches,
+                   bool scaled = false) {
   cudaStream_t st = ctx->stream;
   const bool plain = R.prec == QFS_MIXED && ctx->upsi_fp64;
   if (R.oz && !plain) {
-    CK(launch_oz_product(U, psi, out, (int)R.N, R.M, R.oz, R.err, ctx->num_sms, st));
-    *launches += 4;
+    const int n = (int)R.N, m = R.M, sms = ctx->num_sms;
+    CK(scaled ? launch_oz_scaled(U, psi, out, n, m, R.oz, R.err, sms, st)
+              : launch_oz_product(U, psi, out, n, m, R.oz, R.err, R.rows, sms, st));
+    *launches += oz_launches(n, m, sms) + scaled;
     return QFS_OK;
   }
   if (R.n <= kFxProductQubits && !plain) CK(launch_fx_product(U, psi, out, R.n, R.M, st));
@@ -769,7 +777,7 @@ int target_product(qfs_ctx* ctx, Run& R, const double2* U, const double2* psi, d
 int setup_slot(qfs_ctx* ctx, Run& R, int t) {
   cudaStream_t st = ctx->stream;
   const size_t so = (size_t)t * R.sN, go = (size_t)t * R.spt * R.L * 16;
-  CK(cudaMemsetAsync(R.flag, 0, sizeof(int), st));
+  CK(cudaMemsetAsync(R.flag, 0, 2 * sizeof(int), st));
   {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     launch_nonfinite_check(reinterpret_cast<const double*>(R.psi64 + so), 2 * R.sN, R.flag, st);
@@ -778,11 +786,12 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     launch_nonfinite_check(reinterpret_cast<const double*>(R.g64 + go), 2LL * R.spt * R.L * 16, R.flag, st);
   }
-  {
+  auto product = [&](bool scaled) -> int {
     ProfScope ps(ctx, QFS_PROF_GEMM, 8.0 * R.N * R.N * R.M);  // flops, not bytes
     --ctx->prof.launches[QFS_PROF_GEMM];  // (the scope counts one, the product all of its own)
-    TRY(target_product(ctx, R, R.Uslot[t], R.psi64 + so, R.phil64 + so, &ctx->prof.launches[QFS_PROF_GEMM]));
-  }
+    return target_product(ctx, R, R.Uslot[t], R.psi64 + so, R.phil64 + so, &ctx->prof.launches[QFS_PROF_GEMM], scaled);
+  };
+  TRY(product(false));
   {
     // The product in digits has read all of U: only where it met something out
     // of its scale is there a reason to read it again.  (n = 12: 70 us.)
@@ -793,9 +802,8 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
   if (R.prec == QFS_MIXED) {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     launch_cast_c128_to_c64(R.psi64 + so, R.psi32 + so, R.sN, st);
-    launch_cast_c128_to_c64(R.phil64 + so, R.phil32 + so, R.sN, st);
     launch_cast_c128_to_c64(R.g64 + go, R.g32 + go, (long long)R.spt * R.L * 16, st);
-    ctx->prof.launches[QFS_PROF_OTHER] += 2;
+    ctx->prof.launches[QFS_PROF_OTHER] += 1;
   }
   std::vector<int> ones(R.spt, 1);
   CK(cudaMemcpyAsync(R.active + (size_t)t * R.spt, ones.data(), sizeof(int) * R.spt, cudaMemcpyHostToDevice, st));
@@ -803,19 +811,33 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
     ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
     launch_set_identity4(R.vprev + go, (long long)R.spt * R.L, st);
   }
+  // What follows from the product: its complex64 copy and the scales of the
+  // fixed-point sweeps; and what the kernels so far found.
   int4 sc{0, 0, 0, 0};
-  if (R.cl_scale) {
-    ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
-    CK(cudaMemsetAsync(R.cl_acc + 4, 0, sizeof(unsigned), st));
-    CK(launch_cl_scale(R.n, R.M, R.spt * R.L, R.psi64 + so, R.phil64 + so, R.g64 + go, R.cl_acc, R.cl_scale + t, st));
-    CK(cudaMemcpyAsync(&sc, R.cl_scale + t, sizeof(int4), cudaMemcpyDeviceToHost, st));
+  int words[2] = {0, 0};
+  auto finish = [&]() -> int {
+    if (R.prec == QFS_MIXED) {
+      ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
+      launch_cast_c128_to_c64(R.phil64 + so, R.phil32 + so, R.sN, st);
+    }
+    if (R.cl_scale) {
+      ProfScope ps(ctx, QFS_PROF_OTHER, 0.0);
+      CK(cudaMemsetAsync(R.cl_acc + 4, 0, sizeof(unsigned), st));
+      CK(launch_cl_scale(R.n, R.M, R.spt * R.L, R.psi64 + so, R.phil64 + so, R.g64 + go, R.cl_acc, R.cl_scale + t, st));
+      CK(cudaMemcpyAsync(&sc, R.cl_scale + t, sizeof(int4), cudaMemcpyDeviceToHost, st));
+    }
+    CK(cudaMemcpyAsync(words, R.flag, sizeof(words), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    prof_harvest(ctx);
+    return QFS_OK;
+  };
+  TRY(finish());
+  if (words[0]) return fail(QFS_ENONFINITE, "NaN or Inf in the target, samples or initial gates");
+  if (words[1]) {  // (rows of U that are not of norm 1)
+    TRY(product(true));
+    TRY(finish());
   }
-  int flag = 0;
-  CK(cudaMemcpyAsync(&flag, R.flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  prof_harvest(ctx);
   R.cl_plain[t] = sc.x != 0;
-  if (flag) return fail(QFS_ENONFINITE, "NaN or Inf in the target, samples or initial gates");
   return QFS_OK;
 }
 
@@ -1305,7 +1327,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
   // some start meets the tolerance, so sweeps go out in batches.
   const bool batch = df && p->plateau_window == 0 && !R.validate;
   const bool cl_many = R.cl.C == 1 && rs == R64 && T == 1;
-  int* stop = R.flag + 2;
+  int* stop = R.flag + 3;
   // Complex64 sweeps skip the residual pass of starts whose update-time
   // estimate (error ~1e-7) is far above tol; plateau detection needs every
   // sweep's residual, so it keeps them all.
@@ -1557,12 +1579,15 @@ int instantiate_restarting(qfs_ctx* ctx, const qfs_circuit* c, const double* tar
     if (validate) {
       draw_states(p->training_distribution, sa, 5u, n, M, h.data());
       CK(cudaMemcpyAsync(R.psi_val64, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
-      CK(cudaMemsetAsync(R.err, 0, sizeof(int), st));
-      TRY(target_product(ctx, R, R.U, R.psi_val64, R.phil_val64, &ctx->prof.launches[QFS_PROF_GEMM]));
-      int err = 0;
-      CK(cudaMemcpyAsync(&err, R.err, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      if (err) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", err);
+      CK(cudaMemsetAsync(R.rows, 0, 2 * sizeof(int), st));
+      int words[2] = {0, 0};  // rows out of scale, the error word
+      for (bool scaled : {false, true}) {
+        if (scaled && !words[0]) break;
+        TRY(target_product(ctx, R, R.U, R.psi_val64, R.phil_val64, &ctx->prof.launches[QFS_PROF_GEMM], scaled));
+        CK(cudaMemcpyAsync(words, R.rows, sizeof(words), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (words[1]) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", words[1]);
+      }
     }
     CK(cudaMemcpyAsync(R.g64, G.data(), G.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     TRY(setup_inputs(ctx, R));
@@ -2101,15 +2126,22 @@ int qfs_target_product_dev(qfs_ctx* ctx, int32_t n, int32_t M, const double* tar
   // (Without room for the digits' scratch: the FP64 kernel.)
   const size_t oz = oz_scratch_bytes(N, M, ctx->num_sms);
   if (oz > 0 && ensure_ws(ctx, oz) == QFS_OK) {
-    // (The kernel sets the error word in pinned host memory: no memset before it
-    // and no copy behind it.)
+    // (The kernels set their words in pinned host memory: no memset before them
+    // and no copy behind them.)
     TRY(ensure_pinned(ctx, 1));
-    volatile int* err = reinterpret_cast<volatile int*>(ctx->h_pinned);
-    *err = 0;
-    ctx->prof.launches[QFS_PROF_GEMM] += 4;
-    CK(launch_oz_product(U, P, O, N, M, ctx->ws, const_cast<int*>(err), ctx->num_sms, st));
+    volatile int* words = reinterpret_cast<volatile int*>(ctx->h_pinned);  // error word, rows out of scale
+    words[0] = words[1] = 0;
+    int *err = const_cast<int*>(words), *rows = err + 1;
+    const int launches = oz_launches(N, M, ctx->num_sms);
+    ctx->prof.launches[QFS_PROF_GEMM] += launches;
+    CK(launch_oz_product(U, P, O, N, M, ctx->ws, err, rows, ctx->num_sms, st));
     CK(cudaStreamSynchronize(st));
-    if (*err) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", *err);
+    if (words[1] && !words[0]) {
+      ctx->prof.launches[QFS_PROF_GEMM] += launches + 1;
+      CK(launch_oz_scaled(U, P, O, N, M, ctx->ws, err, ctx->num_sms, st));
+      CK(cudaStreamSynchronize(st));
+    }
+    if (words[0]) return fail(QFS_ETIMEOUT, "a bounded device wait ran out (error word %d)", words[0]);
     return QFS_OK;
   }
   g_err.clear();
@@ -2247,7 +2279,7 @@ extern "C" int qfs_sweep_once_noalloc_limit(void* cuda_stream, const qfs_circuit
   if (R.n <= kFxProductQubits) {
     CK(launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st));
   } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
-    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), nullptr, sms, st));
+    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), nullptr, nullptr, sms, st));
   } else {
     CK(launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st));
   }

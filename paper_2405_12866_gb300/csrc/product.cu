@@ -33,8 +33,13 @@
 //
 // U's digits have a fixed scale, so its rows have to have a norm near 1, as a
 // unitary's do.  The kernel sums their squares on the way; if any is outside
-// [0.81, 1.21] (or not a number), the FP64 kernel runs behind it; so it does where
-// a bounded wait ran out.
+// [0.81, 1.21], a second pass scales every row by a power of two (n = 12, M = 32,
+// such a target: 4.5 ms with the FP64 kernel for it, 0.37 so).  Rows out of
+// FP32's range, Inf and NaN take the FP64 kernel, and so does a product whose
+// bounded waits ran out.
+//
+// Scratch: the digits of Psi and the splits' sums, for as many columns at a time as
+// fit kOzScratch (n = 12, M = 4096: 1.2 GB in one go).
 #include <cuda_fp16.h>
 
 #include "fixed.cuh"
@@ -54,6 +59,7 @@ constexpr int kOzThreads = 288;  // eight warps for digits and sums, one for the
 constexpr int kOzProd = 256;
 constexpr int kABytes = kDig * 128 * kOzK * 2;
 constexpr long long kOzWait = 1LL << 24;
+constexpr size_t kOzScratch = (size_t)256 << 20;
 
 __host__ __device__ constexpr int oz_bbytes(int nb) { return kDig * nb * kOzK * 2; }
 constexpr int oz_smem(int nb) { return 2 * (kABytes + oz_bbytes(nb)) + 128; }
@@ -78,19 +84,19 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, unsigned parity) {
   return false;
 }
 
-// The digits of two numbers |x| < 2 as seven f16 pairs, most significant first.
+// The digits of two numbers 2^-e x, |x| < 2^(e + 1), as seven f16 pairs, most significant first.
 // The kernel's producers are bound by these instructions, so: two 32-bit
 // funnel shifts instead of a 64-bit shift by a variable, no conversions.
-__device__ __forceinline__ void digits2(double x0, double x1, uint32_t (&d)[kDig]) {
+__device__ __forceinline__ void digits2(double x0, double x1, int e, uint32_t (&d)[kDig]) {
   unsigned long long t[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const double x = k ? x1 : x0;
     const int h = __double2hiint(x);
     const uint32_t l = (uint32_t)__double2loint(x), mh = ((uint32_t)h & 0xfffffu) | 0x100000u;
-    // |x| 2^55 = (m << 3) >> (1023 - exponent field) for the 53-bit mantissa m.
+    // |x| 2^(55 - e) = (m << 3) >> (1023 + e - exponent field) for the 53-bit mantissa m.
     const uint32_t m1 = mh << 3 | l >> 29, m0 = l << 3;
-    const int sh = min(max(1023 - ((h >> 20) & 0x7ff), 0), 63);
+    const int sh = min(max(1023 + e - ((h >> 20) & 0x7ff), 0), 63);
     const bool far = sh >= 32;
     const uint32_t a1 = far ? 0u : m1, a0 = far ? m1 : m0;
     const unsigned long long y = (unsigned long long)(a1 >> (sh & 31)) << 32 | __funnelshift_r(a0, a1, sh);
@@ -127,6 +133,10 @@ __device__ __forceinline__ float trunc32(double x) {
   return __uint_as_float(f <= 0 ? 0u : (uint32_t)min(f, 255) << 23 | m);  // (Inf or NaN stays one; the sign is not wanted)
 }
 
+// The scale of a row in the second pass: 2^e with norm^2 in [2^(2e - 1), 2^(2e + 1)).
+__device__ __forceinline__ bool oz_row_ok(float n2) { return n2 > 0x1p-100f && n2 < 0x1p100f; }
+__device__ __forceinline__ int oz_row_exp(float n2) { return oz_row_ok(n2) ? ((int)(__float_as_uint(n2) >> 23) - 126) >> 1 : 0; }
+
 // K-major operand without swizzle: 8 rows x 16 bytes are contiguous, `lead`
 // bytes lie between neighbours along K, 128 between groups of 8 rows.
 __device__ __forceinline__ uint64_t oz_desc(uint32_t saddr, uint32_t lead) {
@@ -161,21 +171,23 @@ __device__ __forceinline__ void tmem_zero16(uint32_t addr) {
 
 }  // namespace
 
-// Psi's digits in the order of the product kernel's stages: [column block]
-// [step][K group of 8][digit][column][8].  Block j takes column j of Psi
-// (j >= M: zeros that fill up the last column block) and a chunk of the rows
-// (blockIdx.y; all of them look over the whole column for its scale expo[j]).
-// Block (0, 0) also zeroes the flag.
-__global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi, int N, int M, int NB, __half* dig, int* expo,
-                                                  float* row2, int* flag) {
+// Digits of M columns of Psi (rows of ld) in the order of the product kernel's
+// stages: [column block][step][K group of 8][digit][column][8].  Block j takes
+// column j (j >= M: zeros that fill up the last column block) and a chunk of the
+// rows (blockIdx.y; all of them look over the whole column for its scale expo[j]).
+// With row2 (nullable) they also zero it and the flags.
+__global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi, int ld, int N, int M, int NB, __half* dig,
+                                                  int* expo, float* row2, int* flags) {
   const int j = blockIdx.x, tid = threadIdx.x;
-  for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + tid; i < N; i += gridDim.x * gridDim.y * blockDim.x)
-    row2[i] = 0.f;
-  if (j == 0 && blockIdx.y == 0 && tid == 0) *flag = 0;
+  if (row2 != nullptr) {
+    for (int i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + tid; i < N; i += gridDim.x * gridDim.y * blockDim.x)
+      row2[i] = 0.f;
+    if (j == 0 && blockIdx.y == 0 && tid < 2) flags[tid] = 0;
+  }
   int top = 0;  // exponent field of the column's largest entry
   if (j < M)
     for (int i = tid; i < N; i += 256) {
-      const double2 z = Psi[(long long)i * M + j];
+      const double2 z = Psi[(long long)i * ld + j];
       top = max(top, max((__double2hiint(z.x) >> 20) & 0x7ff, (__double2hiint(z.y) >> 20) & 0x7ff));
     }
   __shared__ int red[8];
@@ -196,17 +208,17 @@ __global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi
     double2 z[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      z[r] = j < M ? Psi[(long long)(4 * g + r) * M + j] : double2{0.0, 0.0};
+      z[r] = j < M ? Psi[(long long)(4 * g + r) * ld + j] : double2{0.0, 0.0};
       z[r] = double2{scaled(z[r].x), scaled(z[r].y)};
     }
     uint32_t a[kDig][4], b[kDig][4];  // columns 2j: (pr, -pi), 2j + 1: (pi, pr)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       uint32_t d[kDig];
-      digits2(z[r].x, -z[r].y, d);
+      digits2(z[r].x, -z[r].y, 0, d);
 #pragma unroll
       for (int i = 0; i < kDig; ++i) a[i][r] = d[i];
-      digits2(z[r].y, z[r].x, d);
+      digits2(z[r].y, z[r].x, 0, d);
 #pragma unroll
       for (int i = 0; i < kDig; ++i) b[i][r] = d[i];
     }
@@ -221,11 +233,12 @@ __global__ void __launch_bounds__(256) k_oz_prep(const double2* __restrict__ Psi
 }
 
 // Grid (N / 128 row tiles, K splits, column blocks).  part: [split][column
-// block][row][NB] sums in units of 2^-54 of the scaled columns.
-template <int NB>
+// block][row][NB] sums in units of 2^-54 of the scaled rows and columns.  row2: the
+// sums of the rows' squares, which this launch adds to (norms) or, SCALED, scales by.
+template <int NB, bool SCALED>
 __global__ void __launch_bounds__(kOzThreads, 1)
-    k_oz_product(const double* __restrict__ U, const __half* __restrict__ dig, int N, long long* part, float* row2, int* flag,
-                 int* err) {
+    k_oz_product(const double* __restrict__ U, const __half* __restrict__ dig, int N, long long* part, float* row2, int norms,
+                 int* flag, int* err) {
   extern __shared__ __align__(128) unsigned char sm[];
   constexpr int kB = oz_bbytes(NB), kStage = kABytes + kB, HC = NB / 2;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + 2 * kStage);
@@ -308,6 +321,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const double* u1 = u0 + 64LL * 2 * N;
     double2 x[2][4];
     float n0 = 0.f, n1 = 0.f;
+    const int e0 = SCALED ? oz_row_exp(row2[row0 + r]) : 0, e1 = SCALED ? oz_row_exp(row2[row0 + r + 64]) : 0;
     auto load = [&](int h, int k) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) x[h][q] = __ldg(reinterpret_cast<const double2*>((h ? u1 : u0) + (long long)k * kOzK) + q);
@@ -384,9 +398,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         uint32_t d[4][kDig];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          digits2(x[h][q].x, x[h][q].y, d[q]);
-          const float fx = trunc32(x[h][q].x), fy = trunc32(x[h][q].y);
-          (h ? n1 : n0) = fmaf(fx, fx, fmaf(fy, fy, h ? n1 : n0));
+          digits2(x[h][q].x, x[h][q].y, h ? e1 : e0, d[q]);
+          if constexpr (!SCALED) {
+            const float fx = trunc32(x[h][q].x), fy = trunc32(x[h][q].y);
+            (h ? n1 : n0) = fmaf(fx, fx, fmaf(fy, fy, h ? n1 : n0));
+          }
         }
 #pragma unroll
         for (int p = 0; p < kDig; ++p)
@@ -444,7 +460,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
         for (int c = 0; c < 16; c += 2) *reinterpret_cast<longlong2*>(out + 16 * h + c) = longlong2{sum(c), sum(c + 1)};
       }
-      if (blockIdx.z == 0) {
+      if (!SCALED && norms && blockIdx.z == 0) {
         n0 += __shfl_xor_sync(FULL, n0, 8);
         n1 += __shfl_xor_sync(FULL, n1, 8);
         n0 += __shfl_xor_sync(FULL, n0, 16);
@@ -475,10 +491,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   }
 }
 
-// The splits' sums (exact), to FP64; *flag |= 1 when a row of U was not of norm 1.
+// The splits' sums (exact), to FP64, into M columns of out (rows of ld).  *flag
+// |= 1, and *rows = 1 (nullable), when a row of U or a column was out of scale.
+template <bool SCALED>
 __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__ part, const int* __restrict__ expo,
                                                     const float* __restrict__ row2, int N, int M, int NB, int splits, int cblocks,
-                                                    double2* out, int* flag) {
+                                                    double2* out, int ld, int* flag, volatile int* rows) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)N * M) return;
   const int row = (int)(i / M), j = (int)(i - (long long)row * M);
@@ -490,13 +508,17 @@ __global__ void __launch_bounds__(256) k_oz_finish(const long long* __restrict__
     re += v.x;
     im += v.y;
   }
-  const int e = expo[j];
-  out[i] = double2{scale_exp((double)re, e - 54), scale_exp((double)im, e - 54)};
+  const int e = expo[j], er = SCALED ? oz_row_exp(row2[row]) : 0;
+  out[(long long)row * ld + j] = double2{scale_exp((double)re, e + er - 54), scale_exp((double)im, e + er - 54)};
+  bool bad = e == 1 << 20 && row == 0;
   if (j == 0) {
     const float n2 = row2[row];
-    if (!(n2 > 0.81f && n2 < 1.21f)) atomicOr(flag, 1);
+    bad |= SCALED ? !oz_row_ok(n2) : !(n2 > 0.81f && n2 < 1.21f);
   }
-  if (e == 1 << 20 && row == 0) atomicOr(flag, 1);
+  if (bad) {
+    atomicOr(flag, 1);
+    if (rows != nullptr) *rows = 1;
+  }
 }
 
 // out = U Psi for N <= 256 rows (fixed.cuh: FxDot): grid (N / 8 row tiles (at least 1), column tiles).  Where a row's
@@ -559,54 +581,79 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
 namespace {
 
 struct OzShape {
-  int nb, cblocks, splits;
+  int nb, cblocks, splits;  // of a group of columns
+  int cols, groups;         // columns of a group (the last one may have fewer)
   size_t dig, part, row2, expo, total;
 };
 OzShape oz_shape(int N, int M, int num_sms) {
   OzShape s;
   s.nb = 2 * M <= 32 ? 32 : 64;
-  s.cblocks = (2 * M + s.nb - 1) / s.nb;
-  const int steps = 2 * N / kOzK;
-  s.splits = std::max(1, std::min(steps / 2, num_sms / (N / 128 * s.cblocks)));
+  const int all = (2 * M + s.nb - 1) / s.nb, steps = 2 * N / kOzK;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  s.dig = up((size_t)s.cblocks * steps * oz_bbytes(s.nb));
-  s.part = up((size_t)s.splits * s.cblocks * N * s.nb * sizeof(long long));
-  s.row2 = up((size_t)N * sizeof(float));
-  s.expo = up((size_t)s.cblocks * s.nb / 2 * sizeof(int) + 2 * sizeof(int));
-  s.total = s.dig + s.part + s.row2 + s.expo;
+  auto shape = [&](int cblocks) {
+    s.cblocks = cblocks;
+    s.splits = std::max(1, std::min(steps / 2, num_sms / (N / 128 * cblocks)));
+    s.dig = up((size_t)cblocks * steps * oz_bbytes(s.nb));
+    s.part = up((size_t)s.splits * cblocks * N * s.nb * sizeof(long long));
+    s.row2 = up((size_t)N * sizeof(float));
+    s.expo = up((size_t)cblocks * s.nb / 2 * sizeof(int) + 2 * sizeof(int));
+    s.total = s.dig + s.part + s.row2 + s.expo;
+  };
+  for (s.groups = 1;; ++s.groups) {
+    shape((all + s.groups - 1) / s.groups);
+    if (s.total <= kOzScratch || s.cblocks == 1) break;
+  }
+  s.cols = s.cblocks * s.nb / 2;
+  s.groups = (M + s.cols - 1) / s.cols;
   return s;
+}
+
+// One pass over all columns: digits of Psi, product, sums.
+template <bool SCALED>
+cudaError_t oz_pass(const OzShape& s, const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
+                    int* rows, cudaStream_t st) {
+  char* p = static_cast<char*>(scratch);
+  __half* dig = reinterpret_cast<__half*>(p);
+  long long* part = reinterpret_cast<long long*>(p + s.dig);
+  float* row2 = reinterpret_cast<float*>(p + s.dig + s.part);
+  int* flags = reinterpret_cast<int*>(p + s.dig + s.part + s.row2);
+  int *flag = flags + SCALED, *expo = flags + 2;
+  const auto product = s.nb == 64 ? k_oz_product<64, SCALED> : k_oz_product<32, SCALED>;
+  cudaError_t e = allow_smem(product, oz_smem(s.nb));
+  for (int c = 0; c < M && e == cudaSuccess; c += s.cols) {
+    const int m = std::min(s.cols, M - c), cblocks = (2 * m + s.nb - 1) / s.nb;
+    const bool first = !SCALED && c == 0;
+    e = launch_kernel(k_oz_prep, dim3(cblocks * s.nb / 2, std::max(1, std::min(16, N / 512))), 256, 0, st, Psi + c, M, N, m, s.nb,
+                      dig, expo, first ? row2 : nullptr, flags);
+    if (e == cudaSuccess)
+      e = launch_kernel(product, dim3(N / 128, s.splits, cblocks), kOzThreads, oz_smem(s.nb), st, (const double*)U, dig, N, part,
+                        row2, (int)first, flag, err);
+    if (e == cudaSuccess)
+      e = launch_kernel(k_oz_finish<SCALED>, (unsigned)(((long long)N * m + 255) / 256), 256, 0, st, part, expo, row2, N, m, s.nb,
+                        s.splits, cblocks, out + c, M, flag, rows);
+  }
+  return e;
 }
 
 }  // namespace
 
 size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 512 ? 0 : oz_shape(N, M, num_sms).total; }
+int oz_launches(int N, int M, int num_sms) { return 3 * oz_shape(N, M, num_sms).groups; }
 
 const int* oz_flag(const void* scratch, int N, int M, int num_sms) {
   const OzShape s = oz_shape(N, M, num_sms);
   return reinterpret_cast<const int*>(static_cast<const char*>(scratch) + s.dig + s.part + s.row2);
 }
 
-cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
+cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err, int* rows,
                               int num_sms, cudaStream_t st) {
-  const OzShape s = oz_shape(N, M, num_sms);
-  char* p = static_cast<char*>(scratch);
-  __half* dig = reinterpret_cast<__half*>(p);
-  long long* part = reinterpret_cast<long long*>(p + s.dig);
-  float* row2 = reinterpret_cast<float*>(p + s.dig + s.part);
-  int* flag = reinterpret_cast<int*>(p + s.dig + s.part + s.row2);
-  int* expo = flag + 2;
-  cudaError_t e = cudaFuncSetAttribute(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem(s.nb));
-  if (e != cudaSuccess) return e;
-  e = launch_kernel(k_oz_prep, dim3(s.cblocks * s.nb / 2, std::max(1, std::min(16, N / 512))), 256, 0, st, Psi, N, M, s.nb, dig,
-                    expo, row2, flag);
-  if (e != cudaSuccess) return e;
-  e = launch_kernel(s.nb == 64 ? k_oz_product<64> : k_oz_product<32>, dim3(N / 128, s.splits, s.cblocks), kOzThreads,
-                    oz_smem(s.nb), st, (const double*)U, dig, N, part, row2, flag, err);
-  if (e != cudaSuccess) return e;
-  e = launch_kernel(k_oz_finish, (unsigned)(((long long)N * M + 255) / 256), 256, 0, st, part, expo, row2, N, M, s.nb, s.splits,
-                    s.cblocks, out, flag);
-  return e != cudaSuccess ? e : launch_gemm_upsi(U, Psi, out, N, M, st, flag);
+  const cudaError_t e = oz_pass<false>(oz_shape(N, M, num_sms), U, Psi, out, N, M, scratch, err, rows, st);
+  return e != cudaSuccess || rows != nullptr ? e : launch_gemm_upsi(U, Psi, out, N, M, st, oz_flag(scratch, N, M, num_sms));
+}
+cudaError_t launch_oz_scaled(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err, int num_sms,
+                             cudaStream_t st) {
+  const cudaError_t e = oz_pass<true>(oz_shape(N, M, num_sms), U, Psi, out, N, M, scratch, err, nullptr, st);
+  return e != cudaSuccess ? e : launch_gemm_upsi(U, Psi, out, N, M, st, oz_flag(scratch, N, M, num_sms) + 1);
 }
 
 cudaError_t launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st) {

@@ -234,17 +234,24 @@ void launch_gate_update_batch(int count, const double2* envs, const double2* g_o
 cudaError_t launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
                              cudaStream_t st, const int* only_if = nullptr);
 // The same product, for N >= 512, from 8-bit digits on the tensor cores
-// (product.cu), and by k_gemm_upsi behind it if a row of U is not of norm 1 or a
-// bounded wait ran out.  err: device word, bit 0 set when one did (may be null).
-// The word in its scratch that is not zero, once it has run, when the FP64 kernel
-// ran too: for one, whenever U or Psi holds Inf or NaN.
+// (product.cu).  err: word whose bit 0 is set when a bounded wait ran out (may be
+// null).  rows: word set to 1 when a row of U or a column of Psi was out of scale;
+// the caller then has launch_oz_scaled form the product (U is not of norm 1 in each
+// row: a pass that scales them; what that cannot take: the FP64 kernel).  Null for a
+// caller that cannot look: the FP64 kernel is queued behind, to run in that case.
+// Both words may lie in pinned host memory.
+cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err, int* rows,
+                              int num_sms, cudaStream_t st);
+cudaError_t launch_oz_scaled(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err, int num_sms,
+                             cudaStream_t st);
+size_t oz_scratch_bytes(int N, int M, int num_sms);
+int oz_launches(int N, int M, int num_sms);  // kernels of one pass
+// The word in its scratch that is not zero, once it has run, when something was out
+// of scale: for one, whenever U or Psi holds Inf or NaN.
 const int* oz_flag(const void* scratch, int N, int M, int num_sms);
 // The same for n <= 8 in 64-bit fixed point.
 constexpr int kFxProductQubits = 8;
 cudaError_t launch_fx_product(const double2* U, const double2* Psi, double2* out, int n, int M, cudaStream_t st);
-size_t oz_scratch_bytes(int N, int M, int num_sms);
-cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err,
-                              int num_sms, cudaStream_t st);
 
 void launch_cast_c128_to_c64(const double2* in, float2* out, long long count, cudaStream_t st);
 

@@ -30,9 +30,11 @@ def ctx():
 SIZES = [(9, 5), (10, 16), (11, 1), (11, 17), (11, 65), (12, 32), (12, 33), (12, 300), (13, 20), (13, 64)]
 
 
-@pytest.mark.parametrize("n,M", SIZES)
-@pytest.mark.parametrize("alike", [False, True])
-def test_digits_against_exact_integers(ctx, n, M, alike):
+# (12, 2048: more columns than the scratch holds at a time.)
+@pytest.mark.parametrize("n,M,alike,rows", [(n, M, a, 0) for n, M in SIZES for a in (False, True)] + [(12, 2048, False, 0)]
+                         + [(n, M, False, 40) for n, M in [(9, 5), (10, 31), (11, 65), (12, 300), (12, 2048)]])
+def test_digits_against_exact_integers(ctx, n, M, alike, rows):
+    """rows: each row of U times a power of two up to 2^+-rows (the second pass)."""
     import torch
     N = 1 << n
     gen = torch.Generator(device="cuda").manual_seed(100 * n + M)
@@ -47,16 +49,35 @@ def test_digits_against_exact_integers(ctx, n, M, alike):
     else:
         a = int(one * np.sqrt(3.0))
         u, p = ints(-a, a + 1, (2, N, N)), ints(-(1 << 23) + 1, 1 << 23, (2, N, M))
-    U = torch.complex(*(torch.ldexp(x.double(), torch.tensor(-(22 + n // 2), device="cuda")) for x in u))
+    up = torch.randint(-rows, rows + 1, (N, 1), generator=gen, device="cuda")
+    U = torch.complex(*(torch.ldexp(x.double(), up - (22 + n // 2)) for x in u))
     Psi = torch.complex(*(torch.ldexp(x.double(), torch.tensor(-23, device="cuda")) for x in p))
     got = ctx.target_product(n, U, Psi, 0).cpu().numpy()
-    rows = np.unique(np.concatenate([[0, 1, 127, 128, N - 128, N - 1], np.random.default_rng(n).integers(0, N, 18)]))
-    u, p = u[:, torch.from_numpy(rows).cuda()].cpu().numpy(), p.cpu().numpy()
-    unit = 2.0 ** -(45 + n // 2)
+    some = np.unique(np.concatenate([[0, 1, 127, 128, N - 128, N - 1], np.random.default_rng(n).integers(0, N, 18)]))
+    u, p = u[:, torch.from_numpy(some).cuda()].cpu().numpy(), p.cpu().numpy()
+    scale = np.ldexp(1.0, up.cpu().numpy()[some])
+    unit = 2.0 ** -(45 + n // 2) * scale
     want = (u[0] @ p[0] - u[1] @ p[1]).astype(np.longdouble) * unit, (u[0] @ p[1] + u[1] @ p[0]).astype(np.longdouble) * unit
     slack = 2 * N * (3 / 256 * 2.0**-52 + 2.0**-48 / 4096) if alike else 0.0
-    for g, e in zip((got[rows].real, got[rows].imag), want):
-        assert np.all(np.abs(g - e) <= 2.0**-53 * np.abs(e) + 32 * 2.0**-55 + slack)
+    for g, e in zip((got[some].real, got[some].imag), want):
+        assert np.all(np.abs(g - e) <= 2.0**-53 * np.abs(e) + (32 * 2.0**-55 + slack) * scale)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_sweep_of_a_target_with_rows_of_all_sizes(ctx, prec):
+    """A run's set-up takes the second pass too: one sweep at 9 qubits against the oracle, to
+    the tolerances of FP64 and complex64 sweeps of states of norm 1, times U's norm."""
+    from oracle import qfs_oracle as o
+    from paper_2405_12866_gb300 import workloads as w
+    n, M = 9, 8
+    pairs = w.brick_pairs(n, 2)
+    U = w.target_unitary(w.haar_gates(701, w.STREAM_TARGET_GATES, len(pairs)), pairs, n)
+    U *= np.random.default_rng(1).uniform(0.2, 3.0, (1 << n, 1))
+    Psi, G = w.sample_states(702, n, M), w.initial_gates(703, 2, len(pairs))
+    _, env, _ = ctx.sweep_once(n, pairs, U, Psi, G, prec)
+    for s in range(2):
+        r = o.sweep(U @ Psi, Psi, G[s], pairs, n)
+        assert np.max(np.abs(env[s] - r.envs)) < 3.0 * (1e-4 if prec else 1e-10)
 
 
 @pytest.mark.parametrize("n,M", SIZES)
