@@ -267,7 +267,7 @@ struct Run {
   size_t oz_bytes = 0;
   double2* g64 = nullptr;
   float2* g32 = nullptr;
-  double2* vprev = nullptr;  // right singular vectors of each gate's last update
+  double2* vprev = nullptr;  // right singular vectors of each gate's last update (per-step sweeps)
   double* partials = nullptr;
   double* costs = nullptr;
   double* cost_rows = nullptr;   // kSweepBatch x S: the costs of each sweep of a batch
@@ -309,7 +309,7 @@ struct Run {
   bool cl_check = false;         // checks of training states in one launch
   bool cl_fx = false;            // fixed-point sweeps or checks: the scales are wanted
   std::vector<char> cl_plain;    // per slot: its sweeps take the plain FP64 form
-  const void* df_key[4] = {};  // what the uploaded table was built for
+  const void* df_key[3] = {};  // what the uploaded table was built for
   int df_key_r = -1;
   bool lean = false;           // the workspace has room for the smallest buffers only
 };
@@ -459,7 +459,7 @@ bool whole_usable(const qfs_ctx* ctx, const Run& R, Real r) { return R.cl.C > 0 
 // sweep()), chunked so that each step offers about two items per resident
 // CTA.  With null buffers in R it only sizes the table.
 void df_build(const qfs_ctx* ctx, const Run& R, Real r, const void* psi, const void* phil, double2* envs,
-              const int* active, double2* vprev, std::vector<DfStep>& steps, double* bytes) {
+              const int* active, std::vector<DfStep>& steps, double* bytes) {
   steps.clear();
   *bytes = 0.0;
   const size_t es = elem_bytes(r);
@@ -503,7 +503,6 @@ void df_build(const qfs_ctx* ctx, const Run& R, Real r, const void* psi, const v
     u.env_stride = gstride;
     u.S = S;
     u.active = active;
-    u.vprev = vprev ? vprev + (size_t)(k - 1) * 16 : nullptr;
     return u;
   };
   auto distinct = [&](int k) {  // gates k and k + 1 on four distinct qubits
@@ -718,7 +717,7 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
     if (R.cl.C == 0 && df_usable(ctx, R, rs)) {
       std::vector<DfStep> steps;
       double b = 0.0;
-      df_build(ctx, R, rs, nullptr, nullptr, nullptr, nullptr, nullptr, steps, &b);
+      df_build(ctx, R, rs, nullptr, nullptr, nullptr, nullptr, steps, &b);
       R.df_cap = (int)steps.size();
       for (const DfStep& st : steps) {
         R.df_max_nchunk = std::max(R.df_max_nchunk, st.nchunk);
@@ -982,13 +981,13 @@ int sweep(qfs_ctx* ctx, Run& R, Real r, const Slice& sl, double2* g64, float2* g
 // sweep() up to the order of the reduction sums).  The step table is built
 // and uploaded once per (precision, outputs) and reused by later sweeps.
 int df_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, double2* envs, const int* active,
-             double2* vprev, cudaStream_t st, int* stop = nullptr, double stop_tol = 0.0,
+             cudaStream_t st, int* stop = nullptr, double stop_tol = 0.0,
              double* cost_row = nullptr, double resid_skip = 0.0) {
-  const void* key[4] = {psi, envs, active, vprev};
+  const void* key[3] = {psi, envs, active};
   if (R.df_key_r != (int)r || std::memcmp(key, R.df_key, sizeof(key)) != 0) {
     std::vector<DfStep> steps;
     double bytes = 0.0;
-    df_build(ctx, R, r, psi, phil, envs, active, vprev, steps, &bytes);
+    df_build(ctx, R, r, psi, phil, envs, active, steps, &bytes);
     int mx = 0;
     for (const DfStep& s : steps) mx = std::max(mx, s.nchunk);
     if ((int)steps.size() > R.df_cap || mx > R.df_max_nchunk)
@@ -1100,9 +1099,9 @@ int cl_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, do
 
 // One whole-sweep launch without a batch.
 int whole_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, double2* envs, const int* active,
-                double2* vprev, cudaStream_t st, double resid_skip = 0.0) {
+                cudaStream_t st, double resid_skip = 0.0) {
   if (R.cl.C > 0) return cl_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, -1.0, nullptr, resid_skip);
-  return df_sweep(ctx, R, r, psi, phil, envs, active, vprev, st, nullptr, 0.0, nullptr, resid_skip);
+  return df_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, 0.0, nullptr, resid_skip);
 }
 
 // FP64 sample cost of start s's master gates on states psi with
@@ -1356,7 +1355,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
                          per));
         } else {
           for (int b = 0; b < B; ++b)
-            TRY(df_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, stop, ctol,
+            TRY(df_sweep(ctx, R, rs, psi, phil, nullptr, R.active, st, stop, ctol,
                          R.cost_rows + (size_t)b * S, skip));
         }
         TRY(read_rows(ctx, R.cost_rows, S, B, rows, R.err));
@@ -1375,7 +1374,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
         prof_harvest(ctx);
       } else {
         if (df) {
-          TRY(whole_sweep(ctx, R, rs, psi, phil, nullptr, R.active, R.vprev, st, skip));
+          TRY(whole_sweep(ctx, R, rs, psi, phil, nullptr, R.active, st, skip));
         } else {
           CK(cudaGraphLaunch(graph.exec, st));
           for (int i = 0; i < QFS_PROF_KINDS; ++i) ctx->prof.launches[i] += graph.launches[i];
@@ -2067,7 +2066,7 @@ int qfs_sweep_once(qfs_ctx* ctx, const qfs_circuit* circuit, const double* targe
   const void* psi = rs == R32 ? (const void*)R.psi32 : (const void*)R.psi64;
   const void* phil = rs == R32 ? (const void*)R.phil32 : (const void*)R.phil64;
   if (whole_usable(ctx, R, rs))
-    TRY(whole_sweep(ctx, R, rs, psi, phil, R.envs, nullptr, nullptr, st));
+    TRY(whole_sweep(ctx, R, rs, psi, phil, R.envs, nullptr, st));
   else
     TRY(sweep(ctx, R, rs, Slice{0, S, S, ctx->stream}, R.g64, R.g32, psi, phil, R.B, R.phi, R.partials,
               R.nblk_max, R.costs, R.envs, nullptr, R.stream_b, nullptr, R.counters));

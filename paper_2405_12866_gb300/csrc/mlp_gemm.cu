@@ -60,9 +60,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
 // The tanh form of GELU, 0.5 x (1 + tanh u) with u = sqrt(2/pi) (x +
 // 0.044715 x^3), evaluated as the equal x / (1 + exp(-2u)): ten instructions,
 // two of them special functions, ~1e-6 relative, far below the bf16 rounding of
-// the result.  The flushing forms skip the scaling for subnormals: 1 + a
-// subnormal is 1, and a quotient by 2^126 and above is 0 (exp(-2u) = inf for
-// u < -44 gives -0).
+// the result.  The .ftz forms give 0 where a result is subnormal (PTX ISA): 1 + that
+// is 1, and a reciprocal below 2^-126 leaves nothing of x (exp(-2u) = inf for u <
+// -44 gives -0).
 __device__ __forceinline__ float gelu_tanh(float x) {
   const float k0 = 0.7978845608028654f, k1 = 0.044715f;
   const float u = k0 * fmaf(k1 * x, x * x, x);
