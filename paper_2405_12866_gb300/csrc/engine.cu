@@ -308,7 +308,8 @@ struct Run {
   double* cl_parts = nullptr;
   bool cl_check = false;         // checks of training states in one launch
   bool cl_fx = false;            // fixed-point sweeps or checks: the scales are wanted
-  std::vector<char> cl_plain;    // per slot: its sweeps take the plain FP64 form
+  std::vector<char> cl_plain;    // per slot: why its sweeps take the plain FP64 form (kClPlain..., 0: they do not)
+  bool cl_plain_df = false;      // ... which is the dataflow sweep then
   const void* df_key[3] = {};  // what the uploaded table was built for
   int df_key_r = -1;
   bool lean = false;           // the workspace has room for the smallest buffers only
@@ -714,7 +715,13 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
     // FP64 cluster sweeps, and the FP64 checks of complex64 runs.
     R.cl_check = !lean && prec == QFS_MIXED && ctx->dataflow && cl_check_fits(R.n, R.L);
     R.cl_fx = R.cl_check || (R.cl.C > 0 && prec == QFS_FP64);
-    if (R.cl.C == 0 && df_usable(ctx, R, rs)) {
+    // Plain FP64 sweeps are bound by the FP64 pipe, of which a cluster has 16 SMs
+    // at most: with 2048 entries a CTA and more (one start, n = 10, M = 32: 563 us
+    // there, 543 by the dataflow sweep; n = 11: 832 and 462; 8 starts 788 and 790,
+    // 1203 and 953) they take the dataflow sweep.
+    R.cl_plain_df = R.cl.C > 0 && prec == QFS_FP64 && df_usable(ctx, R, rs) &&
+                    (size_t)((M + R.cl.C - 1) / R.cl.C) << R.n >= 2048;
+    if (R.cl_plain_df || (R.cl.C == 0 && df_usable(ctx, R, rs))) {
       std::vector<DfStep> steps;
       double b = 0.0;
       df_build(ctx, R, rs, nullptr, nullptr, nullptr, nullptr, steps, &b);
@@ -836,7 +843,8 @@ int setup_slot(qfs_ctx* ctx, Run& R, int t) {
     TRY(product(true));
     TRY(finish());
   }
-  R.cl_plain[t] = sc.x != 0;
+  // (complex64 runs look at it for FP64 checks, whose gates have been swept.)
+  R.cl_plain[t] = (char)(R.prec == QFS_MIXED && sc.x == kClPlainGates ? 0 : sc.x);
   return QFS_OK;
 }
 
@@ -1097,10 +1105,32 @@ int cl_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, do
   return QFS_OK;
 }
 
+// Whether the next sweeps of all starts go by the dataflow sweep.
+bool by_dataflow(const Run& R) {
+  bool plain = false;
+  for (char c : R.cl_plain) plain |= c != 0;
+  return R.cl.C == 0 || (R.cl_plain_df && plain);
+}
+
+// Whether a slot's starts have initial gates that are not unitary; after one
+// sweep they are, and the next ones can be in fixed point.
+bool cl_first_plain(const Run& R) {
+  return R.cl.C > 0 && R.prec == QFS_FP64 &&
+         std::find(R.cl_plain.begin(), R.cl_plain.end(), (char)kClPlainGates) != R.cl_plain.end();
+}
+int cl_lift_plain(qfs_ctx* ctx, Run& R) {
+  for (int t = 0; t < R.T; ++t) {
+    if (R.cl_plain[t] != kClPlainGates) continue;
+    CK(cudaMemsetAsync(&R.cl_scale[t].x, 0, sizeof(int), ctx->stream));
+    R.cl_plain[t] = 0;
+  }
+  return QFS_OK;
+}
+
 // One whole-sweep launch without a batch.
 int whole_sweep(qfs_ctx* ctx, Run& R, Real r, const void* psi, const void* phil, double2* envs, const int* active,
                 cudaStream_t st, double resid_skip = 0.0) {
-  if (R.cl.C > 0) return cl_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, -1.0, nullptr, resid_skip);
+  if (!by_dataflow(R)) return cl_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, -1.0, nullptr, resid_skip);
   return df_sweep(ctx, R, r, psi, phil, envs, active, st, nullptr, 0.0, nullptr, resid_skip);
 }
 
@@ -1338,11 +1368,13 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
       int room = p->max_sweeps;
       for (int t = 0; t < T; ++t)
         if (busy[t]) room = std::min(room, p->max_sweeps - tsweeps[t]);
-      const int B = batch ? std::max(1, std::min(R.cl.C > 0 ? (cl_many ? kSweepBatch : kClBatch) : kDfBatch, room)) : 1;
+      const bool by_df = by_dataflow(R), first_plain = cl_first_plain(R);
+      const int most = first_plain ? 1 : by_df ? kDfBatch : cl_many ? kSweepBatch : kClBatch;
+      const int B = batch ? std::max(1, std::min(most, room)) : 1;
       if (df && B > 1) {
         int per = 1;  // sweeps per launch
-        CK(cudaMemsetAsync(stop, R.cl.C > 0 ? 0x7f : 0, sizeof(int), st));
-        if (R.cl.C > 0) {
+        CK(cudaMemsetAsync(stop, by_df ? 0 : 0x7f, sizeof(int), st));
+        if (!by_df) {
           // FP64 and one target: the run ends at the sweep that meets the
           // tolerance, so one launch takes the batch and a start that meets
           // it stops there.  Complex64 runs may go on from that sweep (the
@@ -1383,6 +1415,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
         TRY(read_costs(ctx, R.costs, S, rows[0], R.err));
         if (ctx->prof.on && !df) prof_harvest_graph(ctx);
         nrows = 1;
+        if (first_plain) TRY(cl_lift_plain(ctx, R));
       }
       row = 0;
     }

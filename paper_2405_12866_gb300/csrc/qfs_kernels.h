@@ -158,10 +158,13 @@ struct ClArgs {
   int sweep0, nsweeps;                  // sweeps of this launch; several need C = 1 (a start ends with the sweep in
                                         // which it or, seen in between, another met stop_tol)
   int* err; long long wait_limit;       // as DfArgs: polls of an exchange before the kernel gives up; err may be null
-  const int4* scale;                    // FP64: per target {1: the plain FP64 form, exponents of the column norms
-                                        //   of Psi and U Psi, 0} (launch_cl_scale); null: plain
+  const int4* scale;                    // FP64: per target {0 or why the plain FP64 form, exponents of the column
+                                        //   norms of Psi and U Psi, 0} (launch_cl_scale); null: plain
   unsigned char pos[kClMaxGates];       // per gate: row bits of its qubits, a | b << 4
 };
+// Why a target's FP64 sweeps are plain: columns out of range, or initial gates that
+// are not unitary (which ends with the first sweep: its gates are polar factors).
+constexpr int kClPlainRange = 1, kClPlainGates = 2;
 struct ClPlan {
   int C = 0;                            // CTAs per start; 0: the state does not fit
   int threads = 0;

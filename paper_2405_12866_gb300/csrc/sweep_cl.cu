@@ -870,7 +870,8 @@ __global__ void __launch_bounds__(NT) k_cl_check(ClArgs a, double* parts, unsign
   }
 }
 
-// The scales of one target's fixed-point sweeps: out = {plain, e_psi, e_phi, 0}.
+// The scales of one target's fixed-point sweeps: out = {plain, e_psi, e_phi, 0},
+// plain 0 or the reason why its sweeps take the plain FP64 form (kClPlain...).
 // Block j < M: the norm of column j of Psi and of U Psi (FP32 is enough for an
 // exponent); the other blocks: whether every initial gate is unitary to 1e-4.
 // acc (zero before): the largest squared norms' bits, a not-unitary flag, and
@@ -935,14 +936,15 @@ __global__ void k_cl_scale(int N, int M, int gates, const double2* psi, const do
   if (last && tid == 0) {
     __threadfence();
     int e[2];
-    bool plain = atomicOr(acc + 2, 0u) != 0;
+    bool range = true;
     for (int k = 0; k < 2; ++k) {
       const float n2 = __uint_as_float(atomicOr(acc + k, 0u));
-      plain |= !(n2 > 1e-30f && n2 < 1e30f);
+      const bool ok = n2 > 1e-30f && n2 < 1e30f;
+      range &= ok;
       // The least e with norm <= 1.001 2^e.
-      e[k] = plain ? 0 : (int)ceilf(0.5f * log2f(n2) - 1.4e-3f);
+      e[k] = ok ? (int)ceilf(0.5f * log2f(n2) - 1.4e-3f) : 0;
     }
-    *out = int4{plain ? 1 : 0, e[0], e[1], 0};
+    *out = int4{!range ? kClPlainRange : atomicOr(acc + 2, 0u) != 0 ? kClPlainGates : 0, e[0], e[1], 0};
   }
 }
 
