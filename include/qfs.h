@@ -319,7 +319,8 @@ int qfs_gate_update(qfs_ctx* ctx, int32_t count, const double* envs, const doubl
 /* Phi_L = U Psi, the A tensor of Section 3 (the product every instantiation
  * starts from), on device buffers: target_dev N x N and samples_dev N x M
  * complex128 row-major, out_dev N x M (N = 2^n).  Either precision gives the
- * same product, to FP64 accuracy: from n = 9 on by exact products of 8-bit
+ * same product, to FP64 accuracy: from n = 9 on, and at n = 8 for more than 96
+ * columns, by exact products of 8-bit
  * digits on the tensor cores (in a second pass where a row of U is not of norm
  * 1 to 10%), below in 64-bit fixed point, in workspace of the context (at most
  * 256 MB, but for one block of 32 columns at least; without room for it: FP64

@@ -751,8 +751,8 @@ int prepare(qfs_ctx* ctx, Run& R, const qfs_circuit* c, int M, int S_target, int
   return QFS_OK;
 }
 
-// Phi_L = U Psi (Sec. 3, the A tensor), to FP64 accuracy: from 512 rows on by
-// digits on the tensor cores (a call at n = 9, M = 24: 302 us in FP64, 57 so; n =
+// Phi_L = U Psi (Sec. 3, the A tensor), to FP64 accuracy: from 512 rows on (256,
+// for many columns: oz_scratch_bytes) by digits on the tensor cores (a call at n = 9, M = 24: 302 us in FP64, 57 so; n =
 // 12, M = 32: 4.28 ms and 0.19), below in fixed point (n = 8, M = 24: 163 us in
 // FP64, 53 by digits, 40 so).  (Without room for the digits' scratch, or when a
 // mixed run asks for it, the FP64 kernel.)  Adds its launches to *launches.
@@ -1369,7 +1369,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
       for (int t = 0; t < T; ++t)
         if (busy[t]) room = std::min(room, p->max_sweeps - tsweeps[t]);
       const bool by_df = by_dataflow(R), first_plain = cl_first_plain(R);
-      const int most = first_plain ? 1 : by_df ? kDfBatch : cl_many ? kSweepBatch : kClBatch;
+      const int most = first_plain ? 1 : cl_many && !by_df ? kSweepBatch : by_df ? kDfBatch : kClBatch;
       const int B = batch ? std::max(1, std::min(most, room)) : 1;
       if (df && B > 1) {
         int per = 1;  // sweeps per launch

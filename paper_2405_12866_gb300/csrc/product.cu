@@ -27,9 +27,9 @@
 // sums of constant rows and columns were off by up to 1e-11 from n = 13 on, in one
 // split of 8192 products and more.)
 //
-// Up to 256 rows there are at most two tiles to fill: k_fx_product forms the
-// product in 64-bit fixed point (fixed.cuh), a component by one or two threads (n
-// = 6, M = 16: 50 us as FP64, 6 us so).
+// Up to 256 rows there are at most two tiles to fill: unless 256 rows meet many
+// columns, k_fx_product forms the product in 64-bit fixed point (fixed.cuh), a
+// component by one or two threads (n = 6, M = 16: 50 us as FP64, 6 us so).
 //
 // U's digits have a fixed scale, so its rows have to have a norm near 1, as a
 // unitary's do.  The kernel sums their squares on the way; if any is outside
@@ -637,7 +637,11 @@ cudaError_t oz_pass(const OzShape& s, const double2* U, const double2* Psi, doub
 
 }  // namespace
 
-size_t oz_scratch_bytes(int N, int M, int num_sms) { return N < 512 ? 0 : oz_shape(N, M, num_sms).total; }
+// From 512 rows on, and at 256 for more than 96 columns, where fixed point grows
+// with M (a call at M = 64: 48 us, 96: 56, 128: 67, 256: 93) and digits take 50 us.
+size_t oz_scratch_bytes(int N, int M, int num_sms) {
+  return N < 256 || (N == 256 && M <= 96) ? 0 : oz_shape(N, M, num_sms).total;
+}
 int oz_launches(int N, int M, int num_sms) { return 3 * oz_shape(N, M, num_sms).groups; }
 
 const int* oz_flag(const void* scratch, int N, int M, int num_sms) {

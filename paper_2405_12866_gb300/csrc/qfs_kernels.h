@@ -236,7 +236,7 @@ void launch_gate_update_batch(int count, const double2* envs, const double2* g_o
 // only_if (nullable, device): the kernel does nothing when it holds zero.
 cudaError_t launch_gemm_upsi(const double2* U, const double2* Psi, double2* out, int N, int M,
                              cudaStream_t st, const int* only_if = nullptr);
-// The same product, for N >= 512, from 8-bit digits on the tensor cores
+// The same product, for N >= 256, from 8-bit digits on the tensor cores
 // (product.cu).  err: word whose bit 0 is set when a bounded wait ran out (may be
 // null).  rows: word set to 1 when a row of U or a column of Psi was out of scale;
 // the caller then has launch_oz_scaled form the product (U is not of norm 1 in each
@@ -247,7 +247,7 @@ cudaError_t launch_oz_product(const double2* U, const double2* Psi, double2* out
                               int num_sms, cudaStream_t st);
 cudaError_t launch_oz_scaled(const double2* U, const double2* Psi, double2* out, int N, int M, void* scratch, int* err, int num_sms,
                              cudaStream_t st);
-size_t oz_scratch_bytes(int N, int M, int num_sms);
+size_t oz_scratch_bytes(int N, int M, int num_sms);  // 0: sizes that take another form
 int oz_launches(int N, int M, int num_sms);  // kernels of one pass
 // The word in its scratch that is not zero, once it has run, when something was out
 // of scale: for one, whenever U or Psi holds Inf or NaN.

@@ -1,4 +1,4 @@
-"""U Psi from 8-bit digits (n >= 9) against exact integers, at the sizes where a
+"""U Psi from 8-bit digits (n >= 9, and n = 8 from 97 columns on) against exact integers, at the sizes where a
 CTA runs through many chunks, a part of a chunk or a second column block, for
 targets and states whose digits are all alike, so that the digits' sums grow as
 fast as they can.
@@ -27,7 +27,7 @@ def ctx():
         yield c
 
 
-SIZES = [(9, 5), (10, 16), (11, 1), (11, 17), (11, 65), (12, 32), (12, 33), (12, 300), (13, 20), (13, 64)]
+SIZES = [(8, 97), (8, 256), (9, 5), (10, 16), (11, 1), (11, 17), (11, 65), (12, 32), (12, 33), (12, 300), (13, 20), (13, 64)]
 
 
 # (12, 2048: more columns than the scratch holds at a time.)
