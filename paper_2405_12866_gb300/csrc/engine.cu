@@ -238,7 +238,8 @@ void prof_harvest(qfs_ctx* ctx) {
 constexpr int kSweepBatch = 64;  // sweeps per host round trip, at most (room for their costs): one launch of
                                  // the cluster sweep with one CTA per start
 constexpr int kClBatch = 16;     // ... of the cluster sweep, a launch each
-constexpr int kDfBatch = 4;      // ... of the dataflow sweep
+constexpr int kDfBatch = 4;      // ... of the dataflow sweep, and of any at n = 2, where one sweep solves the one pair
+                                 // of qubits (complex64, 1 gate: 283 us with 15 idle launches behind it, 243 with 3)
 
 // Device buffers of one run, carved from the context's workspace.
 struct Run {
@@ -1369,7 +1370,7 @@ int run_multistart(qfs_ctx* ctx, Run& R, const qfs_params* p,
       for (int t = 0; t < T; ++t)
         if (busy[t]) room = std::min(room, p->max_sweeps - tsweeps[t]);
       const bool by_df = by_dataflow(R), first_plain = cl_first_plain(R);
-      const int most = first_plain ? 1 : cl_many && !by_df ? kSweepBatch : by_df ? kDfBatch : kClBatch;
+      const int most = first_plain ? 1 : cl_many && !by_df ? kSweepBatch : by_df || R.n == 2 ? kDfBatch : kClBatch;
       const int B = batch ? std::max(1, std::min(most, room)) : 1;
       if (df && B > 1) {
         int per = 1;  // sweeps per launch
