@@ -975,10 +975,14 @@ ClPlan cl_plan(Real r, int n, int M, int L, int spt, bool keep64) {
     const double t = waves * (fixed + work);
     // More than two rounds of complex64 starts of 1 MiB and more: their B
     // lists are in HBM and the dataflow sweep, which overlaps one start's
-    // update with another's streaming, is the faster one (n = 12, M = 32, 17
-    // gates: 32 starts 625 us here, 491 there; 16 starts 352 and 361; n = 11,
-    // 32 starts 241 and 431).  It takes even M.
-    const bool large = r == R32 && waves > 2 && ((size_t)M << n) >= ((size_t)1 << 17) && M % 2 == 0;
+    // update with another's streaming, is the faster one (a sweep here and
+    // there at n = 12, 17 gates, M = 32: 12 starts 207 us and 306, 16: 341 and
+    // 344, 20: 408 and 362, 24, two rounds again: 406 and 399, 32: 606 and 458;
+    // n = 11, 32 starts 185 and 296).  So it is where a second round of slices of
+    // 16,384 entries is a third full or less (n = 9, M = 512: 6 starts 150 and 249,
+    // 8: 294 and 272, 10: 294 and 291; 10 to 12 qubits alike).  It takes even M.
+    const bool rounds = waves > 2 || (waves == 2 && entries >= 16384.0 && 3 * spt <= 4 * at_once);
+    const bool large = r == R32 && rounds && ((size_t)M << n) >= ((size_t)1 << 17) && M % 2 == 0;
     if (best_t == 0.0 || t < best_t) {
       best_t = t;
       best.C = large ? 0 : C;
