@@ -352,7 +352,7 @@ __device__ int block_exponent(const double2* z, int count, int* red) {
 // Psi and Phi_L.  One block per problem, one component of the product per
 // thread at a time, in fixed point with a scale for every row of U and column
 // of Psi (fixed.cuh: FxDot).  (1024 problems of 3 to 5 qubits: 110 us in FP64,
-// whose pipe it filled by a third, 60 so.)  Error relative to the product's norm
+// whose pipe it filled by a third, 52 so; 96 problems 20.)  Error relative to the product's norm
 // at n = 6: FP64 3.9e-16, with one scale for all of U and all of Psi and without
 // the low x low products 1.2e-15, so 6e-17.  Rows and columns out of the scales'
 // range (Inf, NaN) take the FP64 form.
@@ -366,12 +366,8 @@ __global__ void __launch_bounds__(128) k_batch_prep(BatchArgs a) {
   const double2* U = a.targets + pr.target_off;
   const double2* psi = a.psi64 + pr.state_off;
   if (threadIdx.x == 0) a.s_star[p] = INT_MAX;
-  for (int r = threadIdx.x >> 5; r < N; r += 4) {
-    int t = 0;
-    for (int k = lane; k < N; k += 32) t = max(t, fx_top(U[r * N + k]));
-    t = __reduce_max_sync(FULL, t);
-    if (lane == 0) tu[r] = t;
-  }
+  int4* su = reinterpret_cast<int4*>(dsm);
+  int4* sp = su + N * N;
   for (int j = threadIdx.x; j < M; j += blockDim.x) tp[j] = 0;
   __syncthreads();
   for (int e = threadIdx.x; e < N * M; e += blockDim.x) {
@@ -379,10 +375,23 @@ __global__ void __launch_bounds__(128) k_batch_prep(BatchArgs a) {
     a.psi32[pr.state_off + e] = float2{(float)s.x, (float)s.y};
     atomicMax(&tp[e % M], fx_top(s));
   }
+  // A warp takes four rows of U at a time: their loads, then their exponents.
+  for (int r = 4 * (threadIdx.x >> 5); r < N; r += 16) {
+    double2 z[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) z[i][h] = lane + 32 * h < N ? U[(r + i) * N + lane + 32 * h] : double2{0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = __reduce_max_sync(FULL, max(fx_top(z[i][0]), fx_top(z[i][1])));
+      if (lane == 0) tu[r + i] = t;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (lane + 32 * h < N) su[(r + i) * N + lane + 32 * h] = fx_from2(z[i][h], fx_row_exp(t, n));
+    }
+  }
   __syncthreads();
-  int4* su = reinterpret_cast<int4*>(dsm);
-  int4* sp = su + N * N;
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) su[e] = fx_from2(U[e], fx_row_exp(tu[e >> n], n));
   for (int e = threadIdx.x; e < N * M; e += blockDim.x) sp[e] = fx_from2(psi[e], fx_col_exp(tp[e % M], n));
   __syncthreads();
   for (int c = threadIdx.x; c < 2 * N * M; c += blockDim.x) {
@@ -395,7 +404,7 @@ __global__ void __launch_bounds__(128) k_batch_prep(BatchArgs a) {
       }
     } else {
       FxDot t;
-      for (int k = 0; k < N; ++k) t.add(su[i * N + k], sp[k * M + j], im);
+      t.run<1>(su + i * N, sp + j, M, 0, N, im);
       v = fx_dot_value(t.t.h, t.cross(), fx_row_exp(tu[i], n) + fx_col_exp(tp[j], n));
     }
     reinterpret_cast<double*>(a.phil64 + pr.state_off + e)[im] = v;

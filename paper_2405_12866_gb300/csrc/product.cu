@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(256) k_fx_product(const double2* __restrict__ 
   for (int e = tid; e < 2 * KS * rows * cols; e += 256) {  // (KS = 2: a multiple of 32, so warps are whole)
     const int c = e / KS, part = e % KS, im = c & 1, i = (c >> 1) / cols, j = (c >> 1) % cols;
     FxDot t;
-    for (int k = part; k < N; k += KS) t.add(su[i * N + k], sp[k * cols + j], im);
+    t.run<KS>(su + i * N, sp + j, cols, part, N, im);
     long long high = t.t.h, cross = t.cross();
     if constexpr (KS == 2) {
       high += __shfl_xor_sync(FULL, high, 1);
