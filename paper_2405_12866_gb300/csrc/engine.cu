@@ -2307,12 +2307,15 @@ extern "C" int qfs_sweep_once_noalloc_limit(void* cuda_stream, const qfs_circuit
   if (gates_out_dev != gates_in_dev)
     CK(cudaMemcpyAsync(gates_out_dev, gates_in_dev, (size_t)S * R.L * 16 * sizeof(double2),
                        cudaMemcpyDeviceToDevice, st));
-  // Phi_L = U Psi: digits where their scratch still fits behind the sweep's.
-  const size_t oz = oz_scratch_bytes((int)R.N, M, sms);
+  // Phi_L = U Psi: digits where their scratch still fits behind the sweep's, in
+  // as many splits as do (shaped for fewer SMs).
+  int oz_sms = sms;
+  while (oz_sms > 16 && need + 256 + oz_scratch_bytes((int)R.N, M, oz_sms) > (size_t)QFS_NOALLOC_SCRATCH_BYTES) oz_sms /= 2;
+  const size_t oz = oz_scratch_bytes((int)R.N, M, oz_sms);
   if (R.n <= kFxProductQubits) {
     CK(launch_fx_product(R.U, R.psi64, R.phil64, R.n, M, st));
   } else if (oz > 0 && need + 256 + oz <= (size_t)QFS_NOALLOC_SCRATCH_BYTES) {
-    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), nullptr, nullptr, sms, st));
+    CK(launch_oz_product(R.U, R.psi64, R.phil64, (int)R.N, M, take(oz), nullptr, nullptr, oz_sms, st));
   } else {
     CK(launch_gemm_upsi(R.U, R.psi64, R.phil64, (int)R.N, M, st));
   }

@@ -24,8 +24,8 @@
 // most, so its last additions may round to 2^-52 where every digit is extreme);
 // D_6, 2^-48 of D_0, after every 4096.  D_7 may round, and what is left out (d > 7)
 // is below 2^-60 of the result's scale.  (With D_4 and D_5 read only at the end the
-// sums of constant rows and columns were off by up to 1e-11 from n = 13 on, in one
-// split of 8192 products and more.)
+// sums of constant rows and columns were off in splits of 4096 products and more, by
+// up to 1e-11 at n = 13.)
 //
 // Up to 256 rows there are at most two tiles to fill: unless 256 rows meet many
 // columns, k_fx_product forms the product in 64-bit fixed point (fixed.cuh), a

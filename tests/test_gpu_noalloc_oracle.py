@@ -2,7 +2,7 @@
 what it leaves where a wait runs out.
 
 Routes: the cluster sweep (behind the fixed-point product, and behind the digits
-at 9 qubits) and the per-step launches (more gates than the cluster sweep takes,
+at 9 qubits and, in fewer splits for want of room, at 10) and the per-step launches (more gates than the cluster sweep takes,
 with either product).  Tolerances as for every FP64 sweep: 1e-10 on gates and
 environments, 1e-12 on the cost."""
 import ctypes as C
@@ -43,7 +43,7 @@ def _run(qfs, n, pairs, M, S, seed, wait_limit=None, beta=0.0):
     return code, out[0].cpu().numpy(), out[1].cpu().numpy(), cost.cpu().numpy(), (U, Psi, G)
 
 
-@pytest.mark.parametrize("n, layers, chain, M, S", [(6, 3, 0, 16, 3), (3, 0, 4, 4, 1), (9, 2, 0, 4, 1), (4, 0, 130, 8, 3),
+@pytest.mark.parametrize("n, layers, chain, M, S", [(6, 3, 0, 16, 3), (3, 0, 4, 4, 1), (9, 2, 0, 4, 1), (10, 2, 0, 32, 1), (4, 0, 130, 8, 3),
                                                     (9, 0, 130, 1, 1)])
 def test_routes_match_the_oracle(qfs, n, layers, chain, M, S):
     pairs = w.brick_pairs(n, layers) if layers else w.chain_pairs(n, chain)
